@@ -22,6 +22,7 @@ struct small_ctx {
     unsigned wait_iters;     // limit (polls) of every bounded device-side wait; small_set_wait_limit
     void *tc_cache;          // finished launches of the tensor-core kernel by (shape, mode, tensors); conv_tc.cu
     void *mma_cache;         // the same for the warp-level tensor-core kernel; conv_mma.cu
+    void *i8_cache;          // the same for the quantised convolution; conv_i8.cu
     void *static_workspace;  // device address of the library's built-in workspace array on this device (net_static.cu)
     int branch_overlap;      // small_run_net runs independent neighbouring layers side by side (side stream)
     void *side_stream, *ev_fork, *ev_join;   // cudaStream_t / cudaEvent_t of that
@@ -95,6 +96,7 @@ int make_geom(Geom &g, int N, int C, int K, int H, int W, int FH, int FW, int S,
 
 void free_tc_cache(small_ctx *);             // conv_tc.cu
 void free_mma_cache(small_ctx *);            // conv_mma.cu
+void free_i8_cache(small_ctx *);             // conv_i8.cu
 int resolve_static_workspace(small_ctx *);   // net_static.cu; called by small_init with the context's device current
 
 // ---- kernel launchers (each in its own .cu); all return a small_status ----
@@ -150,6 +152,10 @@ int launch_conv_tc(small_ctx *, const float *in, const float *w_hi, const float 
 bool conv_mma_supported(const Geom &, bool x3);
 int launch_conv_mma(small_ctx *, const float *in, const float *w_hi, const float *w_lo, const float *bias, float *out,
                     const Geom &, bool relu, bool accumulate, unsigned mode, cudaStream_t);
+// quantised full channel reduction (conv_i8.cu): windows 1 or 3 wide, strides 1 and 2; w: [CB][FH*FW][KB*32][32] bytes,
+// w_sums: [K][FH*FW] sums of weight bytes over the channels
+int launch_q_conv(small_ctx *, const uint8_t *in, const uint8_t *w, const int *w_sums, const int *bias, uint8_t *out, const Geom &,
+                  bool relu, int zx, int zw, int zo, int mult, int shift, cudaStream_t);
 // tensor-core filter sections of a group convolution: [F_C/32][FH*FW][G*K][32 ci], TF32 part and residual
 size_t group_conv_w_tc_elems(int F_C, int K, int G, int FH, int FW);
 int launch_pack_group_conv_weights_tc(small_ctx *, const float *w, float *hi, float *lo, int F_C, int K, int G, int FH, int FW, cudaStream_t);

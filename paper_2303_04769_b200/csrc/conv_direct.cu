@@ -20,8 +20,6 @@
 // differ in the low three bits.
 #include <cuda.h>
 
-#include <type_traits>
-
 #include "common.cuh"
 #include "sm100.cuh"
 
@@ -36,12 +34,9 @@ constexpr int kMaxThreads = 256;
 constexpr int kMaxRegs = 168;     // 12 resident warps per SM
 
 struct DirectArgs {
-    const void *bias; void *out; int *status;     // float (quantised form: int32 bias, uint8 output)
+    const float *bias; float *out; int *status;
     int N, C, K, OH, OW, CB, KB, FH, pt, pl;
-    int H, W;                   // input plane (the quantised epilogue needs the taps that fall inside it)
-    const int *q_tab;           // quantised form: per filter and tap the sum of its weight bytes [K][T], then per filter [K]
-    int zx, zw, zo, mult, shift;   // quantised form: zero points of input, weights and output; requantisation multiplier / 2^shift
-    int cpb;                    // stages per 32-channel block (32 / cch; the quantised form takes a whole block per stage)
+    int cpb;                    // stages per 32-channel block (32 / cch)
     int gw, gw_shift;           // column groups (of 8 pixels) of a unit: 1, 2 or 4
     int TH, NI;                 // output rows per image in a unit, images per unit
     int bands, tiles_w, units;  // row bands per image, column tiles per row, all units of the layer
@@ -56,20 +51,14 @@ struct DirectArgs {
     int span, Kg, S_C;          // group convolution: channel blocks a filter block reads, filters per group, channel step
     int relu, accumulate;
     uint32_t wait_iters;        // limit of the bounded waits (polls)
-    int pool;                   // fused 2 x 2 stride-2 max pool behind the layer (float form): out is [N][K][OH/2][OW/2]
+    int pool;                   // fused 2 x 2 stride-2 max pool behind the layer: out is [N][K][OH/2][OW/2]
 };
 
 __device__ __forceinline__ void lds128(uint32_t addr, uint32_t *v) {
     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr));
 }
 
-// Q: the quantised form of the same loop nest (Section 5.5).  A pixel of a channel block is 32 bytes = 8 words of 4
-// channels, so the shared-memory geometry is that of the float form with 8 channels per stage; a word of the input
-// meets a word of 4 channel bytes of a filter in one 4-way dot product with 32-bit accumulation (dp4a) instead of an
-// FMA.  Accumulated are the raw sums of byte products and, per pixel, the sum of the input bytes; the zero points enter
-// in the STORE phase:  sum (x - zx)(w - zw) = sum x w - zw sum x - zx sum_{taps inside the plane} w + taps C zx zw,
-// where pixels outside the plane (TMA's zero fill) take no part, which makes them real zeros.
-template <int FW, int S, bool Q>
+template <int FW, int S>
 __global__ void __maxnreg__(kMaxRegs)
 conv_direct_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ CUtensorMap map_w, const DirectArgs a) {
     constexpr int PXH = S == 1 ? 8 : 4;           // pixels per pass over the registers (stride 2: two passes of 4)
@@ -107,7 +96,7 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_cons
     const int blocks = min(a.span, a.CB - cb0);
     const int cpb = a.cpb;
     const int last_n = min(32, a.C - (cb0 + blocks - 1) * 32);
-    const int n_chunks = Q ? blocks : (blocks - 1) * cpb + (last_n + a.cch - 1) / a.cch;
+    const int n_chunks = (blocks - 1) * cpb + (last_n + a.cch - 1) / a.cch;
 
     auto issue = [&](int q, int s) {       // one thread: arm the stage's barrier, start its copies
         const int cbj = q / cpb, c0 = (q - cbj * cpb) * a.cch;
@@ -132,15 +121,11 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_cons
     if (threadIdx.x == 0)
         for (int q = 0; q < a.stages - 1 && q < n_chunks; ++q) issue(q, q);
 
-    typedef typename std::conditional<Q, uint32_t, float>::type AccT;
-    AccT acc[kPW][kKQ];
-    uint32_t sx[Q ? kPW : 1];                     // quantised form: sum of the input bytes each pixel's window has seen
+    float acc[kPW][kKQ];
 #pragma unroll
-    for (int p = 0; p < kPW; ++p) {
-        if (Q) sx[Q ? p : 0] = 0u;
+    for (int p = 0; p < kPW; ++p)
 #pragma unroll
-        for (int k = 0; k < kKQ; ++k) acc[p][k] = AccT(0);
-    }
+        for (int k = 0; k < kKQ; ++k) acc[p][k] = 0.0f;
 
     // idle lanes read the box's first run: in bounds, never stored
     const int p_base = img < a.NI ? (img * a.th_in + row * S) * a.cols_box + g * kPW * S : 0;
@@ -162,9 +147,7 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_cons
         __syncwarp();
         if (ok) {
             const int cbj = q / cpb, c0 = (q - cbj * cpb) * a.cch;
-            // 16-byte chunks of a pixel that hold real channels: 4 floats, or 16 channel bytes, each
-            const int lanes_n = min(32, a.C - (cb0 + cbj) * 32);
-            const int c4_n = Q ? (lanes_n + 15) >> 4 : (min(a.cch, lanes_n - c0) + 3) >> 2;
+            const int c4_n = (min(a.cch, min(32, a.C - (cb0 + cbj) * 32) - c0) + 3) >> 2;     // 4-channel chunks that hold real channels
             const uint32_t in_u = base + s * a.stage_bytes + pw * a.unit_bytes;       // shared-window addresses
             const uint32_t w_s = base + s * a.stage_bytes + w_off;
             for (int x = 0; x < a.FH; ++x) {
@@ -193,16 +176,9 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_cons
                                 lds128(wa + 16, &w[4]);
 #pragma unroll
                                 for (int p = 0; p < PXH; ++p) {
-                                    const uint32_t xv = v[(p * S + y) * 4 + cc];
-                                    AccT *ac = acc[pass * PXH + p];
-                                    if (Q) {
-                                        sx[Q ? pass * PXH + p : 0] = __dp4a(xv, 0x01010101u, sx[Q ? pass * PXH + p : 0]);
+                                    const float xv = __uint_as_float(v[(p * S + y) * 4 + cc]);
 #pragma unroll
-                                        for (int k = 0; k < kKQ; ++k) ac[k] = (AccT)__dp4a(xv, w[k], (uint32_t)ac[k]);
-                                    } else {
-#pragma unroll
-                                        for (int k = 0; k < kKQ; ++k) ac[k] = (AccT)fmaf(__uint_as_float(xv), __uint_as_float(w[k]), (float)ac[k]);
-                                    }
+                                    for (int k = 0; k < kKQ; ++k) acc[pass * PXH + p][k] = fmaf(xv, __uint_as_float(w[k]), acc[pass * PXH + p][k]);
                                 }
                             }
                         }
@@ -227,25 +203,24 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_cons
     if (kb >= a.KB) return;                       // the same for a whole warp
     const int n = n0 + img, oh = oh0 + row;
     const bool last_group = kq0 + kKQ == a.k_tiles * a.KT;
-    if (!Q && a.pool) {
+    if (a.pool) {
         // Abstract fused layer (Section 6): the 2 x 2 stride-2 max pool behind the convolution is taken in the STORE
         // phase.  A thread holds 8 adjacent columns of one row: column pairs are reduced in its registers; rows 2i and
         // 2i + 1 sit in neighbouring lanes (a unit has an even number of rows per image), so the row pair is one
         // shuffle; the even row's lane stores 4 pooled pixels.  All lanes take part in the shuffles.
-        const float *bias = static_cast<const float *>(a.bias);
         float bv[kKQ];
 #pragma unroll
-        for (int k = 0; k < kKQ; ++k) bv[k] = (bias && kq0 + k < a.K) ? bias[kq0 + k] : 0.0f;
+        for (int k = 0; k < kKQ; ++k) bv[k] = (a.bias && kq0 + k < a.K) ? a.bias[kq0 + k] : 0.0f;
         const int PH = a.OH >> 1, PW = a.OW >> 1;
         const int prow = oh >> 1, pcol0 = (ow0 + g * kPW) >> 1;
         const bool store_lane = valid && !(oh & 1) && prow < PH;
-        float *dst = static_cast<float *>(a.out) + ((((size_t)(valid ? n : 0) * a.KB + kb) * PH + (store_lane ? prow : 0)) * PW + pcol0) * 32 + kl;
+        float *dst = a.out + ((((size_t)(valid ? n : 0) * a.KB + kb) * PH + (store_lane ? prow : 0)) * PW + pcol0) * 32 + kl;
 #pragma unroll
         for (int pp = 0; pp < kPW / 2; ++pp) {
             float m[kKQ];
 #pragma unroll
             for (int k = 0; k < kKQ; ++k) {
-                float r0 = (float)acc[2 * pp][k] + bv[k], r1 = (float)acc[2 * pp + 1][k] + bv[k];
+                float r0 = acc[2 * pp][k] + bv[k], r1 = acc[2 * pp + 1][k] + bv[k];
                 if (a.relu) { r0 = fmaxf(r0, 0.0f); r1 = fmaxf(r1, 0.0f); }
                 m[k] = fmaxf(r0, r1);
                 m[k] = fmaxf(m[k], __shfl_xor_sync(0xffffffffu, m[k], 1));
@@ -262,83 +237,35 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_cons
         return;
     }
     if (!valid) return;
-    if constexpr (Q) {
-        // zero points, bias, one requantisation (round half up of the 64-bit product), clamp, 8 bytes per pixel and thread
-        const int T = a.FH * FW;
-        const int *bias = static_cast<const int *>(a.bias);
-        int bv[kKQ], wall[kKQ];
+    // + bias, + the tensor already in `out` (accumulate), ReLU; 32 bytes per pixel and thread
+    float bv[kKQ];
 #pragma unroll
-        for (int k = 0; k < kKQ; ++k) {
-            const bool real = kq0 + k < a.K;
-            bv[k] = (bias && real) ? bias[kq0 + k] : 0;
-            wall[k] = real ? a.q_tab[a.K * T + kq0 + k] : 0;
+    for (int k = 0; k < kKQ; ++k) bv[k] = (a.bias && kq0 + k < a.K) ? a.bias[kq0 + k] : 0.0f;
+    float *dst = a.out + ((((size_t)n * a.KB + kb) * a.OH + oh) * a.OW + ow0 + g * kPW) * 32 + kl;
+#pragma unroll
+    for (int p = 0; p < kPW; ++p) {
+        if (ow0 + g * kPW + p >= a.OW) break;
+        float4 *d4 = reinterpret_cast<float4 *>(dst + p * 32);
+        float r[kKQ];
+#pragma unroll
+        for (int k = 0; k < kKQ; ++k) r[k] = acc[p][k] + bv[k];
+        if (a.accumulate) {
+            const float4 o0 = d4[0], o1 = d4[1];
+            r[0] += o0.x; r[1] += o0.y; r[2] += o0.z; r[3] += o0.w;
+            r[4] += o1.x; r[5] += o1.y; r[6] += o1.z; r[7] += o1.w;
         }
-        const int ih0 = oh * a.cs - a.pt;
-        const int x0 = max(0, -ih0), x1 = min(a.FH, a.H - ih0);
-        const int lo = a.relu ? a.zo : 0;
-        uint8_t *dst = static_cast<uint8_t *>(a.out) + ((((size_t)n * a.KB + kb) * a.OH + oh) * a.OW + ow0 + g * kPW) * 32 + kl;
+        if (a.relu) {
 #pragma unroll
-        for (int p = 0; p < kPW; ++p) {
-            const int ow = ow0 + g * kPW + p;
-            if (ow >= a.OW) break;
-            const int iw0 = ow * a.cs - a.pl;
-            const int y0 = max(0, -iw0), y1 = min(FW, a.W - iw0);
-            const int nv = (x1 - x0) * (y1 - y0);                 // taps of this pixel's window that lie inside the plane
-            uint32_t packed[2] = {0u, 0u};
-#pragma unroll
-            for (int k = 0; k < kKQ; ++k) {
-                int q = 0;
-                if (kq0 + k < a.K) {
-                    int sw = wall[k];
-                    if (nv != T) {                                // a border pixel: only the taps inside count
-                        sw = 0;
-                        for (int x = x0; x < x1; ++x)
-                            for (int y = y0; y < y1; ++y) sw += a.q_tab[(kq0 + k) * T + x * FW + y];
-                    }
-                    const long long t = (long long)acc[p][k] - (long long)a.zw * (long long)sx[Q ? p : 0] - (long long)a.zx * sw +
-                                        (long long)nv * a.C * a.zx * a.zw + bv[k];
-                    const long long r = (t * (long long)a.mult + (1ll << (a.shift - 1))) >> a.shift;
-                    const long long z = (long long)a.zo + r;
-                    q = (int)(z < lo ? lo : z > 255 ? 255 : z);
-                }
-                packed[k >> 2] |= (uint32_t)q << (8 * (k & 3));
-            }
-            *reinterpret_cast<uint2 *>(dst + p * 32) = make_uint2(packed[0], packed[1]);
-            if (last_group)
-                for (int z = kl + kKQ; z < 32; z += 8) *reinterpret_cast<uint2 *>(dst + p * 32 - kl + z) = make_uint2(0u, 0u);
+            for (int k = 0; k < kKQ; ++k) r[k] = fmaxf(r[k], 0.0f);
         }
-    } else {
-        // + bias, + the tensor already in `out` (accumulate), ReLU; 32 bytes per pixel and thread
-        const float *bias = static_cast<const float *>(a.bias);
-        float bv[kKQ];
+        if (kq0 + kKQ > a.K) {
 #pragma unroll
-        for (int k = 0; k < kKQ; ++k) bv[k] = (bias && kq0 + k < a.K) ? bias[kq0 + k] : 0.0f;
-        float *dst = static_cast<float *>(a.out) + ((((size_t)n * a.KB + kb) * a.OH + oh) * a.OW + ow0 + g * kPW) * 32 + kl;
-#pragma unroll
-        for (int p = 0; p < kPW; ++p) {
-            if (ow0 + g * kPW + p >= a.OW) break;
-            float4 *d4 = reinterpret_cast<float4 *>(dst + p * 32);
-            float r[kKQ];
-#pragma unroll
-            for (int k = 0; k < kKQ; ++k) r[k] = (float)acc[p][k] + bv[k];
-            if (a.accumulate) {
-                const float4 o0 = d4[0], o1 = d4[1];
-                r[0] += o0.x; r[1] += o0.y; r[2] += o0.z; r[3] += o0.w;
-                r[4] += o1.x; r[5] += o1.y; r[6] += o1.z; r[7] += o1.w;
-            }
-            if (a.relu) {
-#pragma unroll
-                for (int k = 0; k < kKQ; ++k) r[k] = fmaxf(r[k], 0.0f);
-            }
-            if (kq0 + kKQ > a.K) {
-#pragma unroll
-                for (int k = 0; k < kKQ; ++k) if (kq0 + k >= a.K) r[k] = 0.0f;
-            }
-            d4[0] = make_float4(r[0], r[1], r[2], r[3]);
-            d4[1] = make_float4(r[4], r[5], r[6], r[7]);
-            if (last_group)
-                for (int z = kl + kKQ; z < 32; z += 4) *reinterpret_cast<float4 *>(dst + p * 32 - kl + z) = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int k = 0; k < kKQ; ++k) if (kq0 + k >= a.K) r[k] = 0.0f;
         }
+        d4[0] = make_float4(r[0], r[1], r[2], r[3]);
+        d4[1] = make_float4(r[4], r[5], r[6], r[7]);
+        if (last_group)
+            for (int z = kl + kKQ; z < 32; z += 4) *reinterpret_cast<float4 *>(dst + p * 32 - kl + z) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
 
@@ -349,13 +276,12 @@ size_t round1k(size_t b) { return (b + 1023) & ~(size_t)1023; }
 // Tile shapes.  The unit of a row warp follows from the plane's width; what is chosen is the number of channels per
 // stage (8 or 16) and of units per block: the smallest blocks (finest work granularity over the SMs) that still keep
 // 12 or more warps resident per SM within shared memory.
-DirectPlan plan_direct(const Geom &g, int span, int Kg, int S_C, size_t max_smem, bool quant = false, bool pool = false) {
+DirectPlan plan_direct(const Geom &g, int span, int Kg, int S_C, size_t max_smem, bool pool = false) {
     DirectPlan best{};
     best.ok = false;
     if ((g.FW != 1 && g.FW != 3) || (g.S != 1 && g.S != 2) || g.FH * g.FW > 256) return best;
     DirectArgs a{};
     a.N = g.N; a.C = g.C; a.K = g.K; a.OH = g.OH; a.OW = g.OW; a.CB = g.CB; a.KB = g.KB; a.FH = g.FH; a.pt = g.pt; a.pl = g.pl;
-    a.H = g.H; a.W = g.W;
     a.span = span > 0 ? span : g.CB; a.Kg = span > 0 ? Kg : 0; a.S_C = S_C;
     a.gw = g.OW <= 8 ? 1 : g.OW <= 16 ? 2 : 4;
     a.gw_shift = a.gw == 1 ? 0 : a.gw == 2 ? 1 : 2;
@@ -363,7 +289,7 @@ DirectPlan plan_direct(const Geom &g, int span, int Kg, int S_C, size_t max_smem
     const int rows_u = 32 / a.gw;
     if (g.OH <= rows_u) { a.TH = g.OH; a.NI = rows_u / g.OH; a.bands = 1; if (a.NI > g.N) a.NI = g.N; }
     else { a.TH = rows_u; a.NI = 1; a.bands = ceil_div(g.OH, rows_u); }
-    if (pool && ((a.TH & 1) || g.OH < 2 || g.OW < 2 || quant || span > 0)) return best;   // row pairs must share a unit
+    if (pool && ((a.TH & 1) || g.OH < 2 || g.OW < 2 || span > 0)) return best;   // row pairs must share a unit
     a.pool = pool ? 1 : 0;
     const long long units = (long long)ceil_div(g.N, a.NI) * a.bands * a.tiles_w;
     if (units > 0x3fffffffLL) return best;
@@ -380,13 +306,12 @@ DirectPlan plan_direct(const Geom &g, int span, int Kg, int S_C, size_t max_smem
     const int T = g.FH * g.FW;
     const int last_n = g.C - (g.CB - 1) * 32;
     int best_warps = 0;
-    // (the quantised form has one geometry: a stage is a whole 32-channel block, 8 words of 4 channel bytes per pixel)
-    for (int cch = quant ? 8 : 16; cch >= 8; cch -= 8) {
-        const int n_chunks = quant ? g.CB : ((span > 0 ? span : g.CB) - 1) * (32 / cch) + ceil_div(last_n, cch);
+    for (int cch = 16; cch >= 8; cch -= 8) {
+        const int n_chunks = ((span > 0 ? span : g.CB) - 1) * (32 / cch) + ceil_div(last_n, cch);
         for (int pwarps = 1; pwarps * kwarps * 32 <= kMaxThreads; ++pwarps) {
             if (pwarps * kwarps < 2) continue;
             DirectArgs c = a;
-            c.cch = cch; c.pwarps = pwarps; c.cpb = quant ? 1 : 32 / cch;
+            c.cch = cch; c.pwarps = pwarps; c.cpb = 32 / cch;
             c.sw_shift = cch == 16 ? 1 : 2; c.sw_mask = cch == 16 ? 3 : 1;
             c.in_box_bytes = (uint32_t)((size_t)a.NI * a.th_in * a.cols_box * cch * 4);
             c.unit_bytes = (uint32_t)round1k(c.in_box_bytes);
@@ -428,22 +353,20 @@ long long conv_direct_blocks(const Geom &g) {
 
 namespace {
 
-// Tensor maps and launch shared by the float and the quantised form.  esize: bytes per channel of the activation
-// tensor (4 or 1); the filter tensor is [KB][span][FH*FW][32][32] 4-byte words in both forms (floats [ci][ko], or
-// words of 4 channel bytes [c4][ko] in the first 8 of the 32 rows' worth - see pack_q_conv_w_kernel).
-int launch_direct(small_ctx *ctx, DirectPlan &p, const Geom &g, const void *in, const void *w, bool quant, cudaStream_t st) {
+// Tensor maps and launch; the packed filters are [KB][span][FH*FW][32 ci][32 ko].
+int launch_direct(small_ctx *ctx, DirectPlan &p, const Geom &g, const float *in, const float *w, cudaStream_t st) {
     DirectArgs &a = p.a;
     a.wait_iters = ctx->wait_iters;
     EncodeTiledFn encode = reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled);
     CUtensorMap map_in, map_w;
     {   // activations [N][CB][H][W][32]: box = one stage's channels x cols_box x th_in x 1 block x NI images, swizzled
-        const cuuint64_t px = quant ? 32 : 128;      // bytes per pixel and channel block
+        const cuuint64_t px = 128;                   // bytes per pixel and channel block
         cuuint64_t dims[5] = {32, (cuuint64_t)g.W, (cuuint64_t)g.H, (cuuint64_t)g.CB, (cuuint64_t)g.N};
         cuuint64_t strides[4] = {px, (cuuint64_t)g.W * px, (cuuint64_t)g.H * g.W * px, (cuuint64_t)g.CB * g.H * g.W * px};
         const cuuint32_t es = (cuuint32_t)a.es;     // element stride 2: a box of 2 cols x 2 rows elements lands as cols x rows pixels
-        cuuint32_t box[5] = {(cuuint32_t)(quant ? 32 : a.cch), (cuuint32_t)a.cols_box * es, (cuuint32_t)a.th_in * es, 1, (cuuint32_t)a.NI};
+        cuuint32_t box[5] = {(cuuint32_t)a.cch, (cuuint32_t)a.cols_box * es, (cuuint32_t)a.th_in * es, 1, (cuuint32_t)a.NI};
         cuuint32_t estr[5] = {1, es, es, 1, 1};
-        CUresult r = encode(&map_in, quant ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<void *>(in), dims,
+        CUresult r = encode(&map_in, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<float *>(in), dims,
                             strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                             a.cch == 16 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -451,22 +374,19 @@ int launch_direct(small_ctx *ctx, DirectPlan &p, const Geom &g, const void *in, 
     }
     {   // packed filters: box = up to 32 filters x one stage's channel rows x all taps
         const int T = g.FH * g.FW;
-        const cuuint64_t rows = quant ? 8 : 32;      // words per filter, tap and channel block
+        const cuuint64_t rows = 32;                  // channels per tap and channel block
         cuuint64_t dims[4] = {32, rows, (cuuint64_t)T, (cuuint64_t)g.KB * a.span};
         cuuint64_t strides[3] = {128, rows * 128, (cuuint64_t)T * rows * 128};
         cuuint32_t box[4] = {(cuuint32_t)(a.KT < 32 ? a.KT : 32), (cuuint32_t)a.cch, (cuuint32_t)T, 1};
         cuuint32_t estr[4] = {1, 1, 1, 1};
-        CUresult r = encode(&map_w, quant ? CU_TENSOR_MAP_DATA_TYPE_INT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void *>(w), dims,
+        CUresult r = encode(&map_w, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float *>(w), dims,
                             strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) { ctx->last_cuda = (int)r; return SMALL_ERR_CUDA; }
     }
     const int S = g.S / a.es;
     void (*kern)(const CUtensorMap, const CUtensorMap, const DirectArgs);
-    if (quant) kern = g.FW == 1 ? (S == 1 ? conv_direct_kernel<1, 1, true> : conv_direct_kernel<1, 2, true>)
-                                : (S == 1 ? conv_direct_kernel<3, 1, true> : conv_direct_kernel<3, 2, true>);
-    else kern = g.FW == 1 ? (S == 1 ? conv_direct_kernel<1, 1, false> : conv_direct_kernel<1, 2, false>)
-                          : (S == 1 ? conv_direct_kernel<3, 1, false> : conv_direct_kernel<3, 2, false>);
+    kern = g.FW == 1 ? (S == 1 ? conv_direct_kernel<1, 1> : conv_direct_kernel<1, 2>) : (S == 1 ? conv_direct_kernel<3, 1> : conv_direct_kernel<3, 2>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SMALL_ERR_CUDA; }
@@ -486,30 +406,18 @@ int launch_conv_direct(small_ctx *ctx, const float *in, const float *w, const fl
     if (!p.ok) return SMALL_ERR_UNSUPPORTED;
     DirectArgs &a = p.a;
     a.bias = bias; a.out = out; a.status = ctx->dev_status; a.relu = relu; a.accumulate = accumulate;
-    return launch_direct(ctx, p, g, in, w, false, st);
+    return launch_direct(ctx, p, g, in, w, st);
 }
 
-bool conv_direct_pool_supported(const Geom &g) { return plan_direct(g, 0, 0, 0, 227 * 1024, false, true).ok; }
+bool conv_direct_pool_supported(const Geom &g) { return plan_direct(g, 0, 0, 0, 227 * 1024, true).ok; }
 
 int launch_conv_direct_pool(small_ctx *ctx, const float *in, const float *w, const float *bias, float *out, const Geom &g,
                             bool relu, cudaStream_t st) {
-    DirectPlan p = plan_direct(g, 0, 0, 0, ctx->max_smem_optin, false, true);
-    if (!p.ok) return SMALL_ERR_UNSUPPORTED;
-    DirectArgs &a = p.a;
-    a.bias = bias; a.out = out; a.status = ctx->dev_status; a.relu = relu; a.accumulate = 0;
-    return launch_direct(ctx, p, g, in, w, false, st);
-}
-
-bool q_conv_supported(const Geom &g) { return plan_direct(g, 0, 0, 0, 227 * 1024, true).ok; }
-
-int launch_q_conv(small_ctx *ctx, const uint8_t *in, const uint32_t *w_words, const int *tables, const int *bias, uint8_t *out,
-                  const Geom &g, bool relu, int zx, int zw, int zo, int mult, int shift, cudaStream_t st) {
     DirectPlan p = plan_direct(g, 0, 0, 0, ctx->max_smem_optin, true);
     if (!p.ok) return SMALL_ERR_UNSUPPORTED;
     DirectArgs &a = p.a;
     a.bias = bias; a.out = out; a.status = ctx->dev_status; a.relu = relu; a.accumulate = 0;
-    a.q_tab = tables; a.zx = zx; a.zw = zw; a.zo = zo; a.mult = mult; a.shift = shift;
-    return launch_direct(ctx, p, g, in, w_words, true, st);
+    return launch_direct(ctx, p, g, in, w, st);
 }
 
 }  // namespace small

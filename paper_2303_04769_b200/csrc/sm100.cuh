@@ -66,6 +66,12 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map
         ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
 }
 
+// Untiled copy of contiguous bytes (addresses and size multiples of 16).
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -90,6 +96,23 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
     int ok = 1;
     if ((threadIdx.x & 31) == 0) ok = mbar_wait<kFast>(bar, parity, abort_flag, status, limit) ? 1 : 0;
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+
+// Roles of one thread (TMA producers, MMA issuers) run as whole warps whose single thread is picked by elect.sync at the
+// instruction itself.  Written as `if (lane == 0) { ... }` around the role, every MMA and copy costs the thread a trip
+// through code that moves its operands to uniform registers for a warp the compiler has to take as divergent: measured 52
+// cycles per MMA at best and 140 to 280 in loops with run-time trip counts; as a uniform warp the pipe's own (128 + N) / 4
+// cycles per 128 x N MMA of 32-byte rows for N <= 128 (40 at N = 32, 48 at N = 64).
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+// Bounded wait of a whole warp, every lane polling; the answer is the same for all lanes.
+template <uint32_t kFast = 64>
+__device__ __forceinline__ bool mbar_wait_uniform(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status, uint32_t limit) {
+    return __all_sync(0xffffffffu, mbar_wait<kFast>(bar, parity, abort_flag, status, limit));
 }
 
 __device__ __forceinline__ void tmem_alloc(uint32_t smem_dst, uint32_t cols) {
