@@ -62,7 +62,7 @@ constexpr int kMaxAStages = 6;         // input strips in flight (at least 2; as
 constexpr int kMaxBStages = 8;
 constexpr int kRawStages = 2;           // fused depthwise: halo tiles in flight
 constexpr int kCtrlBarrierBytes = 24 * kMaxAStages + 16 * kMaxBStages + 16 * kSlots + 16 * kRawStages;   // all mbarriers
-constexpr int kTapTabEntries = 4 * 64;   // original tap of every (phase plane, view tap), -1 where the view tap has none
+constexpr int kMaxTaps = 256;            // taps of the layer's window
 
 struct TcPlan {
     int OH, OW, Wq, Hq;
@@ -94,8 +94,8 @@ struct TcPlan {
 
 struct TcArgs {
     const float *bias; float *out; int *status;
-    int N, K, KB, CB, OH, OW, Wq, Hq, FH, FW, pt, pl;   // CB, FH, FW, pt, pl: the stride-1 view (see Virt)
-    int S, n_phase, CBr, phase_bits, FHo, FWo, pto, plo;  // stride, phase planes, real channel blocks, original window
+    int N, K, KB, CB, OH, OW, Wq, Hq, pt, pl;   // CB, pt, pl: the stride-1 view (see Virt)
+    int S, n_phase, CBr, phase_bits;   // stride, phase planes, real channel blocks
     int nn, px_tile, px_img, tiles_img, m_tiles, n_tiles, strip_px, tail_px, w_rows;
     int a_stages, b_stages, pixel_m, w_tile, cps, b_resident, ks_last;
     int rows_tile;       // whole rows per tile when every tile starts at a row start, else 0
@@ -110,10 +110,14 @@ struct TcArgs {
     uint32_t raw_stage_bytes, raw_box_bytes;
     int x_packed;              // 3xTF32, at most 16 channels: the residual sits in the unused lanes of the same row
     int x3_wide;               // 3xTF32, pixels on M: x_hi meets [w_hi; w_lo] in one MMA of twice the filters (see the issue loop)
-    int alt_tiles;             // one chain per tile: the two MMA threads take alternate tiles (else warp 1 issues everything)
     uint32_t x_lo_off;         // 3xTF32: 16-byte units from a strip's TF32 part to its residual
     int relu, accumulate;
     uint32_t wait_iters;       // limit of every bounded wait (polls)
+    // the layer's taps sorted by phase plane: strip offset (16-byte units: 8 per pixel), original tap; phase p holds the
+    // entries phase_at[p] .. phase_at[p + 1] - 1
+    int phase_at[5];
+    uint16_t tap_off[kMaxTaps];
+    uint8_t tap_id[kMaxTaps];
 };
 
 // ---------------------------------------------------------------------------------------------- kernel
@@ -146,10 +150,8 @@ __device__ __forceinline__ Tile decode_tile(const TcArgs &a, int t) {
 }
 
 // CH: MMA chains per tile (accumulator slots with filters on M, 128-pixel chunks with pixels on M); KS_LAST: K steps
-// of the last channel block that hold real channels (1, 2 or 4); PM: pixels on the MMA's M axis;
-// MASKED: some view taps do not exist (stride-2 layers).  They are template
-// parameters so that the single issuing thread runs straight-line code: with run-time chain and K-step counts every
-// MMA costs it about 100 cycles of branches and selects, more than a small MMA occupies the pipe (measured).
+// of the last channel block that hold real channels (1, 2 or 4); PM: pixels on the MMA's M axis.  They are template
+// parameters so that the issuing warp runs straight-line code between waits.
 // X3: 3xTF32.  Every FP32 operand is split into its TF32 part and the residual (x = x_hi + x_lo, w = w_hi + w_lo) and
 // each K step issues x_lo*w_hi, x_hi*w_lo and x_hi*w_hi into the same FP32 accumulator (x_lo*w_lo is below FP32
 // resolution).  Filters arrive split (packed so); the activations are split in shared memory by four extra warps as
@@ -157,10 +159,10 @@ __device__ __forceinline__ Tile decode_tile(const TcArgs &a, int t) {
 // DW: a depthwise 3x3 (+ bias, ReLU) is computed in front of this 1x1 convolution: TMA loads halo tiles of the layer's
 // input, warps 8-11 compute the depthwise result straight into the strip the MMAs read (and split it for 3xTF32),
 // so the depthwise output never goes to global memory.
-template <int CH, int KS_LAST, bool PM, bool MASKED, bool X3, bool DW>
+template <int CH, int KS_LAST, bool PM, bool X3, bool DW>
 __global__ void __launch_bounds__(DW ? kThreadsDW : X3 ? kThreadsX3 : kThreads, 1)
 conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-               const __grid_constant__ CUtensorMap map_b_lo, const TcArgs a) {
+               const __grid_constant__ CUtensorMap map_b_lo, const __grid_constant__ TcArgs a) {
     constexpr int kNT = DW ? kThreadsDW : X3 ? kThreadsX3 : kThreads;
     constexpr int kXform = DW ? 256 : 128;     // threads that split (3xTF32) or compute (fused depthwise) the strips
     extern __shared__ uint8_t smem_raw[];
@@ -182,28 +184,16 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(ctrl_ptr + kCtrlBarrierBytes);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(ctrl_ptr + kCtrlBarrierBytes + 4);
     float *bias_s = reinterpret_cast<float *>(ctrl_ptr + kCtrlBarrierBytes + 16);
-    volatile short *tap_tab = reinterpret_cast<volatile short *>(ctrl_ptr + kCtrlBarrierBytes + 16 + (size_t)a.KB * 32 * 4);
-    float *dw_s_w = reinterpret_cast<float *>(ctrl_ptr + kCtrlBarrierBytes + 16 + (size_t)a.KB * 32 * 4 + kTapTabEntries * sizeof(short));   // [CB][10][32]: 9 taps + bias
+    float *dw_s_w = reinterpret_cast<float *>(ctrl_ptr + kCtrlBarrierBytes + 16 + (size_t)a.KB * 32 * 4);   // [CB][10][32]: 9 taps + bias
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // Two issuing threads (warps 1 and 3, on different schedulers): issuing a small MMA costs a thread about twice the
-    // cycles the pipe needs to run it.  A tile's MMA chains are split between them; an odd number of chains is split the
-    // other way round on odd tiles (chains [0, kSplit) and [kSplit, CH) on even tiles, [0, CH - kSplit) and the rest on
-    // odd ones), so that both issue the same number of MMAs over two tiles.  With one chain per tile the two threads take
-    // alternate tiles where the MMAs are small enough to be issue-bound (alt_tiles; measured: the 32 -> 32 layer of the
-    // residual CNN 32.4 -> 26.6 us in 3xTF32; the host side leaves it off today, see there), else warp 1 issues alone: a second thread that only walks the barriers
-    // cost the TF32 step 6 us.  Both threads walk every tile and every barrier; only the chains they issue for differ.
-    // (TF32 kernels keep the fixed split and the single thread: alternating measured 7 us slower per step there.)
-    const int kIssuers = (CH >= 2 || (X3 && a.alt_tiles)) ? 2 : 1;
-    constexpr int kSplit = (CH + 1) / 2, kOddSplit = X3 ? CH - kSplit : kSplit;      // chains of warp 1 on even / odd tiles
-    const int T = a.FH * a.FW;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int total_tiles = a.m_tiles * a.n_tiles;
 
     if (threadIdx.x == 0) {
-        // every MMA issuer commits to the stage-empty and slot-full barriers; 4 epilogue warps free a slot
-        for (int s = 0; s < kAStages; ++s) { mbar_init(bar_a_full + 8 * s, 1); mbar_init(bar_a_empty + 8 * s, kIssuers); mbar_init(bar_a_split + 8 * s, kXform); }
-        for (int s = 0; s < a.b_stages; ++s) { mbar_init(bar_b_full + 8 * s, 1); mbar_init(bar_b_empty + 8 * s, kIssuers); }
-        for (int s = 0; s < kSlots; ++s) { mbar_init(bar_slot_full + 8 * s, kIssuers); mbar_init(bar_slot_free + 8 * s, 4); }
+        // the MMA warp commits to the stage-empty and slot-full barriers; 4 epilogue warps free a slot
+        for (int s = 0; s < kAStages; ++s) { mbar_init(bar_a_full + 8 * s, 1); mbar_init(bar_a_empty + 8 * s, 1); mbar_init(bar_a_split + 8 * s, kXform); }
+        for (int s = 0; s < a.b_stages; ++s) { mbar_init(bar_b_full + 8 * s, 1); mbar_init(bar_b_empty + 8 * s, 1); }
+        for (int s = 0; s < kSlots; ++s) { mbar_init(bar_slot_full + 8 * s, 1); mbar_init(bar_slot_free + 8 * s, 4); }
         for (int s = 0; s < kRawStages; ++s) { mbar_init(bar_raw_full + 8 * s, 1); mbar_init(bar_raw_empty + 8 * s, kXform); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -228,13 +218,6 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             const int cb = i / 320, rest = i - cb * 320, tap = rest >> 5, c = rest & 31;
             dw_s_w[i] = tap < 9 ? a.dw_w[(cb * 9 + tap) * 32 + c] : (a.dw_bias && cb * 32 + c < a.dw_C ? a.dw_bias[cb * 32 + c] : 0.0f);
         }
-    // view tap (x', y') of phase plane (ph, pw) is the original tap x = S (x' - pt') + ph + pt, y likewise, if it exists
-    for (int i = threadIdx.x; i < a.n_phase * T; i += kNT) {
-        const int p = i / T, tv = i - p * T, xv = tv / a.FW, yv = tv - xv * a.FW;
-        const int x = a.S * (xv - a.pt) + ((a.phase_bits >> (2 * p)) & 1) + a.pto;
-        const int y = a.S * (yv - a.pl) + ((a.phase_bits >> (2 * p + 1)) & 1) + a.plo;
-        tap_tab[i] = (short)((x >= 0 && x < a.FHo && y >= 0 && y < a.FWo) ? x * a.FWo + y : -1);
-    }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy zeros visible to the tensor core
     if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t *>(tmem_slot)), (uint32_t)(kSlots * kSlotPx));
     tc_fence_before();
@@ -251,10 +234,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     uint32_t armed_mask = 0, armed_parity = 0;
     uint32_t drain_bar = 0;
 
-    // The three single-thread roles below keep their loops free of divisions: stage indices, phase bits and tap
-    // offsets advance incrementally, because every scalar instruction of the one issuing thread is a few cycles that
-    // the tensor pipe may have to wait for.
-    if (warp == 0 && lane == 0) {
+    // The three roles below are one thread's work done by a whole warp, the thread picked at each copy or MMA (see elect_one);
+    // stage indices, phase bits and tap offsets advance incrementally.
+    if (warp == 0) {
         // ---- input strips: one box per (tile, channel block)
         drain_bar = DW ? bar_raw_full : bar_a_full;
         bool alive = true, wrapped = false;
@@ -264,10 +246,12 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             for (int t = blockIdx.x; t < total_tiles && alive; t += gridDim.x) {
                 const Tile tl = decode_tile(a, t);
                 for (int cb = 0; cb < a.CBr; ++cb) {
-                    if (wrapped) alive = mbar_wait(bar_raw_empty + 8 * s, phase ^ 1u, abort_flag, a.status, a.wait_iters);
+                    if (wrapped) alive = mbar_wait_uniform<4>(bar_raw_empty + 8 * s, phase ^ 1u, abort_flag, a.status, a.wait_iters);
                     if (!alive) break;
-                    mbar_expect_tx(bar_raw_full + 8 * s, a.raw_box_bytes);
-                    tma_load_5d(raw_base + s * a.raw_stage_bytes, &map_a, bar_raw_full + 8 * s, 0, -a.dw_pl, tl.row0 * a.dw_s - a.dw_pt, cb, tl.n0);
+                    if (elect_one()) {
+                        mbar_expect_tx(bar_raw_full + 8 * s, a.raw_box_bytes);
+                        tma_load_5d(raw_base + s * a.raw_stage_bytes, &map_a, bar_raw_full + 8 * s, 0, -a.dw_pl, tl.row0 * a.dw_s - a.dw_pt, cb, tl.n0);
+                    }
                     armed_mask |= 1u << s;
                     armed_parity = (armed_parity & ~(1u << s)) | (phase << s);
                     if (++s == (uint32_t)kRawStages) { s = 0; phase ^= 1u; wrapped = true; }
@@ -282,34 +266,33 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             for (int p = 0; p < a.n_phase && alive; ++p) {
                 const int ph = (a.phase_bits >> (2 * p)) & 1, pw = (a.phase_bits >> (2 * p + 1)) & 1;
                 for (int cb = 0; cb < a.CBr; ++cb) {
-                    if (wrapped) alive = mbar_wait(bar_a_empty + 8 * s, phase ^ 1u, abort_flag, a.status, a.wait_iters);
+                    if (wrapped) alive = mbar_wait_uniform<4>(bar_a_empty + 8 * s, phase ^ 1u, abort_flag, a.status, a.wait_iters);
                     if (!alive) break;
-                    mbar_expect_tx(bar_a_full + 8 * s, a.a_box_bytes);
-                    tma_load_5d(a_base + s * a.a_stage_bytes, &map_a, bar_a_full + 8 * s, 0, c1 + pw, c2 + ph, cb + tl.n_tile * a.cb_group, tl.n0);
+                    if (elect_one()) {
+                        mbar_expect_tx(bar_a_full + 8 * s, a.a_box_bytes);
+                        tma_load_5d(a_base + s * a.a_stage_bytes, &map_a, bar_a_full + 8 * s, 0, c1 + pw, c2 + ph, cb + tl.n_tile * a.cb_group, tl.n0);
+                    }
                     armed_mask |= 1u << s;
                     armed_parity = (armed_parity & ~(1u << s)) | (phase << s);
                     if (++s == (uint32_t)kAStages) { s = 0; phase ^= 1u; wrapped = true; }
                 }
             }
         }
-    } else if (warp == 2 && lane == 0) {
-        // ---- filter tiles: w_rows x 128 bytes per (channel block, tap).  Resident: all of them once, on one barrier.
+    } else if (warp == 2) {
+        // ---- filter tiles: w_rows x 128 bytes per (phase plane, channel block, tap).  Resident: all of them once, on one barrier.
         drain_bar = bar_b_full;
         const uint32_t box_bytes = (uint32_t)a.w_rows * 128u;
         if (a.b_resident) {
-            int boxes = 0;
-            for (int i = 0; i < a.n_phase * T; ++i) boxes += tap_tab[i] >= 0 ? 1 : 0;
-            mbar_expect_tx(bar_b_full, box_bytes * (uint32_t)(boxes * a.CBr) * (X3 ? 2u : 1u));
-            uint32_t dst = b_base;
-            for (int p = 0; p < a.n_phase; ++p)
-                for (int cb = 0; cb < a.CBr; ++cb)
-                    for (int tap = 0; tap < T; ++tap, dst += kBStageBytes) {
-                        const int orig = tap_tab[p * T + tap];
-                        if (orig >= 0) {
-                            tma_load_4d(dst, &map_b, bar_b_full, 0, 0, orig, cb);
-                            if (X3) tma_load_4d(dst + a.b_half, &map_b_lo, bar_b_full, 0, 0, orig, cb);
+            if (elect_one()) {
+                mbar_expect_tx(bar_b_full, box_bytes * (uint32_t)(a.phase_at[a.n_phase] * a.CBr) * (X3 ? 2u : 1u));
+                uint32_t dst = b_base;
+                for (int p = 0; p < a.n_phase; ++p)
+                    for (int cb = 0; cb < a.CBr; ++cb)
+                        for (int i = a.phase_at[p]; i < a.phase_at[p + 1]; ++i, dst += kBStageBytes) {
+                            tma_load_4d(dst, &map_b, bar_b_full, 0, 0, a.tap_id[i], cb);
+                            if (X3) tma_load_4d(dst + a.b_half, &map_b_lo, bar_b_full, 0, 0, a.tap_id[i], cb);
                         }
-                    }
+            }
             armed_mask = 1u;
         } else {
             bool alive = true, wrapped = false;
@@ -318,31 +301,28 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 const int row = (t % a.n_tiles) * a.w_tile;
                 for (int p = 0; p < a.n_phase && alive; ++p)
                     for (int cb = 0; cb < a.CBr && alive; ++cb)
-                        for (int tap = 0; tap < T; ++tap) {
-                            const int orig = tap_tab[p * T + tap];
-                            if (orig < 0) continue;
-                            if (wrapped) alive = mbar_wait(bar_b_empty + 8 * s, phase ^ 1u, abort_flag, a.status, a.wait_iters);
+                        for (int i = a.phase_at[p]; i < a.phase_at[p + 1]; ++i) {
+                            if (wrapped) alive = mbar_wait_uniform<4>(bar_b_empty + 8 * s, phase ^ 1u, abort_flag, a.status, a.wait_iters);
                             if (!alive) break;
-                            mbar_expect_tx(bar_b_full + 8 * s, X3 ? 2u * box_bytes : box_bytes);
-                            tma_load_4d(b_base + s * kBStageBytes, &map_b, bar_b_full + 8 * s, 0, row, orig, cb);
-                            if (X3) tma_load_4d(b_base + s * kBStageBytes + a.b_half, &map_b_lo, bar_b_full + 8 * s, 0, row, orig, cb);
+                            if (elect_one()) {
+                                mbar_expect_tx(bar_b_full + 8 * s, X3 ? 2u * box_bytes : box_bytes);
+                                tma_load_4d(b_base + s * kBStageBytes, &map_b, bar_b_full + 8 * s, 0, row, a.tap_id[i], cb);
+                                if (X3) tma_load_4d(b_base + s * kBStageBytes + a.b_half, &map_b_lo, bar_b_full + 8 * s, 0, row, a.tap_id[i], cb);
+                            }
                             armed_mask |= 1u << s;
                             armed_parity = (armed_parity & ~(1u << s)) | (phase << s);
                             if (++s == (uint32_t)a.b_stages) { s = 0; phase ^= 1u; wrapped = true; }
                         }
             }
         }
-    } else if ((warp == 1 || (kIssuers == 2 && warp == 3)) && lane == 0) {
-        // ---- MMA issue: this thread's chains are [C0, C1)
-        auto mma_role = [&](auto c0_tag, auto c1_tag, auto d0_tag, auto d1_tag) {
-        constexpr int C0 = decltype(c0_tag)::value, C1 = decltype(c1_tag)::value;       // chains on even tiles
-        constexpr int D0 = decltype(d0_tag)::value, D1 = decltype(d1_tag)::value;       // chains on odd tiles
+    } else if (warp == 1) {
+        // ---- MMA issue
+        const uint32_t elected = elect_one();
         bool alive = true;
         uint32_t sa = 0, pa = 0, sb = 0, pb = 0;
         uint32_t slot_uses = 0;                   // slots taken so far; slot j of a tile is (slot_uses + j) % 2
         const uint32_t b_step = kBStageBytes >> 4;
         const uint32_t x_half = a.x_lo_off, w_half = a.b_half >> 4;
-        const uint32_t row_wrap = (uint32_t)(a.Wq - a.FW + 1) * 8u;     // tap offset step from the end of a window row
         // N of the MMA: pixels of a slot (filters on M), or the filters of the tile (pixels on M)
         const uint32_t idesc = instr_desc(PM ? a.w_rows : a.n_slot);
         const uint32_t idesc_wide = instr_desc(PM ? 2 * a.w_rows : a.n_slot);   // x3_wide: both filter halves on N
@@ -351,83 +331,74 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         uint32_t xo[CH];
 #pragma unroll
         for (int c = 0; c < CH; ++c) xo[c] = (uint32_t)(c * (PM ? 128 : a.n_slot)) * 8u;
-        if (a.b_resident) alive = mbar_wait(bar_b_full, 0, abort_flag, a.status, a.wait_iters);
+        if (a.b_resident) alive = mbar_wait_uniform(bar_b_full, 0, abort_flag, a.status, a.wait_iters);
 
-        // all taps of one channel block with KS K-steps each; straight-line MMA issue
-        // bit t set: view tap t of the phase plane exists (all of them for stride 1); kept in a register so that the
-        // tap loop reads no memory
-        auto load_mask = [&](int p) {
-            unsigned long long m = 0;
-            for (int tv = 0; tv < T; ++tv) m |= (unsigned long long)(tap_tab[p * T + tv] >= 0 ? 1 : 0) << tv;
-            return m;
-        };
-        const unsigned long long mask0 = MASKED ? load_mask(0) : ~0ull;
-
-        auto issue_block = [&](auto ks_tag, auto lo_tag, auto hi_tag, const uint32_t x_stage, const uint32_t (&acc)[CH], const unsigned long long taps, const uint32_t r_sel, uint32_t &started, uint32_t &w_res) {
-            const uint32_t r_col = r_sel * (uint32_t)(kSlotPx / a.racc);   // this block's accumulator within each slot
-            constexpr int KS = decltype(ks_tag)::value, CL = decltype(lo_tag)::value, CU = decltype(hi_tag)::value;
-            uint32_t off = 0;
-            int y = 0;
-            for (int tap = 0; tap < T; ++tap) {
-                uint32_t w_lo;
-                if (MASKED && !((taps >> tap) & 1ull)) {   // the view has no such tap in this phase plane
-                    if (a.b_resident) w_res += b_step;
-                    if (++y == a.FW) { y = 0; off += row_wrap; } else off += 8u;
-                    continue;
-                }
-                if (a.b_resident) {
-                    w_lo = w_res; w_res += b_step;
+        // the MMAs of one tap of one channel block with KS K steps, all chains; `first`: 0 overwrites the accumulators
+        auto mmas = [&](auto ks_tag, auto wide_tag, const uint32_t x_lo, const uint32_t w_lo, const uint32_t (&acc)[CH], const uint32_t r_col, const uint32_t first) {
+            constexpr int KS = decltype(ks_tag)::value;
+            constexpr bool WIDE = decltype(wide_tag)::value;
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                const uint32_t xs = x_lo + xo[c];
+                const uint32_t da = PM ? xs : w_lo, db = PM ? w_lo : xs;
+                if (!X3) {
+#pragma unroll
+                    for (int k = 0; k < KS; ++k) mma_tf32(acc[c] + r_col, da + 2u * k, db + 2u * k, kDescHi, idesc, k == 0 ? first : 1u);   // K steps of 32 bytes
                 } else {
-                    alive = mbar_wait(bar_b_full + 8 * sb, pb, abort_flag, a.status, a.wait_iters);
-                    if (!alive) return;
-                    w_lo = smem_desc_lo(b_base + sb * kBStageBytes);
-                }
-                const uint32_t x_lo = x_stage + off;
-                const uint32_t first = (started >> r_sel) & 1u;   // 0 for an accumulator's first MMAs of the tile: they overwrite
-                started |= 1u << r_sel;
-#pragma unroll
-                for (int c = CL; c < CU; ++c) {
-                    const uint32_t xs = x_lo + xo[c];
-                    const uint32_t da = PM ? xs : w_lo, db = PM ? w_lo : xs;
-                    if (!X3) {
-                        mma_tf32(acc[c] + r_col, da, db, kDescHi, idesc, first);
-                        if (KS > 1) mma_tf32(acc[c] + r_col, da + 2u, db + 2u, kDescHi, idesc, 1u);        // K steps of 32 bytes
-                        if (KS > 2) mma_tf32(acc[c] + r_col, da + 4u, db + 4u, kDescHi, idesc, 1u);
-                        if (KS > 3) mma_tf32(acc[c] + r_col, da + 6u, db + 6u, kDescHi, idesc, 1u);
-                    } else {
-                        // the residual halves sit x_half / w_half (16-byte units) behind the TF32 halves
-                        const uint32_t da_lo = da + (PM ? x_half : w_half), db_lo = db + (PM ? w_half : x_half);
-                        if (PM && wide) {
-                            // columns [0, w) of the chunk: x_hi w_hi + x_lo w_hi; columns [w, 2w): x_hi w_lo
-#pragma unroll
-                            for (int k = 0; k < KS; ++k) {
-                                mma_tf32(acc[c] + r_col, da + 2u * k, db + 2u * k, kDescHi, idesc_wide, k == 0 ? first : 1u);
-                                mma_tf32(acc[c] + r_col, da_lo + 2u * k, db + 2u * k, kDescHi, idesc, 1u);
-                            }
-                        } else
+                    // the residual halves sit x_half / w_half (16-byte units) behind the TF32 halves
+                    const uint32_t da_lo = da + (PM ? x_half : w_half), db_lo = db + (PM ? w_half : x_half);
+                    if (WIDE) {
+                        // columns [0, w) of the chunk: x_hi w_hi + x_lo w_hi; columns [w, 2w): x_hi w_lo
 #pragma unroll
                         for (int k = 0; k < KS; ++k) {
-                            mma_tf32(acc[c] + r_col, da_lo + 2u * k, db + 2u * k, kDescHi, idesc, k == 0 ? first : 1u);   // small terms first
-                            mma_tf32(acc[c] + r_col, da + 2u * k, db_lo + 2u * k, kDescHi, idesc, 1u);
-                            mma_tf32(acc[c] + r_col, da + 2u * k, db + 2u * k, kDescHi, idesc, 1u);
+                            mma_tf32(acc[c] + r_col, da + 2u * k, db + 2u * k, kDescHi, idesc_wide, k == 0 ? first : 1u);
+                            mma_tf32(acc[c] + r_col, da_lo + 2u * k, db + 2u * k, kDescHi, idesc, 1u);
                         }
+                    } else
+#pragma unroll
+                    for (int k = 0; k < KS; ++k) {
+                        mma_tf32(acc[c] + r_col, da_lo + 2u * k, db + 2u * k, kDescHi, idesc, k == 0 ? first : 1u);   // small terms first
+                        mma_tf32(acc[c] + r_col, da + 2u * k, db_lo + 2u * k, kDescHi, idesc, 1u);
+                        mma_tf32(acc[c] + r_col, da + 2u * k, db + 2u * k, kDescHi, idesc, 1u);
                     }
                 }
-                if (!a.b_resident) {
-                    mma_commit(bar_b_empty + 8 * sb);                // filter stage reusable once these MMAs have read it
+            }
+        };
+        // All taps of one channel block.  With resident filters the loop holds nothing but address steps and MMAs: with the
+        // wait for streamed filters inside it, jumped over, an iteration takes several times as long (instruction fetches).
+        auto issue_block = [&](auto ks_tag, auto wide_tag, const uint32_t x_stage, const uint32_t (&acc)[CH], const int i0, const int i1, const uint32_t r_sel, uint32_t &started, uint32_t &w_res) {
+            const uint32_t r_col = r_sel * (uint32_t)(kSlotPx / a.racc);   // this block's accumulator within each slot
+            uint32_t first = (started >> r_sel) & 1u;   // 0 for an accumulator's first MMAs of the tile: they overwrite
+            started |= 1u << r_sel;
+            if (a.b_resident) {
+                for (int i = i0; i < i1; ++i) {
+                    const uint32_t x_lo = x_stage + a.tap_off[i];
+                    if (elected) mmas(ks_tag, wide_tag, x_lo, w_res, acc, r_col, first);
+                    first = 1u;
+                    w_res += b_step;
+                }
+            } else {
+                for (int i = i0; i < i1; ++i) {
+                    alive = mbar_wait_uniform(bar_b_full + 8 * sb, pb, abort_flag, a.status, a.wait_iters);
+                    if (!alive) return;
+                    const uint32_t x_lo = x_stage + a.tap_off[i];
+                    if (elected) {
+                        mmas(ks_tag, wide_tag, x_lo, smem_desc_lo(b_base + sb * kBStageBytes), acc, r_col, first);
+                        mma_commit(bar_b_empty + 8 * sb);            // filter stage reusable once these MMAs have read it
+                    }
+                    first = 1u;
                     if (++sb == (uint32_t)a.b_stages) { sb = 0; pb ^= 1u; }
                 }
-                if (++y == a.FW) { y = 0; off += row_wrap; } else off += 8u;
             }
         };
 
-        bool odd_tile = false;
-        for (int t = blockIdx.x; t < total_tiles && alive; t += gridDim.x, odd_tile = !odd_tile) {
+        auto role = [&](auto wide_tag) {
+        for (int t = blockIdx.x; t < total_tiles && alive; t += gridDim.x) {
             const Tile tl = decode_tile(a, t);
             // the previous content of the slots this tile takes must have left tensor memory
             for (int j = 0; j < a.slots && alive; ++j) {
                 const uint32_t u = slot_uses + j;
-                if (u >= kSlots) alive = mbar_wait(bar_slot_free + 8 * (u % kSlots), (u / kSlots - 1) & 1, abort_flag, a.status, a.wait_iters);
+                if (u >= kSlots) alive = mbar_wait_uniform(bar_slot_free + 8 * (u % kSlots), (u / kSlots - 1) & 1, abort_flag, a.status, a.wait_iters);
             }
             if (!alive) break;
             tc_fence_after();
@@ -443,34 +414,30 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             }
             uint32_t w_res = smem_desc_lo(b_base), started = 0, r_sel = 0;
             int cb = 0, plane = 0;
-            unsigned long long taps = mask0;
             for (int blk = 0; blk < a.CB && alive; ++blk) {       // blocks = phase planes x real channel blocks
-                alive = mbar_wait(((X3 || DW) ? bar_a_split : bar_a_full) + 8 * sa, pa, abort_flag, a.status, a.wait_iters);   // once split / computed
+                alive = mbar_wait_uniform(((X3 || DW) ? bar_a_split : bar_a_full) + 8 * sa, pa, abort_flag, a.status, a.wait_iters);   // once split / computed
                 if (!alive) break;
+                tc_fence_after();
                 const uint32_t x_stage = smem_desc_lo(a_base + sa * a.a_stage_bytes) + (uint32_t)tl.a0 * 8u;   // 128 bytes per pixel, >> 4
-                if (odd_tile && (D0 != C0 || D1 != C1)) {
-                    if (cb == a.CBr - 1) issue_block(std::integral_constant<int, KS_LAST>{}, d0_tag, d1_tag, x_stage, acc, taps, r_sel, started, w_res);
-                    else issue_block(std::integral_constant<int, 4>{}, d0_tag, d1_tag, x_stage, acc, taps, r_sel, started, w_res);
-                } else {
-                    if (cb == a.CBr - 1) issue_block(std::integral_constant<int, KS_LAST>{}, c0_tag, c1_tag, x_stage, acc, taps, r_sel, started, w_res);
-                    else issue_block(std::integral_constant<int, 4>{}, c0_tag, c1_tag, x_stage, acc, taps, r_sel, started, w_res);
-                }
+                const int i0 = a.phase_at[plane], i1 = a.phase_at[plane + 1];
+                if (KS_LAST != 4 && cb == a.CBr - 1) issue_block(std::integral_constant<int, KS_LAST>{}, wide_tag, x_stage, acc, i0, i1, r_sel, started, w_res);
+                else issue_block(std::integral_constant<int, 4>{}, wide_tag, x_stage, acc, i0, i1, r_sel, started, w_res);
                 if (++r_sel == (uint32_t)a.racc) r_sel = 0;
-                if (alive) mma_commit(bar_a_empty + 8 * sa);
+                if (alive && elected) mma_commit(bar_a_empty + 8 * sa);
                 if (++sa == (uint32_t)kAStages) { sa = 0; pa ^= 1u; }
-                if (++cb == a.CBr) { cb = 0; if (MASKED && ++plane < a.n_phase) taps = load_mask(plane); }
+                if (++cb == a.CBr) { cb = 0; ++plane; }
             }
-            if (alive)
+            if (alive && elected)
                 for (int j = 0; j < a.slots; ++j) mma_commit(bar_slot_full + 8 * ((slot_uses + j) % kSlots));
             slot_uses += a.slots;
         }
         };
-        if (CH == 1 && kIssuers == 1) mma_role(std::integral_constant<int, 0>{}, std::integral_constant<int, CH>{},
-                                               std::integral_constant<int, 0>{}, std::integral_constant<int, CH>{});
-        else if (warp == 1) mma_role(std::integral_constant<int, 0>{}, std::integral_constant<int, kSplit>{},
-                                     std::integral_constant<int, 0>{}, std::integral_constant<int, kOddSplit>{});
-        else mma_role(std::integral_constant<int, kSplit>{}, std::integral_constant<int, CH>{},
-                      std::integral_constant<int, kOddSplit>{}, std::integral_constant<int, CH>{});
+        if constexpr (X3 && PM) {
+            if (wide) role(std::true_type{});
+            else role(std::false_type{});
+        } else {
+            role(std::false_type{});
+        }
     } else if (DW && warp >= 8) {
         // ---- fused depthwise 3x3: halo tile -> strip (FMAs, bias, ReLU, 16-byte stores at the swizzled places of the
         // K-major strip the MMAs read).
@@ -714,7 +681,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         tc_fence_before();
     }
     __syncthreads();
-    if (*abort_flag && armed_mask) {   // a role gave up: let the copies that are still in flight land before the CTA exits
+    if (*abort_flag && armed_mask && lane == 0) {   // a role gave up: let the copies that are still in flight land before the CTA exits
         for (int st = 0; st < 32; ++st)
             if (armed_mask >> st & 1u)
                 for (uint32_t it = 0; it < a.wait_iters && !mbar_try_wait(drain_bar + 8 * st, armed_parity >> st & 1u); ++it) __nanosleep(200);
@@ -727,7 +694,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 }
 
 // ---------------------------------------------------------------------------------------------- host side
-size_t ctrl_bytes(int KB) { return kCtrlBarrierBytes + 16 + (size_t)KB * 32 * 4 + kTapTabEntries * sizeof(short); }
+size_t ctrl_bytes(int KB) { return kCtrlBarrierBytes + 16 + (size_t)KB * 32 * 4; }
 
 // Plan with at most `max_px` pixels per tile in the given orientation; ok = false when it does not fit.
 TcPlan make_plan_with(const Geom &g, size_t max_smem, int max_px, int pixel_m, int S, double taps_eff, bool x3, int racc, bool pack_ok, int group_k, const DwFuse *dw) {
@@ -826,13 +793,14 @@ TcPlan make_plan_with(const Geom &g, size_t max_smem, int max_px, int pixel_m, i
         dw_extra = (size_t)kRawStages * p.raw_stage_bytes + (size_t)g.CB * 320 * sizeof(float);
     }
     const size_t fixed = 1024 + ctrl_bytes(g.KB) + dw_extra;
-    const size_t all_b = (size_t)g.CB * g.FH * g.FW * b_stage;
+    const int boxes = (int)(g.CB * taps_eff + 0.5);       // one per tap that exists and channel block
+    const size_t all_b = (size_t)boxes * b_stage;
     p.b_resident = 0;
     if (p.n_tiles == 1 && fixed + all_b + 2 * (size_t)p.a_stage_bytes <= max_smem) {
         size_t fit = (max_smem - fixed - all_b) / p.a_stage_bytes;
         if (fit > (size_t)kMaxAStages) fit = kMaxAStages;
         const size_t want = g.CB + 1 < 4 ? g.CB + 1 : 4;
-        if (fit >= want) { p.b_resident = 1; p.a_stages = (int)fit; p.b_stages = g.CB * g.FH * g.FW; }
+        if (fit >= want) { p.b_resident = 1; p.a_stages = (int)fit; p.b_stages = boxes; }
     }
     if (!p.b_resident) {
         if (fixed + 2 * (size_t)p.a_stage_bytes + 2 * b_stage > max_smem) return p;
@@ -936,28 +904,27 @@ TcPlan make_plan(const Geom &g, size_t max_smem, int sms, bool out_aligned32, in
 typedef void (*TcKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const TcArgs);
 
 template <int CH, int KS, bool PM>
-TcKernel pick_flags(bool masked, bool x3, bool dw) {
-    if (dw) return masked ? nullptr : x3 ? conv_tc_kernel<CH, KS, PM, false, true, true> : conv_tc_kernel<CH, KS, PM, false, false, true>;
-    if (x3) return masked ? conv_tc_kernel<CH, KS, PM, true, true, false> : conv_tc_kernel<CH, KS, PM, false, true, false>;
-    return masked ? conv_tc_kernel<CH, KS, PM, true, false, false> : conv_tc_kernel<CH, KS, PM, false, false, false>;
+TcKernel pick_flags(bool x3, bool dw) {
+    if (dw) return x3 ? conv_tc_kernel<CH, KS, PM, true, true> : conv_tc_kernel<CH, KS, PM, false, true>;
+    return x3 ? conv_tc_kernel<CH, KS, PM, true, false> : conv_tc_kernel<CH, KS, PM, false, false>;
 }
 template <int CH, bool PM>
-TcKernel pick_ks(int ks, bool masked, bool x3, bool dw) {
+TcKernel pick_ks(int ks, bool x3, bool dw) {
     switch (ks) {
-        case 1: return pick_flags<CH, 1, PM>(masked, x3, dw);
-        case 2: return pick_flags<CH, 2, PM>(masked, x3, dw);
-        case 4: return pick_flags<CH, 4, PM>(masked, x3, dw);
+        case 1: return pick_flags<CH, 1, PM>(x3, dw);
+        case 2: return pick_flags<CH, 2, PM>(x3, dw);
+        case 4: return pick_flags<CH, 4, PM>(x3, dw);
         default: return nullptr;
     }
 }
 // Filters on M: one chain per accumulator slot (1 or 2); pixels on M: one per 128-pixel chunk (1 to 4).
-TcKernel pick_kernel(int chains, int ks, bool pixel_m, bool masked, bool x3, bool dw) {
-    if (!pixel_m) return chains == 1 ? pick_ks<1, false>(ks, masked, x3, dw) : chains == 2 ? pick_ks<2, false>(ks, masked, x3, dw) : nullptr;
+TcKernel pick_kernel(int chains, int ks, bool pixel_m, bool x3, bool dw) {
+    if (!pixel_m) return chains == 1 ? pick_ks<1, false>(ks, x3, dw) : chains == 2 ? pick_ks<2, false>(ks, x3, dw) : nullptr;
     switch (chains) {
-        case 1: return pick_ks<1, true>(ks, masked, x3, dw);
-        case 2: return pick_ks<2, true>(ks, masked, x3, dw);
-        case 3: return pick_ks<3, true>(ks, masked, x3, dw);
-        case 4: return pick_ks<4, true>(ks, masked, x3, dw);
+        case 1: return pick_ks<1, true>(ks, x3, dw);
+        case 2: return pick_ks<2, true>(ks, x3, dw);
+        case 3: return pick_ks<3, true>(ks, x3, dw);
+        case 4: return pick_ks<4, true>(ks, x3, dw);
         default: return nullptr;
     }
 }
@@ -1148,9 +1115,8 @@ int launch_conv_tc(small_ctx *ctx, const float *in, const float *w_hi, const flo
     TcArgs a{};
     a.bias = bias; a.out = out; a.status = ctx->dev_status;
     a.N = g.N; a.K = g.K; a.KB = g.KB; a.CB = g.CB; a.OH = g.OH; a.OW = g.OW; a.Wq = p.Wq; a.Hq = p.Hq;
-    a.FH = g.FH; a.FW = g.FW; a.pt = g.pt; a.pl = g.pl;
+    a.pt = g.pt; a.pl = g.pl;
     a.S = v.S; a.n_phase = v.n_phase; a.CBr = v.CBr; a.phase_bits = v.phase_bits;
-    a.FHo = v.FHo; a.FWo = v.FWo; a.pto = v.S == 1 ? g.pt : v.pto; a.plo = v.S == 1 ? g.pl : v.plo;
     a.nn = p.nn; a.px_tile = p.px_tile; a.px_img = p.px_img; a.tiles_img = p.tiles_img; a.m_tiles = p.m_tiles; a.n_tiles = p.n_tiles;
     a.strip_px = p.strip_px; a.tail_px = p.tail_px; a.w_rows = p.w_rows; a.b_stages = p.b_stages;
     a.a_stages = p.a_stages; a.pixel_m = p.pixel_m; a.w_tile = p.w_tile; a.cps = p.cps; a.b_stage_bytes = p.b_stage_bytes;
@@ -1177,14 +1143,24 @@ int launch_conv_tc(small_ctx *ctx, const float *in, const float *w_hi, const flo
         a.n_slot = ((p.px_tile + a.slots - 1) / a.slots + 15) & ~15;
         chains = a.slots;
     }
-    // the MMA's N: filters of the tile (twice that for x3_wide) or pixels of a slot; up to 128 columns an MMA is issue-bound
-    // Off: alternating paid on the residual CNN's 32 -> 32 layer, which the warp-level kernel has taken since, and cost
-    // the 64 -> 64 pointwise layers of the keyword-spotting and depthwise-separable networks 2-3 % of their step
-    // (219 -> 213 us and 213 -> 209 us with it off).
-    a.alt_tiles = 0;
+    // tap (x, y) reads row oh + floor((x - pt) / S) of phase plane ((x - pt) mod S, (y - pl) mod S)
+    for (int ph = 0, n = 0; ph < v.n_phase; ++ph) {
+        for (int x = 0; x < v.FHo; ++x)
+            for (int y = 0; y < v.FWo; ++y) {
+                int px = x * p.Wq + y, bits = 0;
+                if (v.S == 2) {
+                    bits = ((x - v.pto) & 1) | (((y - v.plo) & 1) << 1);
+                    px = (floor_half(x - v.pto) + g.pt) * p.Wq + floor_half(y - v.plo) + g.pl;
+                }
+                if (bits != ((v.phase_bits >> (2 * ph)) & 3)) continue;
+                a.tap_off[n] = (uint16_t)(px * 8); a.tap_id[n] = (uint8_t)(x * v.FWo + y);
+                ++n;
+            }
+        a.phase_at[ph + 1] = n;
+    }
     const int ks = p.ks_last == 3 ? 4 : p.ks_last;     // a K step of zero channels more is harmless
     a.relu = relu; a.accumulate = accumulate; a.wait_iters = ctx->wait_iters;
-    const TcKernel kern = pick_kernel(chains, ks, p.pixel_m != 0, v.S != 1, x3, dw != nullptr);
+    const TcKernel kern = pick_kernel(chains, ks, p.pixel_m != 0, x3, dw != nullptr);
     if (!kern) return SMALL_ERR_UNSUPPORTED;
     // the attribute belongs to the kernel instance, which other layers share: always the device's limit, so that a
     // launch kept in the cache never finds it lowered by a later layer with a smaller tile
