@@ -145,6 +145,26 @@ def lib():
     return L
 
 
+class _Unloaded:
+    """Stands where the native module goes until the first call: loads the library (with the message above if it is
+    missing) and the module, then is out of the way."""
+
+    def __getattr__(self, name):
+        global _n
+        lib()
+        from . import _native
+        _native.configure(_raise, torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+        _n = _native
+        return getattr(_native, name)
+
+
+def _raise(status, where):
+    raise SmallError(status, where)
+
+
+_n = _Unloaded()
+
+
 def _ptr(t):
     if t is None:
         return None
@@ -183,11 +203,11 @@ def small_channel_block():
 
 
 def small_packed_elems(N, C, H, W):
-    return lib().small_packed_elems(N, C, H, W)
+    return _n.small_packed_elems(N, C, H, W)
 
 
 def small_out_size(I, F, stride, pad_before=0, pad_after=0):
-    return lib().small_out_size(I, F, stride, pad_before, pad_after)
+    return _n.small_out_size(I, F, stride, pad_before, pad_after)
 
 
 def small_set_layer_overlap(ctx, on):
@@ -230,11 +250,11 @@ def small_device_status(ctx, stream=None):
 
 
 def small_pack(ctx, nchw, blk, N, C, H, W, stream=None):
-    _check(lib().small_pack(ctx, _ptr(nchw), _ptr(blk), N, C, H, W, _stream(stream)), "small_pack")
+    _n.small_pack(ctx, nchw, blk, N, C, H, W, stream)
 
 
 def small_unpack(ctx, blk, nchw, N, C, H, W, stream=None):
-    _check(lib().small_unpack(ctx, _ptr(blk), _ptr(nchw), N, C, H, W, _stream(stream)), "small_unpack")
+    _n.small_unpack(ctx, blk, nchw, N, C, H, W, stream)
 
 
 def small_conv_weight_elems(C, K, FH, FW, math=MATH_FP32):
@@ -242,7 +262,7 @@ def small_conv_weight_elems(C, K, FH, FW, math=MATH_FP32):
 
 
 def small_pack_conv_weights(ctx, w_kcrs, w_blk, C, K, FH, FW, math=MATH_FP32, stream=None):
-    _check(lib().small_pack_conv_weights(ctx, _ptr(w_kcrs), _ptr(w_blk), C, K, FH, FW, math, _stream(stream)), "small_pack_conv_weights")
+    _n.small_pack_conv_weights(ctx, w_kcrs, w_blk, C, K, FH, FW, math, stream)
 
 
 def small_dw_weight_elems(C, FH, FW):
@@ -250,7 +270,7 @@ def small_dw_weight_elems(C, FH, FW):
 
 
 def small_pack_dw_weights(ctx, w_crs, w_blk, C, FH, FW, stream=None):
-    _check(lib().small_pack_dw_weights(ctx, _ptr(w_crs), _ptr(w_blk), C, FH, FW, _stream(stream)), "small_pack_dw_weights")
+    _n.small_pack_dw_weights(ctx, w_crs, w_blk, C, FH, FW, stream)
 
 
 def small_fc_weight_elems(J, K, math=MATH_FP32):
@@ -276,13 +296,12 @@ def small_fc_uses_tensor_cores(N, J, K, math):
 
 
 def small_pack_fc_weights(ctx, w_kj, w_blk, J, K, math=MATH_FP32, stream=None):
-    _check(lib().small_pack_fc_weights(ctx, _ptr(w_kj), _ptr(w_blk), J, K, math, _stream(stream)), "small_pack_fc_weights")
+    _n.small_pack_fc_weights(ctx, w_kj, w_blk, J, K, math, stream)
 
 
 def small_conv2d(ctx, inp, w_blk, bias, out, N, C, K, H, W, FH, FW, stride, pad, flags=0, stream=None):
     pt, pb, pl, pr = pad
-    _check(lib().small_conv2d(ctx, _ptr(inp), _ptr(w_blk), _ptr(bias), _ptr(out), N, C, K, H, W, FH, FW, stride,
-                              pt, pb, pl, pr, flags, _stream(stream)), "small_conv2d")
+    _n.small_conv2d(ctx, inp, w_blk, bias, out, N, C, K, H, W, FH, FW, stride, pt, pb, pl, pr, flags, stream)
 
 
 def small_group_count(C, F_C, S_C):
@@ -294,20 +313,17 @@ def small_group_conv_weight_elems(C, F_C, S_C, K, FH, FW):
 
 
 def small_pack_group_conv_weights(ctx, w_gkcrs, w_blk, C, F_C, S_C, K, FH, FW, stream=None):
-    _check(lib().small_pack_group_conv_weights(ctx, _ptr(w_gkcrs), _ptr(w_blk), C, F_C, S_C, K, FH, FW, _stream(stream)),
-           "small_pack_group_conv_weights")
+    _n.small_pack_group_conv_weights(ctx, w_gkcrs, w_blk, C, F_C, S_C, K, FH, FW, stream)
 
 
 def small_group_conv2d(ctx, inp, w_blk, bias, out, N, C, F_C, S_C, K, H, W, FH, FW, stride, pad, flags=0, stream=None):
     pt, pb, pl, pr = pad
-    _check(lib().small_group_conv2d(ctx, _ptr(inp), _ptr(w_blk), _ptr(bias), _ptr(out), N, C, F_C, S_C, K, H, W, FH, FW, stride,
-                                    pt, pb, pl, pr, flags, _stream(stream)), "small_group_conv2d")
+    _n.small_group_conv2d(ctx, inp, w_blk, bias, out, N, C, F_C, S_C, K, H, W, FH, FW, stride, pt, pb, pl, pr, flags, stream)
 
 
 def small_dwpw_conv2d(ctx, inp, dw_w_blk, dw_bias, pw_w_blk, pw_bias, out, scratch, N, C, K, H, W, stride, pad, flags=0, stream=None):
     pt, pb, pl, pr = pad
-    _check(lib().small_dwpw_conv2d(ctx, _ptr(inp), _ptr(dw_w_blk), _ptr(dw_bias), _ptr(pw_w_blk), _ptr(pw_bias), _ptr(out), _ptr(scratch),
-                                   N, C, K, H, W, stride, pt, pb, pl, pr, flags, _stream(stream)), "small_dwpw_conv2d")
+    _n.small_dwpw_conv2d(ctx, inp, dw_w_blk, dw_bias, pw_w_blk, pw_bias, out, scratch, N, C, K, H, W, stride, pt, pb, pl, pr, flags, stream)
 
 
 def small_dwpw_fused(N, C, K, H, W, stride, pad, math):
@@ -317,8 +333,7 @@ def small_dwpw_fused(N, C, K, H, W, stride, pad, math):
 
 def small_conv_maxpool2d(ctx, inp, w_blk, bias, out, scratch, N, C, K, H, W, FH, FW, stride, pad, flags=0, stream=None):
     pt, pb, pl, pr = pad
-    _check(lib().small_conv_maxpool2d(ctx, _ptr(inp), _ptr(w_blk), _ptr(bias), _ptr(out), _ptr(scratch), N, C, K, H, W, FH, FW, stride,
-                                      pt, pb, pl, pr, flags, _stream(stream)), "small_conv_maxpool2d")
+    _n.small_conv_maxpool2d(ctx, inp, w_blk, bias, out, scratch, N, C, K, H, W, FH, FW, stride, pt, pb, pl, pr, flags, stream)
 
 
 def small_conv_maxpool_fused(N, C, K, H, W, FH, FW, stride, pad):
@@ -333,39 +348,36 @@ def small_conv2d_uses_tensor_cores(N, C, K, H, W, FH, FW, stride, pad):
 
 def small_dwconv2d(ctx, inp, w_blk, bias, out, N, C, H, W, FH, FW, stride, pad, flags=0, stream=None):
     pt, pb, pl, pr = pad
-    _check(lib().small_dwconv2d(ctx, _ptr(inp), _ptr(w_blk), _ptr(bias), _ptr(out), N, C, H, W, FH, FW, stride,
-                                pt, pb, pl, pr, flags, _stream(stream)), "small_dwconv2d")
+    _n.small_dwconv2d(ctx, inp, w_blk, bias, out, N, C, H, W, FH, FW, stride, pt, pb, pl, pr, flags, stream)
 
 
 def small_pool2d(ctx, inp, out, idx, N, C, H, W, FH, FW, stride, pad, mode=POOL_MAX, stream=None):
     pt, pb, pl, pr = pad
-    _check(lib().small_pool2d(ctx, _ptr(inp), _ptr(out), _ptr(idx), N, C, H, W, FH, FW, stride, pt, pb, pl, pr, mode,
-                              _stream(stream)), "small_pool2d")
+    _n.small_pool2d(ctx, inp, out, idx, N, C, H, W, FH, FW, stride, pt, pb, pl, pr, mode, stream)
 
 
 def small_relu(ctx, inp, out, N, C, H, W, stream=None):
-    _check(lib().small_relu(ctx, _ptr(inp), _ptr(out), N, C, H, W, _stream(stream)), "small_relu")
+    _n.small_relu(ctx, inp, out, N, C, H, W, stream)
 
 
 def small_scale_shift(ctx, inp, scale, shift, out, N, C, H, W, flags=0, stream=None):
-    _check(lib().small_scale_shift(ctx, _ptr(inp), _ptr(scale), _ptr(shift), _ptr(out), N, C, H, W, flags, _stream(stream)), "small_scale_shift")
+    _n.small_scale_shift(ctx, inp, scale, shift, out, N, C, H, W, flags, stream)
 
 
 def small_upsample_nearest(ctx, inp, out, N, C, H, W, factor, stream=None):
-    _check(lib().small_upsample_nearest(ctx, _ptr(inp), _ptr(out), N, C, H, W, factor, _stream(stream)), "small_upsample_nearest")
+    _n.small_upsample_nearest(ctx, inp, out, N, C, H, W, factor, stream)
 
 
 def small_add(ctx, a, b, out, N, C, H, W, flags=0, stream=None):
-    _check(lib().small_add(ctx, _ptr(a), _ptr(b), _ptr(out), N, C, H, W, flags, _stream(stream)), "small_add")
+    _n.small_add(ctx, a, b, out, N, C, H, W, flags, stream)
 
 
 def small_fc(ctx, inp, w_blk, bias, out, N, J, K, flags=0, stream=None):
-    _check(lib().small_fc(ctx, _ptr(inp), _ptr(w_blk), _ptr(bias), _ptr(out), N, J, K, flags, _stream(stream)), "small_fc")
+    _n.small_fc(ctx, inp, w_blk, bias, out, N, J, K, flags, stream)
 
 
 def small_gap_fc(ctx, inp, w_blk, bias, out, scratch, N, C, H, W, K, flags=0, stream=None):
-    _check(lib().small_gap_fc(ctx, _ptr(inp), _ptr(w_blk), _ptr(bias), _ptr(out), _ptr(scratch), N, C, H, W, K, flags, _stream(stream)),
-           "small_gap_fc")
+    _n.small_gap_fc(ctx, inp, w_blk, bias, out, scratch, N, C, H, W, K, flags, stream)
 
 
 def small_gap_fc_fused(N, C, K, math):
@@ -377,7 +389,7 @@ FUSE_DEFAULT = FUSE_DWPW | FUSE_CONVPOOL | FUSE_FC_CHAIN | FUSE_POOLFC
 
 
 def small_set_net_fusion(ctx, mask):
-    _check(lib().small_set_net_fusion(ctx, mask), "small_set_net_fusion")
+    _n.small_set_net_fusion(ctx, mask)
 
 
 def small_net_launches(ctx, layers, N):
@@ -389,8 +401,7 @@ def small_net_workspace_bytes(layers, N):
 
 
 def small_run_net(ctx, layers, N, in_blk, out_blk, workspace, workspace_bytes, stream=None):
-    _check(lib().small_run_net(ctx, layers, len(layers), N, _ptr(in_blk), _ptr(out_blk), _ptr(workspace), workspace_bytes,
-                               _stream(stream)), "small_run_net")
+    _n.small_run_net(ctx, layers, len(layers), N, in_blk, out_blk, workspace, workspace_bytes, stream)
 
 
 def small_net_host_staging_bytes(N, C, H, W, outC, outH, outW):
@@ -399,8 +410,7 @@ def small_net_host_staging_bytes(N, C, H, W, outC, outH, outW):
 
 def small_run_net_host(ctx, layers, N, in_host, C, H, W, out_host, outC, outH, outW, workspace, workspace_bytes, stream=None):
     """in_host / out_host: CPU tensors (pinned for asynchronous copies)."""
-    _check(lib().small_run_net_host(ctx, layers, len(layers), N, _ptr(in_host), C, H, W, _ptr(out_host), outC, outH, outW,
-                                    _ptr(workspace), workspace_bytes, _stream(stream)), "small_run_net_host")
+    _n.small_run_net_host(ctx, layers, len(layers), N, in_host, C, H, W, out_host, outC, outH, outW, workspace, workspace_bytes, stream)
 
 
 def small_static_workspace_bytes():
@@ -409,8 +419,7 @@ def small_static_workspace_bytes():
 
 def small_run_net_static(ctx, layers, N, in_blk, out_blk, stream=None):
     """small_run_net on the library's built-in workspace: no device allocation by the call (see include/small.h)."""
-    _check(lib().small_run_net_static(ctx, layers, len(layers), N, _ptr(in_blk), _ptr(out_blk), _stream(stream)),
-           "small_run_net_static")
+    _n.small_run_net_static(ctx, layers, len(layers), N, in_blk, out_blk, stream)
 
 
 def small_measure_tf32_peak(ctx, n=128, iters=4096, stream=None):
@@ -426,15 +435,15 @@ def small_measure_tf32_peak(ctx, n=128, iters=4096, stream=None):
 # ---- quantised layers (uint8 tensors; qp = (z_in, z_w, z_out, mult, shift)) ----
 
 def small_q_packed_bytes(N, C, H, W):
-    return lib().small_q_packed_bytes(N, C, H, W)
+    return _n.small_q_packed_bytes(N, C, H, W)
 
 
 def small_q_pack(ctx, nchw, blk, N, C, H, W, stream=None):
-    _check(lib().small_q_pack(ctx, _ptr(nchw), _ptr(blk), N, C, H, W, _stream(stream)), "small_q_pack")
+    _n.small_q_pack(ctx, nchw, blk, N, C, H, W, stream)
 
 
 def small_q_unpack(ctx, blk, nchw, N, C, H, W, stream=None):
-    _check(lib().small_q_unpack(ctx, _ptr(blk), _ptr(nchw), N, C, H, W, _stream(stream)), "small_q_unpack")
+    _n.small_q_unpack(ctx, blk, nchw, N, C, H, W, stream)
 
 
 def small_q_conv_weight_bytes(C, K, FH, FW):
@@ -442,14 +451,13 @@ def small_q_conv_weight_bytes(C, K, FH, FW):
 
 
 def small_q_pack_conv_weights(ctx, w_kcrs, w_blk, C, K, FH, FW, stream=None):
-    _check(lib().small_q_pack_conv_weights(ctx, _ptr(w_kcrs), _ptr(w_blk), C, K, FH, FW, _stream(stream)), "small_q_pack_conv_weights")
+    _n.small_q_pack_conv_weights(ctx, w_kcrs, w_blk, C, K, FH, FW, stream)
 
 
 def small_q_conv2d(ctx, inp, w_blk, bias, out, N, C, K, H, W, FH, FW, stride, pad, qp, flags=0, stream=None):
     pt, pb, pl, pr = pad
     z_in, z_w, z_out, mult, shift = qp
-    _check(lib().small_q_conv2d(ctx, _ptr(inp), _ptr(w_blk), _ptr(bias), _ptr(out), N, C, K, H, W, FH, FW, stride, pt, pb, pl, pr,
-                                z_in, z_w, z_out, mult, shift, flags, _stream(stream)), "small_q_conv2d")
+    _n.small_q_conv2d(ctx, inp, w_blk, bias, out, N, C, K, H, W, FH, FW, stride, pt, pb, pl, pr, z_in, z_w, z_out, mult, shift, flags, stream)
 
 
 def small_q_dw_weight_bytes(C, FH, FW):
@@ -457,20 +465,19 @@ def small_q_dw_weight_bytes(C, FH, FW):
 
 
 def small_q_pack_dw_weights(ctx, w_crs, w_blk, C, FH, FW, stream=None):
-    _check(lib().small_q_pack_dw_weights(ctx, _ptr(w_crs), _ptr(w_blk), C, FH, FW, _stream(stream)), "small_q_pack_dw_weights")
+    _n.small_q_pack_dw_weights(ctx, w_crs, w_blk, C, FH, FW, stream)
 
 
 def small_q_dwconv2d(ctx, inp, w_blk, bias, out, N, C, H, W, FH, FW, stride, pad, qp, flags=0, stream=None):
     pt, pb, pl, pr = pad
     z_in, z_w, z_out, mult, shift = qp
-    _check(lib().small_q_dwconv2d(ctx, _ptr(inp), _ptr(w_blk), _ptr(bias), _ptr(out), N, C, H, W, FH, FW, stride, pt, pb, pl, pr,
-                                  z_in, z_w, z_out, mult, shift, flags, _stream(stream)), "small_q_dwconv2d")
+    _n.small_q_dwconv2d(ctx, inp, w_blk, bias, out, N, C, H, W, FH, FW, stride, pt, pb, pl, pr, z_in, z_w, z_out, mult, shift, flags, stream)
 
 
 def small_q_maxpool2d(ctx, inp, out, N, C, H, W, FH, FW, stride, pad, z, stream=None):
     pt, pb, pl, pr = pad
-    _check(lib().small_q_maxpool2d(ctx, _ptr(inp), _ptr(out), N, C, H, W, FH, FW, stride, pt, pb, pl, pr, z, _stream(stream)), "small_q_maxpool2d")
+    _n.small_q_maxpool2d(ctx, inp, out, N, C, H, W, FH, FW, stride, pt, pb, pl, pr, z, stream)
 
 
 def small_q_relu(ctx, inp, out, N, C, H, W, z, stream=None):
-    _check(lib().small_q_relu(ctx, _ptr(inp), _ptr(out), N, C, H, W, z, _stream(stream)), "small_q_relu")
+    _n.small_q_relu(ctx, inp, out, N, C, H, W, z, stream)

@@ -1,15 +1,19 @@
-"""Builds the CUDA library in-tree: every csrc/*.cu -> _build/*.o (sm_100a), linked into libsmall.so here."""
+"""Builds the CUDA library in-tree: every csrc/*.cu -> _build/*.o (sm_100a), linked into libsmall.so here, and the Python
+module _native (csrc/py_native.cpp) that calls it."""
 from __future__ import annotations
 
 import concurrent.futures
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libsmall.so")
+NATIVE_SRC = os.path.join(CSRC, "py_native.cpp")
+NATIVE = os.path.join(HERE, "_native.so")
 BUILD_DIR = os.path.join(ROOT, "_build")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -60,6 +64,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
         subprocess.check_call([_nvcc(), "-Wno-deprecated-gpu-targets", "-shared", "-o", tmp] + objs +
                               ["-lcudart_static", "-ldl", "-lrt", "-lpthread"])
         os.replace(tmp, OUT)
+    if force or not os.path.exists(NATIVE) or os.path.getmtime(NATIVE) < max(os.path.getmtime(NATIVE_SRC), os.path.getmtime(os.path.join(ROOT, "include", "small.h"))):
+        tmp = NATIVE + f".tmp{os.getpid()}"
+        subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I" + sysconfig.get_paths()["include"],
+                               "-I" + os.path.join(ROOT, "include"), NATIVE_SRC, "-o", tmp, "-L" + HERE, "-l:libsmall.so", "-Wl,-rpath,$ORIGIN"])
+        os.replace(tmp, NATIVE)
     return OUT
 
 
