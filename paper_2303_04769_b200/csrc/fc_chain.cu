@@ -17,24 +17,20 @@
 //   epilogue    = thread = filter: tensor memory -> registers, + bias, ReLU, and the filter's nt values go straight back
 //                 into the B slots as the next layer's operand (for 3xTF32 split into TF32 part and residual); the last
 //                 layer's values go to global memory, a warp writing one image's 32-channel line per store
-// Roles: one thread of warp 0 issues the MMAs; the first lanes of warp 1 stream the first layer's input and every layer's
-// filters, each lane its own loads in lockstep with the others; warps 4 .. (four per 32 images) run the epilogue.
+// Roles: warp 0 issues the MMAs; warp 1 streams the first layer's input and every layer's filters (each one thread's work,
+// done by a uniform warp: see elect_one); warps 4 .. (four per 32 images) run the epilogue.
 //
-// The chain is latency-bound, so the design follows what one thread's instructions were measured to cost: a poll of an
-// mbarrier that is already complete takes a hundred cycles or more, arming a barrier and starting a copy several hundred,
-// and a tcgen05.commit stalls the issuing thread for about 450 cycles - each more than the four MMAs of a channel block.
-// Hence: several producer lanes; the MMA thread starts the polls of up to four blocks together; filter stages are handed
-// back in groups (one commit per group, not per stage), operand slots of a wide first layer in groups of four, and only
-// where a later block reuses them.
+// The chain is latency-bound: per layer the MMAs (16 of 40 to 64 cycles), their completion, the epilogue and its hand-over
+// follow one another.  Roles written as `if (lane == 0)` took some 140 cycles per MMA, several hundred per copy and 450 per
+// commit, and needed several producer lanes and hand-overs in groups to hide it.
 //
 // A layer's MMAs wait for the epilogue of the layer before it, the rewrite of the slots waits for the MMAs that read them
 // (the accumulator's barrier), and an accumulator is reused only after its epilogue.  A barrier's phase is only ever
-// awaited by a thread that has itself seen the phase before (stages, slots and their groups have fixed owners among the
-// producer lanes); what a latecomer may read is a counter (steps_done).  Every wait is bounded; on expiry the kernel
-// records SMALL_ERR_TIMEOUT, lets its copies land, frees its tensor memory and returns.
+// awaited by a warp that has itself seen the phase before; what a latecomer may read is a counter (steps_done).  Every wait
+// is bounded; on expiry the kernel records SMALL_ERR_TIMEOUT, lets its copies land, frees its tensor memory and returns.
 #include <cuda.h>
 
-#include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "sm100.cuh"
@@ -50,8 +46,7 @@ constexpr int kWBlock = 16 * 1024;     // one filter box: 128 rows x 128 bytes
 constexpr int kTmemCols = 256;
 constexpr uint32_t kSpin = 1u << 15;      // polls without back-off for the roles on the layer-to-layer critical path
 constexpr int kMaxThreads = 128 + 16 * 32;
-// control block: barriers (8 bytes each), then the tensor-memory address, the abort flag and the step counter; the bias
-// table follows
+// control block: barriers (8 bytes each), then the tensor-memory address, the abort flag and the step counter
 constexpr int kOffWFull = 0, kOffWEmpty = 64, kOffInFull = 128, kOffSplit = 256, kOffSlotFree = 384, kOffAccFull = 512,
               kOffEpiDone = 576, kOffTmem = 640, kOffAbort = 644, kOffStepsDone = 648, kCtrl = 704;
 
@@ -62,12 +57,9 @@ struct ChainArgs {
     const float *bias[kChainMax];
     int J[kChainMax], K[kChainMax], relu[kChainMax];
     int box_rows[kChainMax];            // filter rows per box: the layer's rows, 128 for a last layer wider than that
-    int first_load[kChainMax + 1];      // loads (one per channel block and chunk) of a tile before layer i; [L] = per tile
     float *out; int *status;
     int L, N, tiles;
     int nt, n_slots, w_stages;          // images per tile, operand slots, filter stages
-    int release;                        // stages handed back per commit; divides w_stages
-    int lanes;                          // producer lanes (4, or 2); divides w_stages, and n_slots where slots are reused
     uint32_t wait_iters;
 };
 
@@ -102,9 +94,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(ctrl_ptr + kOffTmem);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(ctrl_ptr + kOffAbort);
     volatile uint32_t *steps_done = reinterpret_cast<volatile uint32_t *>(ctrl_ptr + kOffStepsDone);   // steps whose MMAs have all completed
-    float *bias_s = reinterpret_cast<float *>(ctrl_ptr + kCtrl);                // [L - 1][128], then the last layer's
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int n_epi_warps = nt >> 3;                     // four warps (one per 32 tensor-memory lanes) per 32 images
     const int JB0 = (a.J[0] + 31) >> 5;
     // the last layer may have more than 128 filters: it runs as chunks of 128, each one more pass over the same operand
@@ -112,18 +103,14 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
     // accumulators in rotation: 256 columns / (nt, or 2 nt for 3xTF32, whose x_lo products land in a second set of columns)
     const uint32_t acc_cols = X3 ? 2u * (uint32_t)nt : (uint32_t)nt;
     const uint32_t nacc_log2 = (nt == 32 ? 3u : nt == 64 ? 2u : 1u) - (X3 ? 1u : 0u), nacc = 1u << nacc_log2;
-    // slots, stages and stages per commit are powers of two
-    const int ns_log2 = 31 - __clz(n_slots);
-    const uint32_t ws_log2 = 31 - __clz(a.w_stages), rel_log2 = 31 - __clz(a.release);
+    const int ns_log2 = 31 - __clz(n_slots);             // slots are a power of two
     // The first layer's channel block cb lies in slot cb mod n_slots, its `cb / n_slots`-th use in the tile.  Slots are
     // handed back for reuse in groups of four (group = slot / 4), once per use that another use in the same tile follows.
     auto slot_uses = [&](int slot) -> uint32_t { return slot < JB0 ? (uint32_t)((JB0 - 1 - slot) >> ns_log2) + 1u : 0u; };
     auto group_uses = [&](int sg) -> uint32_t { return 4 * sg < JB0 ? (uint32_t)((JB0 - 1 - 4 * sg) >> ns_log2) + 1u : 0u; };
 
-    // Set-up.  TF32: in two halves that meet at named barrier 1 - warp 1 initialises the barriers, arrives and goes straight
-    // to its loads; the other warps fill the bias table, allocate tensor memory and wait there for the barriers to exist
-    // (measured on the ten-layer chain: 39.6 -> 37.8 us).  3xTF32 keeps one block-wide barrier after the set-up: the same
-    // change measured slower there (52.5 -> 57.8 us).
+    // Set-up: warp 1 initialises the barriers, arrives at named barrier 1 and goes straight to its loads; the other warps
+    // allocate tensor memory and wait there for the barriers to exist.
     if (threadIdx.x == 32) {
         for (int s = 0; s < 8; ++s) {
             mbar_init(bar_w_full + 8 * s, 1); mbar_init(bar_w_empty + 8 * s, 1);
@@ -137,20 +124,13 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
         mbar_fence_init();
     }
     uint32_t tmem = 0;
-    if (warp == 1 && !X3) {
+    if (warp == 1) {
         __syncwarp();
         asm volatile("bar.arrive 1, %0;" ::"r"(blockDim.x) : "memory");
     } else {
-        // filters and biases are no layer's output: they are read ahead of the wait on the launch before this one
-        const int fillers = X3 ? blockDim.x : blockDim.x - 32;            // every thread, or every thread but warp 1's
-        for (int i = threadIdx.x - (!X3 && warp > 1 ? 32 : 0); i < steps_per_tile * 128; i += fillers) {
-            const int l = min(i >> 7, a.L - 1), k = i - l * 128;
-            bias_s[i] = (a.bias[l] && k < a.K[l]) ? a.bias[l][k] : 0.0f;
-        }
         if (warp == 0) tmem_alloc(smem_u32(const_cast<uint32_t *>(tmem_slot)), (uint32_t)kTmemCols);
         tc_fence_before();
-        if (X3) __syncthreads();
-        else asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
+        asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
         tc_fence_after();
         tmem = *tmem_slot;
     }
@@ -159,93 +139,69 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
     // copies a producer lane started and the parity of each barrier's latest one, kept for the drain after an abort
     uint32_t armed_mask = 0, armed_parity = 0, in_mask = 0, in_par = 0;
 
-    if (warp == 1 && lane < a.lanes) {
-        // ---- first layer: its input blocks; every layer: one filter box (rows x 128 bytes; 3xTF32: two) per channel block.
-        // Lane j takes the loads q = j, j + lanes, ...: stage q mod w_stages is always its own.  The position of a load in
-        // the chain is advanced, not divided out: an integer division costs a lone thread a hundred cycles or more.
-        const uint32_t per_tile = (uint32_t)a.first_load[a.L];
-        const uint32_t my_tiles = blockIdx.x < (uint32_t)a.tiles ? ((uint32_t)a.tiles - blockIdx.x + gridDim.x - 1u) / gridDim.x : 0u;
-        const uint32_t total = my_tiles * per_tile;
-        const uint32_t lanes_mask = (1u << a.lanes) - 1u;
+    if (warp == 1) {
+        // ---- first layer: its input blocks; every layer: one filter box (rows x 128 bytes; 3xTF32: two) per channel block
         bool alive = true, synced = false;
-        uint32_t tile_k = 0, r = (uint32_t)lane;             // this lane's load: tile of this block, position in the tile
-        int l = 0;
-        for (uint32_t q0 = 0; q0 < total; q0 += (uint32_t)a.lanes) {       // every lane runs every round (they meet in it)
-            const uint32_t q = q0 + (uint32_t)lane;
-            const bool mine = q < total;
-            while (r >= per_tile) { r -= per_tile; ++tile_k; l = 0; }
-            while (l + 1 < a.L && (int)r >= a.first_load[l + 1]) ++l;
-            const int JB = (a.J[l] + 31) >> 5;
-            int cb = (int)r - a.first_load[l], ch = 0;
-            while (cb >= JB) { cb -= JB; ++ch; }             // chunks: the last layer only
-            const int t = (int)(blockIdx.x + tile_k * gridDim.x);
-            const uint32_t s = q & (uint32_t)(a.w_stages - 1), turn = q >> ws_log2;           // turn: loads into this stage before
-            // A tile's first loads wait for the tile before to complete, and that needs its last loads, which another lane
-            // may hold in this very round: the lanes that wait for nothing of this round go first.
-            const bool gated = l == 0 && cb < n_slots && tile_k > 0;
-            auto load = [&]() {
-                if (l == 0) {
-                    const int slot = cb & (n_slots - 1), sg = slot >> 2, o = cb >> ns_log2;
-                    const uint32_t use = tile_k * slot_uses(slot) + (uint32_t)o;
-                    // the slot's previous content: this tile's block cb - n_slots, or the previous tile's activations
-                    // (a group's barrier completes once per use that another use of the same tile follows)
-                    if (o > 0)
-                        alive = mbar_wait<kSpin>(bar_slot_free + 8 * sg, (tile_k * (group_uses(sg) - 1u) + (uint32_t)o - 1u) & 1u, abort_flag, a.status, a.wait_iters);
-                    else if (tile_k > 0)
-                        alive = counter_wait(steps_done, tile_k * (uint32_t)steps_per_tile, abort_flag, a.status, a.wait_iters);
-                    if (!alive) return;
-                    if (!synced) { grid_dep_sync(); synced = true; }
-                    mbar_expect_tx(bar_in + 8 * slot, slot_bytes);
-                    tma_load_3d(x_base + slot * slot_pitch, &a.map_in, bar_in + 8 * slot, 0, cb, t * nt);
-                    in_mask |= 1u << slot;
-                    in_par = (in_par & ~(1u << slot)) | ((use & 1u) << slot);
+        uint32_t tile_k = 0, s = 0, pw = 1;                  // filter stage in turn and the parity its release is waited with
+        for (int t = blockIdx.x; t < a.tiles && alive; t += gridDim.x, ++tile_k) {
+            for (int st = 0; st < steps_per_tile && alive; ++st) {
+                const int l = min(st, a.L - 1), ch = st - l, JB = (a.J[l] + 31) >> 5;
+                const uint32_t bytes = (uint32_t)a.box_rows[l] * 128u * (X3 ? 2u : 1u);
+                for (int cb = 0; cb < JB; ++cb) {
+                    if (l == 0) {
+                        const int slot = cb & (n_slots - 1), sg = slot >> 2, o = cb >> ns_log2;
+                        const uint32_t use = tile_k * slot_uses(slot) + (uint32_t)o;
+                        // the slot's previous content: this tile's block cb - n_slots, or the previous tile's activations
+                        // (a group's barrier completes once per use that another use of the same tile follows)
+                        if (o > 0) {
+                            if ((slot & 3) == 0)
+                                alive = mbar_wait_uniform<kSpin>(bar_slot_free + 8 * sg, (tile_k * (group_uses(sg) - 1u) + (uint32_t)o - 1u) & 1u, abort_flag, a.status, a.wait_iters);
+                        } else if (tile_k > 0 && cb == 0) {
+                            alive = __all_sync(0xffffffffu, counter_wait(steps_done, tile_k * (uint32_t)steps_per_tile, abort_flag, a.status, a.wait_iters));
+                        }
+                        if (!alive) break;
+                        if (!synced) { grid_dep_sync(); synced = true; }
+                        if (elect_one()) {
+                            mbar_expect_tx(bar_in + 8 * slot, slot_bytes);
+                            tma_load_3d(x_base + slot * slot_pitch, &a.map_in, bar_in + 8 * slot, 0, cb, t * nt);
+                        }
+                        in_mask |= 1u << slot;
+                        in_par = (in_par & ~(1u << slot)) | ((use & 1u) << slot);
+                    }
+                    alive = mbar_wait_uniform<kSpin>(bar_w_empty + 8 * s, pw, abort_flag, a.status, a.wait_iters);    // passes at once in the first round
+                    if (!alive) break;
+                    if (elect_one()) {
+                        mbar_expect_tx(bar_w_full + 8 * s, bytes);
+                        tma_load_3d(w_base + s * kWStage, &a.map_w[l], bar_w_full + 8 * s, 0, ch * 128, cb);
+                        if (X3) tma_load_3d(w_base + s * kWStage + kWBlock, &a.map_w_lo[l], bar_w_full + 8 * s, 0, ch * 128, cb);
+                    }
+                    armed_mask |= 1u << s;
+                    armed_parity = (armed_parity & ~(1u << s)) | ((pw ^ 1u) << s);
+                    if (++s == (uint32_t)a.w_stages) { s = 0; pw ^= 1u; }
                 }
-                if (turn > 0) alive = mbar_wait<kSpin>(bar_w_empty + 8 * (s >> rel_log2), (turn - 1u) & 1u, abort_flag, a.status, a.wait_iters);
-                if (!alive) return;
-                mbar_expect_tx(bar_w_full + 8 * s, (uint32_t)a.box_rows[l] * 128u * (X3 ? 2u : 1u));
-                tma_load_3d(w_base + s * kWStage, &a.map_w[l], bar_w_full + 8 * s, 0, ch * 128, cb);
-                if (X3) tma_load_3d(w_base + s * kWStage + kWBlock, &a.map_w_lo[l], bar_w_full + 8 * s, 0, ch * 128, cb);
-                armed_mask |= 1u << s;
-                armed_parity = (armed_parity & ~(1u << s)) | ((turn & 1u) << s);
-            };
-            if (mine && alive && !gated) load();
-            __syncwarp(lanes_mask);
-            if (mine && alive && gated) load();
-            r += (uint32_t)a.lanes;
+            }
         }
-    } else if (warp == 0 && lane == 0) {
-        // ---- the MMAs of every step (a layer, or a chunk of 128 filters of the last layer).  This thread's instruction
-        // count is the chain's critical path: descriptors and counters advance by addition, a layer's polls start together.
+    } else if (warp == 0) {
+        // ---- the MMAs of every step (a layer, or a chunk of 128 filters of the last layer)
+        const uint32_t elected = elect_one();
         bool alive = true;
         uint32_t g = 0, tile_k = 0;                        // g: steps so far; accumulator and its barriers = g mod nacc
         const uint32_t idesc = instr_desc(nt), idesc_wide = instr_desc(2 * nt);
         const uint32_t w_desc0 = smem_desc_lo(w_base), x_desc0 = smem_desc_lo(x_base);
         const uint32_t w_step = kWStage >> 4, x_step = slot_pitch >> 4, w_lo = kWBlock >> 4;
-        uint32_t sw = 0, pw = 0, wa = w_desc0;             // filter stage in turn, its parity, its descriptor
-        uint32_t rel_left = (uint32_t)a.release, rel_bar = bar_w_empty;        // stages until the group in turn goes back
-        const int group = min(4, a.w_stages);              // channel blocks whose barriers are polled together
-        auto issue = [&](uint32_t acc, uint32_t xb, int ks, uint32_t &started) {      // the MMAs of one channel block
+        uint32_t sw = 0, pw = 0;                           // filter stage in turn, its parity
+        auto issue = [&](auto ks_tag, uint32_t acc, uint32_t xb, uint32_t wa, uint32_t started) {      // the MMAs of one channel block
+            constexpr int KS = decltype(ks_tag)::value;
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (k < ks) {
-                    if (X3) {
-                        // columns [0, nt): w_hi x_hi + w_lo x_hi; columns [nt, 2 nt): w_hi x_lo - two MMAs for three products
-                        mma_tf32(acc, wa + 2u * k, xb + 2u * k, kDescHi, idesc_wide, started);
-                        mma_tf32(acc, wa + w_lo + 2u * k, xb + 2u * k, kDescHi, idesc, 1u);
-                    } else {
-                        mma_tf32(acc, wa + 2u * k, xb + 2u * k, kDescHi, idesc, started);
-                    }
-                    started = 1u;
+            for (int k = 0; k < KS; ++k) {
+                if (X3) {
+                    // columns [0, nt): w_hi x_hi + w_lo x_hi; columns [nt, 2 nt): w_hi x_lo - two MMAs for three products
+                    mma_tf32(acc, wa + 2u * k, xb + 2u * k, kDescHi, idesc_wide, k == 0 ? started : 1u);
+                    mma_tf32(acc, wa + w_lo + 2u * k, xb + 2u * k, kDescHi, idesc, 1u);
+                } else {
+                    mma_tf32(acc, wa + 2u * k, xb + 2u * k, kDescHi, idesc, k == 0 ? started : 1u);
                 }
-        };
-        auto next_stage = [&]() {                          // the filter stages go back in groups of `release`
-            if (--rel_left == 0) {
-                mma_commit(rel_bar);
-                rel_left = (uint32_t)a.release;
-                rel_bar += 8;
             }
-            wa += w_step;
-            if (++sw == (uint32_t)a.w_stages) { sw = 0; pw ^= 1u; wa = w_desc0; rel_bar = bar_w_empty; }
         };
         for (int t = blockIdx.x; t < a.tiles && alive; t += gridDim.x, ++tile_k) {
             for (int st = 0; st < steps_per_tile && alive; ++st, ++g) {
@@ -253,66 +209,68 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
                 const uint32_t ga = g & (nacc - 1u);
                 const int JB = (a.J[l] + 31) >> 5, ks_last = (a.J[l] - (JB - 1) * 32 + 7) >> 3;      // K steps with real channels
                 const uint32_t acc = tmem + ga * acc_cols;
-                uint32_t started = 0;
-                for (int cb0 = 0; cb0 < JB && alive; cb0 += group) {
-                    const int nb = min(group, JB - cb0);
-                    // start the group's polls together, then wait properly for whatever was not there yet
-                    auto poll_group = [&]() {
-                        uint32_t ready = 0;
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            if (j < nb) {
-                                uint32_t sj = sw + j, pj = pw;
-                                if (sj >= (uint32_t)a.w_stages) { sj -= a.w_stages; pj ^= 1u; }
-                                bool ok = mbar_test_wait(bar_w_full + 8 * sj, pj);
-                                if (l == 0) {
-                                    const int slot = (cb0 + j) & (n_slots - 1);
-                                    const uint32_t use = tile_k * slot_uses(slot) + (uint32_t)((cb0 + j) >> ns_log2);
-                                    ok = mbar_test_wait((X3 ? bar_split : bar_in) + 8 * slot, use & 1u) && ok;
-                                }
-                                ready |= (ok ? 1u : 0u) << j;
-                            }
-                        return ready;
-                    };
-                    uint32_t ready = poll_group();
-                    if (cb0 == 0) {
-                        // Only now (the filters' polls are behind us) wait for the epilogue: the accumulator's previous
-                        // step has been read out, and a new layer's operand is what the epilogue of the step before wrote
-                        // (epilogues finish in order: the second wait covers the first).
-                        if (st > 0 && ch == 0)
-                            alive = mbar_wait<kSpin>(bar_epi + 8 * ((g - 1u) & (nacc - 1u)), ((g - 1u) >> nacc_log2) & 1u, abort_flag, a.status, a.wait_iters);
-                        else if (g >= nacc)
-                            alive = mbar_wait<kSpin>(bar_epi + 8 * ga, ((g >> nacc_log2) - 1u) & 1u, abort_flag, a.status, a.wait_iters);
-                        if (!alive) break;
-                        tc_fence_after();                  // once per step: orders the MMAs after the epilogue's reads of the accumulator
+                // a layer whose filters all fit in the stages: they are waited for before the epilogue is, so that nothing but
+                // MMAs follows the latter
+                const bool ahead = l > 0 && JB <= a.w_stages;
+                if (ahead) {
+                    uint32_t s1 = sw, p1 = pw;
+                    for (int cb = 0; cb < JB && alive; ++cb) {
+                        alive = mbar_wait_uniform<kSpin>(bar_w_full + 8 * s1, p1, abort_flag, a.status, a.wait_iters);
+                        if (++s1 == (uint32_t)a.w_stages) { s1 = 0; p1 ^= 1u; }
                     }
-                    if (l > 0) {
-                        uint32_t xb = x_desc0 + (uint32_t)cb0 * x_step;
-                        for (int j = 0; j < nb; ++j, xb += x_step) {
-                            if (!(ready >> j & 1u)) {
-                                alive = mbar_wait<kSpin>(bar_w_full + 8 * sw, pw, abort_flag, a.status, a.wait_iters);
-                                if (!alive) break;
-                            }
-                            issue(acc, xb, cb0 + j == JB - 1 ? ks_last : 4, started);
-                            next_stage();
-                        }
-                    } else {
-                        for (int j = 0; j < nb; ++j) {
-                            const int cb = cb0 + j, slot = cb & (n_slots - 1);
-                            if (!(ready >> j & 1u)) {
-                                const uint32_t use = tile_k * slot_uses(slot) + (uint32_t)(cb >> ns_log2);
-                                alive = mbar_wait<kSpin>((X3 ? bar_split : bar_in) + 8 * slot, use & 1u, abort_flag, a.status, a.wait_iters);
-                                if (alive) alive = mbar_wait<kSpin>(bar_w_full + 8 * sw, pw, abort_flag, a.status, a.wait_iters);
-                                if (!alive) break;
-                            }
-                            issue(acc, x_desc0 + (uint32_t)slot * x_step, cb == JB - 1 ? ks_last : 4, started);
-                            // a group of four slots that a later block of this layer reuses: signal when its last block is done
-                            if (((cb & 3) == 3 || cb == JB - 1) && (cb & ~3) + n_slots < JB) mma_commit(bar_slot_free + 8 * (slot >> 2));
-                            next_stage();
-                        }
-                    }
+                    if (!alive) break;
                 }
-                if (alive) mma_commit(bar_acc + 8 * ga);
+                // The accumulator's previous step has been read out, and a new layer's operand is what the epilogue of the
+                // step before wrote (epilogues finish in order: the second wait covers the first).
+                if (st > 0 && ch == 0)
+                    alive = mbar_wait_uniform<kSpin>(bar_epi + 8 * ((g - 1u) & (nacc - 1u)), ((g - 1u) >> nacc_log2) & 1u, abort_flag, a.status, a.wait_iters);
+                else if (g >= nacc)
+                    alive = mbar_wait_uniform<kSpin>(bar_epi + 8 * ga, ((g >> nacc_log2) - 1u) & 1u, abort_flag, a.status, a.wait_iters);
+                if (!alive) break;
+                tc_fence_after();                          // orders the MMAs after the epilogue's reads of the accumulator
+                if (ahead) {
+                    uint32_t xb = x_desc0;
+                    for (int cb = 0; cb < JB - 1; ++cb, xb += x_step) {
+                        if (elected) {
+                            issue(std::integral_constant<int, 4>{}, acc, xb, w_desc0 + sw * w_step, cb > 0 ? 1u : 0u);
+                            mma_commit(bar_w_empty + 8 * sw);
+                        }
+                        if (++sw == (uint32_t)a.w_stages) { sw = 0; pw ^= 1u; }
+                    }
+                    if (elected) {
+                        const uint32_t wa = w_desc0 + sw * w_step, started = JB > 1 ? 1u : 0u;
+                        if (ks_last == 4) issue(std::integral_constant<int, 4>{}, acc, xb, wa, started);
+                        else
+                            for (int k = 0; k < ks_last; ++k) issue(std::integral_constant<int, 1>{}, acc, xb + 2u * k, wa + 2u * k, k ? 1u : started);
+                        mma_commit(bar_w_empty + 8 * sw);
+                        mma_commit(bar_acc + 8 * ga);
+                    }
+                    if (++sw == (uint32_t)a.w_stages) { sw = 0; pw ^= 1u; }
+                    continue;
+                }
+                for (int cb = 0; cb < JB; ++cb) {
+                    uint32_t slot = (uint32_t)cb;
+                    if (l == 0) {
+                        slot = (uint32_t)(cb & (n_slots - 1));
+                        const uint32_t use = tile_k * slot_uses((int)slot) + (uint32_t)(cb >> ns_log2);
+                        alive = mbar_wait_uniform<kSpin>((X3 ? bar_split : bar_in) + 8 * slot, use & 1u, abort_flag, a.status, a.wait_iters);
+                        if (!alive) break;
+                    }
+                    alive = mbar_wait_uniform<kSpin>(bar_w_full + 8 * sw, pw, abort_flag, a.status, a.wait_iters);
+                    if (!alive) break;
+                    const uint32_t xb = x_desc0 + slot * x_step, wa = w_desc0 + sw * w_step, started = cb > 0 ? 1u : 0u;
+                    const int ks = cb == JB - 1 ? ks_last : 4;
+                    if (elected) {
+                        if (ks == 4) issue(std::integral_constant<int, 4>{}, acc, xb, wa, started);
+                        else
+                            for (int k = 0; k < ks; ++k) issue(std::integral_constant<int, 1>{}, acc, xb + 2u * k, wa + 2u * k, k ? 1u : started);
+                        mma_commit(bar_w_empty + 8 * sw);
+                        // a group of four slots that a later block of this layer reuses: signal when its last block is done
+                        if (l == 0 && ((cb & 3) == 3 || cb == JB - 1) && (cb & ~3) + n_slots < JB) mma_commit(bar_slot_free + 8 * (slot >> 2));
+                    }
+                    if (++sw == (uint32_t)a.w_stages) { sw = 0; pw ^= 1u; }
+                }
+                if (alive && elected) mma_commit(bar_acc + 8 * ga);
             }
         }
     } else if (warp >= 4 && warp < 4 + n_epi_warps) {
@@ -346,6 +304,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
             for (int st = 0; st < steps_per_tile && alive; ++st, ++g) {
                 const int l = min(st, a.L - 1), ch = st - l;
                 const uint32_t ga = g & (nacc - 1u);
+                const int kf = ch * 128 + quarter * 32 + lane;                        // this thread's filter of the layer
+                const float b = a.bias[l] && kf < a.K[l] ? __ldg(a.bias[l] + kf) : 0.0f;
                 alive = mbar_wait_warp<kSpin>(bar_acc + 8 * ga, (g >> nacc_log2) & 1u, abort_flag, a.status, a.wait_iters);
                 if (!alive) break;
                 // the step's MMAs have completed: its filter stages, and after a tile's last step the slots, may be refilled
@@ -356,14 +316,15 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
                 if (quarter * 32 < K) {                                               // else: no filter of this step in this warp
                     const int k = quarter * 32 + lane;
                     float v[32];
-                    tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + ga * acc_cols + (uint32_t)cg * 32u, v);
+                    const uint32_t at = tmem + ((uint32_t)(quarter * 32) << 16) + ga * acc_cols + (uint32_t)cg * 32u;
                     if (X3) {                                                         // + the x_lo products
                         float u[32];
-                        tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + ga * acc_cols + (uint32_t)nt + (uint32_t)cg * 32u, u);
+                        tmem_ld32x2(at, at + (uint32_t)nt, v, u);
 #pragma unroll
                         for (int e = 0; e < 32; ++e) v[e] += u[e];
+                    } else {
+                        tmem_ld32(at, v);
                     }
-                    const float b = bias_s[st * 128 + k];
                     const bool relu = a.relu[l] != 0, real = k < K;
 #pragma unroll
                     for (int e = 0; e < 32; ++e) {
@@ -401,7 +362,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
         }
     }
     __syncthreads();
-    if (*abort_flag && warp == 1 && lane < a.lanes) {     // a role gave up: each producer lane lets its copies still in flight land
+    if (*abort_flag && warp == 1 && lane == 0) {     // a role gave up: let the copies still in flight land
         for (int st = 0; st < 16; ++st) {
             if (st < 8 && (armed_mask >> st & 1u))
                 for (uint32_t it = 0; it < a.wait_iters && !mbar_try_wait(bar_w_full + 8 * st, armed_parity >> st & 1u); ++it) __nanosleep(200);
@@ -438,27 +399,25 @@ int launch_fc_chain(small_ctx *ctx, const float *in, const float *const *w_blk, 
     // the larger tiles stream the filters fewer times.  A tile whose shared memory does not fit is halved.
     int nt = ctx->fc_chain_tile;
     if (nt == 0) nt = N <= 32 * ctx->sm_count ? 32 : N <= 64 * ctx->sm_count ? 64 : 128;
-    const size_t bias_bytes = ((size_t)L - 1 + ceil_div(widths[L], 128)) * 128 * sizeof(float);
     const size_t stage_bytes = (size_t)kWBlock * (x3 ? 2 : 1);
     const bool wide = widths[0] > 128;
-    int w_stages = 0, release = 0, lanes = 0, n_slots = 0;
+    int w_stages = 0, n_slots = 0;
     size_t smem = 0;
     for (;; nt /= 2) {
         if (nt < 32) return SMALL_ERR_UNSUPPORTED;
         const size_t slot_bytes = (size_t)nt * 128 * (x3 ? 2 : 1);
-        // Filter stages and how many go back per commit: two layers' worth in halves (TF32), one layer's in halves
-        // (3xTF32).  Operand slots: four hold 128 channels; more deepen the stream of a wider first layer, which needs at
-        // least eight (slots go back in groups of four while the four producer lanes run four blocks ahead).
-        w_stages = x3 ? 4 : 8; release = x3 ? 2 : 4; lanes = 4; n_slots = 4;                 // all powers of two
+        // Filter stages: two layers' worth (TF32), one layer's (3xTF32).  Operand slots: four hold 128 channels; more deepen
+        // the stream of a wider first layer, which needs at least eight (slots go back in groups of four).
+        w_stages = x3 ? 4 : 8; n_slots = 4;                                                  // slots: a power of two
         while (n_slots < 16 && (size_t)(2 * n_slots) * slot_bytes <= 64 * 1024) n_slots *= 2;
         if (wide && n_slots < 8) n_slots = 8;
-        const size_t fixed = 1024 + n_slots * slot_bytes + kCtrl + bias_bytes;
-        if (fixed + w_stages * stage_bytes > ctx->max_smem_optin && !wide) { w_stages = 2; release = 1; lanes = 2; }
+        const size_t fixed = 1024 + n_slots * slot_bytes + kCtrl;
+        if (fixed + w_stages * stage_bytes > ctx->max_smem_optin && !wide) w_stages = 2;
         smem = fixed + w_stages * stage_bytes;
         if (smem <= ctx->max_smem_optin) break;
     }
     a.L = L; a.N = N; a.tiles = ceil_div(N, nt); a.out = out; a.status = ctx->dev_status; a.wait_iters = ctx->wait_iters;
-    a.nt = nt; a.n_slots = n_slots; a.w_stages = w_stages; a.release = release; a.lanes = lanes;
+    a.nt = nt; a.n_slots = n_slots; a.w_stages = w_stages;
     {   // the first layer's input, blocked [N][JB][32]: one box = nt images x one 32-channel block
         const int JB = blocks_of(widths[0]);
         cuuint64_t dims[3] = {32, (cuuint64_t)JB, (cuuint64_t)N};
@@ -469,10 +428,6 @@ int launch_fc_chain(small_ctx *ctx, const float *in, const float *const *w_blk, 
                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) { ctx->last_cuda = (int)r; return SMALL_ERR_CUDA; }
-    }
-    for (int l = 0, loads = 0; l <= L; ++l) {
-        a.first_load[l] = loads;
-        if (l < L) loads += blocks_of(widths[l]) * (l == L - 1 ? ceil_div(widths[L], 128) : 1);
     }
     for (int l = 0; l < L; ++l) {
         const int J = widths[l], K = widths[l + 1], CB = blocks_of(J), Kp = blocks_of(K) * 32;
