@@ -4,10 +4,14 @@
 #include <cstring>
 #include <initializer_list>
 #include <new>
+#include <string>
+#include <unordered_map>
 
 #include "common.cuh"
 
 namespace small {
+
+typedef std::unordered_map<std::string, int> PathCache;
 
 int make_geom(Geom &g, int N, int C, int K, int H, int W, int FH, int FW, int S, int pt, int pb, int pl, int pr) {
     if (N < 1 || C < 1 || K < 1 || H < 1 || W < 1 || FH < 1 || FW < 1 || S < 1) return SMALL_ERR_SHAPE;
@@ -104,6 +108,8 @@ SMALL_API int small_init(int device, small_ctx **out) {
     c->tc_cache = nullptr;
     c->mma_cache = nullptr;
     c->i8_cache = nullptr;
+    c->direct_cache = nullptr;
+    c->path_cache = nullptr;
     c->wait_iters = 1u << 22;     // with the polls' nanosleep back-off: seconds
     if (resolve_static_workspace(c) != SMALL_OK) {      // loads the library's device code here, not inside a later call
         cudaFree(block);
@@ -144,6 +150,8 @@ SMALL_API int small_shutdown(small_ctx *ctx) {
     free_tc_cache(ctx);
     free_mma_cache(ctx);
     free_i8_cache(ctx);
+    free_direct_cache(ctx);
+    delete static_cast<PathCache *>(ctx->path_cache);
     if (ctx->ev_fork) cudaEventDestroy(static_cast<cudaEvent_t>(ctx->ev_fork));
     if (ctx->ev_join) cudaEventDestroy(static_cast<cudaEvent_t>(ctx->ev_join));
     if (ctx->side_stream) cudaStreamDestroy(static_cast<cudaStream_t>(ctx->side_stream));
@@ -354,16 +362,18 @@ static bool prefer_cuda_cores(const small_ctx *ctx, const Geom &g, unsigned math
     return g.FH * g.FW == 1 || (math == SMALL_MATH_3XTF32 && g.S == 2);
 }
 
-static int conv2d_path(const small_ctx *ctx, const Geom &g, unsigned math, bool out_aligned32) {
+static int choose_path(const small_ctx *ctx, const Geom &g, unsigned math, bool out_aligned32) {
     if (ctx && ctx->conv_path == SMALL_CONV_PATH_WARP_MMA && math != SMALL_MATH_FP32 && conv_mma_supported(g, math == SMALL_MATH_3XTF32)) return 4;
     if (conv_thin_supported(g)) return 0;          // a reduction of a few dozen terms: CUDA cores in every math mode
     if (ctx && ctx->conv_path == SMALL_CONV_PATH_GENERAL) return 2;
     bool direct = conv_direct_supported(g);
-    // the register-tiled kernel computes runs of 8 output columns per thread and 256 to 2048 outputs x 8 to 64 filters per
-    // thread block: planes narrower than 4 columns leave it mostly idle, and a layer that gives it fewer blocks than half
-    // the SMs runs faster on the general kernel's many small blocks (measured on the depthwise-separable network)
+    // the register-tiled kernel computes runs of 7 or 8 output columns per thread and 256 to 2048 outputs x 8 to 64 filters per
+    // thread block: planes narrower than 4 columns leave it mostly idle (a 1 x 1 layer's plane is viewed with longer rows), and a
+    // layer that gives it fewer blocks than half the SMs runs faster on the general kernel's many small blocks, unless its
+    // threads have many FMAs each: 3 x 3 at stride 1 on planes of 12 columns and more (batch 1, us, general against
+    // register-tiled: 16 -> 16 on 32 x 32 12.9 / 10.5, 64 -> 64 on 28 x 28 41 / 33, but on 8 x 8 27.5 / 30.7 and 1 x 1 on 25 x 5 6.8 / 9.7)
     if (direct && !(ctx && ctx->conv_path == SMALL_CONV_PATH_CUDA_CORES) &&
-        (g.OW < 4 || conv_direct_blocks(g) < (ctx ? ctx->sm_count : 148) / 2))
+        ((g.OW < 4 && g.FH * g.FW > 1) || (conv_direct_blocks(g) < (ctx ? ctx->sm_count : 148) / 2 && !(g.FH == 3 && g.FW == 3 && g.S == 1 && g.OW >= 12))))
         direct = false;
     if (math == SMALL_MATH_FP32) return direct ? 1 : 2;
     // One channel block and at most 32 filters (64 with a 1x1 window): the warp-level MMA (see conv_mma.cu), which measured faster than both
@@ -379,6 +389,19 @@ static int conv2d_path(const small_ctx *ctx, const Geom &g, unsigned math, bool 
     const bool tc = out_aligned32 && conv_tc_supported(g, math == SMALL_MATH_3XTF32);
     if (tc && !(direct && prefer_cuda_cores(ctx, g, math))) return 3;
     return direct ? 1 : 2;
+}
+
+// The choice walks the planners of several kernels; it depends on the shape and two settings alone and is kept per context.
+static int conv2d_path(small_ctx *ctx, const Geom &g, unsigned math, bool out_aligned32) {
+    if (!ctx) return choose_path(ctx, g, math, out_aligned32);
+    const int f[] = {g.N, g.C, g.K, g.H, g.W, g.FH, g.FW, g.S, g.pt, g.pb, g.pl, g.pr, (int)math, out_aligned32 ? 1 : 0, ctx->conv_path};
+    const std::string key(reinterpret_cast<const char *>(f), sizeof(f));
+    if (!ctx->path_cache) ctx->path_cache = new PathCache();
+    PathCache &cache = *static_cast<PathCache *>(ctx->path_cache);
+    auto it = cache.find(key);
+    if (it != cache.end()) return it->second;
+    if (cache.size() >= 65536) cache.clear();
+    return cache[key] = choose_path(ctx, g, math, out_aligned32);
 }
 
 SMALL_API int small_conv2d_uses_tensor_cores(int N, int C, int K, int H, int W, int FH, int FW, int stride,

@@ -22,6 +22,8 @@ struct small_ctx {
     unsigned wait_iters;     // limit (polls) of every bounded device-side wait; small_set_wait_limit
     void *tc_cache;          // finished launches of the tensor-core kernel by (shape, mode, tensors); conv_tc.cu
     void *mma_cache;         // the same for the warp-level tensor-core kernel; conv_mma.cu
+    void *direct_cache;      // the same for the register-tiled FP32 kernel; conv_direct.cu
+    void *path_cache;        // kernel family per shape, mode and path setting; api.cu
     void *i8_cache;          // the same for the quantised convolution; conv_i8.cu
     void *static_workspace;  // device address of the library's built-in workspace array on this device (net_static.cu)
     int branch_overlap;      // small_run_net runs independent neighbouring layers side by side (side stream)
@@ -97,6 +99,7 @@ int make_geom(Geom &g, int N, int C, int K, int H, int W, int FH, int FW, int S,
 void free_tc_cache(small_ctx *);             // conv_tc.cu
 void free_mma_cache(small_ctx *);            // conv_mma.cu
 void free_i8_cache(small_ctx *);             // conv_i8.cu
+void free_direct_cache(small_ctx *);         // conv_direct.cu
 int resolve_static_workspace(small_ctx *);   // net_static.cu; called by small_init with the context's device current
 
 // ---- kernel launchers (each in its own .cu); all return a small_status ----

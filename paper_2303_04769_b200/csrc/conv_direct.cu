@@ -11,14 +11,22 @@
 //   i loop over F_C in F_Cb steps   -> stages of 8 or 16 input channels: TMA copies the halo box of each unit and the
 //                                      filter box of the stage into shared memory, ring of up to 3 stages
 //   x, y, ii kernel loops           -> per 4 channels and filter row: one 16-byte read per input pixel of the run
-//                                      (8 S + FW - S pixels), then 4 x FW x 64 FMAs against filter values that the
-//                                      whole warp reads as broadcasts
+//                                      (8 S + FW - S pixels), then 4 x FW x 32 two-filter FMAs (f32x2) against
+//                                      filter values that the whole warp reads as broadcasts
 // The input box keeps the blocked layout's [pixel][channel] order: nothing is transposed and no thread computes a
 // load address or a bounds check - pixels outside the plane are TMA's zero fill, which is the padding.  Bank
 // conflicts are avoided by the copy's swizzle (16-byte chunk j of pixel p lies at chunk j ^ f(p)) together with an
 // odd box width: the 8 lanes that share a shared-memory wavefront hold 8 consecutive rows, so their pixel indices
 // differ in the low three bits.
+// What bounds it: the FMA pipe and the issue slots beside it.  Two FMAs per instruction leave half the issue slots to operand
+// loads, address steps and the copies of a pixel's value into both halves; runs of 7 pixels on planes of 7, 14, 28 and 56 columns
+// leave an eighth fewer pixels idle, and blocks of 4 warps put 12 warps on an SM where blocks of 8 put 8.  Measured (batch
+// 128, 256 -> 256 on 14 x 14, 3 x 3): 948 us with one FMA per instruction, 840 with two, 662 us with 7-pixel runs and small
+// blocks (60 % of the FMA rate); 64 -> 64 on 25 x 5 at batch 1024, 1 x 1: 94 -> 43 us (rows of 125 pixels).
 #include <cuda.h>
+
+#include <string>
+#include <unordered_map>
 
 #include "common.cuh"
 #include "sm100.cuh"
@@ -27,7 +35,6 @@ namespace small {
 
 namespace {
 
-constexpr int kPW = 8;          // output pixels per thread (adjacent in a row)
 constexpr int kKQ = 8;          // filters per thread
 constexpr int kMaxStages = 3;
 constexpr int kMaxThreads = 256;
@@ -37,7 +44,8 @@ struct DirectArgs {
     const float *bias; float *out; int *status;
     int N, C, K, OH, OW, CB, KB, FH, pt, pl;
     int cpb;                    // stages per 32-channel block (32 / cch)
-    int gw, gw_shift;           // column groups (of 8 pixels) of a unit: 1, 2 or 4
+    int pw;                     // output pixels per thread (adjacent in a row): 8, or 7 where that leaves fewer columns idle
+    int gw, gw_shift;           // column groups (of pw pixels) of a unit: 1, 2 or 4
     int TH, NI;                 // output rows per image in a unit, images per unit
     int bands, tiles_w, units;  // row bands per image, column tiles per row, all units of the layer
     int th_in, cols_box;        // input box of a unit: rows per image, columns (odd)
@@ -54,14 +62,24 @@ struct DirectArgs {
     int pool;                   // fused 2 x 2 stride-2 max pool behind the layer: out is [N][K][OH/2][OW/2]
 };
 
+__device__ __forceinline__ void lds64x2(uint32_t addr, uint64_t *v) {
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "r"(addr));
+}
+// two FMAs per instruction; the pixel's value stands in both halves
+__device__ __forceinline__ uint64_t pair_of(uint32_t x) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "r"(x));
+    return r;
+}
+__device__ __forceinline__ void fma2(uint64_t &c, uint64_t a, uint64_t b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b)); }
 __device__ __forceinline__ void lds128(uint32_t addr, uint32_t *v) {
     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr));
 }
 
-template <int FW, int S>
+template <int FW, int S, int kPW = 8>
 __global__ void __maxnreg__(kMaxRegs)
 conv_direct_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ CUtensorMap map_w, const DirectArgs a) {
-    constexpr int PXH = S == 1 ? 8 : 4;           // pixels per pass over the registers (stride 2: two passes of 4)
+    constexpr int PXH = S == 1 ? kPW : 4;           // pixels per pass over the registers (stride 2: two passes of 4)
     constexpr int NPASS = kPW / PXH;
     constexpr int NINH = (PXH - 1) * S + FW;      // input pixels a pass reads per filter row
     extern __shared__ uint8_t smem_raw[];
@@ -121,11 +139,11 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_cons
     if (threadIdx.x == 0)
         for (int q = 0; q < a.stages - 1 && q < n_chunks; ++q) issue(q, q);
 
-    float acc[kPW][kKQ];
+    uint64_t acc2[kPW][kKQ / 2];                  // pairs of filters
 #pragma unroll
     for (int p = 0; p < kPW; ++p)
 #pragma unroll
-        for (int k = 0; k < kKQ; ++k) acc[p][k] = 0.0f;
+        for (int k = 0; k < kKQ / 2; ++k) acc2[p][k] = 0ull;
 
     // idle lanes read the box's first run: in bounds, never stored
     const int p_base = img < a.NI ? (img * a.th_in + row * S) * a.cols_box + g * kPW * S : 0;
@@ -170,15 +188,15 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_cons
                         for (int cc = 0; cc < 4; ++cc) {
 #pragma unroll
                             for (int y = 0; y < FW; ++y) {
-                                uint32_t w[8];
+                                uint64_t w[4];
                                 const uint32_t wa = w_s + (uint32_t)(((x * FW + y) * a.cch + 4 * j + cc) * KTb) * 4u;
-                                lds128(wa, &w[0]);
-                                lds128(wa + 16, &w[4]);
+                                lds64x2(wa, &w[0]);
+                                lds64x2(wa + 16, &w[2]);
 #pragma unroll
                                 for (int p = 0; p < PXH; ++p) {
-                                    const float xv = __uint_as_float(v[(p * S + y) * 4 + cc]);
+                                    const uint64_t xv = pair_of(v[(p * S + y) * 4 + cc]);
 #pragma unroll
-                                    for (int k = 0; k < kKQ; ++k) acc[pass * PXH + p][k] = fmaf(xv, __uint_as_float(w[k]), acc[pass * PXH + p][k]);
+                                    for (int k = 0; k < kKQ / 2; ++k) fma2(acc2[pass * PXH + p][k], xv, w[k]);
                                 }
                             }
                         }
@@ -196,6 +214,11 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_cons
         return;
     }
 
+    float acc[kPW][kKQ];
+#pragma unroll
+    for (int p = 0; p < kPW; ++p)
+#pragma unroll
+        for (int k = 0; k < kKQ / 2; ++k) { acc[p][2 * k] = __uint_as_float((uint32_t)acc2[p][k]); acc[p][2 * k + 1] = __uint_as_float((uint32_t)(acc2[p][k] >> 32)); }
     // STORE phase.  Lanes of the last filter block beyond K stay zero: the thread holding the launch's last filter group
     // writes them.
     const int kq0 = k0 + kw * kKQ;
@@ -203,7 +226,7 @@ conv_direct_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_cons
     if (kb >= a.KB) return;                       // the same for a whole warp
     const int n = n0 + img, oh = oh0 + row;
     const bool last_group = kq0 + kKQ == a.k_tiles * a.KT;
-    if (a.pool) {
+    if (kPW % 2 == 0 && a.pool) {
         // Abstract fused layer (Section 6): the 2 x 2 stride-2 max pool behind the convolution is taken in the STORE
         // phase.  A thread holds 8 adjacent columns of one row: column pairs are reduced in its registers; rows 2i and
         // 2i + 1 sit in neighbouring lanes (a unit has an even number of rows per image), so the row pair is one
@@ -273,67 +296,109 @@ struct DirectPlan { DirectArgs a; size_t smem; int threads; long long blocks; bo
 
 size_t round1k(size_t b) { return (b + 1023) & ~(size_t)1023; }
 
-// Tile shapes.  The unit of a row warp follows from the plane's width; what is chosen is the number of channels per
-// stage (8 or 16) and of units per block: the smallest blocks (finest work granularity over the SMs) that still keep
-// 12 or more warps resident per SM within shared memory.
-DirectPlan plan_direct(const Geom &g, int span, int Kg, int S_C, size_t max_smem, bool pool = false) {
+// Tile shapes: pixels per thread (7 where a multiple of 7 columns would leave an eighth of the threads' pixels idle), filters
+// per block, channels per stage (8 or 16) and units per block, by the estimated time of the layer: a warp's FMAs (two per
+// instruction) with the operand loads beside them, how well the resident warps of an SM keep its pipes busy (at 160 registers 12
+// warps fit in small blocks, 8 in blocks of 8 warps), and whole waves of blocks where they are few.
+DirectPlan plan_direct_view(const Geom &g, int span, int Kg, int S_C, size_t max_smem, bool pool, double &best_cost) {
     DirectPlan best{};
     best.ok = false;
     if ((g.FW != 1 && g.FW != 3) || (g.S != 1 && g.S != 2) || g.FH * g.FW > 256) return best;
     DirectArgs a{};
     a.N = g.N; a.C = g.C; a.K = g.K; a.OH = g.OH; a.OW = g.OW; a.CB = g.CB; a.KB = g.KB; a.FH = g.FH; a.pt = g.pt; a.pl = g.pl;
     a.span = span > 0 ? span : g.CB; a.Kg = span > 0 ? Kg : 0; a.S_C = S_C;
-    a.gw = g.OW <= 8 ? 1 : g.OW <= 16 ? 2 : 4;
-    a.gw_shift = a.gw == 1 ? 0 : a.gw == 2 ? 1 : 2;
-    a.tiles_w = ceil_div(g.OW, a.gw * kPW);
-    const int rows_u = 32 / a.gw;
-    if (g.OH <= rows_u) { a.TH = g.OH; a.NI = rows_u / g.OH; a.bands = 1; if (a.NI > g.N) a.NI = g.N; }
-    else { a.TH = rows_u; a.NI = 1; a.bands = ceil_div(g.OH, rows_u); }
-    if (pool && ((a.TH & 1) || g.OH < 2 || g.OW < 2 || span > 0)) return best;   // row pairs must share a unit
-    a.pool = pool ? 1 : 0;
-    const long long units = (long long)ceil_div(g.N, a.NI) * a.bands * a.tiles_w;
-    if (units > 0x3fffffffLL) return best;
-    a.units = (int)units;
     a.cs = g.S;
     a.es = (g.FH == 1 && g.FW == 1) ? g.S : 1;      // 1 x 1 windows: the copy itself skips the pixels a stride leaves out
     const int S = g.S / a.es;                       // stride the kernel sees in shared memory
-    a.th_in = (a.TH - 1) * S + g.FH;
-    a.cols_box = ((a.gw * kPW - 1) * S + g.FW) | 1;
-    if (a.th_in * a.es > 256 || a.cols_box * a.es > 256 || a.NI > 256) return best;
-    a.KT = g.K <= 8 ? 8 : g.K <= 16 ? 16 : (g.K <= 32 || span > 0) ? 32 : 64;
-    a.k_tiles = ceil_div(g.K, a.KT);
-    const int kwarps = a.KT / kKQ;
+    a.pool = pool ? 1 : 0;
     const int T = g.FH * g.FW;
     const int last_n = g.C - (g.CB - 1) * 32;
-    int best_warps = 0;
-    for (int cch = 16; cch >= 8; cch -= 8) {
-        const int n_chunks = ((span > 0 ? span : g.CB) - 1) * (32 / cch) + ceil_div(last_n, cch);
-        for (int pwarps = 1; pwarps * kwarps * 32 <= kMaxThreads; ++pwarps) {
-            if (pwarps * kwarps < 2) continue;
-            DirectArgs c = a;
-            c.cch = cch; c.pwarps = pwarps; c.cpb = 32 / cch;
-            c.sw_shift = cch == 16 ? 1 : 2; c.sw_mask = cch == 16 ? 3 : 1;
-            c.in_box_bytes = (uint32_t)((size_t)a.NI * a.th_in * a.cols_box * cch * 4);
-            c.unit_bytes = (uint32_t)round1k(c.in_box_bytes);
-            const int KTb = a.KT < 32 ? a.KT : 32;
-            c.w_box_bytes = (uint32_t)((size_t)T * cch * KTb * 4);
-            c.w_bytes = c.w_box_bytes * (uint32_t)ceil_div(a.KT, 32);
-            c.stage_bytes = (uint32_t)round1k((size_t)pwarps * c.unit_bytes + c.w_bytes);
-            c.stages = n_chunks < kMaxStages ? n_chunks : kMaxStages;
-            size_t smem = (size_t)c.stages * c.stage_bytes + 1024;
-            while (smem > 110 * 1024 && c.stages > 2) { --c.stages; smem = (size_t)c.stages * c.stage_bytes + 1024; }
-            if (smem > max_smem) continue;
-            const int warps = pwarps * kwarps;
-            int per_sm = (int)((225 * 1024) / (smem + 1024));
-            if (per_sm * warps > 12) per_sm = 12 / warps;             // registers: kMaxRegs allows 12 warps per SM
-            const int resident = per_sm * warps > 12 ? 12 : per_sm * warps;   // beyond 12 warps per SM nothing is gained
-            if (resident > best_warps) {
-                best_warps = resident;
-                best.a = c; best.smem = smem; best.threads = 32 * warps;
-                best.blocks = (long long)ceil_div(a.units, pwarps) * a.k_tiles;
-                best.ok = best.blocks <= 0x7fffffffLL;
+    const int channels = ((span > 0 ? span : g.CB) - 1) * 32 + last_n;
+    best_cost = 0.0;
+    for (int pw = 8; pw >= (S == 1 && !pool ? 7 : 8); --pw) {
+        a.pw = pw;
+        a.gw = g.OW <= pw ? 1 : g.OW <= 2 * pw ? 2 : 4;
+        a.gw_shift = a.gw == 1 ? 0 : a.gw == 2 ? 1 : 2;
+        a.tiles_w = ceil_div(g.OW, a.gw * pw);
+        const int rows_u = 32 / a.gw;
+        if (g.OH <= rows_u) { a.TH = g.OH; a.NI = rows_u / g.OH; a.bands = 1; if (a.NI > g.N) a.NI = g.N; }
+        else { a.TH = rows_u; a.NI = 1; a.bands = ceil_div(g.OH, rows_u); }
+        if (pool && ((a.TH & 1) || g.OH < 2 || g.OW < 2 || span > 0)) return best;   // row pairs must share a unit
+        const long long units = (long long)ceil_div(g.N, a.NI) * a.bands * a.tiles_w;
+        if (units > 0x3fffffffLL) return best;
+        a.units = (int)units;
+        a.th_in = (a.TH - 1) * S + g.FH;
+        a.cols_box = ((a.gw * pw - 1) * S + g.FW) | 1;
+        if (a.th_in * a.es > 256 || a.cols_box * a.es > 256 || a.NI > 256) continue;
+        for (int kt = g.K <= 8 ? 8 : g.K <= 16 ? 16 : (g.K <= 32 || span > 0) ? 32 : 64; kt >= (g.K > 32 ? 32 : g.K <= 8 ? 8 : g.K <= 16 ? 16 : 32); kt /= 2)
+        for (int cch = 16; cch >= 8; cch -= 8) {
+            a.KT = kt;
+            a.k_tiles = ceil_div(g.K, kt);
+            const int kwarps = kt / kKQ;
+            const int n_chunks = ((span > 0 ? span : g.CB) - 1) * (32 / cch) + ceil_div(last_n, cch);
+            for (int pwarps = 1; pwarps * kwarps * 32 <= kMaxThreads; ++pwarps) {
+                if (pwarps * kwarps < 2) continue;
+                DirectArgs c = a;
+                c.cch = cch; c.pwarps = pwarps; c.cpb = 32 / cch;
+                c.sw_shift = cch == 16 ? 1 : 2; c.sw_mask = cch == 16 ? 3 : 1;
+                c.in_box_bytes = (uint32_t)((size_t)a.NI * a.th_in * a.cols_box * cch * 4);
+                c.unit_bytes = (uint32_t)round1k(c.in_box_bytes);
+                const int KTb = a.KT < 32 ? a.KT : 32;
+                c.w_box_bytes = (uint32_t)((size_t)T * cch * KTb * 4);
+                c.w_bytes = c.w_box_bytes * (uint32_t)ceil_div(a.KT, 32);
+                c.stage_bytes = (uint32_t)round1k((size_t)pwarps * c.unit_bytes + c.w_bytes);
+                c.stages = n_chunks < kMaxStages ? n_chunks : kMaxStages;
+                size_t smem = (size_t)c.stages * c.stage_bytes + 1024;
+                while (smem > 73 * 1024 && c.stages > 2) { --c.stages; smem = (size_t)c.stages * c.stage_bytes + 1024; }
+                if (smem > max_smem) continue;
+                const int warps = pwarps * kwarps;
+                int per_sm = (int)((225 * 1024) / (smem + 1024));
+                if (per_sm * warps > 12) per_sm = 12 / warps;             // registers: kMaxRegs allows 12 warps per SM
+                if (per_sm < 1) per_sm = 1;
+                const long long blocks = (long long)ceil_div(a.units, pwarps) * a.k_tiles;
+                const int resident = per_sm * warps;
+                const double eff = resident >= 12 ? 1.0 : resident >= 8 ? 0.85 + 0.0375 * (resident - 8) : 0.12 * resident;
+                const double warp = (double)channels * T * (8.0 * pw + 10.0 + (g.FW == 1 ? 2.0 * pw : 0.5 * pw)) + 2500.0;
+                const double set = warp * resident / 4.0 / eff;
+                const double waves = (double)blocks / (148.0 * per_sm);
+                // with few waves the last one counts whole, but its blocks have the SMs to themselves where it is not full
+                const double whole = (double)(long long)waves, rest = waves - whole;
+                double cost;
+                if (waves <= 1.0) {
+                    const int here = (int)((blocks + 147) / 148);         // blocks of the busiest SM
+                    const int r = here * warps;
+                    cost = warp * r / 4.0 / (r >= 12 ? 1.0 : r >= 8 ? 0.85 + 0.0375 * (r - 8) : 0.12 * r);
+                } else {
+                    cost = set * (whole + (rest > 0.0 ? (waves > 8.0 ? rest : 0.5 + 0.5 * rest) : 0.0));
+                }
+                // few stages: loads overlap other blocks' arithmetic only, so many small blocks
+                if (n_chunks <= 3) cost *= 1.0 + 0.03 * warps;
+                if (!best.ok || cost < best_cost) {
+                    best.a = c; best.smem = smem; best.threads = 32 * warps; best.blocks = blocks;
+                    best.ok = blocks <= 0x7fffffffLL;
+                    best_cost = cost;
+                }
             }
         }
+    }
+    return best;
+}
+
+// A 1 x 1 window at stride 1 without padding may view the plane with any row length that divides it: the one that leaves
+// the fewest threads idle (25 x 5 planes as rows of 125: 97 instead of 49 % of the pixels of a unit).
+DirectPlan plan_direct(Geom &g, int span, int Kg, int S_C, size_t max_smem, bool pool = false) {
+    double cost = 0.0;
+    DirectPlan best = plan_direct_view(g, span, Kg, S_C, max_smem, pool, cost);
+    if (!best.ok || g.FH * g.FW != 1 || g.S != 1 || (g.pt | g.pb | g.pl | g.pr) || pool) return best;
+    const int hw = g.H * g.W;
+    const Geom orig = g;
+    for (int h = 1; h <= 32 && h <= hw; ++h) {
+        if (hw % h) continue;
+        Geom v = orig;
+        v.H = v.OH = h; v.W = v.OW = hw / h;
+        double c = 0.0;
+        const DirectPlan p = plan_direct_view(v, span, Kg, S_C, max_smem, false, c);
+        if (p.ok && c < 0.98 * cost) { best = p; cost = c; g = v; }
     }
     return best;
 }
@@ -343,22 +408,55 @@ using sm100::EncodeTiledFn;
 }  // namespace
 
 bool conv_direct_supported(const Geom &g, int span, int Kg, int S_C) {
-    return plan_direct(g, span, Kg, S_C, 227 * 1024).ok;
+    double cost;
+    return plan_direct_view(g, span, Kg, S_C, 227 * 1024, false, cost).ok;
 }
 
-long long conv_direct_blocks(const Geom &g) {
+long long conv_direct_blocks(const Geom &g_in) {
+    Geom g = g_in;
     const DirectPlan p = plan_direct(g, 0, 0, 0, 227 * 1024);
     return p.ok ? p.blocks : 0;
 }
 
+// A finished launch - plan, tensor maps, arguments, kernel - is kept per context by (shape, flags, tensors), so that a
+// repeated call only launches.
 namespace {
 
-// Tensor maps and launch; the packed filters are [KB][span][FH*FW][32 ci][32 ko].
-int launch_direct(small_ctx *ctx, DirectPlan &p, const Geom &g, const float *in, const float *w, cudaStream_t st) {
+typedef void (*DirectKernel)(const CUtensorMap, const CUtensorMap, const DirectArgs);
+struct DirectLaunch { CUtensorMap map_in, map_w; DirectArgs a; DirectKernel kern; unsigned grid, threads; size_t smem; };
+typedef std::unordered_map<std::string, DirectLaunch> DirectCache;
+
+int start(small_ctx *ctx, const DirectLaunch &L, cudaStream_t st) {
+    // an ordinary launch whose successor starts only as its blocks leave, like the general FP32 kernel
+    const int dependent = ctx->dependent;
+    ctx->dependent = 0;
+    launch_kernel(ctx, L.kern, dim3(L.grid), dim3(L.threads), L.smem, st, L.map_in, L.map_w, L.a);
+    ctx->dependent = dependent;
+    return check_launch(ctx);
+}
+
+int launch_direct(small_ctx *ctx, const Geom &g_in, const float *in, const float *w, const float *bias, float *out, bool relu, bool accumulate,
+                  bool pool, int span, int Kg, int S_C, cudaStream_t st) {
+    std::string key;
+    {
+        const int f[] = {g_in.N, g_in.C, g_in.K, g_in.H, g_in.W, g_in.FH, g_in.FW, g_in.S, g_in.pt, g_in.pb, g_in.pl, g_in.pr, relu ? 1 : 0,
+                         accumulate ? 1 : 0, pool ? 1 : 0, span, Kg, S_C, (int)ctx->wait_iters};
+        const void *ptrs[] = {in, w, bias, out};
+        key.append(reinterpret_cast<const char *>(f), sizeof(f));
+        key.append(reinterpret_cast<const char *>(ptrs), sizeof(ptrs));
+    }
+    if (!ctx->direct_cache) ctx->direct_cache = new DirectCache();
+    DirectCache &cache = *static_cast<DirectCache *>(ctx->direct_cache);
+    auto it = cache.find(key);
+    if (it != cache.end()) return start(ctx, it->second, st);
+    Geom g = g_in;                                   // (a pointwise layer's plane may be viewed with another row length)
+    DirectPlan p = plan_direct(g, span, Kg, S_C, ctx->max_smem_optin, pool);
+    if (!p.ok) return SMALL_ERR_UNSUPPORTED;
     DirectArgs &a = p.a;
-    a.wait_iters = ctx->wait_iters;
+    a.bias = bias; a.out = out; a.status = ctx->dev_status; a.relu = relu; a.accumulate = accumulate; a.wait_iters = ctx->wait_iters;
+    DirectLaunch L;
+    CUtensorMap &map_in = L.map_in, &map_w = L.map_w;
     EncodeTiledFn encode = reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled);
-    CUtensorMap map_in, map_w;
     {   // activations [N][CB][H][W][32]: box = one stage's channels x cols_box x th_in x 1 block x NI images, swizzled
         const cuuint64_t px = 128;                   // bytes per pixel and channel block
         cuuint64_t dims[5] = {32, (cuuint64_t)g.W, (cuuint64_t)g.H, (cuuint64_t)g.CB, (cuuint64_t)g.N};
@@ -385,39 +483,38 @@ int launch_direct(small_ctx *ctx, DirectPlan &p, const Geom &g, const float *in,
         if (r != CUDA_SUCCESS) { ctx->last_cuda = (int)r; return SMALL_ERR_CUDA; }
     }
     const int S = g.S / a.es;
-    void (*kern)(const CUtensorMap, const CUtensorMap, const DirectArgs);
-    kern = g.FW == 1 ? (S == 1 ? conv_direct_kernel<1, 1> : conv_direct_kernel<1, 2>) : (S == 1 ? conv_direct_kernel<3, 1> : conv_direct_kernel<3, 2>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    DirectKernel kern;
+    if (a.pw == 7) kern = g.FW == 1 ? conv_direct_kernel<1, 1, 7> : conv_direct_kernel<3, 1, 7>;
+    else kern = g.FW == 1 ? (S == 1 ? conv_direct_kernel<1, 1> : conv_direct_kernel<1, 2>) : (S == 1 ? conv_direct_kernel<3, 1> : conv_direct_kernel<3, 2>);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->max_smem_optin - 1024);   // the kernel has static shared memory too
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SMALL_ERR_CUDA; }
-    // an ordinary launch whose successor starts only as its blocks leave, like the general FP32 kernel
-    const int dependent = ctx->dependent;
-    ctx->dependent = 0;
-    launch_kernel(ctx, kern, dim3((unsigned)p.blocks), dim3(p.threads), p.smem, st, map_in, map_w, a);
-    ctx->dependent = dependent;
-    return check_launch(ctx);
+    if (cache.size() >= 4096) cache.clear();
+    L.a = a; L.kern = kern; L.grid = (unsigned)p.blocks; L.threads = (unsigned)p.threads; L.smem = p.smem;
+    cache[key] = L;
+    return start(ctx, L, st);
 }
 
 }  // namespace
 
-int launch_conv_direct(small_ctx *ctx, const float *in, const float *w, const float *bias, float *out, const Geom &g,
-                       bool relu, bool accumulate, cudaStream_t st, int span, int Kg, int S_C) {
-    DirectPlan p = plan_direct(g, span, Kg, S_C, ctx->max_smem_optin);
-    if (!p.ok) return SMALL_ERR_UNSUPPORTED;
-    DirectArgs &a = p.a;
-    a.bias = bias; a.out = out; a.status = ctx->dev_status; a.relu = relu; a.accumulate = accumulate;
-    return launch_direct(ctx, p, g, in, w, st);
+void free_direct_cache(small_ctx *ctx) {
+    delete static_cast<DirectCache *>(ctx->direct_cache);
+    ctx->direct_cache = nullptr;
 }
 
-bool conv_direct_pool_supported(const Geom &g) { return plan_direct(g, 0, 0, 0, 227 * 1024, true).ok; }
+int launch_conv_direct(small_ctx *ctx, const float *in, const float *w, const float *bias, float *out, const Geom &g,
+                       bool relu, bool accumulate, cudaStream_t st, int span, int Kg, int S_C) {
+    return launch_direct(ctx, g, in, w, bias, out, relu, accumulate, false, span, Kg, S_C, st);
+}
+
+bool conv_direct_pool_supported(const Geom &g) {
+    double cost;
+    return plan_direct_view(g, 0, 0, 0, 227 * 1024, true, cost).ok;
+}
 
 int launch_conv_direct_pool(small_ctx *ctx, const float *in, const float *w, const float *bias, float *out, const Geom &g,
                             bool relu, cudaStream_t st) {
-    DirectPlan p = plan_direct(g, 0, 0, 0, ctx->max_smem_optin, true);
-    if (!p.ok) return SMALL_ERR_UNSUPPORTED;
-    DirectArgs &a = p.a;
-    a.bias = bias; a.out = out; a.status = ctx->dev_status; a.relu = relu; a.accumulate = 0;
-    return launch_direct(ctx, p, g, in, w, st);
+    return launch_direct(ctx, g, in, w, bias, out, relu, false, true, 0, 0, 0, st);
 }
 
 }  // namespace small
