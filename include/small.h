@@ -390,12 +390,14 @@ typedef struct small_layer {
  * full reductions whose inner widths are at most 128 under a tensor-core math mode (SMALL_FUSE_FC_CHAIN, see small_fc_chain), and
  * a global average pool with the full reduction behind it, in every math mode (SMALL_FUSE_POOLFC, see small_gap_fc).  The skipped
  * intermediate tensors are then not written.  Default: all four (without DWPW_ALWAYS); 0 runs every layer on its own.
+ * With every kind on, a whole run of convolutions and depthwise 3x3 layers that ends the list in a global average pool and a full
+ * reduction may run as one kernel that keeps each image's activations on chip (small batches; where it was measured to pay).
  * Results stay within each math mode's tolerance either way. */
 enum { SMALL_FUSE_DWPW = 1u, SMALL_FUSE_DWPW_ALWAYS = 2u, SMALL_FUSE_CONVPOOL = 4u, SMALL_FUSE_FC_CHAIN = 8u,
        SMALL_FUSE_POOLFC = 16u };   /* a global average pool and the full reduction behind it (small_gap_fc) */
 int small_set_net_fusion(small_ctx *ctx, unsigned mask);
 /* Number of kernel launches small_run_net makes for these layers at batch N under the context's fusion setting (one per
- * layer or fused pair); -1 for invalid arguments. */
+ * layer or fused pair; fewer are made where a run of layers is kept on chip as one kernel); -1 for invalid arguments. */
 int small_net_launches(small_ctx *ctx, const small_layer *layers, int n_layers, int N);
 /* Bytes of workspace for `layers` at batch N: slot s is as large as the largest tensor any layer reads
  * from or writes to it, rounded up to 256 bytes; slots are laid out back to back.  0 on invalid input. */

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <cstddef>
 #include <cstdint>
+#include <functional>
 
 #include "small.h"
 
@@ -22,6 +23,7 @@ struct small_ctx {
     unsigned wait_iters;     // limit (polls) of every bounded device-side wait; small_set_wait_limit
     void *tc_cache;          // finished launches of the tensor-core kernel by (shape, mode, tensors); conv_tc.cu
     void *mma_cache;         // the same for the warp-level tensor-core kernel; conv_mma.cu
+    void *resident_state;    // plans of the resident network kernel; net_resident.cu
     void *direct_cache;      // the same for the register-tiled FP32 kernel; conv_direct.cu
     void *path_cache;        // kernel family per shape, mode and path setting; api.cu
     void *i8_cache;          // the same for the quantised convolution; conv_i8.cu
@@ -100,6 +102,7 @@ void free_tc_cache(small_ctx *);             // conv_tc.cu
 void free_mma_cache(small_ctx *);            // conv_mma.cu
 void free_i8_cache(small_ctx *);             // conv_i8.cu
 void free_direct_cache(small_ctx *);         // conv_direct.cu
+void free_resident_state(small_ctx *);       // net_resident.cu
 int resolve_static_workspace(small_ctx *);   // net_static.cu; called by small_init with the context's device current
 
 // ---- kernel launchers (each in its own .cu); all return a small_status ----
@@ -155,6 +158,11 @@ int launch_conv_tc(small_ctx *, const float *in, const float *w_hi, const float 
 bool conv_mma_supported(const Geom &, bool x3);
 int launch_conv_mma(small_ctx *, const float *in, const float *w_hi, const float *w_lo, const float *bias, float *out,
                     const Geom &, bool relu, bool accumulate, unsigned mode, cudaStream_t);
+// a run of layers up to the end of the list as one kernel (net_resident.cu): the first layer of the run at or behind `from`
+// (-1: none), and its launch, which reads and writes whole tensors through rd / wr (slot -> address)
+int resident_from(small_ctx *, const small_layer *layers, int n, int from, int N);
+int launch_resident(small_ctx *, const small_layer *layers, int n, int from, int N, const std::function<const float *(int)> &rd,
+                    const std::function<float *(int)> &wr, cudaStream_t);
 // quantised full channel reduction (conv_i8.cu): windows 1 or 3 wide, strides 1 and 2; w: [CB][FH*FW][KB*32][32] bytes,
 // w_sums: [K][FH*FW] sums of weight bytes over the channels
 int launch_q_conv(small_ctx *, const uint8_t *in, const uint8_t *w, const int *w_sums, const int *bias, uint8_t *out, const Geom &,

@@ -1,0 +1,355 @@
+// Host side of the resident network kernel (net_resident.cuh): which run of layers at the end of a list it takes, where the
+// tensors lie in shared memory, how many thread blocks share an image, and the launch.
+#include <algorithm>
+#include <cstring>
+#include <map>
+#include <vector>
+
+#include "net_resident.cuh"
+
+namespace small {
+
+using namespace resident;
+
+namespace {
+
+struct Tensor { int C, H, W, pitch, size, off, last_use; bool external; int slot; };
+
+uint32_t multiplier(int d) { return d <= 1 ? 0u : (uint32_t)((1ull << 32) / (unsigned)d) + 1u; }      // see quotient
+
+int act_pitch(int C) { return ((C + 7) & ~7) + 4; }
+
+// Can this layer run on chip?  `last`: it ends the list.
+bool op_supported(const small_layer &L, int N, bool last, unsigned &math, Geom &g) {
+    switch (L.op) {
+        case SMALL_OP_CONV:
+            if (make_geom(g, N, L.C, L.K, L.H, L.W, L.FH, L.FW, L.stride, L.pad_t, L.pad_b, L.pad_l, L.pad_r)) return false;
+            // (fewer than 8 channels: a K step would be mostly padding, and such layers have a kernel of their own)
+            if (L.C < 8 || L.C > 256 || L.K > 512 || L.FH * L.FW > 25 || L.FH * L.FW * ((L.C + 7) / 8) > kMaxSteps) return false;
+            break;
+        case SMALL_OP_DWCONV:
+            if (make_geom(g, N, L.C, L.C, L.H, L.W, L.FH, L.FW, L.stride, L.pad_t, L.pad_b, L.pad_l, L.pad_r)) return false;
+            return L.FH == 3 && L.FW == 3 && L.stride <= 2 && L.C <= 256;      // (filters and bias fit in one stage)
+        case SMALL_OP_POOL:
+            if (make_geom(g, N, L.C, L.C, L.H, L.W, L.FH, L.FW, L.stride, L.pad_t, L.pad_b, L.pad_l, L.pad_r)) return false;
+            return !last && L.pool_mode == SMALL_POOL_AVG && L.FH == L.H && L.FW == L.W && L.C <= 512 && !(L.pad_t | L.pad_b | L.pad_l | L.pad_r);
+        case SMALL_OP_FC:
+            if (!last || L.C < 1 || L.C > 512 || L.K < 1 || L.K > 256) return false;
+            break;
+        default: return false;
+    }
+    const unsigned m = L.flags & SMALL_MATH_MASK;
+    if (math == ~0u) math = m;
+    return m == math;
+}
+
+struct Plan { Args a; size_t smem; int from; bool ok; int out_slot; int in_slot[kMaxInputs]; unsigned math; };
+
+// Layers from .. n - 1 as one kernel; ok = false where they do not fit.
+Plan plan_run(const small_layer *layers, int n, int from, int N, size_t max_smem, bool keep) {
+    Plan p{};
+    p.ok = false;
+    p.from = from;
+    // only runs that end in the classifier head: what a list ends in is a result, and a run's other tensors are not written
+    if (n - from < 2 || n - from > kMaxOps || layers[n - 1].op != SMALL_OP_FC) return p;
+    if (layers[from].op != SMALL_OP_CONV && layers[from].op != SMALL_OP_DWCONV) return p;      // the filter stream starts with the first operation
+    unsigned math = ~0u;
+    std::vector<Tensor> t;
+    std::map<int, int> at;                               // slot -> tensor it holds
+    struct Use { int src, dst; Geom g; };
+    std::vector<Use> use;
+    auto external = [&](int slot, int C, int H, int W) {
+        t.push_back(Tensor{C, H, W, act_pitch(C), 0, 0, -1, true, slot});
+        return at[slot] = (int)t.size() - 1;
+    };
+    Args &a = p.a;
+    for (int i = from; i < n; ++i) {
+        const small_layer &L = layers[i];
+        Use u{};
+        if (!op_supported(L, N, i == n - 1, math, u.g)) return p;
+        if (L.op == SMALL_OP_POOL && (layers[i + 1].op != SMALL_OP_FC || layers[i + 1].src != L.dst || layers[i + 1].C != L.C)) return p;
+        if (L.op == SMALL_OP_FC && (i == from || layers[i - 1].op != SMALL_OP_POOL)) return p;
+        if (L.dst == SMALL_SLOT_OUTPUT && i != n - 1) return p;
+        u.src = at.count(L.src) ? at[L.src] : external(L.src, L.C, L.H, L.W);
+        if (t[u.src].C != L.C || t[u.src].H != L.H || t[u.src].W != L.W) return p;
+        t[u.src].last_use = i;
+        const int OH = L.op == SMALL_OP_FC ? 1 : u.g.OH, OW = L.op == SMALL_OP_FC ? 1 : u.g.OW, K = L.op == SMALL_OP_CONV || L.op == SMALL_OP_FC ? L.K : L.C;
+        if (L.op == SMALL_OP_CONV && (L.flags & SMALL_ACCUMULATE)) {
+            u.dst = at.count(L.dst) ? at[L.dst] : external(L.dst, K, OH, OW);
+            if (t[u.dst].C != K || t[u.dst].H != OH || t[u.dst].W != OW) return p;
+        } else {
+            t.push_back(Tensor{K, OH, OW, act_pitch(K), 0, 0, -1, false, L.dst});
+            u.dst = (int)t.size() - 1;
+            at[L.dst] = u.dst;
+        }
+        t[u.dst].last_use = i;
+        use.push_back(u);
+    }
+    int n_ext = 0;
+    for (Tensor &x : t) {
+        if ((long long)x.H * x.W * x.pitch > (1 << 20)) return p;
+        x.size = (x.H * x.W * x.pitch + 3) & ~3;
+        if (x.external && ++n_ext > kMaxInputs) return p;
+    }
+    // first fit; external tensors are loaded before the first operation
+    const long long limit = (long long)(max_smem - 1024) / 4;
+    struct Block { int off, size, tensor; };
+    std::vector<Block> live;
+    long long top = 0;
+    auto place = [&](int ti) {
+        long long off = 0;
+        std::sort(live.begin(), live.end(), [](const Block &x, const Block &y) { return x.off < y.off; });
+        for (const Block &b : live)
+            if (off + t[ti].size > b.off) off = std::max(off, (long long)b.off + b.size);
+            else break;
+        t[ti].off = (int)off;
+        live.push_back(Block{(int)off, t[ti].size, ti});
+        top = std::max(top, off + t[ti].size);
+    };
+    a.zero = 0; a.ops = kZeroFloats; a.steps = a.ops + (int)(sizeof(a.op) / sizeof(float)); a.ring = a.steps + 2 * kMaxSteps; a.scratch = a.ring + kStages * kStageFloats;      // (scratch behind the ring: see mma_steps)
+    live.push_back(Block{0, a.scratch + kScratchFloats, -1});
+    for (int i = 0; i < (int)t.size(); ++i)
+        if (t[i].external) {
+            place(i);
+            a.in[a.n_in] = Input{nullptr, t[i].C, t[i].H, t[i].W, t[i].off, t[i].pitch};
+            p.in_slot[a.n_in++] = t[i].slot;
+        }
+    std::vector<Block> since;                            // what depthwise layers read since the last exchange
+    for (int i = from; i < n; ++i) {
+        const small_layer &L = layers[i];
+        const Use &u = use[i - from];
+        bool placed = false;
+        for (const Block &b : live) placed = placed || b.tensor == u.dst;
+        if (!placed && L.op != SMALL_OP_FC) place(u.dst);
+        if (top > limit) return p;
+        Op &o = a.op[a.n_ops++];
+        o.kind = L.op == SMALL_OP_CONV ? kConv : L.op == SMALL_OP_DWCONV ? kDw : L.op == SMALL_OP_POOL ? kGap : kFc;
+        o.C = L.C; o.K = t[u.dst].C; o.H = L.H; o.W = L.W; o.OH = t[u.dst].H; o.OW = t[u.dst].W;
+        o.FH = L.FH; o.FW = L.FW; o.S = L.stride; o.pt = L.pad_t; o.pl = L.pad_l;
+        o.src = t[u.src].off; o.sp = t[u.src].pitch; o.dst = t[u.dst].off; o.dp = t[u.dst].pitch;
+        o.relu = (L.flags & SMALL_RELU) ? 1 : 0; o.accumulate = (L.flags & SMALL_ACCUMULATE) ? 1 : 0;
+        o.w = L.w_blk; o.bias = L.bias;
+        const int C4 = ((o.C + 7) & ~7) >> 2;
+        o.by_ow = multiplier(o.OW); o.by_c4 = multiplier(C4); o.by_cols = multiplier(o.OW * C4);
+        if (o.kind == kDw) {
+            // runs of rows: as many as give every thread one, of at least two rows
+            o.segs = std::max(1, std::min(kThreads / (o.OW * C4), (o.OH + 1) / 2));
+            o.seg_rows = ceil_div(o.OH, o.segs);
+            o.segs = ceil_div(o.OH, o.seg_rows);
+        } else if (o.kind == kGap) {
+            o.segs = std::min(std::min(kThreads / C4, kScratchFloats / (C4 * 4)), 32);      // groups of pixels
+        }
+        if (o.kind == kDw) since.push_back(Block{t[u.src].off, t[u.src].size, u.src});
+        if (o.kind == kConv) {
+            // the blocks of a cluster store into each other's copies of this output: where it takes the place of something a
+            // slower block may still be reading, they meet before it
+            for (const Block &b : since)
+                if (t[u.dst].off < b.off + b.size && b.off < t[u.dst].off + t[u.dst].size) a.op[a.n_ops - 2].exchange = 1;
+            since.clear();
+        }
+        // (what a depthwise layer read stays for one operation more where there is room, so that the convolution behind it does
+        // not take its place)
+        live.erase(std::remove_if(live.begin(), live.end(), [&](const Block &b) {
+                       return b.tensor >= 0 && i < n - 1 && t[b.tensor].last_use + (keep && t[b.tensor].size < limit / 8 && layers[t[b.tensor].last_use].op == SMALL_OP_DWCONV ? 1 : 0) <= i;
+                   }), live.end());
+    }
+    p.out_slot = layers[n - 1].dst;
+    a.n_stream = a.n_ops - 2;
+    a.N = N;
+    p.smem = (size_t)top * 4;
+    p.math = math;
+    p.ok = true;
+    return p;
+}
+
+Kernel kernel_of(unsigned math) {
+    return math == SMALL_MATH_FP32 ? resident_kernel_fp32() : math == SMALL_MATH_TF32 ? resident_kernel_tf32() : resident_kernel_x3();
+}
+
+// How every convolution is split over the G blocks of an image and their warps, and the estimated cycles of one image.
+double tile_ops(Args &a, unsigned math, int G) {
+    double total = 3000.0;
+    for (int i = 0; i < a.n_ops; ++i) {
+        Op &o = a.op[i];
+        const int P = o.OH * o.OW, T = o.FH * o.FW, CB = blocks_of(o.C), tail = (o.C - (CB - 1) * 32 + 7) & ~7;
+        if (o.kind != kConv) {
+            // a block computes these whole: about 20 (four channels of a pixel) per cycle; the head waits for memory
+            total += o.kind == kDw ? (double)P * ((o.C + 3) / 4) / 12.0 + 500.0 : 1500.0;
+            continue;
+        }
+        o.rows = T * ((CB - 1) * 32 + tail);
+        const int Kr = o.K <= 8 ? 8 : o.K <= 16 ? 16 : blocks_of(o.K) * 32;        // filters padded to a part's widths
+        double best = -1.0;
+        Op pick = o;
+        for (int parts = 1; parts <= G; parts *= 2) {
+            if (Kr % parts || (Kr / parts) % 8 || (Kr / parts > 32 && (Kr / parts) % 32) || (Kr / parts < 32 && Kr / parts != 8 && Kr / parts != 16)) continue;
+            Op c = o;
+            c.n_parts = parts; c.n_w = Kr / parts;
+            c.lg_parts = 0;
+            while ((1 << c.lg_parts) < parts) ++c.lg_parts;
+            const int pw = c.n_w < 32 ? c.n_w : 32, panels = c.n_w / pw;
+            c.pitch = pw == 32 ? 40 : pw == 16 ? 24 : 8;
+            c.chunk_rows = kStageFloats / (panels * c.pitch) & ~7;
+            if (c.chunk_rows < 8) continue;
+            if (c.chunk_rows > c.rows) c.chunk_rows = c.rows;
+            c.panel = c.chunk_rows * c.pitch;
+            c.chunks = ceil_div(c.rows, c.chunk_rows);
+            const int m_parts = G / parts, F = ceil_div(P, 16);
+            const double ksteps = c.rows / 8.0;
+            auto consider = [&](int mf, int nf, int m_all, int n_units, double step, int part_floats) {
+                Op d = c;
+                d.mf = mf; d.nf = nf; d.m_units = ceil_div(m_all, m_parts); d.n_units = n_units; d.by_units = multiplier(n_units);
+                const int units = d.m_units * n_units;
+                d.rounds = ceil_div(units, kWarps);
+                d.lg_split = 0;
+                while (d.lg_split < 2 && (units << (d.lg_split + 1)) <= kWarps && units * ((2 << d.lg_split) - 1) * part_floats <= kScratchFloats) ++d.lg_split;
+                d.split = 1 << d.lg_split;
+                // a scheduler's warps of a round share its pipes; a lone warp waits out its own latencies
+                const int per = ceil_div(units < kWarps ? units * d.split : kWarps, 4);
+                const double pass = ceil_div((int)ksteps, d.split) * (step * per > 80.0 ? step * per : 80.0) + d.chunks * 150.0 + 500.0;
+                const double stream = (double)d.chunks * d.chunk_rows * panels * pw * 4.0 / 30.0;        // bytes through the ring
+                const double t = d.rounds * (pass > stream ? pass : stream) + (double)P * o.K * (math == SMALL_MATH_FP32 ? 1.0 : 0.4) * (G == 8 ? 0.35 : G == 4 ? 0.2 : G == 2 ? 0.1 : 0.0);      // and the exchange
+                if (best < 0.0 || t < best) { best = t; pick = d; }
+            };
+            if (math == SMALL_MATH_FP32) {
+                const int px = 8 * (32 / pw);
+                for (int q = 1; q <= (panels % 2 == 0 ? 2 : 1); ++q) consider(1, q, ceil_div(P, px), panels / q, 64.0 * q + 60.0, q * 256);
+            } else {
+                const bool x3 = math == SMALL_MATH_3XTF32;
+                static const int tiles[3][2] = {{1, 1}, {1, 2}, {2, 2}};
+                for (auto &t : tiles)
+                    if (t[1] <= c.n_w / 8)
+                        consider(t[0], t[1], ceil_div(F, t[0]), c.n_w / 8 / t[1], t[0] * t[1] * (x3 ? 24.0 : 8.0) + 6.0 * t[1] + 8.0 * t[0] + 10.0, t[0] * t[1] * 128);
+            }
+        }
+        if (best < 0.0) return -1.0;
+        o = pick;
+        total += best + (G > 1 ? 1000.0 : 200.0);
+    }
+    return total;
+}
+
+struct Entry { std::vector<unsigned char> key; Plan p; };
+struct State {
+    int clusters[3][4] = {};                             // resident clusters of 1, 2, 4, 8 blocks per math mode; 0: not asked yet
+    std::vector<Entry> plans;                            // finished plans, the latest first
+};
+State &state_of(small_ctx *ctx) {
+    if (!ctx->resident_state) ctx->resident_state = new State();
+    return *static_cast<State *>(ctx->resident_state);
+}
+
+int clusters_of(small_ctx *ctx, unsigned math, int lg) {
+    State &s = state_of(ctx);
+    int &c = s.clusters[math == SMALL_MATH_FP32 ? 0 : math == SMALL_MATH_TF32 ? 1 : 2][lg];
+    if (c) return c;
+    if (lg == 0) return c = ctx->sm_count;
+    const Kernel k = kernel_of(math);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctx->sm_count / (1 << lg) * (1 << lg)); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = ctx->max_smem_optin - 1024;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1u << lg; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->max_smem_optin - 1024);
+    if (cudaOccupancyMaxActiveClusters(&c, k, &cfg) != cudaSuccess || c < 1) { cudaGetLastError(); c = 1; }
+    return c;
+}
+
+// Where the run is faster on chip than layer by layer.  `one_round`: every image has its own thread blocks; with more images
+// than that the layer kernels, which see the whole batch, win.  Measured (us, on chip / layer by layer): keyword spotting,
+// batch 37: FP32 50 / 70, TF32 36 / 51, 3xTF32 41 / 58, batch 148 39 / 74 in TF32; depthwise-separable network, batch 1: FP32 129 /
+// 178, TF32 105 / 103, batch 37 TF32 138 / 135: its filters (700 KB) stream through every block, which the tensor-core kernels
+// share between images; residual network, batch 1 (8 blocks per image): FP32 97 / 115, 3xTF32 73 / 66, batch 16 (4 blocks) FP32 125 / 124:
+// without depthwise layers nothing is computed without an exchange.
+bool worth_it(const Args &a, unsigned math, int G, bool one_round) {
+    if (!one_round) return false;
+    size_t filters = 0;
+    int depthwise = 0;
+    for (int i = 0; i < a.n_ops; ++i) {
+        depthwise += a.op[i].kind == kDw ? 1 : 0;
+        if (a.op[i].kind == kConv) filters += (size_t)a.op[i].C * a.op[i].K * a.op[i].FH * a.op[i].FW * 4;
+    }
+    if (!depthwise) return math == SMALL_MATH_FP32 && G == 8;
+    return math == SMALL_MATH_FP32 || filters <= 256 * 1024;
+}
+
+const Plan *find_plan(small_ctx *ctx, const small_layer *layers, int n, int from, int N) {
+    State &s = state_of(ctx);
+    const int head[2] = {N, from};
+    const size_t lb = sizeof(small_layer) * (size_t)n;
+    for (size_t i = 0; i < s.plans.size(); ++i) {
+        const Entry &e = s.plans[i];
+        if (e.key.size() == lb + sizeof(head) && !memcmp(e.key.data(), head, sizeof(head)) && !memcmp(e.key.data() + sizeof(head), layers, lb)) {
+            if (i) std::rotate(s.plans.begin(), s.plans.begin() + i, s.plans.begin() + i + 1);
+            return &s.plans.front().p;
+        }
+    }
+    Entry e;
+    e.key.resize(lb + sizeof(head));
+    memcpy(e.key.data(), head, sizeof(head));
+    memcpy(e.key.data() + sizeof(head), layers, lb);
+    e.p.ok = false;
+    for (int s0 = from; s0 < n; ++s0) {
+        e.p = plan_run(layers, n, s0, N, ctx->max_smem_optin, true);
+        if (!e.p.ok) e.p = plan_run(layers, n, s0, N, ctx->max_smem_optin, false);
+        if (e.p.ok) break;
+    }
+    if (e.p.ok) {
+        Args &a = e.p.a;
+        double best = 0.0;
+        int best_g = 0;
+        for (int lg = 0; lg < 4; ++lg) {
+            const int c = clusters_of(ctx, e.p.math, lg);
+            const double t = (double)ceil_div(N, c) * tile_ops(a, e.p.math, 1 << lg);
+            if (t > 0.0 && (!best_g || t < best)) { best = t; best_g = 1 << lg; }
+        }
+        a.G = best_g;
+        if (!best_g || !worth_it(a, e.p.math, best_g, N <= clusters_of(ctx, e.p.math, best_g == 8 ? 3 : best_g == 4 ? 2 : best_g - 1))) e.p.ok = false;
+        else tile_ops(a, e.p.math, best_g);
+    }
+    if (s.plans.size() >= 32) s.plans.pop_back();
+    s.plans.insert(s.plans.begin(), std::move(e));
+    return &s.plans.front().p;
+}
+
+}  // namespace
+
+void free_resident_state(small_ctx *ctx) {
+    delete static_cast<State *>(ctx->resident_state);
+    ctx->resident_state = nullptr;
+}
+
+int resident_from(small_ctx *ctx, const small_layer *layers, int n, int from, int N) {
+    const Plan *p = find_plan(ctx, layers, n, from, N);
+    return p->ok ? p->from : -1;
+}
+
+int launch_resident(small_ctx *ctx, const small_layer *layers, int n, int from, int N, const std::function<const float *(int)> &rd,
+                    const std::function<float *(int)> &wr, cudaStream_t st) {
+    const Plan *p = find_plan(ctx, layers, n, from, N);
+    if (!p->ok) return SMALL_ERR_UNSUPPORTED;
+    Args a = p->a;
+    for (int i = 0; i < a.n_in; ++i) a.in[i].g = rd(p->in_slot[i]);
+    a.out = wr(p->out_slot);
+    const Kernel k = kernel_of(p->math);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->max_smem_optin - 1024);
+    if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SMALL_ERR_CUDA; }
+    int lg = 0;
+    while ((1 << lg) < a.G) ++lg;
+    const int clusters = std::min(N, clusters_of(ctx, p->math, lg));
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(clusters * a.G)); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = p->smem; cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)a.G; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = ctx->dependent ? 2 : 1;
+    e = cudaLaunchKernelEx(&cfg, k, a);
+    (void)e;                                             // picked up by check_launch through cudaGetLastError
+    return check_launch(ctx);
+}
+
+}  // namespace small

@@ -1,0 +1,58 @@
+"""Runs of layers kept on chip as one kernel, against the oracle and against the same network launched layer by layer: ragged
+channel counts and planes, strides, residual joins, one to eight thread blocks per image and several images per block."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import nets
+from synth import configs
+from synth.configs import P0, P1, _conv, _dw, _fc, _gap
+from paper_2303_04769_b200 import binding as B
+from paper_2303_04769_b200.net import Net
+from gpu_util import TOL, ctx, from_blk, rel_err, to_blk
+
+pytestmark = pytest.mark.gpu
+
+
+def separable(H, W, C, K):
+    """Depthwise and 1x1 layers whose channels are no multiples of anything, a 3x3 behind them, a strided pair."""
+    L = [_conv("c0", "in", "a", C, K, 1, 1, P0, True), _dw("d1", "a", "b", K, 1), _conv("p1", "b", "c", K, C, 1, 1, P0, True),
+         _dw("d2", "c", "d", C, 2), _conv("p2", "d", "e", C, K + 9, 1, 1, P0, True), _conv("c3", "e", "f", K + 9, 24, 3, 1, P1, True),
+         _gap("gap", "f", "g", 24), _fc("fc", "g", "out", 24, 37)]
+    return dict(name="separable", batch=1, input=(C, H, W), input_dist=("uniform", -1.0, 1.0), weight_dist="he_normal", layers=L)
+
+
+def joined():
+    """A residual join and a strided shortcut without depthwise layers (FP32, one image on eight blocks)."""
+    L = [_conv("a", "in", "x", 20, 12, 3, 1, P1, True), _conv("b", "x", "y", 12, 40, 3, 2, P1, True), _conv("s", "x", "z", 12, 40, 1, 2, P0, False),
+         _conv("c", "y", "z", 40, 40, 3, 1, P1, True, accumulate=True), _gap("gap", "z", "g", 40), _fc("fc", "g", "out", 40, 5)]
+    return dict(name="joined", batch=1, input=(20, 13, 11), input_dist=("uniform", -1.0, 1.0), weight_dist="he_normal", layers=L)
+
+
+@pytest.mark.parametrize("math", ["fp32", "tf32", "3xtf32"])
+@pytest.mark.parametrize("net,batch", [(separable(9, 7, 20, 33), 1), (separable(6, 16, 40, 64), 30), (separable(5, 5, 8, 100), 70),
+                                       (separable(11, 3, 33, 17), 148), (joined(), 3)])
+def test_on_chip_runs_match(net, batch, math):
+    params = configs.make_params(net)
+    x = configs.make_input(net, batch)
+    ref = nets.run_net(net, params, x)["out"]
+    blk = to_blk(x)
+    got = from_blk(Net(ctx(), net, params, batch=batch, math=math).run(blk), batch, *ref.shape[1:])
+    apart = from_blk(Net(ctx(), net, params, batch=batch, math=math, fuse_poolfc=False).run(blk), batch, *ref.shape[1:])
+    assert rel_err(got, ref) <= TOL[math] and rel_err(apart, ref) <= TOL[math]
+    assert B.small_device_status(ctx()) == 0
+
+
+def test_on_chip_run_repeats_its_bits_in_a_graph():
+    net = configs.kws_cnn(batch=40)
+    gnet = Net(ctx(), net, configs.make_params(net), math="3xtf32")
+    blk = to_blk(configs.make_input(net))
+    want = gnet.run(blk).clone()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        out = gnet.run(blk)
+    for _ in range(3):
+        out.fill_(float("nan"))
+        g.replay()
+        assert torch.equal(out, want)
