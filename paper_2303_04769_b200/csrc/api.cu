@@ -109,6 +109,7 @@ SMALL_API int small_init(int device, small_ctx **out) {
     c->mma_cache = nullptr;
     c->i8_cache = nullptr;
     c->direct_cache = nullptr;
+    c->dw_cache = nullptr;
     c->path_cache = nullptr;
     c->resident_state = nullptr;
     c->wait_iters = 1u << 22;     // with the polls' nanosleep back-off: seconds
@@ -152,6 +153,7 @@ SMALL_API int small_shutdown(small_ctx *ctx) {
     free_mma_cache(ctx);
     free_i8_cache(ctx);
     free_direct_cache(ctx);
+    free_dw_cache(ctx);
     delete static_cast<PathCache *>(ctx->path_cache);
     free_resident_state(ctx);
     if (ctx->ev_fork) cudaEventDestroy(static_cast<cudaEvent_t>(ctx->ev_fork));

@@ -25,6 +25,7 @@ struct small_ctx {
     void *mma_cache;         // the same for the warp-level tensor-core kernel; conv_mma.cu
     void *resident_state;    // plans of the resident network kernel; net_resident.cu
     void *direct_cache;      // the same for the register-tiled FP32 kernel; conv_direct.cu
+    void *dw_cache;          // the same for the depthwise 3x3 kernel; dwconv.cu
     void *path_cache;        // kernel family per shape, mode and path setting; api.cu
     void *i8_cache;          // the same for the quantised convolution; conv_i8.cu
     void *static_workspace;  // device address of the library's built-in workspace array on this device (net_static.cu)
@@ -102,6 +103,7 @@ void free_tc_cache(small_ctx *);             // conv_tc.cu
 void free_mma_cache(small_ctx *);            // conv_mma.cu
 void free_i8_cache(small_ctx *);             // conv_i8.cu
 void free_direct_cache(small_ctx *);         // conv_direct.cu
+void free_dw_cache(small_ctx *);             // dwconv.cu
 void free_resident_state(small_ctx *);       // net_resident.cu
 int resolve_static_workspace(small_ctx *);   // net_static.cu; called by small_init with the context's device current
 
