@@ -386,12 +386,15 @@ static int choose_path(const small_ctx *ctx, const Geom &g, unsigned math, bool 
     // 12.2 / 15.8; 1x1 stride 2 16->32 10.2 / 14.3 against 7.1 / 7.6; 3x3 32->32 on 16x16 planes 15.5 / 27.2 against
     // 14.8 / 23.9, on 8x8 planes 10.2 / 13.4 against 8.1 / 9.1; 1x1 stride 2 32->64 8.3 / 9.8 against 7.1 / 7.7; but 3x3
     // stride 2 32->64 15.4 / 18.4 against 15.4 / 23.6, so 3x3 layers with more than 32 filters stay where they were).
-    // 3x3 in 3xTF32 with more than 16 channels and more than 16 filters is the block-level kernel's at stride 1 (32->32 on 16x16
-    // planes, batch 1 / 8 / 64 / 256: 8.3 / 8.5 / 12.4 / 22.6 against 10.3 / 10.3 / 12.4 / 24.7; on 8x8 planes 8.3 / 8.3 / 8.3 /
-    // 12.4 against 10.3 / 10.3 / 10.3 / 12.4): 108 dependent MMAs per fragment are the warp's chain, the block's roles share them.
-    const bool block_3x = math == SMALL_MATH_3XTF32 && g.FH == 3 && g.FW == 3 && g.S == 1 && g.C > 16 && g.K > 16 && out_aligned32 &&
-                          conv_tc_supported(g, true) && !(ctx && ctx->conv_path == SMALL_CONV_PATH_WARP_MMA);
-    if (!block_3x && !(ctx && (ctx->conv_path == SMALL_CONV_PATH_TENSOR || ctx->conv_path == SMALL_CONV_PATH_CUDA_CORES)) &&
+    // 3x3 at stride 1 with more than 16 channels and more than 16 filters is the block-level kernel's in 3xTF32 (32->32, us,
+    // warp-level against block-level: 16x16 planes, batch 1 / 8 / 64 / 256 10.3 / 10.3 / 12.4 / 24.7 against 8.3 / 8.5 / 12.4 /
+    // 22.6, batch 300 5x5 18.4 / 9.1, 13x13 32.8 / 19.5, 24x23 69.9 / 34.9, 33x33 145 / 62, batch 60 56x56 61.6 / 38.2, 30x70
+    // 52.4 / 32.8) up to 72 columns (80x80 127 against 176: fewer of its strips fit), and in TF32 on large planes of many
+    // pixels in all (batch 60 32x32 12.5 / 14.4, 48x48 27.1 / 19.7, 30x70 24.7 / 18.5, 80x80 55.4 / 34.9; batch 256 16x16 14.2 / 14.4).
+    const bool block = g.FH == 3 && g.FW == 3 && g.S == 1 && g.C > 16 && g.K > 16 && out_aligned32 &&
+                       (math == SMALL_MATH_3XTF32 ? g.OW <= 72 : g.OW >= 30 && (long long)g.N * g.OH * g.OW >= 100000) &&
+                       conv_tc_supported(g, math == SMALL_MATH_3XTF32);
+    if (!block && !(ctx && (ctx->conv_path == SMALL_CONV_PATH_TENSOR || ctx->conv_path == SMALL_CONV_PATH_CUDA_CORES)) &&
         ((ctx && ctx->conv_path == SMALL_CONV_PATH_WARP_MMA) || g.K <= 32 || (g.K <= 64 && g.FH * g.FW == 1)) && conv_mma_supported(g, math == SMALL_MATH_3XTF32))
         return 4;
     if (ctx && ctx->conv_path == SMALL_CONV_PATH_WARP_MMA) return direct ? 1 : 2;
