@@ -81,11 +81,12 @@ static bool slot_dead_after(const small_layer *layers, int n_layers, int from, i
     return true;
 }
 
-// Fusing a depthwise 3x3 with the 1x1 convolution behind it pays where the two separate launches are short (measured:
-// a few percent on the depthwise-separable network at batch 64, a loss on large intermediate tensors, where the fused
-// kernel's eight depthwise warps per SM cannot keep up with two full-size kernels); above this size of the
-// intermediate tensor the pair runs as two layers unless SMALL_FUSE_DWPW_ALWAYS is set.
-static const size_t kFuseDwpwMaxBytes = 24u << 20;
+// Fusing a depthwise 3x3 with the 1x1 convolution behind it pays where launches are all there is to the two layers, at a few
+// small images: the fused kernel has eight depthwise warps per SM and half the strips, the two kernels have whole SMs.  Networks,
+// us, fused / separate: depthwise-separable 3xTF32 batch 1 121.5 / 122.0, 4 125.9 / 122.2, 16 146 / 142, 64 185 / 174, TF32 batch 4
+// 113.7 / 114.8, 64 166 / 158; keyword spotting 3xTF32 batch 150 105 / 67, 400 156 / 100, 700 234 / 140, TF32 146 / 128.
+static const int kFuseDwpwMaxImages = 4;
+static const size_t kFuseDwpwMaxBytes = 1u << 20;      // of the intermediate tensor
 
 // Two layers may run at the same time when neither writes a tensor the other one reads or writes.
 static bool independent(const small_layer &A, const small_layer &Bn) {
@@ -110,7 +111,7 @@ static int fused_pair(const small_ctx *ctx, const small_layer *layers, int n_lay
         if ((Bn.flags & SMALL_ACCUMULATE) || Bn.C != A.C || math == SMALL_MATH_FP32) return 0;
         if (make_geom(g, N, A.C, A.C, A.H, A.W, 3, 3, A.stride, A.pad_t, A.pad_b, A.pad_l, A.pad_r)) return 0;
         if (Bn.H != g.OH || Bn.W != g.OW) return 0;
-        if (!(ctx->net_fusion & SMALL_FUSE_DWPW_ALWAYS) && sizeof(float) * packed_elems(N, A.C, g.OH, g.OW) > kFuseDwpwMaxBytes) return 0;
+        if (!(ctx->net_fusion & SMALL_FUSE_DWPW_ALWAYS) && (N > kFuseDwpwMaxImages || sizeof(float) * packed_elems(N, A.C, g.OH, g.OW) > kFuseDwpwMaxBytes)) return 0;
         return small_dwpw_fused(N, A.C, Bn.K, A.H, A.W, A.stride, A.pad_t, A.pad_b, A.pad_l, A.pad_r, math) ? SMALL_OP_DWPW : 0;
     }
     if (A.op == SMALL_OP_CONV && Bn.op == SMALL_OP_POOL && (ctx->net_fusion & SMALL_FUSE_CONVPOOL)) {
