@@ -30,8 +30,8 @@
 // transform between the copy and the MMAs (see the X3 and DW template flags).
 //
 // Persistent CTAs (one per SM) walk the tile list with stride gridDim.x.  Roles: warp 0 = TMA producer for input
-// strips, warp 2 = TMA producer for filter tiles, warps 1 and 3 = MMA issuers (one thread each; a tile's chains are
-// split between them), warps 4-7 = epilogue, warps 8 and up = strip transform where there is one.  The producers run
+// strips, warp 2 = TMA producer for filter tiles, warp 1 = MMA issuer (each a uniform warp whose thread is elected
+// at the instruction), warps 4-7 = epilogue, warps 8 and up = strip transform where there is one.  The producers run
 // ahead across tiles; accumulator slots are handed back to the issuers as soon as the epilogue has read them out of
 // tensor memory, so the next tile's MMAs overlap the current tile's stores (one-slot tiles alternate between the two
 // slots).  Every mbarrier wait is bounded; on expiry the kernel records SMALL_ERR_TIMEOUT in the context's status
