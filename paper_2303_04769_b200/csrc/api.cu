@@ -391,8 +391,13 @@ static int choose_path(const small_ctx *ctx, const Geom &g, unsigned math, bool 
     // 22.6, batch 300 5x5 18.4 / 9.1, 13x13 32.8 / 19.5, 24x23 69.9 / 34.9, 33x33 145 / 62, batch 60 56x56 61.6 / 38.2, 30x70
     // 52.4 / 32.8) up to 72 columns (80x80 127 against 176: fewer of its strips fit), and in TF32 on large planes of many
     // pixels in all (batch 60 32x32 12.5 / 14.4, 48x48 27.1 / 19.7, 30x70 24.7 / 18.5, 80x80 55.4 / 34.9; batch 256 16x16 14.2 / 14.4).
-    const bool block = g.FH == 3 && g.FW == 3 && g.S == 1 && g.C > 16 && g.K > 16 && out_aligned32 &&
-                       (math == SMALL_MATH_3XTF32 ? g.OW <= 72 : g.OW >= 30 && (long long)g.N * g.OH * g.OW >= 100000) &&
+    // So are 1x1 layers of 33 to 64 filters at stride 1 from some 32,000 pixels on, where the warp-level kernel reads every pixel
+    // once per 32 filters (32->64, TF32 / 3xTF32, warp-level against block-level: 12x12 batch 64 6.2 / 6.3 against 8.3 / 8.3, batch 256
+    // 12.4 / 14.3 against 10.2 / 12.4, 28x28 batch 16 6.2 / 6.4 against 8.3 / 8.5, batch 256 32.8 / 39.1 against 24.8 / 26.9).
+    const long long pixels = (long long)g.N * g.OH * g.OW;
+    const bool block = g.S == 1 && g.C > 16 && out_aligned32 &&
+                       (g.FH == 3 && g.FW == 3 ? g.K > 16 && (math == SMALL_MATH_3XTF32 ? g.OW <= 72 : g.OW >= 30 && pixels >= 100000)
+                                               : g.FH == 1 && g.FW == 1 && g.K > 32 && pixels >= 32768) &&
                        conv_tc_supported(g, math == SMALL_MATH_3XTF32);
     if (!block && !(ctx && (ctx->conv_path == SMALL_CONV_PATH_TENSOR || ctx->conv_path == SMALL_CONV_PATH_CUDA_CORES)) &&
         ((ctx && ctx->conv_path == SMALL_CONV_PATH_WARP_MMA) || g.K <= 32 || (g.K <= 64 && g.FH * g.FW == 1)) && conv_mma_supported(g, math == SMALL_MATH_3XTF32))
