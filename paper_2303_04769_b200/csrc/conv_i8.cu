@@ -437,7 +437,9 @@ struct I8Plan { I8Args a; int ch; unsigned grid; size_t smem; int es_w, es_h; bo
 
 int floor_half(int v) { return v >= 0 ? v / 2 : -((1 - v) / 2); }
 
-// The cheapest tiling over the chunks per tile (1, 2 or 4) and the filters per tile (32 to 128).
+// The cheapest tiling over the chunks per tile (1, 2 or 4) and the filters per tile (32 to 128).  Where the filter tiles share
+// the SMs, a block of each walks its part of the pixel tiles; more filter tiles than SMs (above 18,944 filters on 148 SMs, any
+// tiling) take one block each, which walks all pixel tiles, and the blocks follow one another over the SMs.
 I8Plan plan_i8(const Geom &g, size_t max_smem, int sms) {
     I8Plan best{};
     best.ok = false;
@@ -467,6 +469,7 @@ I8Plan plan_i8(const Geom &g, size_t max_smem, int sms) {
     const int maxh = b.ptv > pbv ? b.ptv : pbv, minh = b.ptv < pbv ? b.ptv : pbv;
     const int lim = 256 / g.S;                                   // pixels a box spans in one dimension
     double best_cost = 0.0;
+    for (int many = 0; many < 2 && !best.ok; ++many)         // first tilings of no more filter tiles than SMs, else any
     for (int ch = 4; ch >= 1; ch >>= 1) {
         I8Args a = b;
         const int px = ch * 128;
@@ -524,7 +527,7 @@ I8Plan plan_i8(const Geom &g, size_t max_smem, int sms) {
             if (a.slots > kMaxSlots) a.slots = kMaxSlots;
             a.epi = a.slots * ch >= kEpi ? kEpi : 2;
             a.n_tiles = ceil_div(g.KB * 32, kt);
-            if (a.n_tiles > sms) continue;
+            if ((a.n_tiles > sms) != (many == 1)) continue;
             a.b_box = (uint32_t)(kt + kOnesRows) * 32u;
             const bool table = classes * kt * 4 <= 32 * 1024;
             a.row_classes = table ? (g.pt + 1) * (g.pb + 1) : 0; a.col_classes = table ? (g.pl + 1) * (g.pr + 1) : 0;
@@ -543,8 +546,8 @@ I8Plan plan_i8(const Geom &g, size_t max_smem, int sms) {
             if (a.a_stages > kMaxA) a.a_stages = kMaxA;
             // cycles of the busiest block: MMAs (128 x N x 32: 32 + N / 4 cycles of operand reads, some more to issue)
             // beside the requantisation (about 350 cycles per 128 pixels and 32 filters for one group of four warps)
-            const int per = sms / a.n_tiles;
-            const double tiles = (double)ceil_div(a.m_tiles, per < a.m_tiles ? per : a.m_tiles);
+            const int per = many ? 1 : sms / a.n_tiles;
+            const double tiles = (double)ceil_div(a.m_tiles, per < a.m_tiles ? per : a.m_tiles) * ceil_div(a.n_tiles, sms);
             const double mma = (double)ch * a.CB * a.T * (48.0 + (kt + kOnesRows) / 4.0);
             const double epi = (double)ch * (kt / 32) * (a.epi == kEpi ? 200.0 : 300.0);
             const double load = ((double)a.CB * a.n_phase * a.strip_px * 32 + (a.resident ? 0.0 : (double)all_b)) / 40.0;

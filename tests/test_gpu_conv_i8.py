@@ -1,6 +1,7 @@
 """The quantised convolution's tilings at their edges, bit-exact against the oracle: column tiles of wide planes, filter tiles
 with a remainder, filters that stream instead of staying resident, several images per tile, windows whose border classes
-are too many for the table, windows taller than one input box, and every form of the requantising shift."""
+are too many for the table, windows taller than one input box, more filter tiles than the chip has SMs, and every form of the
+requantising shift."""
 import numpy as np
 import pytest
 import torch
@@ -22,6 +23,8 @@ CASES = [  # N, C, K, H, W, FH, FW, S, pad, shift
     (1, 8, 40, 25, 12, 9, 3, 1, (8, 8, 2, 2), 33),       # 729 border classes
     (1, 4, 8, 200, 5, 180, 1, 1, (3, 0, 0, 0), 40),      # a tall window
     (1, 4, 8, 256, 3, 256, 1, 2, (1, 0, 0, 0), 41),      # the tallest, over phase planes: two boxes per strip
+    (2, 5, 18977, 12, 11, 3, 3, 1, (1, 1, 1, 1), 39),    # more filter tiles than SMs
+    (3, 33, 37900, 7, 5, 1, 1, 2, (0, 0, 0, 0), 36),     # more than two per SM, the last one ragged
 ]
 
 
