@@ -167,10 +167,12 @@ __global__ void __launch_bounds__(kDwThreads, 2) dwconv3x3_tma_kernel(const __gr
     bool alive = true;
     ulonglong2 w[9], bias2 = make_ulonglong2(0ull, 0ull);
     ulonglong2 px[kPx], A[2], B[2];
-    // The next input row.  Its slot is released at the row after it: by then the sums have taken the pixels, which a release
-    // right behind the loads does not wait for.
+    // The next input row.  Its slot is released at the row after it, so that no warp waits for its own loads to release it.  One
+    // lane hands the slot back for the warp: the barrier in front of it puts the other lanes' reads of the slot before its arrival
+    // (41.8 us with it and without, 64 channels on 56 x 56, batch 128).
     auto load = [&]() {
         alive = sm100::mbar_wait_uniform(full + 8 * s, par, &abort_flag, a.status, a.wait_iters);
+        __syncwarp();
         if (prev >= 0 && (threadIdx.x & 31) == 0) sm100::mbar_arrive(empty + 8 * prev);
         const uint8_t *from = mine + s * a.slot_bytes;
 #pragma unroll

@@ -39,3 +39,26 @@ def test_depthwise_3x3(case):
         B.small_dwconv2d(ctx(), xb, wb, dev(b), out, N, C, H, W, 3, 3, S, pad, B.RELU)
         assert rel_err(from_blk(out, N, C, OH, OW), ref) <= 1e-5
         assert pad_lanes_are_zero(out, N, C, OH, OW)
+
+
+@pytest.mark.parametrize("case", [(128, 64, 56, 56, 1), (96, 64, 25, 5, 1), (64, 128, 56, 56, 2), (200, 96, 7, 7, 1)])
+def test_depthwise_3x3_repeats_its_bits(case):
+    """A slot of the ring that were refilled while a lane still reads it would change bits now and then: the same layer some
+    hundred times, back to back on a full chip, against its own first result (which the oracle checks on one image)."""
+    N, C, H, W, S = case
+    x, w, b = synth.uniform((N, C, H, W), -1, 1, 4, seed=77), synth.uniform((C, 3, 3), -1, 1, 5, seed=77), synth.uniform((C,), -1, 1, 6, seed=77)
+    OH, OW = B.small_out_size(H, 3, S, 1, 1), B.small_out_size(W, 3, S, 1, 1)
+    wb, bias = torch.empty(B.small_dw_weight_elems(C, 3, 3), device="cuda"), dev(b)
+    B.small_pack_dw_weights(ctx(), dev(w), wb, C, 3, 3)
+    xb = to_blk(x)
+    out, first, wrong = new_blk(N, C, OH, OW), None, torch.zeros((), dtype=torch.int64, device="cuda")
+    for i in range(400):
+        out.fill_(float("nan"))
+        B.small_dwconv2d(ctx(), xb, wb, bias, out, N, C, H, W, 3, 3, S, (1, 1, 1, 1), B.RELU)
+        if first is None:
+            first = out.clone()
+        wrong += (out.view(torch.int32) != first.view(torch.int32)).sum()
+    assert int(wrong) == 0
+    n = N // 2
+    assert rel_err(from_blk(first, N, C, OH, OW)[n:n + 1], oracle.dwconv2d(x[n:n + 1], w, b, S, (1, 1, 1, 1), True)) <= 1e-5
+    assert B.small_device_status(ctx()) == 0
