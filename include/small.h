@@ -419,7 +419,11 @@ size_t small_net_host_staging_bytes(int N, int C, int H, int W, int outC, int ou
  * `stream` before reading the result, and keep in_nchw_host unchanged until then.
  * The input copy runs on a stream of the context's own into one of two staging areas of the workspace, so that with
  * back-to-back calls on one workspace the copy of a call's input overlaps the layers of the call before it; the caller's
- * stream waits for the copy by an event.  (While `stream` is being captured the copy stays on `stream`.) */
+ * stream waits for the copy by an event.  (While `stream` is being captured the copy stays on `stream`.)  Several networks may
+ * be called in turn, each on a workspace of its own: up to eight keep that overlap.  The first call on a workspace waits for all
+ * work queued on `stream` before it; from then on the part of the workspace behind its first small_net_workspace_bytes belongs
+ * to these calls, and memory that was used for something else meanwhile (freed and allocated again, say) may be handed back
+ * as the same workspace only when that use has finished. */
 int small_run_net_host(small_ctx *ctx, const small_layer *layers, int n_layers, int N,
                        const float *in_nchw_host, int C, int H, int W,
                        float *out_nchw_host, int outC, int outH, int outW,

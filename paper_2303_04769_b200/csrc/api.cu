@@ -131,14 +131,18 @@ SMALL_API int small_init(int device, small_ctx **out) {
         if (cudaEventCreateWithFlags(&f, cudaEventDisableTiming) == cudaSuccess) c->ev_fork = f;
         if (cudaEventCreateWithFlags(&j, cudaEventDisableTiming) == cudaSuccess) c->ev_join = j;
         if (!c->side_stream || !c->ev_fork || !c->ev_join) c->branch_overlap = 0;
-        c->copy_stream = nullptr; c->host_ws = nullptr; c->host_parity = 0; c->host_used[0] = c->host_used[1] = 0;
+        c->copy_stream = c->ev_h2d = c->ev_start = nullptr;
         cudaStream_t cs;
         bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess;
-        for (int i = 0; i < 2; ++i) {
-            cudaEvent_t a = nullptr, b = nullptr;
-            ok = ok && cudaEventCreateWithFlags(&a, cudaEventDisableTiming) == cudaSuccess && cudaEventCreateWithFlags(&b, cudaEventDisableTiming) == cudaSuccess;
-            c->ev_h2d[i] = a; c->ev_pack[i] = b;
-        }
+        auto event = [&ok](void *&ev) {
+            cudaEvent_t e = nullptr;
+            ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+            ev = e;
+        };
+        event(c->ev_h2d);
+        event(c->ev_start);
+        for (small_host_stage &h : c->host_stage)
+            for (int i = 0; i < 2; ++i) event(h.ev_read[i]);
         if (ok) c->copy_stream = cs;
     }
     *out = c;
@@ -159,10 +163,11 @@ SMALL_API int small_shutdown(small_ctx *ctx) {
     if (ctx->ev_fork) cudaEventDestroy(static_cast<cudaEvent_t>(ctx->ev_fork));
     if (ctx->ev_join) cudaEventDestroy(static_cast<cudaEvent_t>(ctx->ev_join));
     if (ctx->side_stream) cudaStreamDestroy(static_cast<cudaStream_t>(ctx->side_stream));
-    for (int i = 0; i < 2; ++i) {
-        if (ctx->ev_h2d[i]) cudaEventDestroy(static_cast<cudaEvent_t>(ctx->ev_h2d[i]));
-        if (ctx->ev_pack[i]) cudaEventDestroy(static_cast<cudaEvent_t>(ctx->ev_pack[i]));
-    }
+    if (ctx->ev_h2d) cudaEventDestroy(static_cast<cudaEvent_t>(ctx->ev_h2d));
+    if (ctx->ev_start) cudaEventDestroy(static_cast<cudaEvent_t>(ctx->ev_start));
+    for (small_host_stage &h : ctx->host_stage)
+        for (int i = 0; i < 2; ++i)
+            if (h.ev_read[i]) cudaEventDestroy(static_cast<cudaEvent_t>(h.ev_read[i]));
     if (ctx->copy_stream) cudaStreamDestroy(static_cast<cudaStream_t>(ctx->copy_stream));
     delete ctx;
     return SMALL_OK;

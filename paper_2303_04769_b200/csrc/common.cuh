@@ -11,6 +11,18 @@
 #define SMALL_CB 32          // channel block of the blocked layout (floats): one 128-byte line
 #define SMALL_API extern "C" __attribute__((visibility("default")))
 
+// A workspace that small_run_net_host was called on: its two input staging areas (see there).
+struct small_host_stage {
+    const char *base;        // nullptr: entry free
+    size_t bytes;            // of the workspace that the calls use
+    const char *in;          // the first staging area; the second one lies behind it
+    size_t in_bytes;
+    int next, used[2];       // area of the next call; whether an area was read yet
+    int ordered;             // a call on this memory was captured: its replays read the first area at times unknown here
+    void *ev_read[2];        // cudaEvent_t: the layer that read the area last has finished
+    unsigned long long last; // call that used the entry last
+};
+
 struct small_ctx {
     int device;
     int last_cuda;           // last cudaError_t / CUresult seen
@@ -31,8 +43,10 @@ struct small_ctx {
     void *static_workspace;  // device address of the library's built-in workspace array on this device (net_static.cu)
     int branch_overlap;      // small_run_net runs independent neighbouring layers side by side (side stream)
     void *side_stream, *ev_fork, *ev_join;   // cudaStream_t / cudaEvent_t of that
-    void *copy_stream, *ev_h2d[2], *ev_pack[2];   // small_run_net_host: input copies on their own stream, two staging areas
-    void *host_ws; int host_parity, host_used[2];
+    void *copy_stream, *ev_h2d, *ev_start;   // small_run_net_host: input copies on their own stream
+    small_host_stage host_stage[8];          // the workspaces it was called on latest
+    unsigned long long host_calls;
+    int host_ordered;        // an entry with `ordered` set had to make room: every copy keeps the caller's order from then on
     unsigned net_fusion;     // SMALL_FUSE_*: which neighbouring layers small_run_net runs as one fused layer
     int conv_path;           // SMALL_CONV_PATH_*: automatic, or one kernel family forced where it takes the shape
     int fc_chain_tile;       // images per thread block of the fused chain of full reductions: 0 = by batch size, else 32, 64 or 128

@@ -346,11 +346,32 @@ SMALL_API size_t small_net_host_staging_bytes(int N, int C, int H, int W, int ou
            round256(sizeof(float) * packed_elems(N, outC, outH, outW)) + round256(sizeof(float) * (size_t)N * outC * outH * outW);
 }
 
+// The staging areas of a workspace: the entry of the calls before on the same memory, laid out alike, or a new one (`fresh`),
+// which takes the place of every entry whose memory it overlaps, or of the one unused for longest.
+static small_host_stage &host_stage(small_ctx *ctx, const char *base, size_t bytes, const char *in, size_t in_bytes, bool &fresh) {
+    const unsigned long long now = ++ctx->host_calls;
+    for (small_host_stage &h : ctx->host_stage)
+        if (h.base == base && h.bytes == bytes && h.in == in && h.in_bytes == in_bytes) { fresh = false; h.last = now; return h; }
+    int ordered = 0;
+    small_host_stage *pick = nullptr;
+    auto rank = [](const small_host_stage &h) { return h.base ? (h.ordered ? 2 : 1) : 0; };
+    for (small_host_stage &h : ctx->host_stage) {
+        if (h.base && base < h.base + h.bytes && h.base < base + bytes) { ordered |= h.ordered; h.base = nullptr; }
+        if (!pick || rank(h) < rank(*pick) || (rank(h) == rank(*pick) && h.last < pick->last)) pick = &h;
+    }
+    if (rank(*pick) == 2) ctx->host_ordered = 1;
+    pick->base = base; pick->bytes = bytes; pick->in = in; pick->in_bytes = in_bytes;
+    pick->next = pick->used[0] = pick->used[1] = 0; pick->ordered = ordered; pick->last = now;
+    fresh = true;
+    return *pick;
+}
+
 // The host-buffer call keeps the copy engine busy next to the SMs: the NCHW input goes to one of two staging areas on
 // the context's copy stream, so the copy of call i + 1 runs while the layers of call i are still computing on the caller's
 // stream; the caller's stream waits for its own input by an event, and a staging area is not overwritten before the
-// pack that read it last has finished.  Everything else (pack, layers, unpack, the result's copy back) stays in order on
-// the caller's stream.  While the caller's stream is being captured, the input copy stays on that stream.
+// layer that read it last has finished.  The first copy into a workspace waits for everything in front of it on the caller's
+// stream, which may still use that memory for something else, and so does every copy once a call was captured on it.  Everything else (pack, layers, unpack, the result's copy back)
+// stays in order on the caller's stream.  While the caller's stream is being captured, the input copy stays on that stream.
 SMALL_API int small_run_net_host(small_ctx *ctx, const small_layer *layers, int n_layers, int N,
                                  const float *in_host, int C, int H, int W,
                                  float *out_host, int outC, int outH, int outW,
@@ -383,18 +404,33 @@ SMALL_API int small_run_net_host(small_ctx *ctx, const small_layer *layers, int 
     cudaStreamIsCapturing(st, &cap);
     const bool piped = ctx->copy_stream && cap == cudaStreamCaptureStatusNone;
     int par = 0;
+    bool fresh = true;
+    small_host_stage *stage = nullptr;
+    if (ctx->copy_stream) {
+        stage = &host_stage(ctx, static_cast<const char *>(workspace), net_b + stage_b, reinterpret_cast<const char *>(d_in_nchw[0]), in_nchw_b, fresh);
+        if (!piped) stage->ordered = 1;
+        if (stage->ordered || ctx->host_ordered) fresh = true;
+    }
     if (piped) {
-        if (ctx->host_ws != workspace) { ctx->host_ws = workspace; ctx->host_parity = 0; ctx->host_used[0] = ctx->host_used[1] = 0; }
-        par = ctx->host_parity;
+        par = stage->next;
         cudaStream_t cs = static_cast<cudaStream_t>(ctx->copy_stream);
-        if (ctx->host_used[par]) e = cudaStreamWaitEvent(cs, static_cast<cudaEvent_t>(ctx->ev_pack[par]), 0);
+        if (fresh) {           // behind everything queued so far
+            e = cudaEventRecord(static_cast<cudaEvent_t>(ctx->ev_start), st);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, static_cast<cudaEvent_t>(ctx->ev_start), 0);
+        } else if (stage->used[par]) {
+            e = cudaStreamWaitEvent(cs, static_cast<cudaEvent_t>(stage->ev_read[par]), 0);
+        }
         if (e == cudaSuccess) e = cudaMemcpyAsync(d_in_nchw[par], in_host, in_nchw_b, cudaMemcpyHostToDevice, cs);
-        if (e == cudaSuccess) e = cudaEventRecord(static_cast<cudaEvent_t>(ctx->ev_h2d[par]), cs);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, static_cast<cudaEvent_t>(ctx->ev_h2d[par]), 0);
+        if (e == cudaSuccess) e = cudaEventRecord(static_cast<cudaEvent_t>(ctx->ev_h2d), cs);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, static_cast<cudaEvent_t>(ctx->ev_h2d), 0);
     } else {
         e = cudaMemcpyAsync(d_in_nchw[0], in_host, in_nchw_b, cudaMemcpyHostToDevice, st);
     }
-    if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SMALL_ERR_CUDA; }
+    if (e != cudaSuccess) {
+        if (stage && !stage->ordered) stage->base = nullptr;
+        ctx->last_cuda = (int)e;
+        return SMALL_ERR_CUDA;
+    }
     // A first layer with at most four input channels (an image, a spectrogram) reads the NCHW tensor itself: its kernel
     // gathers the real channels into shared memory either way, so the blocked copy of the input - 32 lanes for one to four
     // channels - is never made.  The values and their order of summation are those of the blocked path.
@@ -420,10 +456,10 @@ SMALL_API int small_run_net_host(small_ctx *ctx, const small_layer *layers, int 
     if (!first)
         if (int s = small_pack(ctx, d_in_nchw[par], d_in_blk, N, C, H, W, stream)) return s;
     if (piped) {
-        e = cudaEventRecord(static_cast<cudaEvent_t>(ctx->ev_pack[par]), st);
+        e = cudaEventRecord(static_cast<cudaEvent_t>(stage->ev_read[par]), st);
         if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SMALL_ERR_CUDA; }
-        ctx->host_used[par] = 1;
-        ctx->host_parity = par ^ 1;
+        stage->used[par] = 1;
+        stage->next = par ^ 1;
     }
     if (first) {
         // the rest of the list over the same slots: its plan must be the whole list's (slot sizes come from all layers)

@@ -100,7 +100,6 @@ class Net:
             self.layer_rows.append(dict(name=L["name"], op=L["op"], C=L["C"], K=L["K"], H=h, W=wd, FH=fh, FW=fw,
                                         stride=L["stride"], pad=L["pad"], OH=oh, OW=ow, dst=L["dst"], first=li, upto=li + 1))
             descs.append(d)
-        torch.cuda.synchronize()
         self.dims = dims
         self.out_shape = dims["out"]
         self.layers = (B.small_layer * len(descs))(*descs)
@@ -111,6 +110,7 @@ class Net:
         self.workspace = torch.empty(self.ws_bytes + self.stage_bytes + 256, dtype=torch.uint8, device=device)
         assert self.workspace.data_ptr() % 256 == 0
         self.out_blk = torch.empty(B.small_packed_elems(self.N, oc, oh, ow), device=device)
+        torch.cuda.synchronize()      # the filters are packed, and nothing queued before still uses the workspace's memory (see run_host)
 
     def launches(self):
         """Kernel launches of one run under this network's fusion setting."""
@@ -132,6 +132,8 @@ class Net:
         return out_blk
 
     def run_host(self, in_host, out_host, stream=None):
+        """From host memory to host memory.  The input is copied into this network's workspace on a stream of the library's own,
+        ahead of the calls still running: nothing else may use the workspace's staging areas."""
         c, h, w = self.in_shape
         oc, oh, ow = self.out_shape
         B.small_set_net_fusion(self.ctx, self.fusion)

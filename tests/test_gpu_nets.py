@@ -204,3 +204,37 @@ def test_run_net_rejects_bad_workspace_and_descriptors():
     assert L.small_run_net(ctx(), bad, len(bad), 2, x.data_ptr(), gnet.out_blk.data_ptr(), gnet.workspace.data_ptr(),
                            gnet.ws_bytes, st) == 1
     torch.cuda.synchronize()
+
+
+def test_host_calls_in_turn_on_several_workspaces():
+    """Networks called in turn from host buffers, back to back: a call's input is copied while calls before it still run, and must
+    not land in a staging area that one of them has yet to read.  Captured and direct calls on one workspace mix as well."""
+    batch = 384
+    net = configs.kws_cnn(batch=batch)
+    gnets = [Net(ctx(), net, configs.make_params(net, seed), batch=batch, math="3xtf32") for seed in (1, 2, 3)]
+    ins = [torch.from_numpy(configs.make_input(net, batch, seed)).pin_memory() for seed in range(12)]
+    new_out = lambda: torch.full((batch,) + tuple(gnets[0].out_shape), float("nan")).pin_memory()
+    want = {}
+    for g in range(3):
+        for i in range(12):
+            want[g, i] = new_out()
+            gnets[g].run_host(ins[i], want[g, i])
+            torch.cuda.synchronize()
+    calls = [(c % k, (5 * c + c // 7) % 12) for k in (2, 3) for c in range(48)]
+    outs = [new_out() for _ in calls]
+    for (g, i), out in zip(calls, outs):
+        gnets[g].run_host(ins[i], out)
+    torch.cuda.synchronize()
+    assert all(torch.equal(out, want[call]) for call, out in zip(calls, outs))
+    replayed = new_out()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        gnets[0].run_host(ins[0], replayed)
+    outs = [new_out() for _ in range(24)]
+    for c, out in enumerate(outs):
+        graph.replay()
+        gnets[0].run_host(ins[1 + c % 11], out)
+    torch.cuda.synchronize()
+    assert torch.equal(replayed, want[0, 0])
+    assert all(torch.equal(out, want[0, 1 + c % 11]) for c, out in enumerate(outs))
+    assert B.small_device_status(ctx()) == 0
