@@ -376,13 +376,14 @@ static int choose_path(const small_ctx *ctx, const Geom &g, unsigned math, bool 
     if (conv_thin_supported(g)) return 0;          // a reduction of a few dozen terms: CUDA cores in every math mode
     if (ctx && ctx->conv_path == SMALL_CONV_PATH_GENERAL) return 2;
     bool direct = conv_direct_supported(g);
+    const int sms = ctx ? ctx->sm_count : kSmCount;
     // the register-tiled kernel computes runs of 7 or 8 output columns per thread and 256 to 2048 outputs x 8 to 64 filters per
     // thread block: planes narrower than 4 columns leave it mostly idle (a 1 x 1 layer's plane is viewed with longer rows), and a
     // layer that gives it fewer blocks than half the SMs runs faster on the general kernel's many small blocks, unless its
     // threads have many FMAs each: 3 x 3 at stride 1 on planes of 12 columns and more (batch 1, us, general against
     // register-tiled: 16 -> 16 on 32 x 32 12.9 / 10.5, 64 -> 64 on 28 x 28 41 / 33, but on 8 x 8 27.5 / 30.7 and 1 x 1 on 25 x 5 6.8 / 9.7)
     if (direct && !(ctx && ctx->conv_path == SMALL_CONV_PATH_CUDA_CORES) &&
-        ((g.OW < 4 && g.FH * g.FW > 1) || (conv_direct_blocks(g) < (ctx ? ctx->sm_count : 148) / 2 && !(g.FH == 3 && g.FW == 3 && g.S == 1 && g.OW >= 12))))
+        ((g.OW < 4 && g.FH * g.FW > 1) || (conv_direct_blocks(g, sms) < sms / 2 && !(g.FH == 3 && g.FW == 3 && g.S == 1 && g.OW >= 12))))
         direct = false;
     if (math == SMALL_MATH_FP32) return direct ? 1 : 2;
     // One channel block and at most 32 filters (64 with a 1x1 window): the warp-level MMA (see conv_mma.cu), which measured faster than both

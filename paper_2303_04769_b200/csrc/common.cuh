@@ -54,6 +54,8 @@ struct small_ctx {
 
 namespace small {
 
+constexpr int kSmCount = 148;      // of a B200: for questions about a shape that are asked without a context
+
 static inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 static inline int blocks_of(int C) { return (C + SMALL_CB - 1) / SMALL_CB; }
 static inline size_t packed_elems(int N, int C, int H, int W) {
@@ -143,7 +145,7 @@ int launch_conv_fp32(small_ctx *, const float *in, const float *w, const float *
                      bool relu, bool accumulate, cudaStream_t, int span = 0, int Kg = 0, int S_C = 0);
 // register-tiled FP32 kernel: windows 1 or 3 wide, strides 1 and 2 (group convolutions as launch_conv_fp32 takes them)
 bool conv_direct_supported(const Geom &, int span = 0, int Kg = 0, int S_C = 0);
-long long conv_direct_blocks(const Geom &);     // thread blocks its plan launches (0: shape not taken)
+long long conv_direct_blocks(const Geom &, int sms);     // thread blocks its plan launches (0: shape not taken)
 int launch_conv_direct(small_ctx *, const float *in, const float *w, const float *bias, float *out, const Geom &,
                        bool relu, bool accumulate, cudaStream_t, int span = 0, int Kg = 0, int S_C = 0);
 // the same kernel with a 2 x 2 stride-2 max pool taken in its STORE phase: out is [N][K][OH/2][OW/2]

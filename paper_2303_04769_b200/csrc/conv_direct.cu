@@ -300,7 +300,7 @@ size_t round1k(size_t b) { return (b + 1023) & ~(size_t)1023; }
 // per block, channels per stage (8 or 16) and units per block, by the estimated time of the layer: a warp's FMAs (two per
 // instruction) with the operand loads beside them, how well the resident warps of an SM keep its pipes busy (at 160 registers 12
 // warps fit in small blocks, 8 in blocks of 8 warps), and whole waves of blocks where they are few.
-DirectPlan plan_direct_view(const Geom &g, int span, int Kg, int S_C, size_t max_smem, bool pool, double &best_cost) {
+DirectPlan plan_direct_view(const Geom &g, int span, int Kg, int S_C, size_t max_smem, int sms, bool pool, double &best_cost) {
     DirectPlan best{};
     best.ok = false;
     if ((g.FW != 1 && g.FW != 3) || (g.S != 1 && g.S != 2) || g.FH * g.FW > 256) return best;
@@ -360,12 +360,12 @@ DirectPlan plan_direct_view(const Geom &g, int span, int Kg, int S_C, size_t max
                 const double eff = resident >= 12 ? 1.0 : resident >= 8 ? 0.85 + 0.0375 * (resident - 8) : 0.12 * resident;
                 const double warp = (double)channels * T * (8.0 * pw + 10.0 + (g.FW == 1 ? 2.0 * pw : 0.5 * pw)) + 2500.0;
                 const double set = warp * resident / 4.0 / eff;
-                const double waves = (double)blocks / (148.0 * per_sm);
+                const double waves = (double)blocks / ((double)sms * per_sm);
                 // with few waves the last one counts whole, but its blocks have the SMs to themselves where it is not full
                 const double whole = (double)(long long)waves, rest = waves - whole;
                 double cost;
                 if (waves <= 1.0) {
-                    const int here = (int)((blocks + 147) / 148);         // blocks of the busiest SM
+                    const int here = (int)((blocks + sms - 1) / sms);         // blocks of the busiest SM
                     const int r = here * warps;
                     cost = warp * r / 4.0 / (r >= 12 ? 1.0 : r >= 8 ? 0.85 + 0.0375 * (r - 8) : 0.12 * r);
                 } else {
@@ -386,9 +386,9 @@ DirectPlan plan_direct_view(const Geom &g, int span, int Kg, int S_C, size_t max
 
 // A 1 x 1 window at stride 1 without padding may view the plane with any row length that divides it: the one that leaves
 // the fewest threads idle (25 x 5 planes as rows of 125: 97 instead of 49 % of the pixels of a unit).
-DirectPlan plan_direct(Geom &g, int span, int Kg, int S_C, size_t max_smem, bool pool = false) {
+DirectPlan plan_direct(Geom &g, int span, int Kg, int S_C, size_t max_smem, int sms, bool pool = false) {
     double cost = 0.0;
-    DirectPlan best = plan_direct_view(g, span, Kg, S_C, max_smem, pool, cost);
+    DirectPlan best = plan_direct_view(g, span, Kg, S_C, max_smem, sms, pool, cost);
     if (!best.ok || g.FH * g.FW != 1 || g.S != 1 || (g.pt | g.pb | g.pl | g.pr) || pool) return best;
     const int hw = g.H * g.W;
     const Geom orig = g;
@@ -397,7 +397,7 @@ DirectPlan plan_direct(Geom &g, int span, int Kg, int S_C, size_t max_smem, bool
         Geom v = orig;
         v.H = v.OH = h; v.W = v.OW = hw / h;
         double c = 0.0;
-        const DirectPlan p = plan_direct_view(v, span, Kg, S_C, max_smem, false, c);
+        const DirectPlan p = plan_direct_view(v, span, Kg, S_C, max_smem, sms, false, c);
         if (p.ok && c < 0.98 * cost) { best = p; cost = c; g = v; }
     }
     return best;
@@ -409,12 +409,12 @@ using sm100::EncodeTiledFn;
 
 bool conv_direct_supported(const Geom &g, int span, int Kg, int S_C) {
     double cost;
-    return plan_direct_view(g, span, Kg, S_C, 227 * 1024, false, cost).ok;
+    return plan_direct_view(g, span, Kg, S_C, 227 * 1024, kSmCount, false, cost).ok;
 }
 
-long long conv_direct_blocks(const Geom &g_in) {
+long long conv_direct_blocks(const Geom &g_in, int sms) {
     Geom g = g_in;
-    const DirectPlan p = plan_direct(g, 0, 0, 0, 227 * 1024);
+    const DirectPlan p = plan_direct(g, 0, 0, 0, 227 * 1024, sms);
     return p.ok ? p.blocks : 0;
 }
 
@@ -450,7 +450,7 @@ int launch_direct(small_ctx *ctx, const Geom &g_in, const float *in, const float
     auto it = cache.find(key);
     if (it != cache.end()) return start(ctx, it->second, st);
     Geom g = g_in;                                   // (a pointwise layer's plane may be viewed with another row length)
-    DirectPlan p = plan_direct(g, span, Kg, S_C, ctx->max_smem_optin, pool);
+    DirectPlan p = plan_direct(g, span, Kg, S_C, ctx->max_smem_optin, ctx->sm_count, pool);
     if (!p.ok) return SMALL_ERR_UNSUPPORTED;
     DirectArgs &a = p.a;
     a.bias = bias; a.out = out; a.status = ctx->dev_status; a.relu = relu; a.accumulate = accumulate; a.wait_iters = ctx->wait_iters;
@@ -509,7 +509,7 @@ int launch_conv_direct(small_ctx *ctx, const float *in, const float *w, const fl
 
 bool conv_direct_pool_supported(const Geom &g) {
     double cost;
-    return plan_direct_view(g, 0, 0, 0, 227 * 1024, true, cost).ok;
+    return plan_direct_view(g, 0, 0, 0, 227 * 1024, kSmCount, true, cost).ok;
 }
 
 int launch_conv_direct_pool(small_ctx *ctx, const float *in, const float *w, const float *bias, float *out, const Geom &g,

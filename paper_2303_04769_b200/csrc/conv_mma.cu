@@ -132,7 +132,7 @@ MmaPlan plan_mma(const Geom &g, bool x3, size_t max_smem, int sms) {
 
 }  // namespace
 
-bool conv_mma_supported(const Geom &g, bool x3) { return plan_mma(g, x3, 227 * 1024, 148).ok; }
+bool conv_mma_supported(const Geom &g, bool x3) { return plan_mma(g, x3, 227 * 1024, kSmCount).ok; }
 
 // A finished launch - plan, tensor maps, arguments, kernel - is kept per context by (shape, mode, flags, tensors), so that
 // a repeated call (a network step) only launches.

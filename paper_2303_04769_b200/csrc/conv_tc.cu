@@ -991,10 +991,10 @@ static bool make_virt(const Geom &g_in, Virt &v, bool keep_rows = false) {
 static bool conv_tc_supported_uncached(const Geom &g, bool x3, int groups, const DwFuse *dw) {
     Virt v;
     if (!make_virt(g, v, dw != nullptr)) return false;
-    if (dw) return groups == 1 && make_plan(v.g, 227 * 1024, 148, false, v.S, v.taps_eff, x3, false, 0, dw).ok;
+    if (dw) return groups == 1 && make_plan(v.g, 227 * 1024, kSmCount, false, v.S, v.taps_eff, x3, false, 0, dw).ok;
     if (groups > 1) return (g.C % 32 == 0) && (g.K % (32 * groups) == 0) &&
-                           make_plan(v.g, 227 * 1024, 148, false, v.S, v.taps_eff, x3, false, g.K / groups).ok;
-    return make_plan(v.g, 227 * 1024, 148, false, v.S, v.taps_eff, x3, v.CBr == 1 && g.C <= 16).ok;
+                           make_plan(v.g, 227 * 1024, kSmCount, false, v.S, v.taps_eff, x3, false, g.K / groups).ok;
+    return make_plan(v.g, 227 * 1024, kSmCount, false, v.S, v.taps_eff, x3, v.CBr == 1 && g.C <= 16).ok;
 }
 
 // Planning a layer walks two orientations x eight tile sizes; its answers depend on the shape alone, so they are kept:
