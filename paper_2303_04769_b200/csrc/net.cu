@@ -81,12 +81,20 @@ static bool slot_dead_after(const small_layer *layers, int n_layers, int from, i
     return true;
 }
 
-// Fusing a depthwise 3x3 with the 1x1 convolution behind it pays where launches are all there is to the two layers, at a few
-// small images: the fused kernel has eight depthwise warps per SM and half the strips, the two kernels have whole SMs.  Networks,
-// us, fused / separate: depthwise-separable 3xTF32 batch 1 121.5 / 122.0, 4 125.9 / 122.2, 16 146 / 142, 64 185 / 174, TF32 batch 4
-// 113.7 / 114.8, 64 166 / 158; keyword spotting 3xTF32 batch 150 105 / 67, 400 156 / 100, 700 234 / 140, TF32 146 / 128.
-static const int kFuseDwpwMaxImages = 4;
+// Fusing a depthwise 3x3 with the 1x1 convolution behind it: one launch instead of two, but the fused kernel has eight depthwise
+// warps per SM and half the strips, where the two kernels have whole SMs.  At a few small images the two forms take the same time
+// and fusing halves the host's (depthwise-separable network called directly, us, separate / fused: TF32 batch 1 110.7 / 111.8,
+// 2 110.0 / 109.9, 3 114.3 / 113.9, 4 115.2 / 114.2, 8 118.0 / 121.5; 3xTF32 1 122.1 / 122.6, 2 122.1 / 121.8, 3 124.6 / 124.9,
+// 4 124.3 / 126.2, 8 130.0 / 134.2; host time of a call 65 / 39; replayed from a graph, where the host counts for nothing, fused is
+// 2 to 5 % behind).  Single pairs, batch 1: 128 channels on 28 x 28 in 3xTF32 14.6 / 12.4, 256 on 14 x 14 TF32 13.5 / 16.5, 3xTF32
+// 20.5 / 18.6, but 512 on 7 x 7 14.5 / 28.8 and 18.6 / 34.3, where a block has the filters of all 16 channel blocks to stream:
+// hence the bound on channels and filters.
+static const int kFuseDwpwMaxImages = 4, kFuseDwpwMaxImagesX3 = 3, kFuseDwpwMaxChannels = 256;
 static const size_t kFuseDwpwMaxBytes = 1u << 20;      // of the intermediate tensor
+static bool dwpw_pays(int N, int C, int K, int OH, int OW, unsigned math) {
+    return N <= (math == SMALL_MATH_3XTF32 ? kFuseDwpwMaxImagesX3 : kFuseDwpwMaxImages) && C <= kFuseDwpwMaxChannels && K <= kFuseDwpwMaxChannels &&
+           sizeof(float) * packed_elems(N, C, OH, OW) <= kFuseDwpwMaxBytes;
+}
 
 // Two layers may run at the same time when neither writes a tensor the other one reads or writes.
 static bool independent(const small_layer &A, const small_layer &Bn) {
@@ -111,7 +119,7 @@ static int fused_pair(const small_ctx *ctx, const small_layer *layers, int n_lay
         if ((Bn.flags & SMALL_ACCUMULATE) || Bn.C != A.C || math == SMALL_MATH_FP32) return 0;
         if (make_geom(g, N, A.C, A.C, A.H, A.W, 3, 3, A.stride, A.pad_t, A.pad_b, A.pad_l, A.pad_r)) return 0;
         if (Bn.H != g.OH || Bn.W != g.OW) return 0;
-        if (!(ctx->net_fusion & SMALL_FUSE_DWPW_ALWAYS) && (N > kFuseDwpwMaxImages || sizeof(float) * packed_elems(N, A.C, g.OH, g.OW) > kFuseDwpwMaxBytes)) return 0;
+        if (!(ctx->net_fusion & SMALL_FUSE_DWPW_ALWAYS) && !dwpw_pays(N, A.C, Bn.K, g.OH, g.OW, math)) return 0;
         return small_dwpw_fused(N, A.C, Bn.K, A.H, A.W, A.stride, A.pad_t, A.pad_b, A.pad_l, A.pad_r, math) ? SMALL_OP_DWPW : 0;
     }
     if (A.op == SMALL_OP_CONV && Bn.op == SMALL_OP_POOL && (ctx->net_fusion & SMALL_FUSE_CONVPOOL)) {

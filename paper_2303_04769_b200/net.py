@@ -37,7 +37,7 @@ def assign_slots(layers):
 
 class Net:
     """A network resident on the device: packed filters, plain layer descriptors and workspace.  Which neighbouring
-    layers run as one fused layer is the library's decision inside small_run_net; fuse_dwpw (True: where it pays, "all":
+    layers run as one fused layer is the library's decision inside small_run_net; fuse_dwpw (True: where it costs nothing, "all":
     wherever the fused kernel takes the shape, False: never) and fuse_convpool only select the library's fusion setting
     for this network's runs."""
 
