@@ -241,11 +241,12 @@ def test_host_calls_in_turn_on_several_workspaces():
 
 
 def test_depthwise_pairs_fuse_for_a_few_small_images_only():
-    """Where small_run_net forms the depthwise / 1x1 pair by itself: batch 4 in TF32, 3 in 3xTF32, at most 256 channels."""
+    """Where small_run_net forms the depthwise / 1x1 pair by itself: batch 4 in TF32, 3 in 3xTF32, at most 256 channels and 1 MB
+    (the first pair's tensor takes 1.2 MB at batch 4)."""
     net = configs.dwsep_cnn(batch=3)
     params = configs.make_params(net)
     counts = {(m, b): Net(ctx(), net, params, batch=b, math=m).launches() for m in ("tf32", "3xtf32") for b in (3, 4, 5)}
-    assert counts == {("tf32", 3): 15, ("tf32", 4): 15, ("tf32", 5): 28, ("3xtf32", 3): 15, ("3xtf32", 4): 28, ("3xtf32", 5): 28}
+    assert counts == {("tf32", 3): 15, ("tf32", 4): 16, ("tf32", 5): 28, ("3xtf32", 3): 15, ("3xtf32", 4): 28, ("3xtf32", 5): 28}
     for c, launches in ((256, 1), (257, 2), (512, 2)):
         layers = [configs._dw("d", "in", "a", c, 1), configs._conv("p", "a", "out", c, 64, 1, 1, configs.P0, True)]
         pair = dict(name="pair", batch=1, input=(c, 7, 7), input_dist=("uniform", -1.0, 1.0), weight_dist="he_normal", layers=layers)
