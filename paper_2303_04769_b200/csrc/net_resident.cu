@@ -257,21 +257,39 @@ int clusters_of(small_ctx *ctx, unsigned math, int lg) {
 }
 
 // Where the run is faster on chip than layer by layer.  `one_round`: every image has its own thread blocks; with more images
-// than that the layer kernels, which see the whole batch, win.  Measured (us, on chip / layer by layer): keyword spotting,
-// batch 37: FP32 50 / 70, TF32 36 / 51, 3xTF32 41 / 58, batch 148 39 / 74 in TF32; depthwise-separable network, batch 1: FP32 129 /
-// 178, TF32 105 / 103, batch 37 TF32 138 / 135: its filters (700 KB) stream through every block, which the tensor-core kernels
-// share between images; residual network, batch 1 (8 blocks per image): FP32 97 / 115, 3xTF32 73 / 66, batch 16 (4 blocks) FP32 125 / 124:
-// without depthwise layers nothing is computed without an exchange.
+// than that the layer kernels, which see the whole batch, win.  Measured called directly, us, layer by layer / on chip, on stacks of
+// a 10 x 4 stem and n pairs of a depthwise and a 1x1 layer of C channels on 25 x 5 (the keyword-spotting network: C = 64, n = 4):
+//   Tensor-core modes: what counts is a layer's work on an image, which one to eight SMs do with warp-level MMAs while the layer
+//   kernels use block-level ones, and the exchange, which grows with G.  3xTF32: C = 48 batch 1 (G = 8) 44.0 / 36.9, 148 (G = 1)
+//   58.4 / 41.6; C = 64 8 42.2 / 47.3, 18 (G = 4) 44.1 / 43.1, 74 (G = 2) 51.5 / 45.1, 148 57.6 / 47.1; C = 72 8 48.8 / 55.2, 148
+//   70.8 / 93.4; C = 96 8 49.4 / 67.9, 37 56.2 / 61.5, 148 72.0 / 112.7; C = 128 148 82.7 / 139.4; TF32 C = 64 8 38.0 / 41.0, 24 40.2 /
+//   43.3, 48 44.1 / 41.2, 148 52.3 / 41.1.  So 600,000 products per layer and image, 2.4 million times blocks (C = 64 at G = 4 is 2.05
+//   million, C = 48 at G = 8 2.3).  The 700 KB of filters of the depthwise-separable network stream through every block; that
+//   network stays with the layer kernels, which share them between images.
+//   FP32: the layer kernels are as far from their peak as this one.  C = 64 batch 1 51.4 / 52.0, 37 70.3 / 53.5, 148 93.7 / 57.6;
+//   C = 128 24 102.6 / 78.0, 74 128 / 91.6, 148 (G = 1) 166 / 176; depthwise-separable network 1 200 / 131, 64 308 / 213, 100 (G = 1) 337 /
+//   350.  Filters are dealt to the blocks by halves of whole blocks of 32: C = 96 batch 18 77.9 / 64.9, but 37 (G = 2) 86.1 / 96.1, 148
+//   119.6 / 139.4; C = 160, whose five blocks of filters all stay together, 1 67.8 / 119, 37 94.5 / 288, 148 168 / 478.  Without depthwise
+//   layers nothing is computed without an exchange: residual network batch 1 (G = 8) 131 / 98, 12 132 / 105, 16 (G = 4) 125 / 124;
+//   3xTF32 batch 1 66 / 73.
 bool worth_it(const Args &a, unsigned math, int G, bool one_round) {
     if (!one_round) return false;
     size_t filters = 0;
-    int depthwise = 0;
+    double most = 0.0;                                   // products of a layer and image
+    int depthwise = 0, uneven = 0;                       // uneven: the most filters, in whole blocks, of layers where these are no power of two
     for (int i = 0; i < a.n_ops; ++i) {
-        depthwise += a.op[i].kind == kDw ? 1 : 0;
-        if (a.op[i].kind == kConv) filters += (size_t)a.op[i].C * a.op[i].K * a.op[i].FH * a.op[i].FW * 4;
+        const Op &o = a.op[i];
+        depthwise += o.kind == kDw ? 1 : 0;
+        if (o.kind != kConv) continue;
+        const int Kr = blocks_of(o.K) * 32;
+        const size_t f = (size_t)o.C * o.K * o.FH * o.FW;
+        filters += f * 4;
+        most = std::max(most, (double)f * o.OH * o.OW);
+        if (Kr & (Kr - 1)) uneven = std::max(uneven, Kr);
     }
-    if (!depthwise) return math == SMALL_MATH_FP32 && G == 8;
-    return math == SMALL_MATH_FP32 || filters <= 256 * 1024;
+    if (math != SMALL_MATH_FP32) return depthwise && filters <= 256 * 1024 && most <= 600e3 && most * G <= 2.4e6;
+    if (uneven > 96 || (uneven && G < 4) || (G == 1 && most > 550e3)) return false;
+    return depthwise || G == 8;
 }
 
 const Plan *find_plan(small_ctx *ctx, const small_layer *layers, int n, int from, int N) {

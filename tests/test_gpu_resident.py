@@ -56,3 +56,27 @@ def test_on_chip_run_repeats_its_bits_in_a_graph():
         out.fill_(float("nan"))
         g.replay()
         assert torch.equal(out, want)
+
+
+def stack(C, n):
+    L = [_conv("stem", "in", "p0", 1, C, (10, 4), 2, (4, 5, 1, 1), True)]
+    for i in range(n):
+        L += [_dw(f"d{i}", f"p{i}", f"m{i}", C, 1), _conv(f"c{i}", f"m{i}", f"p{i + 1}", C, C, 1, 1, P0, True)]
+    L += [_gap("gap", f"p{n}", "g", C), _fc("fc", "g", "out", C, 12)]
+    return dict(name="stack", batch=1, input=(1, 49, 10), input_dist=("normal", 0.0, 1.0), weight_dist="he_normal", layers=L)
+
+
+@pytest.mark.parametrize("C,batch,math,on_chip", [(64, 9, "fp32", True), (64, 148, "3xtf32", True), (64, 60, "tf32", True), (48, 9, "tf32", True),
+                                                  (64, 9, "3xtf32", False), (96, 148, "tf32", False), (128, 9, "3xtf32", False),
+                                                  (96, 9, "fp32", True), (96, 60, "fp32", False), (128, 148, "fp32", False), (160, 9, "fp32", False)])
+def test_which_runs_stay_on_chip(C, batch, math, on_chip):
+    """Either side of the lines between the two forms.  The on-chip kernel adds up in another order, so a result has the bits of
+    the layers launched one by one exactly where those run."""
+    net = stack(C, 2)
+    params, x = configs.make_params(net), configs.make_input(net, batch)
+    blk = to_blk(x)
+    got = Net(ctx(), net, params, batch=batch, math=math).run(blk)
+    apart = Net(ctx(), net, params, batch=batch, math=math, fuse_dwpw=False).run(blk)
+    assert torch.equal(got, apart) == (not on_chip)
+    ref = nets.run_net(net, params, x)["out"]
+    assert rel_err(from_blk(got, batch, *ref.shape[1:]), ref) <= TOL[math]
