@@ -3,6 +3,8 @@
 #include <algorithm>
 #include <cstring>
 #include <map>
+#include <memory>
+#include <unordered_map>
 #include <vector>
 
 #include "net_resident.cuh"
@@ -229,10 +231,10 @@ double tile_ops(Args &a, unsigned math, int G) {
     return total;
 }
 
-struct Entry { std::vector<unsigned char> key; Plan p; };
+struct Entry { std::vector<unsigned char> key; std::unique_ptr<Plan> p; };      // no plan: the run is not taken
 struct State {
     int clusters[3][4] = {};                             // resident clusters of 1, 2, 4, 8 blocks per math mode; 0: not asked yet
-    std::vector<Entry> plans;                            // finished plans, the latest first
+    std::unordered_multimap<size_t, Entry> plans;        // finished plans by a few words of (batch, layers); the key has all of them
 };
 State &state_of(small_ctx *ctx) {
     if (!ctx->resident_state) ctx->resident_state = new State();
@@ -292,43 +294,51 @@ bool worth_it(const Args &a, unsigned math, int G, bool one_round) {
     return depthwise || G == 8;
 }
 
+// The plan for layers from .. n - 1, nullptr where they do not run on chip.  Every call of a network asks, so what can be seen
+// without a plan is answered first; plans are made once per batch and list (2 to 25 us each).
 const Plan *find_plan(small_ctx *ctx, const small_layer *layers, int n, int from, int N) {
+    if (N > ctx->sm_count || n - from < 2 || layers[n - 1].op != SMALL_OP_FC || layers[n - 2].op != SMALL_OP_POOL) return nullptr;
+    if ((layers[n - 1].flags & SMALL_MATH_MASK) != SMALL_MATH_FP32) {
+        int i = from;
+        while (i < n && layers[i].op != SMALL_OP_DWCONV) ++i;
+        if (i == n) return nullptr;
+    }
     State &s = state_of(ctx);
     const int head[2] = {N, from};
     const size_t lb = sizeof(small_layer) * (size_t)n;
-    for (size_t i = 0; i < s.plans.size(); ++i) {
-        const Entry &e = s.plans[i];
-        if (e.key.size() == lb + sizeof(head) && !memcmp(e.key.data(), head, sizeof(head)) && !memcmp(e.key.data() + sizeof(head), layers, lb)) {
-            if (i) std::rotate(s.plans.begin(), s.plans.begin() + i, s.plans.begin() + i + 1);
-            return &s.plans.front().p;
-        }
+    const size_t words = ((size_t)N * 64 + from) * 64 + n + ((reinterpret_cast<size_t>(layers[n - 1].w_blk) ^ reinterpret_cast<size_t>(layers[0].w_blk)) << 16);
+    const auto range = s.plans.equal_range(words);
+    for (auto it = range.first; it != range.second; ++it) {
+        const Entry &e = it->second;
+        if (e.key.size() == lb + sizeof(head) && !memcmp(e.key.data(), head, sizeof(head)) && !memcmp(e.key.data() + sizeof(head), layers, lb)) return e.p.get();
     }
     Entry e;
     e.key.resize(lb + sizeof(head));
     memcpy(e.key.data(), head, sizeof(head));
     memcpy(e.key.data() + sizeof(head), layers, lb);
-    e.p.ok = false;
+    Plan p{};
+    p.ok = false;
     for (int s0 = from; s0 < n; ++s0) {
-        e.p = plan_run(layers, n, s0, N, ctx->max_smem_optin, true);
-        if (!e.p.ok) e.p = plan_run(layers, n, s0, N, ctx->max_smem_optin, false);
-        if (e.p.ok) break;
+        p = plan_run(layers, n, s0, N, ctx->max_smem_optin, true);
+        if (!p.ok) p = plan_run(layers, n, s0, N, ctx->max_smem_optin, false);
+        if (p.ok) break;
     }
-    if (e.p.ok) {
-        Args &a = e.p.a;
+    if (p.ok) {
+        Args &a = p.a;
         double best = 0.0;
         int best_g = 0;
         for (int lg = 0; lg < 4; ++lg) {
-            const int c = clusters_of(ctx, e.p.math, lg);
-            const double t = (double)ceil_div(N, c) * tile_ops(a, e.p.math, 1 << lg);
+            const int c = clusters_of(ctx, p.math, lg);
+            const double t = (double)ceil_div(N, c) * tile_ops(a, p.math, 1 << lg);
             if (t > 0.0 && (!best_g || t < best)) { best = t; best_g = 1 << lg; }
         }
         a.G = best_g;
-        if (!best_g || !worth_it(a, e.p.math, best_g, N <= clusters_of(ctx, e.p.math, best_g == 8 ? 3 : best_g == 4 ? 2 : best_g - 1))) e.p.ok = false;
-        else tile_ops(a, e.p.math, best_g);
+        if (!best_g || !worth_it(a, p.math, best_g, N <= clusters_of(ctx, p.math, best_g == 8 ? 3 : best_g == 4 ? 2 : best_g - 1))) p.ok = false;
+        else tile_ops(a, p.math, best_g);
     }
-    if (s.plans.size() >= 32) s.plans.pop_back();
-    s.plans.insert(s.plans.begin(), std::move(e));
-    return &s.plans.front().p;
+    if (p.ok) e.p.reset(new Plan(p));
+    if (s.plans.size() >= 512) s.plans.clear();
+    return s.plans.emplace(words, std::move(e))->second.p.get();
 }
 
 }  // namespace
@@ -340,13 +350,13 @@ void free_resident_state(small_ctx *ctx) {
 
 int resident_from(small_ctx *ctx, const small_layer *layers, int n, int from, int N) {
     const Plan *p = find_plan(ctx, layers, n, from, N);
-    return p->ok ? p->from : -1;
+    return p ? p->from : -1;
 }
 
 int launch_resident(small_ctx *ctx, const small_layer *layers, int n, int from, int N, const std::function<const float *(int)> &rd,
                     const std::function<float *(int)> &wr, cudaStream_t st) {
     const Plan *p = find_plan(ctx, layers, n, from, N);
-    if (!p->ok) return SMALL_ERR_UNSUPPORTED;
+    if (!p) return SMALL_ERR_UNSUPPORTED;
     Args a = p->a;
     for (int i = 0; i < a.n_in; ++i) a.in[i].g = rd(p->in_slot[i]);
     a.out = wr(p->out_slot);
