@@ -385,8 +385,8 @@ typedef struct small_layer {
  * two neighbouring layers as one fused layer when the first one's result is read by the second one only (no later layer
  * reads that slot before it is written again), the pair's output slot differs from its input slot, and the fused kernel
  * takes the shape: a depthwise 3x3 and the 1x1 convolution behind it under a tensor-core math mode (SMALL_FUSE_DWPW: only
- * for up to four images, three in 3xTF32, of at most 256 channels and filters whose intermediate tensor takes at most 1 MB, where it
- * costs nothing and halves the launches; SMALL_FUSE_DWPW_ALWAYS: wherever the kernel takes the shape), a convolution and the 2x2 stride-2 max pool behind it (SMALL_FUSE_CONVPOOL), and a run of 2 to 12
+ * for up to four images of at most 256 channels and filters whose intermediate tensor takes at most 1 MB, small layers in TF32, in
+ * 3xTF32 those of one channel block and large ones, where it is faster or costs nothing and halves the launches; SMALL_FUSE_DWPW_ALWAYS: wherever the kernel takes the shape), a convolution and the 2x2 stride-2 max pool behind it (SMALL_FUSE_CONVPOOL), and a run of 2 to 12
  * full reductions whose inner widths are at most 128 under a tensor-core math mode (SMALL_FUSE_FC_CHAIN, see small_fc_chain), and
  * a global average pool with the full reduction behind it, in every math mode (SMALL_FUSE_POOLFC, see small_gap_fc).  The skipped
  * intermediate tensors are then not written.  Default: all four (without DWPW_ALWAYS); 0 runs every layer on its own.

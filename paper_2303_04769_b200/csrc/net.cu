@@ -82,18 +82,21 @@ static bool slot_dead_after(const small_layer *layers, int n_layers, int from, i
 }
 
 // Fusing a depthwise 3x3 with the 1x1 convolution behind it: one launch instead of two, but the fused kernel has eight depthwise
-// warps per SM and half the strips, where the two kernels have whole SMs.  At a few small images the two forms take the same time
-// and fusing halves the host's (depthwise-separable network called directly, us, separate / fused: TF32 batch 1 110.7 / 111.8,
-// 2 110.0 / 109.9, 3 114.3 / 113.9, 4 115.2 / 114.2, 8 118.0 / 121.5; 3xTF32 1 122.1 / 122.6, 2 122.1 / 121.8, 3 124.6 / 124.9,
-// 4 124.3 / 126.2, 8 130.0 / 134.2; host time of a call 65 / 39; replayed from a graph, where the host counts for nothing, fused is
-// 2 to 5 % behind).  Single pairs, batch 1: 128 channels on 28 x 28 in 3xTF32 14.6 / 12.4, 256 on 14 x 14 TF32 13.5 / 16.5, 3xTF32
-// 20.5 / 18.6, but 512 on 7 x 7 14.5 / 28.8 and 18.6 / 34.3, where a block has the filters of all 16 channel blocks to stream:
-// hence the bound on channels and filters.
-static const int kFuseDwpwMaxImages = 4, kFuseDwpwMaxImagesX3 = 3, kFuseDwpwMaxChannels = 256;
+// warps per SM and half the strips, where the two kernels have whole SMs.  Measured called directly, us, separate / fused:
+//   3xTF32, single pairs, batch 1: 64 channels on 56 x 56 12.2 / 10.4, 128 on 28 x 28 14.6 / 12.4, 256 on 14 x 14 20.5 / 18.6, but 64 on
+//   14 x 14 10.5 / 10.4, on 7 x 7 7.2 / 9.4, keyword-spotting network 42 / 48: it pays from some 50,000 values per image on, and for
+//   one channel block between other layers: depthwise-separable network none / its four pairs of at most 32 channels / all fused,
+//   batch 1 125.8 / 124.2 / 126.0, 2 126.1 / 121.9 / 125.1, 3 129.6 / 122.8 / 126.7, 4 129.6 / 123.7 / 128.6.
+//   TF32, where the two kernels are shorter: 64 on 56 x 56 10.4 / 10.4 (batch 4 11.6 / 12.4), 128 on 28 x 28 12.5 / 12.4, 256 on 14 x 14
+//   13.5 / 16.5; networks of small layers take the same time and half of the host's, depthwise-separable batch 1 110.7 / 111.8, 2 110.0 /
+//   109.9, 3 114.3 / 113.9, 4 115.2 / 114.2, 8 118.0 / 121.5 (host 65 / 39; replayed from a graph fused is 3 % behind): up to 20,000 values.
+//   512 channels on 7 x 7 18.6 / 34.3 and 14.5 / 28.8: a block streams the filters of all 16 channel blocks.
+static const int kFuseDwpwMaxImages = 4, kFuseDwpwMaxChannels = 256;
 static const size_t kFuseDwpwMaxBytes = 1u << 20;      // of the intermediate tensor
 static bool dwpw_pays(int N, int C, int K, int OH, int OW, unsigned math) {
-    return N <= (math == SMALL_MATH_3XTF32 ? kFuseDwpwMaxImagesX3 : kFuseDwpwMaxImages) && C <= kFuseDwpwMaxChannels && K <= kFuseDwpwMaxChannels &&
-           sizeof(float) * packed_elems(N, C, OH, OW) <= kFuseDwpwMaxBytes;
+    if (N > kFuseDwpwMaxImages || C > kFuseDwpwMaxChannels || K > kFuseDwpwMaxChannels || sizeof(float) * packed_elems(N, C, OH, OW) > kFuseDwpwMaxBytes) return false;
+    const long long values = (long long)C * OH * OW;
+    return math == SMALL_MATH_3XTF32 ? C <= 32 || values >= 50000 : values <= 20000;
 }
 
 // Two layers may run at the same time when neither writes a tensor the other one reads or writes.

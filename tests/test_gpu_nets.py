@@ -240,17 +240,17 @@ def test_host_calls_in_turn_on_several_workspaces():
     assert B.small_device_status(ctx()) == 0
 
 
-def test_depthwise_pairs_fuse_for_a_few_small_images_only():
-    """Where small_run_net forms the depthwise / 1x1 pair by itself: batch 4 in TF32, 3 in 3xTF32, at most 256 channels and 1 MB
-    (the first pair's tensor takes 1.2 MB at batch 4)."""
+def test_depthwise_pairs_fuse_for_a_few_images_only():
+    """Where small_run_net forms the depthwise / 1x1 pair by itself: up to batch 4, 256 channels and 1 MB, small layers in TF32, one
+    channel block and large layers in 3xTF32 (the network's first pair is above 1 MB at batch 4)."""
     net = configs.dwsep_cnn(batch=3)
     params = configs.make_params(net)
     counts = {(m, b): Net(ctx(), net, params, batch=b, math=m).launches() for m in ("tf32", "3xtf32") for b in (3, 4, 5)}
-    assert counts == {("tf32", 3): 15, ("tf32", 4): 16, ("tf32", 5): 28, ("3xtf32", 3): 15, ("3xtf32", 4): 28, ("3xtf32", 5): 28}
-    for c, launches in ((256, 1), (257, 2), (512, 2)):
+    assert counts == {("tf32", 3): 15, ("tf32", 4): 16, ("tf32", 5): 28, ("3xtf32", 3): 24, ("3xtf32", 4): 25, ("3xtf32", 5): 28}
+    for c, hw, math, launches in ((256, 7, "tf32", 1), (257, 7, "tf32", 2), (64, 18, "tf32", 2), (32, 7, "3xtf32", 1), (33, 7, "3xtf32", 2), (256, 14, "3xtf32", 1), (256, 13, "3xtf32", 2), (260, 14, "3xtf32", 2)):
         layers = [configs._dw("d", "in", "a", c, 1), configs._conv("p", "a", "out", c, 64, 1, 1, configs.P0, True)]
-        pair = dict(name="pair", batch=1, input=(c, 7, 7), input_dist=("uniform", -1.0, 1.0), weight_dist="he_normal", layers=layers)
-        gnet = Net(ctx(), pair, configs.make_params(pair), math="tf32")
-        assert gnet.launches() == launches
-        x = configs.make_input(pair)
-        assert rel_err(from_blk(gnet.run(to_blk(x)), 1, 64, 7, 7), nets.run_net(pair, configs.make_params(pair), x)["out"]) <= TOL["tf32"]
+        pair = dict(name="pair", batch=1, input=(c, hw, hw), input_dist=("uniform", -1.0, 1.0), weight_dist="he_normal", layers=layers)
+        pair_params, x = configs.make_params(pair), configs.make_input(pair)
+        gnet = Net(ctx(), pair, pair_params, math=math)
+        assert gnet.launches() == launches, (c, hw, math)
+        assert rel_err(from_blk(gnet.run(to_blk(x)), 1, 64, hw, hw), nets.run_net(pair, pair_params, x)["out"]) <= TOL[math]
