@@ -269,8 +269,8 @@ int clusters_of(small_ctx *ctx, unsigned math, int lg) {
 //   million, C = 48 at G = 8 2.3).  The 700 KB of filters of the depthwise-separable network stream through every block; that
 //   network stays with the layer kernels, which share them between images.
 //   FP32: the layer kernels are as far from their peak as this one.  C = 64 batch 1 51.4 / 52.0, 37 70.3 / 53.5, 148 93.7 / 57.6;
-//   C = 128 24 102.6 / 78.0, 74 128 / 91.6, 148 (G = 1) 166 / 176; depthwise-separable network 1 200 / 131, 64 308 / 213, 100 (G = 1) 337 /
-//   350.  Filters are dealt to the blocks by halves of whole blocks of 32: C = 96 batch 18 77.9 / 64.9, but 37 (G = 2) 86.1 / 96.1, 148
+//   C = 128 24 102.6 / 78.0, 74 128 / 91.6, 148 (G = 1) 166 / 176; depthwise-separable network (at most 590,000 products) 1 200 / 131,
+//   64 308 / 213, 80 (G = 1) 356 / 333, 100 337 / 351, 148 376 / 380.  Filters are dealt to the blocks by halves of whole blocks of 32: C = 96 batch 18 77.9 / 64.9, but 37 (G = 2) 86.1 / 96.1, 148
 //   119.6 / 139.4; C = 160, whose five blocks of filters all stay together, 1 67.8 / 119, 37 94.5 / 288, 148 168 / 478.  Without depthwise
 //   layers nothing is computed without an exchange: residual network batch 1 (G = 8) 131 / 98, 12 132 / 105, 16 (G = 4) 125 / 124;
 //   3xTF32 batch 1 66 / 73.
@@ -290,7 +290,7 @@ bool worth_it(const Args &a, unsigned math, int G, bool one_round) {
         if (Kr & (Kr - 1)) uneven = std::max(uneven, Kr);
     }
     if (math != SMALL_MATH_FP32) return depthwise && filters <= 256 * 1024 && most <= 600e3 && most * G <= 2.4e6;
-    if (uneven > 96 || (uneven && G < 4) || (G == 1 && most > 550e3)) return false;
+    if (uneven > 96 || (uneven && G < 4) || (G == 1 && most > 1e6)) return false;
     return depthwise || G == 8;
 }
 
