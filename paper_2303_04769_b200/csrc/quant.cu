@@ -74,20 +74,14 @@ __global__ void pack_q_conv_w_kernel(const uint8_t *__restrict__ w, uint32_t *__
     }
 }
 
-// per filter and tap the sum of the weight bytes over the channels [K][T], then per filter over everything [K]
+// per filter and tap the sum of the weight bytes over the channels [K][T]
 __global__ void q_conv_tables_kernel(const uint8_t *__restrict__ w, int *__restrict__ tab, int C, int K, int T) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < K * T) {
-        const int k = i / T, t = i - k * T;
-        int s = 0;
-        for (int c = 0; c < C; ++c) s += w[((size_t)k * C + c) * T + t];
-        tab[i] = s;
-    } else if (i < K * T + K) {
-        const int k = i - K * T;
-        int s = 0;
-        for (int j = 0; j < C * T; ++j) s += w[(size_t)k * C * T + j];
-        tab[i] = s;
-    }
+    if (i >= K * T) return;
+    const int k = i / T, t = i - k * T;
+    int s = 0;
+    for (int c = 0; c < C; ++c) s += w[((size_t)k * C + c) * T + t];
+    tab[i] = s;
 }
 
 // depthwise filters [C][FH][FW] bytes -> [CB][T][32] bytes, pad lanes 0
@@ -366,7 +360,7 @@ SMALL_API int small_q_unpack(small_ctx *ctx, const uint8_t *blk, uint8_t *nchw, 
 
 SMALL_API size_t small_q_conv_weight_bytes(int C, int K, int FH, int FW) {
     if (C < 1 || K < 1 || FH < 1 || FW < 1) return 0;
-    return q_conv_words(C, K, FH, FW) * 4 + ((size_t)K * FH * FW + K) * sizeof(int);
+    return q_conv_words(C, K, FH, FW) * 4 + ((size_t)K * FH * FW + K) * sizeof(int);      // (the last K words are spare)
 }
 
 SMALL_API int small_q_pack_conv_weights(small_ctx *ctx, const uint8_t *w, void *wb, int C, int K, int FH, int FW, void *stream) {
@@ -379,7 +373,7 @@ SMALL_API int small_q_pack_conv_weights(small_ctx *ctx, const uint8_t *w, void *
     const size_t words = q_conv_words(C, K, FH, FW);
     const int T = FH * FW;
     pack_q_conv_w_kernel<<<grid_for(ctx, words), 256, 0, st>>>(w, static_cast<uint32_t *>(wb), C, K, T, words);
-    q_conv_tables_kernel<<<(K * T + K + 127) / 128, 128, 0, st>>>(w, reinterpret_cast<int *>(static_cast<uint32_t *>(wb) + words), C, K, T);
+    q_conv_tables_kernel<<<(K * T + 127) / 128, 128, 0, st>>>(w, reinterpret_cast<int *>(static_cast<uint32_t *>(wb) + words), C, K, T);
     return check_launch(ctx);
 }
 
