@@ -356,14 +356,12 @@ SMALL_API int small_pack_fc_weights(small_ctx *ctx, const float *w, float *wb, i
 }
 
 // ---- layers ----
-// Which kernel family a full channel reduction takes under a tensor-core math mode.  The tensor-core kernel's MMAs are
-// 128 x N x 8 with N = the layer's filters: with few channels each still occupies the pipe for its floor of 40 to 50
-// cycles, and a launch carries some microseconds of pipeline set-up and drain.  The register-tiled FP32 kernel (whose
-// result meets every mode's tolerance) has neither cost but sustains about half the FP32 FMA rate.  Measured on the
-// residual network's layers at batch 256 (tensor cores TF32 / 3xTF32 against CUDA cores, microseconds): 1x1 stride 2
-// 16->32: 9.9 / 13.6 against 8.8; 3x3 stride 2 16->32: 20.1 / 29.5 against 25.3; 3x3 16->16: 25.7 / 39.3 against 44.4;
-// 1x1 stride 2 32->64: 8.1 / 9.0 against 11.0.  Hence: CUDA cores for C * K <= 512 when the window is 1 x 1, or when the
-// mode is 3xTF32 and the stride 2 (the stride-2 view spends two or three MMAs per product on four phase planes).
+// Layers that neither the stem kernel nor the warp-level one takes and that have few products per pixel (C * K <= 512: in effect
+// more than 32 channels into at most 15 filters, or few channels into many filters) go to the register-tiled FP32 kernel where the
+// window is 1 x 1, or in 3xTF32 the stride 2.  That was the faster kernel when the block-level one paid 52 cycles and more for an
+// MMA.  It is not any more for most of them (24 x 24 planes, us, block-level TF32 / 3xTF32 against CUDA cores: 1x1 40->12 batch 64
+// 7.2 / 9.0 against 11.7, 256 13.5 / 17.5 against 16.3; 1x1 64->8 7.1 / 9.7 against 12.0 and 13.8 / 18.5 against 18.3; 3x3 stride 2 40->12 in
+// 3xTF32, batch 256, 20.4 against 33.9), but their results are FP32's, more accurate than the mode asks for, and stay so.
 static bool prefer_cuda_cores(const small_ctx *ctx, const Geom &g, unsigned math) {
     if (ctx && ctx->conv_path == SMALL_CONV_PATH_TENSOR) return false;
     if (ctx && ctx->conv_path == SMALL_CONV_PATH_CUDA_CORES) return true;
@@ -386,15 +384,15 @@ static int choose_path(const small_ctx *ctx, const Geom &g, unsigned math, bool 
         ((g.OW < 4 && g.FH * g.FW > 1) || (conv_direct_blocks(g, sms) < sms / 2 && !(g.FH == 3 && g.FW == 3 && g.S == 1 && g.OW >= 12))))
         direct = false;
     if (math == SMALL_MATH_FP32) return direct ? 1 : 2;
-    // One channel block and at most 32 filters (64 with a 1x1 window): the warp-level MMA (see conv_mma.cu), which measured faster than both
-    // other families on such layers (residual CNN at batch 256, microseconds, TF32 / 3xTF32, block-level tensor-core
-    // kernel against warp-level: 3x3 16->16 25.3 / 37.4 against 17.3 / 28.7; 3x3 stride 2 16->32 19.9 / 28.3 against
-    // 12.2 / 15.8; 1x1 stride 2 16->32 10.2 / 14.3 against 7.1 / 7.6; 3x3 32->32 on 16x16 planes 15.5 / 27.2 against
-    // 14.8 / 23.9, on 8x8 planes 10.2 / 13.4 against 8.1 / 9.1; 1x1 stride 2 32->64 8.3 / 9.8 against 7.1 / 7.7; but 3x3
-    // stride 2 32->64 15.4 / 18.4 against 15.4 / 23.6, so 3x3 layers with more than 32 filters stay where they were).
+    // One channel block and at most 32 filters (64 with a 1x1 window): the warp-level MMA (see conv_mma.cu), faster on such layers
+    // (us, TF32 / 3xTF32, block-level kernel against warp-level, CUDA cores: 3x3 16->16 on 32x32 batch 1 5.8 / 7.4 against 4.1 / 6.3, 10.4;
+    // 64 10.1 / 15.1 against 5.7 / 9.0, 13.2; 256 20.1 / 29.0 against 14.1 / 24.2, 37.5; on 56x56 256 42.7 / 76.7 against 39.7 / 75.1; 3x3 stride
+    // 2 16->32 on 32x32 256 11.9 / 20.4 against 9.3 / 14.1, 24.4; 1x1 stride 2 16->32 7.2 / 10.1 against 5.1 / 5.6, 7.5; 1x1 stride 2 32->64 on
+    // 16x16 5.9 / 6.6 against 4.4 / 5.3, 9.1; 1x1 16->32 on 48x48 30.8 / 37.9 against 29.0 / 32.5, 42.5; 3x3 32->32 on 16x16 in TF32 12.1
+    // against 11.2; but 3x3 stride 2 32->64 256 10.5 / 12.8 against 17.4 / 29.7, so 3x3 layers with more than 32 filters stay where they were).
     // 3x3 at stride 1 with more than 16 channels and more than 16 filters is the block-level kernel's in 3xTF32 (32->32, us,
-    // warp-level against block-level: 16x16 planes, batch 1 / 8 / 64 / 256 10.3 / 10.3 / 12.4 / 24.7 against 8.3 / 8.5 / 12.4 /
-    // 22.6, batch 300 5x5 18.4 / 9.1, 13x13 32.8 / 19.5, 24x23 69.9 / 34.9, 33x33 145 / 62, batch 60 56x56 61.6 / 38.2, 30x70
+    // warp-level against block-level: 16x16 planes, batch 1 / 8 / 64 / 256 9.1 / 9.3 / 9.9 / 22.1 against 7.4 / 7.6 / 10.8 /
+    // 20.0, batch 300 5x5 18.4 / 9.1, 13x13 32.8 / 19.5, 24x23 69.9 / 34.9, 33x33 145 / 62, batch 60 56x56 61.6 / 38.2, 30x70
     // 52.4 / 32.8) up to 72 columns (80x80 127 against 176: fewer of its strips fit), and in TF32 on large planes of many
     // pixels in all (batch 60 32x32 12.5 / 14.4, 48x48 27.1 / 19.7, 30x70 24.7 / 18.5, 80x80 55.4 / 34.9; batch 256 16x16 14.2 / 14.4).
     // So are 1x1 layers of 33 to 64 filters at stride 1 from some 32,000 pixels on, where the warp-level kernel reads every pixel
