@@ -156,6 +156,9 @@ Plan plan_run(const small_layer *layers, int n, int from, int N, size_t max_smem
                    }), live.end());
     }
     p.out_slot = layers[n - 1].dst;
+    // an image's result must not land where another image's input is still to be read
+    for (int i = 0; i < a.n_in; ++i)
+        if (p.in_slot[i] == p.out_slot) return p;
     a.n_stream = a.n_ops - 2;
     p.smem = (size_t)top * 4;
     p.math = math;

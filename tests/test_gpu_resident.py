@@ -43,6 +43,27 @@ def test_on_chip_runs_match(net, batch, math):
     assert B.small_device_status(ctx()) == 0
 
 
+@pytest.mark.parametrize("batch", [3, 100])
+def test_result_in_the_slot_of_the_runs_input(batch):
+    """A list may end in the slot that its last layers' input came from: images do not wait for one another on chip, so the run has
+    to start at a later layer, which reads another slot."""
+    net = configs.kws_cnn(batch=batch)
+    params, blk = configs.make_params(net), to_blk(configs.make_input(net, batch))
+    gnet = Net(ctx(), net, params, batch=batch)
+    want = gnet.run(blk).clone()
+    last = len(gnet.layers) - 1
+    slot = 1 + max(L.dst for L in gnet.layers)
+    gnet.layers[0].dst = gnet.layers[1].src = gnet.layers[last].dst = slot
+    size = B.small_net_workspace_bytes(gnet.layers, batch)
+    workspace = torch.empty(size + 256, dtype=torch.uint8, device="cuda")
+    start = size - (B.small_packed_elems(batch, 64, 25, 5) * 4 + 255) // 256 * 256          # the last slot, as large as the input
+    for _ in range(20):
+        workspace[start:].fill_(255)
+        B.small_run_net(ctx(), gnet.layers, batch, blk, gnet.out_blk, workspace, size)
+        got = workspace[start:start + 4 * want.numel()].view(torch.float32)
+        assert rel_err(from_blk(got, batch, *gnet.out_shape), from_blk(want, batch, *gnet.out_shape)) <= TOL["fp32"]
+
+
 def test_on_chip_run_repeats_its_bits_in_a_graph():
     net = configs.kws_cnn(batch=40)
     gnet = Net(ctx(), net, configs.make_params(net), math="3xtf32")
