@@ -31,30 +31,38 @@ FLUSH_BYTES = 256 << 20            # larger than the 126 MB L2
 TOL = {"fp32": 1e-5, "tf32": 2e-3, "3xtf32": 1e-5}
 
 # DRAM traffic per launch of the dominant kernel (dram__bytes_read.sum + dram__bytes_write.sum from one ncu capture of
-# this file's network step, averaged over the kernel's launches in one step).  It is reported only while the kernel's
-# source still has the hash it had when the counters were taken.
+# this file's network step, averaged over the kernel's launches in one step).  It is reported only while the kernel and its
+# planner still have the hash they had when the counters were taken and a step has as many of its launches.
+CSRC = "paper_2303_04769_b200/csrc/"
 TRAFFIC = {
-    "conv_3xtf32_warp_mma": {"bytes_per_launch": 27034410.7, "source": "paper_2303_04769_b200/csrc/conv_mma.cuh",
-                             "sha256": "527a631d999499591cd9734e5b054a66bad05b1cbc1ae99376edb6c78c01de45"},
-    "conv_tf32_warp_mma": {"bytes_per_launch": 27010986.7, "source": "paper_2303_04769_b200/csrc/conv_mma.cuh",
-                           "sha256": "527a631d999499591cd9734e5b054a66bad05b1cbc1ae99376edb6c78c01de45"},
-    "conv_3xtf32_tensor": {"bytes_per_launch": 22910037.0, "source": "paper_2303_04769_b200/csrc/conv_tc.cu",
-                           "sha256": "46edea15c263baabda86068dc7269c4601c27973edc2dd8509505bfd06924f4c"},
-    "conv_tf32_tensor": {"bytes_per_launch": 24391387.0, "source": "paper_2303_04769_b200/csrc/conv_tc.cu",
-                         "sha256": "46edea15c263baabda86068dc7269c4601c27973edc2dd8509505bfd06924f4c"},
+    "conv_3xtf32_warp_mma": {"bytes_per_launch": 29065369.6, "launches": 5, "sources": ["conv_mma.cuh", "conv_mma.cu"],
+                             "sha256": "0e66de7151f4225d27af89bcccc74ec331f0b6d86be6c29b4b2070b235a19560"},
+    "conv_tf32_warp_mma": {"bytes_per_launch": 27006848.0, "launches": 6, "sources": ["conv_mma.cuh", "conv_mma.cu"],
+                           "sha256": "0e66de7151f4225d27af89bcccc74ec331f0b6d86be6c29b4b2070b235a19560"},
+    "conv_3xtf32_tensor": {"bytes_per_launch": 11419050.7, "launches": 3, "sources": ["conv_tc.cu"],
+                           "sha256": "e26c523d2dd0e7220a03d6e16c21855acb8a6a6adb91aff2a3db8fbcd4a5cbf5"},
+    "conv_tf32_tensor": {"bytes_per_launch": 8548352.0, "launches": 2, "sources": ["conv_tc.cu"],
+                         "sha256": "e26c523d2dd0e7220a03d6e16c21855acb8a6a6adb91aff2a3db8fbcd4a5cbf5"},
 }
 
 
-def measured_traffic(kernel):
+def source_hash(sources):
     import hashlib
+    h = hashlib.sha256()
+    for name in sources:
+        with open(os.path.join(ROOT, CSRC, name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()
+
+
+def measured_traffic(kernel, launches):
     t = TRAFFIC.get(kernel)
-    if not t or t["bytes_per_launch"] is None:
+    if not t or t["launches"] != launches:
         return None
     try:
-        h = hashlib.sha256(open(os.path.join(ROOT, t["source"]), "rb").read()).hexdigest()
+        return t["bytes_per_launch"] if source_hash(t["sources"]) == t["sha256"] else None
     except OSError:
         return None
-    return t["bytes_per_launch"] if h == t["sha256"] else None
 
 
 def load_peaks():
@@ -400,12 +408,12 @@ def gpu_main(args):
         peak = mode_peak_tflops(mode, peaks, sm_count)
         ach = dom["flops"] / (dom["ms"] * 1e-3) / 1e12
         roofline = {"bound": "alu" if mode == "fp32" else "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
-                    "frac": ach / peak, "traffic": measured_traffic(dom_name), "kernel": dom_name, "launches_per_step": dom["launches"],
+                    "frac": ach / peak, "traffic": measured_traffic(dom_name, dom["launches"]), "kernel": dom_name, "launches_per_step": dom["launches"],
                     "peak_source": f"{peaks['source']}: " + ("SMs x 128 x 2 x max SM clock" if mode == "fp32" else "BF16 burst x 0.5 (TF32)" + (" / 3" if mode == "3xtf32" else ""))}
     else:
         ach = dom["bytes"] / (dom["ms"] * 1e-3) / 1e9
         roofline = {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": ach / peaks["hbm_gbs"],
-                    "traffic": measured_traffic(dom_name), "kernel": dom_name, "launches_per_step": dom["launches"],
+                    "traffic": measured_traffic(dom_name, dom["launches"]), "kernel": dom_name, "launches_per_step": dom["launches"],
                     "peak_source": f"{peaks['source']}: copy bandwidth"}
     if dom_name.endswith("warp_mma"):
         # context: the warp-level MMA this kernel issues runs at 512 TF32 multiply-adds per clock and SM (measured with a

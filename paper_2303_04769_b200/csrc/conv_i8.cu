@@ -19,11 +19,14 @@
 // fit: a block keeps one filter tile and walks the pixel tiles), warp 1 issues the MMAs, warps 4-19 requantise and store.
 // Two to eight accumulator slots, so the MMAs of the next tiles run beside the requantisation of the ones before them.
 //
-// What bounds it: the requantisation - per output one three-input add, one 64-bit multiply-add (rounding, bias and zero
-// point in its addend), a shift, a maximum and half a saturating pack - and the latency of a small kernel, against CB *
-// taps MMAs of 128 x N x 32 at (128 + N) / 4 cycles per 128 pixels; hence sixteen epilogue warps.  Measured (batch 128,
-// 64 -> 64 on 28 x 28, 3 x 3): 13.9 us, of which an empty layer takes 4.8; the 4-way byte dot products on CUDA cores that
-// ran such layers before took 258 us.  512 x 64 -> 64 on 25 x 5, 1 x 1: 7.4 us.
+// What bounds it: the start.  Measured (batch 128, 64 -> 64 on 28 x 28, 3 x 3): 13.9 us, of which an empty layer takes 4.8; an SM
+// has five or six chunks, 18 MMAs of 128 x 80 x 32 each ((128 + N) / 4 cycles of operand reads and some to issue, about 1200 cycles a
+// chunk, 4 us in all), behind the arrival of all filters and the tables.  Tensor pipe 19 % of the active cycles, issue slots 45 %.
+// The requantisation - per output one three-input add, one 64-bit multiply-add (rounding, bias and zero point in its addend), a
+// shift, a maximum and half a saturating pack - runs beside the MMAs on sixteen warps, 400 cycles a chunk, and is the longer part
+// of 1 x 1 layers alone (512 x 64 -> 64 on 25 x 5: 7.4 us, tensor pipe 2 %).  Half of its shared-memory wavefronts are bank
+// conflicts: lanes of different border classes read rows of the same banks.  The 4-way byte dot products on CUDA cores that
+// ran such layers before took 258 us.
 #include <cuda.h>
 
 #include <cstring>

@@ -30,6 +30,9 @@ struct ThinArgs {
 
 // Threads per block: four warps.  A block loads a tile, then computes on it, with nothing in flight meanwhile, so
 // memory-level parallelism comes from many small blocks per SM being at different points of that cycle.
+// What bounds it: 10 x 4 stem, batch 1024, 42.5 us: FMA pipe 37 % of the active cycles, issue slots 65 % (27.4 M warp instructions
+// for 10.2 M FMAs: operand loads, the position of every loaded pixel by division), the rest of the time at the two barriers
+// of a tile.
 constexpr int kThinThreads = 128;
 
 template <int C, int FH, int FW, int S, int PIX, int KPT>

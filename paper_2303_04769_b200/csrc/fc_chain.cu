@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
     }
     grid_dep_trigger();
 
-    // copies a producer lane started and the parity of each barrier's latest one, kept for the drain after an abort
+    // copies the producer started and the parity of each barrier's latest one, kept for the drain after an abort
     uint32_t armed_mask = 0, armed_parity = 0, in_mask = 0, in_par = 0;
 
     if (warp == 1) {

@@ -67,3 +67,13 @@ def test_whole_job_throughput_two_ranks_gloo():
         value, ms = out[r]
         assert ms == pytest.approx(3.0) and value == pytest.approx(512 / 3e-3)
     assert bench.whole_job_throughput(256, 2.0, 1) == (pytest.approx(128000.0), 2.0)
+
+
+def test_measured_traffic_is_of_the_launches_it_was_counted_over(monkeypatch):
+    for kernel, t in bench.TRAFFIC.items():
+        monkeypatch.setitem(bench.TRAFFIC, kernel, dict(t, sha256=bench.source_hash(t["sources"])))
+        assert bench.measured_traffic(kernel, t["launches"]) == t["bytes_per_launch"]
+        assert bench.measured_traffic(kernel, t["launches"] + 1) is None
+        monkeypatch.setitem(bench.TRAFFIC, kernel, dict(t, sha256="0" * 64))
+        assert bench.measured_traffic(kernel, t["launches"]) is None
+    assert bench.measured_traffic("pool", 1) is None
