@@ -160,6 +160,7 @@ Plan plan_run(const small_layer *layers, int n, int from, int N, size_t max_smem
     for (int i = 0; i < a.n_in; ++i)
         if (p.in_slot[i] == p.out_slot) return p;
     a.n_stream = a.n_ops - 2;
+    a.N = N;
     p.smem = (size_t)top * 4;
     p.math = math;
     p.ok = true;
@@ -365,8 +366,11 @@ int launch_resident(small_ctx *ctx, const small_layer *layers, int n, int from, 
     const Kernel k = kernel_of(p->math);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->max_smem_optin - 1024);
     if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SMALL_ERR_CUDA; }
+    int lg = 0;
+    while ((1 << lg) < a.G) ++lg;
+    const int clusters = std::min(N, clusters_of(ctx, p->math, lg));
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(N * a.G)); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = p->smem; cfg.stream = st;
+    cfg.gridDim = dim3((unsigned)(clusters * a.G)); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = p->smem; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)a.G; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;

@@ -6,10 +6,10 @@
 // ten to thirty times: a launch takes 4 to 13 us whatever the batch, most of it start-up, the first copy's latency, and
 // the last tile.  A layer here ends with a barrier of one thread block, or of the few that share an image.
 //
-// Work split.  A cluster of G thread blocks (1, 2, 4 or 8: as many as the batch leaves SMs for) takes one image.  Every block
-// of a cluster holds ALL activations of the image; it computes its share of a convolution's output (filters split over the
-// blocks, then pixels) and stores each value into every block's copy (distributed shared memory), then a cluster barrier.
-// Depthwise layers are cheap and computed by every block for itself: no exchange.
+// Work split.  A cluster of G thread blocks (1, 2, 4 or 8: as many as the batch leaves SMs for) takes one image after the
+// other.  Every block of a cluster holds ALL activations of the image; it computes its share of a convolution's output
+// (filters split over the blocks, then pixels) and stores each value into every block's copy (distributed shared memory),
+// then a cluster barrier.  Depthwise layers are cheap and computed by every block for itself: no exchange.
 //
 // Layout of an activation: [pixel][pitch] floats, pitch = channels rounded up to 8, plus 4: the 16-byte chunks that eight
 // consecutive pixels hold at one channel then lie in eight different bank groups for every channel count, so ldmatrix and
@@ -57,7 +57,7 @@ struct Input { const float *g; int C, H, W, off, pitch; };
 struct Args {
     Op op[kMaxOps];
     Input in[kMaxInputs];
-    int n_ops, n_stream, n_in, G;           // n_stream: operations with streamed filters (all but the head)
+    int n_ops, n_stream, n_in, N, G;        // n_stream: operations with streamed filters (all but the head)
     int zero, scratch, ring, steps, ops;    // offsets (floats)
     float *out;                             // the full reduction's result, blocked [N][KB][1][1][32]
 };
@@ -116,12 +116,12 @@ __device__ __forceinline__ uint32_t tap_mask(const Op &o, int ih0, int iw0) {
 
 // The stream of filter chunks: (op, round, chunk) is the next one to be copied, `put` and `get` count stages.
 struct Stream {
-    int op, round, chunk, put, get;
+    int op, round, chunk, put, get, left;                // left: images whose filters are still to be streamed
 };
 
 // Copies the next chunk into its stage (one commit group per call, empty at the end).
 __device__ __forceinline__ void stream_issue(const Args &a, const Op *ops, Stream &st, const uint32_t sm, const int rank) {
-    if (st.op < a.n_stream) {
+    if (st.left > 0) {
         const Op &o = ops[st.op];
         const uint32_t dst = sm + (uint32_t)(a.ring + st.put * kStageFloats) * 4u;
         const int CB = (o.C + 31) >> 5;
@@ -153,7 +153,7 @@ __device__ __forceinline__ void stream_issue(const Args &a, const Op *ops, Strea
         if (++st.put == kStages) st.put = 0;
         if (o.kind == kDw || (++st.chunk == o.chunks && (st.chunk = 0, ++st.round) == o.rounds)) {
             st.round = 0;
-            ++st.op;
+            if (++st.op == a.n_stream) { st.op = 0; --st.left; }
         }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -596,8 +596,8 @@ __global__ void __launch_bounds__(kThreads, 1) net_resident_kernel(const __grid_
     const int G = a.G;
     int rank = 0;
     if (G > 1) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    const int n = blockIdx.x / G;                                   // this cluster's image
-    Stream st{0, 0, 0, 0, 0};
+    const int first = blockIdx.x / G, step = gridDim.x / G;
+    Stream st{0, 0, 0, 0, 0, first < a.N ? (a.N - first + step - 1) / step : 0};
     Op *ops = reinterpret_cast<Op *>(smem + a.ops);
     for (int i = threadIdx.x; i < a.n_ops * (int)(sizeof(Op) / 4); i += kThreads) reinterpret_cast<int *>(ops)[i] = reinterpret_cast<const int *>(a.op)[i];
     __syncthreads();
@@ -606,35 +606,38 @@ __global__ void __launch_bounds__(kThreads, 1) net_resident_kernel(const __grid_
     for (int i = threadIdx.x; i < kZeroFloats; i += kThreads) smem[a.zero + i] = 0.0f;
     grid_dep_sync();
     grid_dep_trigger();
+    for (int n = first; n < a.N; n += step) {
 #pragma unroll 1
-    for (int t = 0; t < a.n_in; ++t) {
-        const Input &in = a.in[t];
-        const int P = in.H * in.W, C4 = ((in.C + 7) & ~7) >> 2, CB = (in.C + 31) >> 5;
-        const float4 *g = reinterpret_cast<const float4 *>(in.g) + (size_t)n * CB * P * 8;
+        for (int t = 0; t < a.n_in; ++t) {
+            const Input &in = a.in[t];
+            const int P = in.H * in.W, C4 = ((in.C + 7) & ~7) >> 2, CB = (in.C + 31) >> 5;
+            const float4 *g = reinterpret_cast<const float4 *>(in.g) + (size_t)n * CB * P * 8;
 #pragma unroll 4
-        for (int i = threadIdx.x; i < P * C4; i += kThreads) {
-            const int p = i / C4, c4 = i - p * C4;
-            *reinterpret_cast<float4 *>(smem + in.off + p * in.pitch + c4 * 4) = g[((size_t)(c4 >> 3) * P + p) * 8 + (c4 & 7)];
+            for (int i = threadIdx.x; i < P * C4; i += kThreads) {
+                const int p = i / C4, c4 = i - p * C4;
+                *reinterpret_cast<float4 *>(smem + in.off + p * in.pitch + c4 * 4) = g[((size_t)(c4 >> 3) * P + p) * 8 + (c4 & 7)];
+            }
         }
-    }
-    // the image's inputs are in place
-    if (G > 1) cluster_sync(); else __syncthreads();
+        // the image's inputs are in place, and no block still works on the image before
+        if (G > 1) cluster_sync(); else __syncthreads();
 #pragma unroll 1
-    for (int l = 0; l < a.n_ops; ++l) {
-        const Op o = ops[l];                                    // in registers: fields read from the launch's constants where they are used cost a cache miss each
-        if (o.kind == kConv) {
-            int *tab = reinterpret_cast<int *>(smem) + a.steps + (l & 1) * kMaxSteps;      // (the operation before may still be reading its own)
-            if constexpr (MODE == 0) conv_fma(a, ops, o, st, sm, smem, rank, tab);
-            else conv_mma<MODE == 2>(a, ops, o, st, sm, smem, rank, tab);
-            if (G > 1) cluster_sync();                          // one block: the next operation's first chunk is waited for by all
-        } else if (o.kind == kDw) {
-            const int wat = stream_next(a, ops, st, sm, rank);
-            if (o.S == 1) dw_layer<1>(a, o, smem, wat); else dw_layer<2>(a, o, smem, wat);
-            if (G > 1 && o.exchange) cluster_sync();
-        } else if (rank == 0) {                                 // the classifier head: one block's work
-            __syncthreads();
-            if (o.kind == kGap) gap_layer(a, o, smem); else fc_layer(a, o, smem, n);
+        for (int l = 0; l < a.n_ops; ++l) {
+            const Op o = ops[l];                                    // in registers: fields read from the launch's constants where they are used cost a cache miss each
+            if (o.kind == kConv) {
+                int *tab = reinterpret_cast<int *>(smem) + a.steps + (l & 1) * kMaxSteps;      // (the operation before may still be reading its own)
+                if constexpr (MODE == 0) conv_fma(a, ops, o, st, sm, smem, rank, tab);
+                else conv_mma<MODE == 2>(a, ops, o, st, sm, smem, rank, tab);
+                if (G > 1) cluster_sync();                          // one block: the next operation's first chunk is waited for by all
+            } else if (o.kind == kDw) {
+                const int wat = stream_next(a, ops, st, sm, rank);
+                if (o.S == 1) dw_layer<1>(a, o, smem, wat); else dw_layer<2>(a, o, smem, wat);
+                if (G > 1 && o.exchange) cluster_sync();
+            } else if (rank == 0) {                                 // the classifier head: one block's work
+                __syncthreads();
+                if (o.kind == kGap) gap_layer(a, o, smem); else fc_layer(a, o, smem, n);
+            }
         }
+        __syncthreads();
     }
     if (G > 1) cluster_sync();                                      // no block leaves while another may still store into it
 }
