@@ -606,6 +606,8 @@ __global__ void __launch_bounds__(kThreads, 1) net_resident_kernel(const __grid_
     for (int i = threadIdx.x; i < kZeroFloats; i += kThreads) smem[a.zero + i] = 0.0f;
     grid_dep_sync();
     grid_dep_trigger();
+    // (Runs are chosen so that every cluster has one image, see worth_it, and the loop turns once.  Written without it, the FP32
+    // kernel's code comes out slower: keyword-spotting network, batch 75, 55.4 -> 57.4 us, and seven other ways no better.)
     for (int n = first; n < a.N; n += step) {
 #pragma unroll 1
         for (int t = 0; t < a.n_in; ++t) {

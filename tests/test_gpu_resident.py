@@ -1,5 +1,5 @@
 """Runs of layers kept on chip as one kernel, against the oracle and against the same network launched layer by layer: ragged
-channel counts and planes, strides, residual joins, one to eight thread blocks per image and several images per block."""
+channel counts and planes, strides, residual joins, one to eight thread blocks per image."""
 import numpy as np
 import pytest
 import torch
