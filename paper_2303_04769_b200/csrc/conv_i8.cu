@@ -436,7 +436,7 @@ conv_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 }
 
 // ---------------------------------------------------------------------------------------------- host side
-struct I8Plan { I8Args a; int ch; unsigned grid; size_t smem; int es_w, es_h; bool ok; };
+struct I8Plan { I8Args a; int ch; unsigned grid; size_t smem; bool ok; };
 
 int floor_half(int v) { return v >= 0 ? v / 2 : -((1 - v) / 2); }
 
