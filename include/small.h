@@ -391,7 +391,8 @@ typedef struct small_layer {
  * a global average pool with the full reduction behind it, in every math mode (SMALL_FUSE_POOLFC, see small_gap_fc).  The skipped
  * intermediate tensors are then not written.  Default: all four (without DWPW_ALWAYS); 0 runs every layer on its own.
  * With every kind on, a whole run of convolutions and depthwise 3x3 layers that ends the list in a global average pool and a full
- * reduction may run as one kernel that keeps each image's activations on chip (small batches; where it was measured to pay).
+ * reduction may run as one kernel that keeps each image's activations on chip (small batches; where it was measured to pay), and so
+ * may, at any batch and place of the list, a run of three or more depthwise 3x3 -> 1x1 pairs under a tensor-core math mode.
  * Results stay within each math mode's tolerance either way. */
 enum { SMALL_FUSE_DWPW = 1u, SMALL_FUSE_DWPW_ALWAYS = 2u, SMALL_FUSE_CONVPOOL = 4u, SMALL_FUSE_FC_CHAIN = 8u,
        SMALL_FUSE_POOLFC = 16u };   /* a global average pool and the full reduction behind it (small_gap_fc) */

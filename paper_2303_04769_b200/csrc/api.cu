@@ -112,6 +112,7 @@ SMALL_API int small_init(int device, small_ctx **out) {
     c->dw_cache = nullptr;
     c->path_cache = nullptr;
     c->resident_state = nullptr;
+    c->chain_state = nullptr;
     c->wait_iters = 1u << 22;     // with the polls' nanosleep back-off: seconds
     if (resolve_static_workspace(c) != SMALL_OK) {      // loads the library's device code here, not inside a later call
         cudaFree(block);
@@ -160,6 +161,7 @@ SMALL_API int small_shutdown(small_ctx *ctx) {
     free_dw_cache(ctx);
     delete static_cast<PathCache *>(ctx->path_cache);
     free_resident_state(ctx);
+    free_chain_state(ctx);
     if (ctx->ev_fork) cudaEventDestroy(static_cast<cudaEvent_t>(ctx->ev_fork));
     if (ctx->ev_join) cudaEventDestroy(static_cast<cudaEvent_t>(ctx->ev_join));
     if (ctx->side_stream) cudaStreamDestroy(static_cast<cudaStream_t>(ctx->side_stream));

@@ -36,6 +36,7 @@ struct small_ctx {
     void *tc_cache;          // finished launches of the tensor-core kernel by (shape, mode, tensors); conv_tc.cu
     void *mma_cache;         // the same for the warp-level tensor-core kernel; conv_mma.cu
     void *resident_state;    // plans of the resident network kernel; net_resident.cu
+    void *chain_state;       // plans and finished launches of runs of depthwise and 1x1 pairs; sep_chain.cu
     void *direct_cache;      // the same for the register-tiled FP32 kernel; conv_direct.cu
     void *dw_cache;          // the same for the depthwise 3x3 kernel; dwconv.cu
     void *path_cache;        // kernel family per shape, mode and path setting; api.cu
@@ -121,6 +122,7 @@ void free_i8_cache(small_ctx *);             // conv_i8.cu
 void free_direct_cache(small_ctx *);         // conv_direct.cu
 void free_dw_cache(small_ctx *);             // dwconv.cu
 void free_resident_state(small_ctx *);       // net_resident.cu
+void free_chain_state(small_ctx *);          // sep_chain.cu
 int resolve_static_workspace(small_ctx *);   // net_static.cu; called by small_init with the context's device current
 
 // ---- kernel launchers (each in its own .cu); all return a small_status ----
@@ -181,6 +183,12 @@ int launch_conv_mma(small_ctx *, const float *in, const float *w_hi, const float
 int resident_from(small_ctx *, const small_layer *layers, int n, int from, int N);
 int launch_resident(small_ctx *, const small_layer *layers, int n, int from, int N, const std::function<const float *(int)> &rd,
                     const std::function<float *(int)> &wr, cudaStream_t);
+// no layer from `from` on reads the slot before it is written again (net.cu)
+bool slot_dead_after(const small_layer *layers, int n_layers, int from, int slot);
+// a run of depthwise 3x3 -> 1x1 pairs as one kernel (sep_chain.cu): how many layers the run at layer i covers (0: none), with a
+// global average pool and full reduction behind it where it ends in those, and its launch
+int sep_chain_layers(small_ctx *, const small_layer *layers, int n, int i, int N);
+int launch_sep_chain(small_ctx *, const small_layer *layers, int n, int i, int N, const float *in, float *out, cudaStream_t);
 // quantised full channel reduction (conv_i8.cu): windows 1 or 3 wide, strides 1 and 2; w: [CB][FH*FW][KB*32][32] bytes,
 // w_sums: [K][FH*FW] sums of weight bytes over the channels
 int launch_q_conv(small_ctx *, const uint8_t *in, const uint8_t *w, const int *w_sums, const int *bias, uint8_t *out, const Geom &,

@@ -72,7 +72,7 @@ static bool plan_slots(const small_layer *layers, int n_layers, int N, SlotPlan 
 // ---- abstract fused layers (Section 6) chosen by the runner itself: the caller describes plain layers.
 // A layer's result may stay on chip when the next layer is its only reader: nothing after that reads the slot before
 // it is written again, and the pair's output slot is not the pair's input slot.
-static bool slot_dead_after(const small_layer *layers, int n_layers, int from, int slot) {
+bool slot_dead_after(const small_layer *layers, int n_layers, int from, int slot) {
     for (int j = from; j < n_layers; ++j) {
         const small_layer &L = layers[j];
         if (L.src == slot || (L.op == SMALL_OP_ADD && L.src2 == slot)) return false;
@@ -163,12 +163,10 @@ static int fc_chain_len(const small_ctx *ctx, const small_layer *layers, int n_l
     return L >= 2 ? L : 0;
 }
 
-// First layer of the run that is kept on chip (net_resident.cu), -1 for none: where every kind of fusion is on.
-static int resident_start(small_ctx *ctx, const small_layer *layers, int n_layers, int from, int N) {
+// Runs of layers are kept on chip as one kernel where every kind of fusion is on.
+static bool runs_allowed(const small_ctx *ctx) {
     const unsigned rest = SMALL_FUSE_CONVPOOL | SMALL_FUSE_FC_CHAIN | SMALL_FUSE_POOLFC;
-    if ((ctx->net_fusion & rest) != rest || !(ctx->net_fusion & (SMALL_FUSE_DWPW | SMALL_FUSE_DWPW_ALWAYS)) || ctx->conv_path != SMALL_CONV_PATH_AUTO)
-        return -1;
-    return resident_from(ctx, layers, n_layers, from, N);
+    return (ctx->net_fusion & rest) == rest && (ctx->net_fusion & (SMALL_FUSE_DWPW | SMALL_FUSE_DWPW_ALWAYS)) && ctx->conv_path == SMALL_CONV_PATH_AUTO;
 }
 
 }  // namespace small
@@ -277,13 +275,26 @@ static int run_layers(small_ctx *ctx, const small_layer *layers, int n_layers, i
         return SMALL_ERR_INVALID_ARG;
     };
     bool after_join = false;
-    const int on_chip = resident_start(ctx, layers, n_layers, from, N);
+    // a run of depthwise / 1x1 pairs (sep_chain.cu); without one, a run up to the end of the list (net_resident.cu)
+    int chain = -1, chain_layers = 0, on_chip = -1;
+    if (runs_allowed(ctx)) {
+        for (int i = from; i < n_layers && !chain_layers; ++i)
+            if ((chain_layers = sep_chain_layers(ctx, layers, n_layers, i, N)) > 0) chain = i;
+        if (!chain_layers) on_chip = resident_from(ctx, layers, n_layers, from, N);
+    }
     for (int i = from; i < n_layers; ++i) {
         const small_layer &L = layers[i];
         int s = SMALL_OK;
         // every layer behind the first may start its set-up while the layer in front of it drains (see launch_kernel)
         ctx->dependent = ctx->overlap && i > 0 && !after_join;
         after_join = false;
+        if (i == chain) {
+            s = launch_sep_chain(ctx, layers, n_layers, i, N, rd(L.src), wr(layers[i + chain_layers - 1].dst), static_cast<cudaStream_t>(stream));
+            ctx->dependent = 0;
+            if (s != SMALL_OK) return s;
+            i += chain_layers - 1;
+            continue;
+        }
         if (i == on_chip) {
             s = launch_resident(ctx, layers, n_layers, from, N, rd, wr, static_cast<cudaStream_t>(stream));
             ctx->dependent = 0;
@@ -305,7 +316,7 @@ static int run_layers(small_ctx *ctx, const small_layer *layers, int n_layers, i
                 }
             }
         }
-        if (const int fused = i + 1 == on_chip ? 0 : fused_pair(ctx, layers, n_layers, i, N)) {
+        if (const int fused = i + 1 == on_chip || i + 1 == chain ? 0 : fused_pair(ctx, layers, n_layers, i, N)) {
             const small_layer &Nx = layers[i + 1];
             if (fused == SMALL_OP_DWPW) {
                 const unsigned fl = ((L.flags & SMALL_RELU) ? SMALL_RELU_MID : 0u) | (Nx.flags & (SMALL_RELU | SMALL_MATH_MASK));
@@ -327,7 +338,7 @@ static int run_layers(small_ctx *ctx, const small_layer *layers, int n_layers, i
         // shortcut) run side by side: the second one on the context's side stream, forked from and joined to the caller's
         // stream by events, so that a short layer hides behind a long one.  Both are ordinary launches, and so is the
         // layer behind the join.
-        if (ctx->branch_overlap && ctx->side_stream && i + 1 < n_layers && i + 1 != on_chip && independent(L, layers[i + 1]) &&
+        if (ctx->branch_overlap && ctx->side_stream && i + 1 < n_layers && i + 1 != on_chip && i + 1 != chain && independent(L, layers[i + 1]) &&
             !fused_pair(ctx, layers, n_layers, i + 1, N)) {
             cudaStream_t main_st = static_cast<cudaStream_t>(stream), side = static_cast<cudaStream_t>(ctx->side_stream);
             cudaError_t e = cudaEventRecord(static_cast<cudaEvent_t>(ctx->ev_fork), main_st);
