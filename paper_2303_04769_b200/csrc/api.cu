@@ -110,6 +110,7 @@ SMALL_API int small_init(int device, small_ctx **out) {
     c->i8_cache = nullptr;
     c->direct_cache = nullptr;
     c->dw_cache = nullptr;
+    c->thin_cache = nullptr;
     c->path_cache = nullptr;
     c->resident_state = nullptr;
     c->chain_state = nullptr;
@@ -159,6 +160,7 @@ SMALL_API int small_shutdown(small_ctx *ctx) {
     free_i8_cache(ctx);
     free_direct_cache(ctx);
     free_dw_cache(ctx);
+    free_thin_cache(ctx);
     delete static_cast<PathCache *>(ctx->path_cache);
     free_resident_state(ctx);
     free_chain_state(ctx);

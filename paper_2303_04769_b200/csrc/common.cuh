@@ -39,6 +39,7 @@ struct small_ctx {
     void *chain_state;       // plans and finished launches of runs of depthwise and 1x1 pairs; sep_chain.cu
     void *direct_cache;      // the same for the register-tiled FP32 kernel; conv_direct.cu
     void *dw_cache;          // the same for the depthwise 3x3 kernel; dwconv.cu
+    void *thin_cache;        // the same for the kernel of few input channels; conv_thin.cu
     void *path_cache;        // kernel family per shape, mode and path setting; api.cu
     void *i8_cache;          // the same for the quantised convolution; conv_i8.cu
     void *static_workspace;  // device address of the library's built-in workspace array on this device (net_static.cu)
@@ -121,6 +122,7 @@ void free_mma_cache(small_ctx *);            // conv_mma.cu
 void free_i8_cache(small_ctx *);             // conv_i8.cu
 void free_direct_cache(small_ctx *);         // conv_direct.cu
 void free_dw_cache(small_ctx *);             // dwconv.cu
+void free_thin_cache(small_ctx *);           // conv_thin.cu
 void free_resident_state(small_ctx *);       // net_resident.cu
 void free_chain_state(small_ctx *);          // sep_chain.cu
 int resolve_static_workspace(small_ctx *);   // net_static.cu; called by small_init with the context's device current
