@@ -17,10 +17,11 @@
 //   epilogue    = thread = filter: tensor memory -> registers, + bias, ReLU, and the filter's nt values go straight back
 //                 into the B slots as the next layer's operand (for 3xTF32 split into TF32 part and residual); the last
 //                 layer's values go to global memory, a warp writing one image's 32-channel line per store
-// Roles: warp 0 issues the MMAs; warp 1 streams the first layer's input and every layer's filters (each one thread's work,
+// Roles: warp 0 issues the MMAs; warp 1 streams every layer's filters, warp 2 the first layer's input (each one thread's work,
 // done by a uniform warp: see elect_one); warps 4 .. (four per 32 images) run the epilogue.
 //
-// The chain is latency-bound: per layer the MMAs (16 of 40 to 64 cycles), their completion, the epilogue and its hand-over
+// The chain is latency-bound (batch 4096, TF32: 26.6 us with a barrier per box, 22.6 now; 16 epilogue warps, whose polls stand in the
+// way of the MMAs, 24.7): per layer the MMAs (16 of 40 to 64 cycles), their completion, the epilogue and its hand-over
 // follow one another.  Roles written as `if (lane == 0)` took some 140 cycles per MMA, several hundred per copy and 450 per
 // commit, and needed several producer lanes and hand-overs in groups to hide it.
 //
@@ -81,13 +82,14 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *base_ptr = smem_raw + (base - smem_u32(smem_raw));
-    constexpr uint32_t kWStage = X3 ? 2 * kWBlock : kWBlock;
+    constexpr uint32_t kWBlockAll = X3 ? 2 * kWBlock : kWBlock;      // a channel block's filters
+    constexpr int BPS = X3 ? 1 : 2;                                  // channel blocks of a stage (32 KB either way)
     const int nt = a.nt, n_slots = a.n_slots;
     // a slot: the tile's nt rows of one channel block; 3xTF32: the residuals' nt rows right behind them, so that one
     // descriptor of 2 nt rows covers both
     const uint32_t slot_bytes = (uint32_t)nt * 128u, slot_pitch = X3 ? 2u * slot_bytes : slot_bytes;
     const uint32_t x_base = base, w_base = base + (uint32_t)n_slots * slot_pitch;
-    const uint32_t ctrl = w_base + (uint32_t)a.w_stages * kWStage;
+    const uint32_t ctrl = w_base + (uint32_t)a.w_stages * BPS * kWBlockAll;
     uint8_t *ctrl_ptr = base_ptr + (ctrl - base);
     const uint32_t bar_w_full = ctrl + kOffWFull, bar_w_empty = ctrl + kOffWEmpty, bar_in = ctrl + kOffInFull, bar_split = ctrl + kOffSplit,
                    bar_slot_free = ctrl + kOffSlotFree, bar_acc = ctrl + kOffAccFull, bar_epi = ctrl + kOffEpiDone;
@@ -140,40 +142,27 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
     uint32_t armed_mask = 0, armed_parity = 0, in_mask = 0, in_par = 0;
 
     if (warp == 1) {
-        // ---- first layer: its input blocks; every layer: one filter box (rows x 128 bytes; 3xTF32: two) per channel block
-        bool alive = true, synced = false;
-        uint32_t tile_k = 0, s = 0, pw = 1;                  // filter stage in turn and the parity its release is waited with
-        for (int t = blockIdx.x; t < a.tiles && alive; t += gridDim.x, ++tile_k) {
+        // ---- every layer's filters: one box (rows x 128 bytes; 3xTF32: two) per channel block, two boxes a stage: waiting for a stage
+        // and arming its barrier take some 200 cycles, a copy more 15 (TF32 with one box a stage: 26.7 us for 22.6)
+        bool alive = true;
+        uint32_t s = 0, pw = 1;                              // filter stage in turn and the parity its release is waited with
+        for (int t = blockIdx.x; t < a.tiles && alive; t += gridDim.x) {
             for (int st = 0; st < steps_per_tile && alive; ++st) {
                 const int l = min(st, a.L - 1), ch = st - l, JB = (a.J[l] + 31) >> 5;
                 const uint32_t bytes = (uint32_t)a.box_rows[l] * 128u * (X3 ? 2u : 1u);
-                for (int cb = 0; cb < JB; ++cb) {
-                    if (l == 0) {
-                        const int slot = cb & (n_slots - 1), sg = slot >> 2, o = cb >> ns_log2;
-                        const uint32_t use = tile_k * slot_uses(slot) + (uint32_t)o;
-                        // the slot's previous content: this tile's block cb - n_slots, or the previous tile's activations
-                        // (a group's barrier completes once per use that another use of the same tile follows)
-                        if (o > 0) {
-                            if ((slot & 3) == 0)
-                                alive = mbar_wait_uniform<kSpin>(bar_slot_free + 8 * sg, (tile_k * (group_uses(sg) - 1u) + (uint32_t)o - 1u) & 1u, abort_flag, a.status, a.wait_iters);
-                        } else if (tile_k > 0 && cb == 0) {
-                            alive = __all_sync(0xffffffffu, counter_wait(steps_done, tile_k * (uint32_t)steps_per_tile, abort_flag, a.status, a.wait_iters));
-                        }
-                        if (!alive) break;
-                        if (!synced) { grid_dep_sync(); synced = true; }
-                        if (elect_one()) {
-                            mbar_expect_tx(bar_in + 8 * slot, slot_bytes);
-                            tma_load_3d(x_base + slot * slot_pitch, &a.map_in, bar_in + 8 * slot, 0, cb, t * nt);
-                        }
-                        in_mask |= 1u << slot;
-                        in_par = (in_par & ~(1u << slot)) | ((use & 1u) << slot);
-                    }
+                for (int cb = 0; cb < JB; cb += BPS) {
+                    const int nb = min(BPS, JB - cb);
                     alive = mbar_wait_uniform<kSpin>(bar_w_empty + 8 * s, pw, abort_flag, a.status, a.wait_iters);    // passes at once in the first round
                     if (!alive) break;
                     if (elect_one()) {
-                        mbar_expect_tx(bar_w_full + 8 * s, bytes);
-                        tma_load_3d(w_base + s * kWStage, &a.map_w[l], bar_w_full + 8 * s, 0, ch * 128, cb);
-                        if (X3) tma_load_3d(w_base + s * kWStage + kWBlock, &a.map_w_lo[l], bar_w_full + 8 * s, 0, ch * 128, cb);
+                        const uint32_t bar = bar_w_full + 8 * s, dst = w_base + s * BPS * kWBlockAll;
+                        mbar_expect_tx(bar, nb * bytes);
+                        tma_load_3d(dst, &a.map_w[l], bar, 0, ch * 128, cb);
+                        if (X3) tma_load_3d(dst + kWBlock, &a.map_w_lo[l], bar, 0, ch * 128, cb);
+                        if (nb == 2) {
+                            tma_load_3d(dst + kWBlockAll, &a.map_w[l], bar, 0, ch * 128, cb + 1);
+                            if (X3) tma_load_3d(dst + kWBlockAll + kWBlock, &a.map_w_lo[l], bar, 0, ch * 128, cb + 1);
+                        }
                     }
                     armed_mask |= 1u << s;
                     armed_parity = (armed_parity & ~(1u << s)) | ((pw ^ 1u) << s);
@@ -181,6 +170,33 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
                 }
             }
         }
+    } else if (warp == 2) {
+        // ---- the first layer's input: two channel blocks per barrier
+        bool alive = true;
+        uint32_t tile_k = 0;
+        grid_dep_sync();
+        for (int t = blockIdx.x; t < a.tiles && alive; t += gridDim.x, ++tile_k)
+            for (int cb = 0; cb < JB0; cb += 2) {
+                const int nb = min(2, JB0 - cb);
+                const int slot = cb & (n_slots - 1), sg = slot >> 2, o = cb >> ns_log2;
+                const uint32_t use = tile_k * slot_uses(slot) + (uint32_t)o;
+                // the slots' previous content: this tile's blocks cb - n_slots, or the previous tile's activations
+                // (a group's barrier completes once per use that another use of the same tile follows)
+                if (o > 0) {
+                    if ((slot & 3) == 0)
+                        alive = mbar_wait_uniform<kSpin>(bar_slot_free + 8 * sg, (tile_k * (group_uses(sg) - 1u) + (uint32_t)o - 1u) & 1u, abort_flag, a.status, a.wait_iters);
+                } else if (tile_k > 0 && cb == 0) {
+                    alive = __all_sync(0xffffffffu, counter_wait(steps_done, tile_k * (uint32_t)steps_per_tile, abort_flag, a.status, a.wait_iters));
+                }
+                if (!alive) break;
+                if (elect_one()) {
+                    mbar_expect_tx(bar_in + 8 * slot, nb * slot_bytes);
+                    tma_load_3d(x_base + slot * slot_pitch, &a.map_in, bar_in + 8 * slot, 0, cb, t * nt);
+                    if (nb == 2) tma_load_3d(x_base + (slot + 1) * slot_pitch, &a.map_in, bar_in + 8 * slot, 0, cb + 1, t * nt);
+                }
+                in_mask |= 1u << slot;
+                in_par = (in_par & ~(1u << slot)) | ((use & 1u) << slot);
+            }
     } else if (warp == 0) {
         // ---- the MMAs of every step (a layer, or a chunk of 128 filters of the last layer)
         const uint32_t elected = elect_one();
@@ -188,7 +204,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
         uint32_t g = 0, tile_k = 0;                        // g: steps so far; accumulator and its barriers = g mod nacc
         const uint32_t idesc = instr_desc(nt), idesc_wide = instr_desc(2 * nt);
         const uint32_t w_desc0 = smem_desc_lo(w_base), x_desc0 = smem_desc_lo(x_base);
-        const uint32_t w_step = kWStage >> 4, x_step = slot_pitch >> 4, w_lo = kWBlock >> 4;
+        const uint32_t w_step = kWBlockAll >> 4, x_step = slot_pitch >> 4, w_lo = kWBlock >> 4;
         uint32_t sw = 0, pw = 0;                           // filter stage in turn, its parity
         auto issue = [&](auto ks_tag, uint32_t acc, uint32_t xb, uint32_t wa, uint32_t started) {      // the MMAs of one channel block
             constexpr int KS = decltype(ks_tag)::value;
@@ -211,10 +227,11 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
                 const uint32_t acc = tmem + ga * acc_cols;
                 // a layer whose filters all fit in the stages: they are waited for before the epilogue is, so that nothing but
                 // MMAs follows the latter
-                const bool ahead = l > 0 && JB <= a.w_stages;
+                const int stages = (JB + BPS - 1) / BPS;
+                const bool ahead = l > 0 && stages <= a.w_stages, late = ahead && 2 * stages <= a.w_stages;
                 if (ahead) {
                     uint32_t s1 = sw, p1 = pw;
-                    for (int cb = 0; cb < JB && alive; ++cb) {
+                    for (int i = 0; i < stages && alive; ++i) {
                         alive = mbar_wait_uniform<kSpin>(bar_w_full + 8 * s1, p1, abort_flag, a.status, a.wait_iters);
                         if (++s1 == (uint32_t)a.w_stages) { s1 = 0; p1 ^= 1u; }
                     }
@@ -228,49 +245,43 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
                     alive = mbar_wait_uniform<kSpin>(bar_epi + 8 * ga, ((g >> nacc_log2) - 1u) & 1u, abort_flag, a.status, a.wait_iters);
                 if (!alive) break;
                 tc_fence_after();                          // orders the MMAs after the epilogue's reads of the accumulator
-                if (ahead) {
-                    uint32_t xb = x_desc0;
-                    for (int cb = 0; cb < JB - 1; ++cb, xb += x_step) {
-                        if (elected) {
-                            issue(std::integral_constant<int, 4>{}, acc, xb, w_desc0 + sw * w_step, cb > 0 ? 1u : 0u);
-                            mma_commit(bar_w_empty + 8 * sw);
-                        }
-                        if (++sw == (uint32_t)a.w_stages) { sw = 0; pw ^= 1u; }
-                    }
-                    if (elected) {
-                        const uint32_t wa = w_desc0 + sw * w_step, started = JB > 1 ? 1u : 0u;
-                        if (ks_last == 4) issue(std::integral_constant<int, 4>{}, acc, xb, wa, started);
-                        else
-                            for (int k = 0; k < ks_last; ++k) issue(std::integral_constant<int, 1>{}, acc, xb + 2u * k, wa + 2u * k, k ? 1u : started);
-                        mma_commit(bar_w_empty + 8 * sw);
-                        mma_commit(bar_acc + 8 * ga);
-                    }
-                    if (++sw == (uint32_t)a.w_stages) { sw = 0; pw ^= 1u; }
-                    continue;
-                }
-                for (int cb = 0; cb < JB; ++cb) {
-                    uint32_t slot = (uint32_t)cb;
-                    if (l == 0) {
-                        slot = (uint32_t)(cb & (n_slots - 1));
+                for (int cb = 0; cb < JB; cb += BPS) {
+                    const int nb = min(BPS, JB - cb);
+                    const uint32_t slot = l == 0 ? (uint32_t)(cb & (n_slots - 1)) : (uint32_t)cb;
+                    if (l == 0 && (cb & 1) == 0) {                    // two blocks of the input share a barrier
                         const uint32_t use = tile_k * slot_uses((int)slot) + (uint32_t)(cb >> ns_log2);
                         alive = mbar_wait_uniform<kSpin>((X3 ? bar_split : bar_in) + 8 * slot, use & 1u, abort_flag, a.status, a.wait_iters);
                         if (!alive) break;
                     }
-                    alive = mbar_wait_uniform<kSpin>(bar_w_full + 8 * sw, pw, abort_flag, a.status, a.wait_iters);
-                    if (!alive) break;
-                    const uint32_t xb = x_desc0 + slot * x_step, wa = w_desc0 + sw * w_step, started = cb > 0 ? 1u : 0u;
-                    const int ks = cb == JB - 1 ? ks_last : 4;
+                    if (!ahead) {
+                        alive = mbar_wait_uniform<kSpin>(bar_w_full + 8 * sw, pw, abort_flag, a.status, a.wait_iters);
+                        if (!alive) break;
+                    }
+                    const uint32_t xb = x_desc0 + slot * x_step, wa = w_desc0 + BPS * sw * w_step, started = cb > 0 ? 1u : 0u;
+                    const bool full = cb + nb < JB || ks_last == 4;
                     if (elected) {
-                        if (ks == 4) issue(std::integral_constant<int, 4>{}, acc, xb, wa, started);
-                        else
-                            for (int k = 0; k < ks; ++k) issue(std::integral_constant<int, 1>{}, acc, xb + 2u * k, wa + 2u * k, k ? 1u : started);
-                        mma_commit(bar_w_empty + 8 * sw);
+                        if (nb == BPS && full) {
+                            issue(std::integral_constant<int, 4>{}, acc, xb, wa, started);
+                            if (BPS == 2) issue(std::integral_constant<int, 4>{}, acc, xb + x_step, wa + w_step, 1u);
+                        } else {
+                            for (int i = 0; i < nb; ++i) {
+                                const int ks = cb + i == JB - 1 ? ks_last : 4;
+                                for (int k = 0; k < ks; ++k) issue(std::integral_constant<int, 1>{}, acc, xb + i * x_step + 2u * k, wa + i * w_step + 2u * k, i + k ? 1u : started);
+                            }
+                        }
+                        if (!late) mma_commit(bar_w_empty + 8 * sw);
                         // a group of four slots that a later block of this layer reuses: signal when its last block is done
-                        if (l == 0 && ((cb & 3) == 3 || cb == JB - 1) && (cb & ~3) + n_slots < JB) mma_commit(bar_slot_free + 8 * (slot >> 2));
+                        if (l == 0 && (((cb + BPS) & 3) == 0 || cb + BPS >= JB) && (cb & ~3) + n_slots < JB) mma_commit(bar_slot_free + 8 * (slot >> 2));
                     }
                     if (++sw == (uint32_t)a.w_stages) { sw = 0; pw ^= 1u; }
                 }
-                if (alive && elected) mma_commit(bar_acc + 8 * ga);
+                if (alive && elected) {
+                    mma_commit(bar_acc + 8 * ga);
+                    // (a commit takes the issuing thread some 120 cycles: the epilogue's comes first, a layer's stages go back behind it
+                    // where as many again hold the next one's)
+                    if (late)
+                        for (int i = stages; i > 0; --i) mma_commit(bar_w_empty + 8 * ((sw + a.w_stages - i) % a.w_stages));
+                }
             }
         }
     } else if (warp >= 4 && warp < 4 + n_epi_warps) {
@@ -284,13 +295,14 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
         grid_dep_sync();                                              // before the first write to global memory
         for (int t = blockIdx.x; t < a.tiles && alive; t += gridDim.x, ++tile_k) {
             if (X3)
-                for (int cb = 0; cb < JB0 && alive; ++cb) {
-                    const int slot = cb & (n_slots - 1);
+                for (int cb = 0; cb < JB0 && alive; cb += 2) {
+                    const int slot = cb & (n_slots - 1), nb = min(2, JB0 - cb);
                     const uint32_t use = tile_k * slot_uses(slot) + (uint32_t)(cb >> ns_log2);
                     alive = mbar_wait_warp<kSpin>(bar_in + 8 * slot, use & 1u, abort_flag, a.status, a.wait_iters);
                     if (!alive) break;
-                    for (int idx = tid_e; idx < nt * 8; idx += n_epi) {               // 16-byte chunks of the block
-                        float4 *p = reinterpret_cast<float4 *>(x_ptr + (size_t)slot * slot_pitch + (size_t)idx * 16);
+                    for (int idx = tid_e; idx < nb * nt * 8; idx += n_epi) {          // 16-byte chunks of the blocks
+                        const int second = idx >= nt * 8 ? 1 : 0;
+                        float4 *p = reinterpret_cast<float4 *>(x_ptr + (size_t)(slot + second) * slot_pitch + (size_t)(idx - second * nt * 8) * 16);
                         const float4 v = *p;
                         const float4 h = make_float4(__uint_as_float(__float_as_uint(v.x) & 0xffffe000u), __uint_as_float(__float_as_uint(v.y) & 0xffffe000u),
                                                      __uint_as_float(__float_as_uint(v.z) & 0xffffe000u), __uint_as_float(__float_as_uint(v.w) & 0xffffe000u));
@@ -362,7 +374,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
         }
     }
     __syncthreads();
-    if (*abort_flag && warp == 1 && lane == 0) {     // a role gave up: let the copies still in flight land
+    if (*abort_flag && (warp == 1 || warp == 2) && lane == 0) {     // a role gave up: let the copies still in flight land
         for (int st = 0; st < 16; ++st) {
             if (st < 8 && (armed_mask >> st & 1u))
                 for (uint32_t it = 0; it < a.wait_iters && !mbar_try_wait(bar_w_full + 8 * st, armed_parity >> st & 1u); ++it) __nanosleep(200);
@@ -399,7 +411,7 @@ int launch_fc_chain(small_ctx *ctx, const float *in, const float *const *w_blk, 
     // the larger tiles stream the filters fewer times.  A tile whose shared memory does not fit is halved.
     int nt = ctx->fc_chain_tile;
     if (nt == 0) nt = N <= 32 * ctx->sm_count ? 32 : N <= 64 * ctx->sm_count ? 64 : 128;
-    const size_t stage_bytes = (size_t)kWBlock * (x3 ? 2 : 1);
+    const size_t stage_bytes = (size_t)2 * kWBlock;
     const bool wide = widths[0] > 128;
     int w_stages = 0, n_slots = 0;
     size_t smem = 0;
@@ -408,7 +420,7 @@ int launch_fc_chain(small_ctx *ctx, const float *in, const float *const *w_blk, 
         const size_t slot_bytes = (size_t)nt * 128 * (x3 ? 2 : 1);
         // Filter stages: two layers' worth (TF32), one layer's (3xTF32).  Operand slots: four hold 128 channels; more deepen
         // the stream of a wider first layer, which needs at least eight (slots go back in groups of four).
-        w_stages = x3 ? 4 : 8; n_slots = 4;                                                  // slots: a power of two
+        w_stages = 4; n_slots = 4;                                                  // slots: a power of two
         while (n_slots < 16 && (size_t)(2 * n_slots) * slot_bytes <= 64 * 1024) n_slots *= 2;
         if (wide && n_slots < 8) n_slots = 8;
         const size_t fixed = 1024 + n_slots * slot_bytes + kCtrl;
