@@ -95,11 +95,11 @@ int small_out_size(int I, int F, int stride, int pad_before, int pad_after);
 const char *small_strerror(int status);
 /* Last cudaError_t / CUresult seen by this context (0 if none). */
 int small_last_cuda_error(small_ctx *ctx);
-/* Layer overlap inside small_run_net (on by default; `on` = 0 switches it off).  When on, every layer behind the
- * first is launched with programmatic stream serialisation: its thread blocks may become resident and set up shared
- * memory, barriers and tensor memory while the layer in front of it is still draining, and they wait on the device
- * until that layer has completed before they read or write a tensor.  Results are the same either way.  The paper
- * has no counterpart. */
+/* Layer overlap (on by default; `on` = 0 switches it off).  When on, layers - called on their own or by small_run_net - are
+ * launched with programmatic stream serialisation: their thread blocks may become resident and set up shared memory,
+ * barriers and tensor memory while the kernel in front of them in the stream is still draining, and they wait on the
+ * device until that kernel has completed before they read or write a tensor.  (Filters and biases are read earlier only
+ * behind a layer of the same network.)  Results are the same either way.  The paper has no counterpart. */
 int small_set_layer_overlap(small_ctx *ctx, int on);
 /* Branch overlap inside small_run_net (on by default; `on` = 0 switches it off).  When on, two neighbouring layers of the
  * list that share no tensor except as readers - a residual stage's convolution and its shortcut convolution - run at the

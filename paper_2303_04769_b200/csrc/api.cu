@@ -122,6 +122,7 @@ SMALL_API int small_init(int device, small_ctx **out) {
     }
     c->overlap = 1;
     c->dependent = 0;
+    c->in_net = 0;
     c->conv_path = SMALL_CONV_PATH_AUTO;
     c->net_fusion = SMALL_FUSE_DWPW | SMALL_FUSE_CONVPOOL | SMALL_FUSE_FC_CHAIN | SMALL_FUSE_POOLFC;
     c->branch_overlap = 1;
@@ -309,6 +310,7 @@ SMALL_API int small_group_conv2d(small_ctx *ctx, const float *in, const float *w
                                  int N, int C, int F_C, int S_C, int K, int H, int W, int FH, int FW, int stride,
                                  int pt, int pb, int pl, int pr, unsigned flags, void *stream) {
     if (!ctx) return SMALL_ERR_NOT_INIT;
+    CallOfItsOwn call(ctx);
     if (flags & ~(SMALL_RELU | SMALL_ACCUMULATE | SMALL_MATH_MASK)) return SMALL_ERR_INVALID_ARG;
     if (!math_valid(math_of(flags))) return SMALL_ERR_INVALID_ARG;
     if (int s = check_ptrs({in, w, out}, {bias})) return s;
@@ -447,6 +449,7 @@ SMALL_API int small_conv2d(small_ctx *ctx, const float *in, const float *w, cons
                            int N, int C, int K, int H, int W, int FH, int FW, int stride,
                            int pt, int pb, int pl, int pr, unsigned flags, void *stream) {
     if (!ctx) return SMALL_ERR_NOT_INIT;
+    CallOfItsOwn call(ctx);
     if (flags & ~(SMALL_RELU | SMALL_ACCUMULATE | SMALL_MATH_MASK)) return SMALL_ERR_INVALID_ARG;
     unsigned math = math_of(flags);
     if (!math_valid(math)) return SMALL_ERR_INVALID_ARG;
@@ -486,6 +489,7 @@ SMALL_API int small_conv_maxpool2d(small_ctx *ctx, const float *in, const float 
                                    int N, int C, int K, int H, int W, int FH, int FW, int stride,
                                    int pt, int pb, int pl, int pr, unsigned flags, void *stream) {
     if (!ctx) return SMALL_ERR_NOT_INIT;
+    CallOfItsOwn call(ctx);
     if (flags & ~(SMALL_RELU | SMALL_MATH_MASK)) return SMALL_ERR_INVALID_ARG;
     if (!math_valid(math_of(flags))) return SMALL_ERR_INVALID_ARG;
     if (int s = check_ptrs({in, w, out}, {bias, scratch})) return s;
@@ -509,6 +513,7 @@ SMALL_API int small_dwconv2d(small_ctx *ctx, const float *in, const float *w, co
                              int N, int C, int H, int W, int FH, int FW, int stride,
                              int pt, int pb, int pl, int pr, unsigned flags, void *stream) {
     if (!ctx) return SMALL_ERR_NOT_INIT;
+    CallOfItsOwn call(ctx);
     if (flags & ~(SMALL_RELU | SMALL_MATH_MASK)) return SMALL_ERR_INVALID_ARG;
     if (!math_valid(math_of(flags))) return SMALL_ERR_INVALID_ARG;
     if (int s = check_ptrs({in, w, out}, {bias})) return s;
@@ -539,6 +544,7 @@ SMALL_API int small_dwpw_conv2d(small_ctx *ctx, const float *in, const float *dw
                                 int N, int C, int K, int H, int W, int stride,
                                 int pt, int pb, int pl, int pr, unsigned flags, void *stream) {
     if (!ctx) return SMALL_ERR_NOT_INIT;
+    CallOfItsOwn call(ctx);
     if (flags & ~(SMALL_RELU | SMALL_RELU_MID | SMALL_MATH_MASK)) return SMALL_ERR_INVALID_ARG;
     const unsigned math = math_of(flags);
     if (!math_valid(math)) return SMALL_ERR_INVALID_ARG;
@@ -573,6 +579,7 @@ SMALL_API int small_pool2d(small_ctx *ctx, const float *in, float *out, int32_t 
                            int N, int C, int H, int W, int FH, int FW, int stride,
                            int pt, int pb, int pl, int pr, int mode, void *stream) {
     if (!ctx) return SMALL_ERR_NOT_INIT;
+    CallOfItsOwn call(ctx);
     if (mode != SMALL_POOL_MAX && mode != SMALL_POOL_AVG) return SMALL_ERR_INVALID_ARG;
     if (idx && mode != SMALL_POOL_MAX) return SMALL_ERR_INVALID_ARG;
     if (int s = check_ptrs({in, out}, {idx})) return s;
@@ -586,6 +593,7 @@ SMALL_API int small_pool2d(small_ctx *ctx, const float *in, float *out, int32_t 
 
 SMALL_API int small_relu(small_ctx *ctx, const float *in, float *out, int N, int C, int H, int W, void *stream) {
     if (!ctx) return SMALL_ERR_NOT_INIT;
+    CallOfItsOwn call(ctx);
     if (int s = check_ptrs({in, out})) return s;
     size_t n = packed_elems(N, C, H, W);
     if (n == 0) return SMALL_ERR_SHAPE;
@@ -618,6 +626,7 @@ SMALL_API int small_upsample_nearest(small_ctx *ctx, const float *in, float *out
 SMALL_API int small_add(small_ctx *ctx, const float *a, const float *b, float *out, int N, int C, int H, int W,
                         unsigned flags, void *stream) {
     if (!ctx) return SMALL_ERR_NOT_INIT;
+    CallOfItsOwn call(ctx);
     if (flags & ~SMALL_RELU) return SMALL_ERR_INVALID_ARG;
     if (int s = check_ptrs({a, b, out})) return s;
     size_t n = packed_elems(N, C, H, W);
@@ -643,6 +652,7 @@ SMALL_API int small_fc_uses_tensor_cores(int N, int J, int K, unsigned math) {
 SMALL_API int small_fc(small_ctx *ctx, const float *in, const float *w, const float *bias, float *out,
                        int N, int J, int K, unsigned flags, void *stream) {
     if (!ctx) return SMALL_ERR_NOT_INIT;
+    CallOfItsOwn call(ctx);
     if (flags & ~(SMALL_RELU | SMALL_MATH_MASK)) return SMALL_ERR_INVALID_ARG;
     const unsigned math = math_of(flags);
     if (!math_valid(math)) return SMALL_ERR_INVALID_ARG;
@@ -671,6 +681,7 @@ SMALL_API int small_gap_fc_fused(int N, int C, int K, unsigned math) {
 SMALL_API int small_gap_fc(small_ctx *ctx, const float *in, const float *w, const float *bias, float *out, float *scratch,
                            int N, int C, int H, int W, int K, unsigned flags, void *stream) {
     if (!ctx) return SMALL_ERR_NOT_INIT;
+    CallOfItsOwn call(ctx);
     if (flags & ~(SMALL_RELU | SMALL_MATH_MASK)) return SMALL_ERR_INVALID_ARG;
     const unsigned math = math_of(flags);
     if (!math_valid(math)) return SMALL_ERR_INVALID_ARG;
@@ -701,6 +712,7 @@ SMALL_API int small_fc_chain_fused(const int *widths, int L, unsigned math) {
 SMALL_API int small_fc_chain(small_ctx *ctx, const float *in, const float *const *w_blk, const float *const *bias, const int *widths,
                              const int *relu, float *out, float *scratch, int L, int N, unsigned flags, void *stream) {
     if (!ctx) return SMALL_ERR_NOT_INIT;
+    CallOfItsOwn call(ctx);
     if (flags & ~SMALL_MATH_MASK) return SMALL_ERR_INVALID_ARG;
     const unsigned math = math_of(flags);
     if (!math_valid(math) || !w_blk || !widths || !relu || L < 1 || L > 64) return SMALL_ERR_INVALID_ARG;

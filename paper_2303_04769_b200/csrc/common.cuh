@@ -31,7 +31,8 @@ struct small_ctx {
     int sm_count;
     size_t max_smem_optin;
     int overlap;             // small_run_net launches every layer after the first as a dependent launch (see launch_kernel)
-    int dependent;           // set by small_run_net while it issues those layers
+    int dependent;           // how the next layer is launched: 0 the ordinary way, 1 and 2 as a dependent launch (see launch_kernel)
+    int in_net;              // small_run_net is issuing layers: it sets `dependent`
     unsigned wait_iters;     // limit (polls) of every bounded device-side wait; small_set_wait_limit
     void *tc_cache;          // finished launches of the tensor-core kernel by (shape, mode, tensors); conv_tc.cu
     void *mma_cache;         // the same for the warp-level tensor-core kernel; conv_mma.cu
@@ -89,6 +90,11 @@ static inline int check_launch(small_ctx *ctx) {
 // grid_dep_sync() until the earlier kernel has completed and its writes are visible.  Launched the ordinary way,
 // both instructions do nothing.  Chains stay ordered: a kernel cannot complete before its own grid_dep_sync()
 // returns, so completion of kernel i implies completion of every kernel before it.
+// What a layer may do in front of grid_dep_sync() depends on the kernel before it.  Behind a layer of the same network
+// (ctx->dependent = 1) it may read its filters and biases: that layer does not write them, and has seen to it that everything
+// older is finished (its own trigger comes behind its wait).  Behind any other kernel of the stream (2: a call of its own, a
+// network's first layer) it reads nothing: the kernel in front may be what writes the filters.  Kernels that read constants early
+// take that as `late` and wait first.
 #ifdef __CUDACC__
 __device__ __forceinline__ void grid_dep_sync() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -107,6 +113,14 @@ static inline void launch_kernel(small_ctx *ctx, void (*kern)(KArgs...), dim3 gr
     (void)e;   // picked up by check_launch through cudaGetLastError
 }
 #endif
+
+// A layer called on its own: a dependent launch of the second kind where those are on.  (Inside a network the network decides.)
+struct CallOfItsOwn {
+    small_ctx *ctx;
+    int before;
+    explicit CallOfItsOwn(small_ctx *c) : ctx(c), before(c->dependent) { if (!c->in_net) c->dependent = c->overlap ? 2 : 0; }
+    ~CallOfItsOwn() { ctx->dependent = before; }
+};
 
 // Geometry of one windowed layer, validated once on the host and passed to kernels by value.
 struct Geom {

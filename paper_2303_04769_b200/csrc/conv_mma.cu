@@ -162,7 +162,8 @@ int launch_conv_mma(small_ctx *ctx, const float *in, const float *w_hi, const fl
     {
         auto it = cache.find(key);
         if (it != cache.end()) {
-            const MmaLaunch &L = it->second;
+            MmaLaunch &L = it->second;
+            L.a.late = ctx->dependent == 2;
             launch_kernel(ctx, L.kern, dim3(L.grid), dim3(L.threads), L.smem, st, L.map_in, L.map_w, L.map_w_lo, L.a);
             return check_launch(ctx);
         }
@@ -170,7 +171,7 @@ int launch_conv_mma(small_ctx *ctx, const float *in, const float *w_hi, const fl
     MmaPlan p = plan_mma(g, x3, ctx->max_smem_optin, ctx->sm_count);
     if (!p.ok) return SMALL_ERR_UNSUPPORTED;
     MmaArgs &a = p.a;
-    a.bias = bias; a.out = out; a.status = ctx->dev_status; a.relu = relu; a.accumulate = accumulate; a.wait_iters = ctx->wait_iters;
+    a.bias = bias; a.out = out; a.status = ctx->dev_status; a.relu = relu; a.accumulate = accumulate; a.wait_iters = ctx->wait_iters; a.late = ctx->dependent == 2;
     sm100::EncodeTiledFn encode = reinterpret_cast<sm100::EncodeTiledFn>(ctx->encode_tiled);
     const CUtensorMapSwizzle swz = p.CW == 16 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
     CUtensorMap map_in, map_w, map_w_lo;

@@ -27,6 +27,7 @@ struct MmaArgs {
     uint32_t w_box_bytes, w_half_bytes;   // bytes of one filter box (TF32 part or residual) and its 1 KB-rounded place
     int relu, accumulate;
     uint32_t wait_iters;
+    int late;                   // wait for the kernel in front before reading constants
 };
 
 __device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t (&r)[4]) {
@@ -87,7 +88,8 @@ conv_mma_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constan
         failed = 0;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {       // the filters are the layer's own constants: no earlier kernel of the stream writes them
+    if (a.late) grid_dep_sync();
+    if (threadIdx.x == 0) {       // the filters are the layer's own constants
         sm100::mbar_expect_tx(bar_w, a.w_box_bytes * (X3 ? 2u : 1u));
         sm100::tma_load_4d(w_hi_s, &map_w, bar_w, 0, kt * 32, 0, 0);
         if (X3) sm100::tma_load_4d(w_lo_s, &map_w_lo, bar_w, 0, kt * 32, 0, 0);

@@ -113,6 +113,7 @@ struct TcArgs {
     uint32_t x_lo_off;         // 3xTF32: 16-byte units from a strip's TF32 part to its residual
     int relu, accumulate;
     uint32_t wait_iters;       // limit of every bounded wait (polls)
+    int late;                  // wait for the kernel in front before reading constants
     // the layer's taps sorted by phase plane: strip offset (16-byte units: 8 per pixel), original tap; phase p holds the
     // entries phase_at[p] .. phase_at[p + 1] - 1
     int phase_at[5];
@@ -212,6 +213,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 if (X3) rest[i + a.b_half / 16] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
+    if (a.late) grid_dep_sync();
     for (int i = threadIdx.x; i < a.KB * 32; i += kNT) bias_s[i] = (a.bias && i < a.K) ? a.bias[i] : 0.0f;
     if (DW)
         for (int i = threadIdx.x; i < a.CBr * 10 * 32; i += kNT) {
@@ -1062,7 +1064,8 @@ int launch_conv_tc(small_ctx *ctx, const float *in, const float *w_hi, const flo
     {
         auto it = cache.find(key);
         if (it != cache.end()) {
-            const TcLaunch &L = it->second;
+            TcLaunch &L = it->second;
+            L.a.late = ctx->dependent == 2;
             launch_kernel(ctx, L.kern, dim3(L.grid), dim3(L.threads), L.smem, st, L.map_a, L.map_b, L.map_b_lo, L.a);
             return check_launch(ctx);
         }
@@ -1159,7 +1162,7 @@ int launch_conv_tc(small_ctx *ctx, const float *in, const float *w_hi, const flo
         a.phase_at[ph + 1] = n;
     }
     const int ks = p.ks_last == 3 ? 4 : p.ks_last;     // a K step of zero channels more is harmless
-    a.relu = relu; a.accumulate = accumulate; a.wait_iters = ctx->wait_iters;
+    a.relu = relu; a.accumulate = accumulate; a.wait_iters = ctx->wait_iters; a.late = ctx->dependent == 2;
     const TcKernel kern = pick_kernel(chains, ks, p.pixel_m != 0, x3, dw != nullptr);
     if (!kern) return SMALL_ERR_UNSUPPORTED;
     // the attribute belongs to the kernel instance, which other layers share: always the device's limit, so that a

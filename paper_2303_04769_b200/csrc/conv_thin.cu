@@ -42,6 +42,7 @@ struct ThinArgs {
     bool tma;                                // planes of at most 256 columns with their pads, blocked
     bool nchw;                               // the input is the NCHW tensor float[N][C][H][W] itself (the network's edge)
     uint32_t wait_iters;                     // limit of the bounded waits (polls)
+    int late;                                // wait for the kernel in front before reading constants
 };
 
 constexpr int kThinThreads = 128;
@@ -74,6 +75,7 @@ __global__ void __launch_bounds__(kThinThreads, thin_blocks(C *FH *FW, PIX, (PIX
     // the last group's second one may not exist)
     const int kb = LANES == 32 ? (int)blockIdx.y * 2 + (fl >> 4) : 0, k0 = kb * 32 + 2 * (fl & 15);
     const bool line_exists = LANES < 32 || kb < a.KB;
+    if (a.late) grid_dep_sync();
     // filters: [kb][0][x][y][ci][ko], a pair per 8-byte load (two 4-byte ones put together are put together again at every use)
     uint64_t wr[C][FH][FW];
 #pragma unroll
@@ -277,13 +279,15 @@ int launch_conv_thin(small_ctx *ctx, const float *in, const float *w, const floa
     {
         auto it = cache.find(key);
         if (it != cache.end()) {
-            const ThinLaunch &L = it->second;
+            ThinLaunch &L = it->second;
+            L.a.late = ctx->dependent == 2;
             launch_kernel(ctx, L.kern, L.grid, dim3(kThinThreads), L.smem, st, L.map, L.a);
             return check_launch(ctx);
         }
     }
     ThinLaunch made{};
     ThinArgs &a = made.a;
+    a.late = ctx->dependent == 2;
     a.in = in; a.w = w; a.bias = bias; a.out = out; a.status = ctx->dev_status; a.wait_iters = ctx->wait_iters;
     a.N = g.N; a.K = g.K; a.KB = g.KB; a.H = g.H; a.W = g.W; a.OH = g.OH; a.OW = g.OW; a.pt = g.pt; a.pl = g.pl;
     a.relu = relu; a.accumulate = accumulate; a.nchw = nchw_in;

@@ -62,6 +62,7 @@ struct ChainArgs {
     int L, N, tiles;
     int nt, n_slots, w_stages;          // images per tile, operand slots, filter stages
     uint32_t wait_iters;
+    int late;                           // wait for the kernel in front before reading constants
 };
 
 // Bounded wait for a counter in shared memory to reach `need` (a count, unlike a barrier's phase parity, can be read
@@ -125,6 +126,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fc_chain_kernel(const __grid_c
         *steps_done = 0;
         mbar_fence_init();
     }
+    if (a.late) grid_dep_sync();
     uint32_t tmem = 0;
     if (warp == 1) {
         __syncwarp();
@@ -428,7 +430,7 @@ int launch_fc_chain(small_ctx *ctx, const float *in, const float *const *w_blk, 
         smem = fixed + w_stages * stage_bytes;
         if (smem <= ctx->max_smem_optin) break;
     }
-    a.L = L; a.N = N; a.tiles = ceil_div(N, nt); a.out = out; a.status = ctx->dev_status; a.wait_iters = ctx->wait_iters;
+    a.L = L; a.N = N; a.tiles = ceil_div(N, nt); a.out = out; a.status = ctx->dev_status; a.wait_iters = ctx->wait_iters; a.late = ctx->dependent == 2;
     a.nt = nt; a.n_slots = n_slots; a.w_stages = w_stages;
     {   // the first layer's input, blocked [N][JB][32]: one box = nt images x one 32-channel block
         const int JB = blocks_of(widths[0]);

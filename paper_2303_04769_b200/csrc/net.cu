@@ -274,6 +274,11 @@ static int run_layers(small_ctx *ctx, const small_layer *layers, int n_layers, i
         }
         return SMALL_ERR_INVALID_ARG;
     };
+    struct InNet {
+        small_ctx *ctx;
+        ~InNet() { ctx->in_net = 0; ctx->dependent = 0; }
+    } in_net{ctx};
+    ctx->in_net = 1;
     bool after_join = false;
     // a run of depthwise / 1x1 pairs (sep_chain.cu); without one, a run up to the end of the list (net_resident.cu)
     int chain = -1, chain_layers = 0, on_chip = -1;
@@ -285,8 +290,8 @@ static int run_layers(small_ctx *ctx, const small_layer *layers, int n_layers, i
     for (int i = from; i < n_layers; ++i) {
         const small_layer &L = layers[i];
         int s = SMALL_OK;
-        // every layer behind the first may start its set-up while the layer in front of it drains (see launch_kernel)
-        ctx->dependent = ctx->overlap && i > 0 && !after_join;
+        // every layer may start its set-up while the kernel in front of it drains (see launch_kernel)
+        ctx->dependent = !ctx->overlap || after_join ? 0 : i > 0 ? 1 : 2;
         after_join = false;
         if (i == chain) {
             s = launch_sep_chain(ctx, layers, n_layers, i, N, rd(L.src), wr(layers[i + chain_layers - 1].dst), static_cast<cudaStream_t>(stream));

@@ -377,7 +377,7 @@ int launch_resident(small_ctx *ctx, const small_layer *layers, int n, int from, 
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = ctx->dependent ? 2 : 1;
+    cfg.numAttrs = ctx->dependent == 1 ? 2 : 1;      // (the filter stream starts in front of the wait)
     e = cudaLaunchKernelEx(&cfg, k, a);
     (void)e;                                             // picked up by check_launch through cudaGetLastError
     return check_launch(ctx);

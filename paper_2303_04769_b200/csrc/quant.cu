@@ -381,6 +381,7 @@ SMALL_API int small_q_conv2d(small_ctx *ctx, const uint8_t *in, const void *w_bl
                              int N, int C, int K, int H, int W, int FH, int FW, int stride, int pt, int pb, int pl, int pr,
                              int z_in, int z_w, int z_out, int mult, int shift, unsigned flags, void *stream) {
     if (!ctx) return SMALL_ERR_NOT_INIT;
+    CallOfItsOwn call(ctx);
     if (flags & ~SMALL_RELU) return SMALL_ERR_INVALID_ARG;
     if (!in || !w_blk || !out || !qparams_ok(z_in, z_w, z_out, mult, shift)) return SMALL_ERR_INVALID_ARG;
     if (!aligned16(in) || !aligned16(w_blk) || !aligned16(out) || (bias && (reinterpret_cast<uintptr_t>(bias) & 3u))) return SMALL_ERR_ALIGN;
@@ -413,6 +414,7 @@ SMALL_API int small_q_dwconv2d(small_ctx *ctx, const uint8_t *in, const uint8_t 
                                int N, int C, int H, int W, int FH, int FW, int stride, int pt, int pb, int pl, int pr,
                                int z_in, int z_w, int z_out, int mult, int shift, unsigned flags, void *stream) {
     if (!ctx) return SMALL_ERR_NOT_INIT;
+    CallOfItsOwn call(ctx);
     if (flags & ~SMALL_RELU) return SMALL_ERR_INVALID_ARG;
     if (!in || !w_blk || !out || !qparams_ok(z_in, z_w, z_out, mult, shift)) return SMALL_ERR_INVALID_ARG;
     if (!aligned16(in) || !aligned16(w_blk) || !aligned16(out) || (bias && (reinterpret_cast<uintptr_t>(bias) & 3u))) return SMALL_ERR_ALIGN;
@@ -441,6 +443,7 @@ SMALL_API int small_q_dwconv2d(small_ctx *ctx, const uint8_t *in, const uint8_t 
 SMALL_API int small_q_maxpool2d(small_ctx *ctx, const uint8_t *in, uint8_t *out, int N, int C, int H, int W, int FH, int FW,
                                 int stride, int pt, int pb, int pl, int pr, int z, void *stream) {
     if (!ctx) return SMALL_ERR_NOT_INIT;
+    CallOfItsOwn call(ctx);
     if (!in || !out || z < 0 || z > 255) return SMALL_ERR_INVALID_ARG;
     if (!aligned16(in) || !aligned16(out)) return SMALL_ERR_ALIGN;
     Geom g;

@@ -76,6 +76,7 @@ struct Args {
     // classifier behind the run (head_K > 0): packed FP32 filters [KB][CB][32][32]
     const float *head_w, *head_bias; int head_K, head_relu, head_b_at;
     uint32_t wait_iters;
+    int late;                       // wait for the kernel in front before reading constants
 };
 
 __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {      // two FMAs
@@ -308,6 +309,7 @@ __global__ void __launch_bounds__(256, PER_SM) sep_chain_kernel(const __grid_con
         *abort_flag = 0;
         mbar_fence_init();
     }
+    if (a.late) grid_dep_sync();
     {   // biases of every layer and of the head, zero in the pad lanes (the layers' own constants); copies that nothing waits for one by one
         auto bring = [&](int at, const float *src, int real, int n) {
             for (int i = threadIdx.x; i < n; i += kThreads) {
@@ -806,7 +808,7 @@ int launch_sep_chain(small_ctx *ctx, const small_layer *layers, int n, int i, in
         made = &e.made.back();
     }
     Args a = e.p->a;
-    a.out = out; a.status = ctx->dev_status; a.wait_iters = ctx->wait_iters;
+    a.out = out; a.status = ctx->dev_status; a.wait_iters = ctx->wait_iters; a.late = ctx->dependent == 2;
     const bool two = e.p->per_sm == 2;
     auto kern = x3 ? (two ? sep_chain_kernel<true, 2> : sep_chain_kernel<true, 1>) : (two ? sep_chain_kernel<false, 2> : sep_chain_kernel<false, 1>);
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->max_smem_optin);
