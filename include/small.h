@@ -128,7 +128,8 @@ int small_set_conv_path(small_ctx *ctx, int path);
 /* Which kernel small_conv2d runs for this shape and math mode (with a 32-byte aligned output) under the context's
  * path setting: 0 = few-input-channel kernel (network stems), 1 = register-tiled FP32 kernel, 2 = general FP32 kernel,
  * 3 = block-level tensor-core kernel (tcgen05), 4 = warp-level tensor-core kernel (few channels and filters);
- * -1 for invalid arguments. */
+ * -1 for invalid arguments.  Under AUTO, layers of 3 and 4 with so few output pixels that their tiles would leave most of the
+ * GPU idle run as warp-level MMAs with the reduction split over warps; the number reported stays the one of the shape's family. */
 int small_conv2d_path(small_ctx *ctx, int N, int C, int K, int H, int W, int FH, int FW, int stride,
                       int pad_t, int pad_b, int pad_l, int pad_r, unsigned math);
 /* Synchronises `stream`, then reads and clears the device status word: *status is SMALL_OK or

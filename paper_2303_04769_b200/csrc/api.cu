@@ -375,7 +375,7 @@ static bool prefer_cuda_cores(const small_ctx *ctx, const Geom &g, unsigned math
     return g.FH * g.FW == 1 || (math == SMALL_MATH_3XTF32 && g.S == 2);
 }
 
-static int choose_path(const small_ctx *ctx, const Geom &g, unsigned math, bool out_aligned32) {
+static int choose_whole(const small_ctx *ctx, const Geom &g, unsigned math, bool out_aligned32) {
     if (ctx && ctx->conv_path == SMALL_CONV_PATH_WARP_MMA && math != SMALL_MATH_FP32 && conv_mma_supported(g, math == SMALL_MATH_3XTF32)) return 4;
     if (conv_thin_supported(g)) return 0;          // a reduction of a few dozen terms: CUDA cores in every math mode
     if (ctx && ctx->conv_path == SMALL_CONV_PATH_GENERAL) return 2;
@@ -418,6 +418,16 @@ static int choose_path(const small_ctx *ctx, const Geom &g, unsigned math, bool 
     return direct ? 1 : 2;
 }
 
+// kSplit on top: a tensor-core layer of few pixels, whose reduction is split over warps (conv_split.cu).  (Layers that the rules above
+// leave to FP32 arithmetic stay there.)
+constexpr int kSplit = 8;
+static int choose_path(const small_ctx *ctx, const Geom &g, unsigned math, bool out_aligned32) {
+    const int path = choose_whole(ctx, g, math, out_aligned32);
+    const bool split = path >= 3 && (!ctx || ctx->conv_path == SMALL_CONV_PATH_AUTO) &&
+                       conv_split_preferred(g, math == SMALL_MATH_3XTF32, path == 4, ctx ? ctx->sm_count : kSmCount);
+    return split ? path + kSplit : path;
+}
+
 // The choice walks the planners of several kernels; it depends on the shape and two settings alone and is kept per context.
 static int conv2d_path(small_ctx *ctx, const Geom &g, unsigned math, bool out_aligned32) {
     if (!ctx) return choose_path(ctx, g, math, out_aligned32);
@@ -442,7 +452,7 @@ SMALL_API int small_conv2d_path(small_ctx *ctx, int N, int C, int K, int H, int 
                                 int pt, int pb, int pl, int pr, unsigned math) {
     Geom g;
     if (!ctx || !math_valid(math) || make_geom(g, N, C, K, H, W, FH, FW, stride, pt, pb, pl, pr) != SMALL_OK) return -1;
-    return conv2d_path(ctx, g, math, true);
+    return conv2d_path(ctx, g, math, true) & (kSplit - 1);
 }
 
 SMALL_API int small_conv2d(small_ctx *ctx, const float *in, const float *w, const float *bias, float *out,
@@ -473,6 +483,11 @@ SMALL_API int small_conv2d(small_ctx *ctx, const float *in, const float *w, cons
             const float *w_hi = w + conv_w_fp32_elems(C, K, FH, FW);
             const float *w_lo = w_hi + conv_w_tc_elems(C, K, FH, FW);
             return launch_conv_mma(ctx, in, w_hi, math == SMALL_MATH_3XTF32 ? w_lo : nullptr, bias, out, g, relu, acc, math, st);
+        }
+        case 3 + kSplit: case 4 + kSplit: {
+            const float *w_hi = w + conv_w_fp32_elems(C, K, FH, FW);
+            const float *w_lo = w_hi + conv_w_tc_elems(C, K, FH, FW);
+            return launch_conv_split(ctx, in, w_hi, math == SMALL_MATH_3XTF32 ? w_lo : nullptr, bias, out, g, relu, acc, math, st);
         }
         default: return launch_conv_fp32(ctx, in, w, bias, out, g, relu, acc, st);
     }

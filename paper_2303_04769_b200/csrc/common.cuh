@@ -194,6 +194,11 @@ int launch_conv_tc(small_ctx *, const float *in, const float *w_hi, const float 
 bool conv_mma_supported(const Geom &, bool x3);
 int launch_conv_mma(small_ctx *, const float *in, const float *w_hi, const float *w_lo, const float *bias, float *out,
                     const Geom &, bool relu, bool accumulate, unsigned mode, cudaStream_t);
+// warp-level tensor-core kernel for few pixels (conv_split.cu), whose rule says where it is the fastest of the tensor-core kernels;
+// any channels, filters, window and stride; reads the same filter sections
+bool conv_split_preferred(const Geom &, bool x3, bool warp_level, int sms);     // warp_level: instead of conv_mma.cu, else conv_tc.cu
+int launch_conv_split(small_ctx *, const float *in, const float *w_hi, const float *w_lo, const float *bias, float *out,
+                      const Geom &, bool relu, bool accumulate, unsigned mode, cudaStream_t);
 // a run of layers up to the end of the list as one kernel (net_resident.cu): the first layer of the run at or behind `from`
 // (-1: none), and its launch, which reads and writes whole tensors through rd / wr (slot -> address)
 int resident_from(small_ctx *, const small_layer *layers, int n, int from, int N);

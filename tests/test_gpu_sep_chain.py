@@ -60,7 +60,9 @@ def test_run_matches_the_oracle(name, math, batch):
 @pytest.mark.parametrize("math", ["tf32", "3xtf32"])
 def test_many_images_match_the_layers_one_by_one(name, math, batch):
     """Several images per thread block, two blocks per SM: the stream of filters crosses the images' ends.  Both forms round alike but
-    for the order of sums, so they agree far inside the tolerance (FP32 sums of at most 256 products: 1e-5)."""
+    for the order of sums, so they agree far inside the tolerance: FP32 sums of at most 256 products, 1e-5.  In TF32 such a difference
+    can take an operand of the next layer across a rounding boundary: one product is then off by 2^-10 of its size, which is at most
+    the MAX_ELEMENT_FACTOR = 8 rms that rel_err divides by."""
     net = RUNS[name]
     params, x = configs.make_params(net), configs.make_input(net, batch)
     blk = to_blk(x)
@@ -68,7 +70,7 @@ def test_many_images_match_the_layers_one_by_one(name, math, batch):
     shape = (batch,) + tuple(gnet.out_shape)
     want = from_blk(apart.run(blk), *shape)
     got = gnet.run(blk)
-    assert rel_err(from_blk(got, *shape), want) <= 1e-5
+    assert rel_err(from_blk(got, *shape), want) <= (1e-5 if math == "3xtf32" else 2.0 ** -10)
     first = got.clone()
     for _ in range(3):
         assert torch.equal(gnet.run(blk), first)
