@@ -418,13 +418,13 @@ static int choose_whole(const small_ctx *ctx, const Geom &g, unsigned math, bool
     return direct ? 1 : 2;
 }
 
-// kSplit on top: a tensor-core layer of few pixels, whose reduction is split over warps (conv_split.cu).  (Layers that the rules above
-// leave to FP32 arithmetic stay there.)
+// kSplit on top: a layer of few pixels, whose reduction is split over warps - on the tensor cores (conv_split.cu), or in FP32 where the
+// rules above choose FP32 arithmetic (conv_split_fp32.cu)
 constexpr int kSplit = 8;
 static int choose_path(const small_ctx *ctx, const Geom &g, unsigned math, bool out_aligned32) {
-    const int path = choose_whole(ctx, g, math, out_aligned32);
-    const bool split = path >= 3 && (!ctx || ctx->conv_path == SMALL_CONV_PATH_AUTO) &&
-                       conv_split_preferred(g, math == SMALL_MATH_3XTF32, path == 4, ctx ? ctx->sm_count : kSmCount);
+    const int path = choose_whole(ctx, g, math, out_aligned32), sms = ctx ? ctx->sm_count : kSmCount;
+    if (path == 0 || (ctx && ctx->conv_path != SMALL_CONV_PATH_AUTO)) return path;
+    const bool split = path >= 3 ? conv_split_preferred(g, math == SMALL_MATH_3XTF32, path == 4, sms) : conv_split_fp32_preferred(g, sms);
     return split ? path + kSplit : path;
 }
 
@@ -484,6 +484,7 @@ SMALL_API int small_conv2d(small_ctx *ctx, const float *in, const float *w, cons
             const float *w_lo = w_hi + conv_w_tc_elems(C, K, FH, FW);
             return launch_conv_mma(ctx, in, w_hi, math == SMALL_MATH_3XTF32 ? w_lo : nullptr, bias, out, g, relu, acc, math, st);
         }
+        case 1 + kSplit: case 2 + kSplit: return launch_conv_split_fp32(ctx, in, w, bias, out, g, relu, acc, st);
         case 3 + kSplit: case 4 + kSplit: {
             const float *w_hi = w + conv_w_fp32_elems(C, K, FH, FW);
             const float *w_lo = w_hi + conv_w_tc_elems(C, K, FH, FW);

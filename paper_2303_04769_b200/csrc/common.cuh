@@ -199,6 +199,10 @@ int launch_conv_mma(small_ctx *, const float *in, const float *w_hi, const float
 bool conv_split_preferred(const Geom &, bool x3, bool warp_level, int sms);     // warp_level: instead of conv_mma.cu, else conv_tc.cu
 int launch_conv_split(small_ctx *, const float *in, const float *w_hi, const float *w_lo, const float *bias, float *out,
                       const Geom &, bool relu, bool accumulate, unsigned mode, cudaStream_t);
+// FP32 kernel for few pixels (conv_split_fp32.cu): the same for the layers that the other FP32 kernels would take
+bool conv_split_fp32_preferred(const Geom &, int sms);
+int launch_conv_split_fp32(small_ctx *, const float *in, const float *w, const float *bias, float *out, const Geom &,
+                           bool relu, bool accumulate, cudaStream_t);
 // a run of layers up to the end of the list as one kernel (net_resident.cu): the first layer of the run at or behind `from`
 // (-1: none), and its launch, which reads and writes whole tensors through rd / wr (slot -> address)
 int resident_from(small_ctx *, const small_layer *layers, int n, int from, int N);

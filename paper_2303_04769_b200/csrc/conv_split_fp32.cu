@@ -1,0 +1,211 @@
+// Full channel reduction in FP32 over few output pixels (paper Algorithms 1 and 2), any window and stride: the reduction of an output
+// tile is split over the warps of a thread block.
+//
+// Why a third FP32 kernel.  conv_direct.cu and conv_fp32.cu give a tile of 64 and more pixels x 32 filters its whole reduction in one
+// block, channel block after channel block with barriers between: at a batch of a few images that chain is the layer's time (64 -> 64
+// 3x3 on 8x8: 27 us whether 1 or 37 images) while most of the chip idles.  Here a tile is 8 pixels x 32 filters and its (channel
+// block, window position) pairs are dealt to up to 16 warps; one pass through shared memory adds up the warps' partial sums in a fixed
+// order.
+//
+// Within a warp a lane computes 4 filters x all pixels of the tile over a quarter of the channels.  What a lane is handed from cache
+// and shared memory is the limit - 32 lanes x 4 bytes a clock for an SM, broadcast or not, against 128 FMAs - so a value has to serve
+// several FMAs: with a filter per lane, every pixel handed to all of them, the kernel took three times as long.  The pixels go through
+// the warp's own piece of shared memory, channel by channel, so that 16 bytes are two packed pairs of pixels: an FMA instruction does
+// two (fma.rn.f32x2, rounded as two FMAs).  The next step's pixels and filters are on their way while a step is computed, filters into
+// the registers of those just used.
+//
+// us, whole-tile kernels and now, one image: 16 -> 16 3x3 on 32x32 10.3 / 2.5, 64 -> 64 on 8x8 27.1 / 3.7, 256 -> 256 on 7x7 104 / 9.1,
+// 64 -> 128 1x1 stride 2 on 56x56 18.6 / 2.8, 512 -> 512 1x1 on 7x7 41 / 3.6.  Small partial sums also round less: relative error of the
+// 256-channel 3x3 layer 8.2e-7 before, 1.4e-7 now.
+#include "common.cuh"
+
+namespace small {
+
+namespace {
+
+struct SplitFp32Args {
+    const float *in, *w, *bias;
+    float *out;
+    int K, KB, CB, H, W, OH, OW, FH, FW, S, pt, pl;
+    int pixels, chunks;          // output pixels of all images; (channel block, window position) pairs
+    int relu, accumulate, late;
+};
+
+__device__ __forceinline__ void fma2(uint64_t &c, uint64_t a, uint64_t b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b)); }
+__device__ __forceinline__ float2 plus(uint64_t a, uint64_t b) {
+    float2 x, y;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x.x), "=f"(x.y) : "l"(a));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(y.x), "=f"(y.y) : "l"(b));
+    return make_float2(x.x + y.x, x.y + y.y);
+}
+
+constexpr int P = 8;             // pixels of a tile: 16 take twice as long per step and leave room for fewer warps
+constexpr int kMaxWarps = 16;
+
+// CI: channels of a block that are computed (16: layers of at most 16 channels)
+template <int CI>
+struct Room { static constexpr int kFloats = CI * (P + 4) > P * 32 ? CI * (P + 4) : P * 32; };     // of a warp
+
+template <int CI>
+__global__ void __launch_bounds__(32 * kMaxWarps) conv_split_fp32_kernel(const SplitFp32Args a) {
+    constexpr int PITCH = P + 4, NX = P * CI / 128, NC = CI / 4;    // floats from channel to channel; 16-byte pixel loads of a lane; its channels
+    extern __shared__ __align__(16) float smem[];                   // a warp's pixels [channel][pixel], then its sums [pixel][filter]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5, taps = a.FH * a.FW;
+    const int p0 = blockIdx.x * P, kb = blockIdx.y, quarter = lane >> 3;
+    float *mine = smem + warp * Room<CI>::kFloats;
+    const size_t plane = (size_t)a.H * a.W * 32;
+    const float *w_lane = a.w + (size_t)kb * a.chunks * 1024 + quarter * NC * 32 + (lane & 7) * 4;
+
+    // the pixel this lane brings, 16 bytes of four channels at a time
+    const int p = p0 + lane % P, q = p < a.pixels ? p : 0;
+    const int n = q / (a.OH * a.OW), r = q - n * a.OH * a.OW, oy = r / a.OW;
+    const int iy = p < a.pixels ? oy * a.S - a.pt : -0x10000000;       // rows of pixels that do not exist are outside the plane
+    const int ix = (r - oy * a.OW) * a.S - a.pl;
+    const float *img = a.in + (size_t)n * a.CB * plane;
+
+    float4 px[NX], w[NC];
+    auto load_w = [&](const int c, const int i) { w[i] = *reinterpret_cast<const float4 *>(w_lane + (size_t)c * 1024 + i * 32); };
+    auto load_px = [&](const int c) {
+        const int cb = c / taps, tap = c - cb * taps, dy = tap / a.FW, y = iy + dy, x = ix + tap - dy * a.FW;
+        const bool in = (unsigned)y < (unsigned)a.H && (unsigned)x < (unsigned)a.W;
+        const float *s = img + (size_t)cb * plane + (size_t)(in ? y * a.W + x : 0) * 32 + lane / P * 4;
+#pragma unroll
+        for (int j = 0; j < NX; ++j) px[j] = in ? *reinterpret_cast<const float4 *>(s + j * (32 / P) * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+
+    if (a.late) grid_dep_sync();
+    if (warp < a.chunks)                          // the filters are the layer's own constants
+#pragma unroll
+        for (int i = 0; i < NC; ++i) load_w(warp, i);
+    grid_dep_sync();
+    grid_dep_trigger();
+    if (warp < a.chunks) load_px(warp);
+
+    uint64_t acc[P / 2][4];                       // pairs of pixels x filters
+#pragma unroll
+    for (int j = 0; j < P / 2; ++j)
+#pragma unroll
+        for (int f = 0; f < 4; ++f) acc[j][f] = 0;
+    for (int c = warp; c < a.chunks; c += warps) {
+        const int next = c + warps;
+        float *x_store = mine + lane / P * 4 * PITCH + lane % P;
+#pragma unroll
+        for (int j = 0; j < NX; ++j) {
+            float *d = x_store + j * (32 / P) * 4 * PITCH;
+            d[0] = px[j].x; d[PITCH] = px[j].y; d[2 * PITCH] = px[j].z; d[3 * PITCH] = px[j].w;
+        }
+        __syncwarp();
+        if (next < a.chunks) load_px(next);
+        const float *x_lane = mine + quarter * NC * PITCH;
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+            uint64_t ww[4];
+            asm("mov.b64 %0, {%1, %1};" : "=l"(ww[0]) : "f"(w[i].x));
+            asm("mov.b64 %0, {%1, %1};" : "=l"(ww[1]) : "f"(w[i].y));
+            asm("mov.b64 %0, {%1, %1};" : "=l"(ww[2]) : "f"(w[i].z));
+            asm("mov.b64 %0, {%1, %1};" : "=l"(ww[3]) : "f"(w[i].w));
+#pragma unroll
+            for (int j = 0; j < P / 4; ++j) {
+                const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(x_lane + i * PITCH + 4 * j);
+#pragma unroll
+                for (int f = 0; f < 4; ++f) { fma2(acc[2 * j][f], x.x, ww[f]); fma2(acc[2 * j + 1][f], x.y, ww[f]); }
+            }
+            if (next < a.chunks) load_w(next, i);
+        }
+        __syncwarp();
+    }
+    // the quarters' sums: each hands three quarters of its pixels over and keeps the totals of one
+    float2 half[P / 4][4], sum[P / 8][4];
+#pragma unroll
+    for (int j = 0; j < P / 4; ++j)
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            const bool up = lane & 16;
+            half[j][f] = plus(up ? acc[j + P / 4][f] : acc[j][f], __shfl_xor_sync(0xffffffffu, up ? acc[j][f] : acc[j + P / 4][f], 16));
+        }
+#pragma unroll
+    for (int j = 0; j < P / 8; ++j)
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            const bool up = lane & 8;
+            const float2 give = up ? half[j][f] : half[j + P / 8][f], keep = up ? half[j + P / 8][f] : half[j][f];
+            sum[j][f].x = keep.x + __shfl_xor_sync(0xffffffffu, give.x, 8);
+            sum[j][f].y = keep.y + __shfl_xor_sync(0xffffffffu, give.y, 8);
+        }
+    const int from = ((lane & 16) ? P / 2 : 0) + ((lane & 8) ? P / 4 : 0);
+#pragma unroll
+    for (int j = 0; j < P / 8; ++j) {
+        float *d = mine + (from + 2 * j) * 32 + (lane & 7) * 4;
+        *reinterpret_cast<float4 *>(d) = make_float4(sum[j][0].x, sum[j][1].x, sum[j][2].x, sum[j][3].x);
+        *reinterpret_cast<float4 *>(d + 32) = make_float4(sum[j][0].y, sum[j][1].y, sum[j][2].y, sum[j][3].y);
+    }
+    __syncthreads();
+
+    const int k = kb * 32 + lane;
+    const float bv = a.bias && k < a.K ? a.bias[k] : 0.0f;
+    for (int i = warp; i < P && p0 + i < a.pixels; i += warps) {
+        const int m = (p0 + i) / (a.OH * a.OW);
+        float *dst = a.out + (((size_t)m * a.KB + kb) * a.OH * a.OW + (p0 + i - m * a.OH * a.OW)) * 32 + lane;
+        float s = smem[i * 32 + lane];
+#pragma unroll 4
+        for (int u = 1; u < warps; ++u) s += smem[u * Room<CI>::kFloats + i * 32 + lane];
+        s += bv;
+        if (a.accumulate) s += *dst;
+        if (a.relu) s = s > 0.f ? s : 0.f;
+        *dst = k < a.K ? s : 0.0f;                // pad lanes stay +0
+    }
+}
+
+template <int CI>
+void launch_form(small_ctx *ctx, const SplitFp32Args &a, dim3 grid, int warps, cudaStream_t st) {
+    launch_kernel(ctx, conv_split_fp32_kernel<CI>, grid, dim3(32 * warps), (size_t)warps * Room<CI>::kFloats * sizeof(float), st, a);
+}
+
+// How a layer is cut: warps that share a tile's reduction, and the time expected of it in us (of 88 measured layers, most within a fifth).
+struct SplitFp32Plan { int warps; unsigned px_tiles; double us; };
+
+SplitFp32Plan plan_split_fp32(const Geom &g, int sms) {
+    SplitFp32Plan best{};
+    const int chunks = g.CB * g.FH * g.FW, resident = g.C <= 16 ? 20 : 16;     // warps an SM's registers hold
+    const long long px = ((long long)g.N * g.OH * g.OW + P - 1) / P, tiles = px * g.KB, on_sm = (tiles + sms - 1) / sms;
+    int last = 0;
+    for (int rounds = 1; rounds <= chunks; ++rounds) {
+        const int warps = (chunks + rounds - 1) / rounds;
+        if (warps > kMaxWarps || warps == last) continue;
+        last = warps;
+        const int per_sm = resident / warps;       // blocks
+        const long long waves = (tiles + (long long)sms * per_sm - 1) / ((long long)sms * per_sm);
+        const int busy = (int)(on_sm < per_sm ? on_sm : per_sm) * warps;
+        // a round: its latency, and what the resident warps are handed from cache and shared memory
+        const double us = 0.6 + (double)waves * (1.2 + rounds * (g.C <= 16 ? 0.42 + 0.04 * busy : 0.46 + 0.062 * busy));
+        if (!best.warps || us < best.us) best = SplitFp32Plan{warps, (unsigned)px, us};
+    }
+    return best;
+}
+
+}  // namespace
+
+// Few pixels: where the split cut beats the whole-tile kernels clearly.  Those take a tile's whole reduction one channel after the
+// other, 4.5 + 0.043 us per channel and window position for windows of several positions and some 5 + 0.07 for 1 x 1, at any number of
+// pixels that fits the chip at once.  us, whole-tile against split, 1 / 4 / 16 / 37 images: 64 -> 64 3x3 on 16x16 30.8 / 30.9 / 31.1 / 31.3
+// against 3.8 / 5.6 / 16.0 / 30.2; 16 -> 16 on 32x32 10.3 / 10.5 / 10.6 against 2.5 / 5.6 / 17.8; 256 -> 256 1x1 on 14x14 32.8 / 32.9 / 30.8 /
+// 39.2 against 3.5 / 9.0 / 29.3 / 64.2; 64 -> 64 1x1 on 28x28 9.8 / 10.0 / 11.1 / 15.1 against 2.4 / 4.0 / 10.1 / 20.5.
+bool conv_split_fp32_preferred(const Geom &g, int sms) {
+    if ((long long)g.N * g.OH * g.OW > 1 << 20 || (long long)g.H * g.W > 1 << 24 || g.K > 1 << 16) return false;
+    const int taps = g.FH * g.FW;
+    const double whole = taps > 1 ? 4.5 + 0.043 * g.C * taps : 5.0 + 0.07 * g.C < 40.0 ? 5.0 + 0.07 * g.C : 40.0;
+    return plan_split_fp32(g, sms).us < 0.75 * whole;
+}
+
+int launch_conv_split_fp32(small_ctx *ctx, const float *in, const float *w, const float *bias, float *out, const Geom &g,
+                           bool relu, bool accumulate, cudaStream_t st) {
+    const SplitFp32Args a{in, w, bias, out, g.K, g.KB, g.CB, g.H, g.W, g.OH, g.OW, g.FH, g.FW, g.S, g.pt, g.pl,
+                          g.N * g.OH * g.OW, g.CB * g.FH * g.FW, relu, accumulate, ctx->dependent == 2};
+    const SplitFp32Plan p = plan_split_fp32(g, ctx->sm_count);
+    const dim3 grid(p.px_tiles, (unsigned)g.KB);
+    if (g.C <= 16) launch_form<16>(ctx, a, grid, p.warps, st);
+    else launch_form<32>(ctx, a, grid, p.warps, st);
+    return check_launch(ctx);
+}
+
+}  // namespace small

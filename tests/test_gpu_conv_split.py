@@ -1,4 +1,4 @@
-"""Layers of few output pixels in the tensor-core modes: the reduction of a tile split over warps, at the edges of tiles, filter
+"""Layers of few output pixels: the reduction of a tile split over warps, on the tensor cores and in FP32, at the edges of tiles, filter
 blocks and splits, against the oracle; with the pad lanes, the join and an output that is only 16-byte aligned."""
 import pytest
 import torch
@@ -9,7 +9,7 @@ from paper_2303_04769_b200 import binding as B
 from gpu_util import ctx, dev, to_blk, from_blk, rel_err, pad_lanes_are_zero, conv_path
 
 pytestmark = pytest.mark.gpu
-TOL = {"tf32": 2e-3, "3xtf32": 1e-5}
+TOL = {"fp32": 1e-5, "tf32": 2e-3, "3xtf32": 1e-5}
 
 CASES = [  # N, C, K, H, W, FH, FW, stride, pad (t, b, l, r)
     (1, 16, 16, 32, 32, 3, 3, 1, (1, 1, 1, 1)),
@@ -24,7 +24,7 @@ CASES = [  # N, C, K, H, W, FH, FW, stride, pad (t, b, l, r)
 ]
 
 
-@pytest.mark.parametrize("math", ["tf32", "3xtf32"])
+@pytest.mark.parametrize("math", ["fp32", "tf32", "3xtf32"])
 @pytest.mark.parametrize("case", CASES)
 def test_few_pixels(case, math):
     N, C, K, H, W, FH, FW, S, pad = case
@@ -50,18 +50,33 @@ def test_few_pixels(case, math):
     assert pad_lanes_are_zero(acc, N, K, OH, OW)
 
 
-def test_split_sums_are_closer_than_one_chain():
-    N, C, K, H = 1, 256, 64, 7
+def test_values_without_a_number_stay_where_they_are():
+    """FP32: an infinite or missing input reaches the pixels whose window holds it and no other."""
+    x, w = synth.uniform((1, 40, 9, 9), -1, 1, 1, seed=4), abs(synth.uniform((33, 40, 3, 3), -1, 1, 2, seed=4)) + 0.1
+    x[0, 3, 0, 0], x[0, 39, 8, 4] = float("inf"), float("nan")
+    wb = torch.empty(B.small_conv_weight_elems(40, 33, 3, 3, B.MATH_FP32), device="cuda")
+    B.small_pack_conv_weights(ctx(), dev(w), wb, 40, 33, 3, 3, B.MATH_FP32)
+    out = torch.empty(B.small_packed_elems(1, 33, 9, 9), device="cuda")
+    B.small_conv2d(ctx(), to_blk(x), wb, None, out, 1, 40, 33, 9, 9, 3, 3, 1, (1, 1, 1, 1), B.MATH_FP32)
+    got = torch.from_numpy(from_blk(out, 1, 33, 9, 9))
+    want = torch.nn.functional.conv2d(torch.from_numpy(x).double(), torch.from_numpy(w).double(), padding=1)
+    assert torch.equal(got.isinf(), want.isinf()) and torch.equal(got.isnan(), want.isnan())
+    assert got.isinf().sum() == 33 * 4 and got.isnan().sum() == 33 * 6
+
+
+@pytest.mark.parametrize("math,path", [("3xtf32", "tensor"), ("fp32", "cuda_cores")])
+def test_split_sums_are_closer_than_one_chain(math, path):
+    N, C, K, H, m = 1, 256, 64, 7, B.MATH[math]
     x, w = synth.uniform((N, C, H, H), -1, 1, 1, seed=3), synth.uniform((K, C, 3, 3), -1, 1, 2, seed=3)
     ref = oracle.conv2d(x, w, None, 1, (1, 1, 1, 1))
-    wb = torch.empty(B.small_conv_weight_elems(C, K, 3, 3, B.MATH_3XTF32), device="cuda")
-    B.small_pack_conv_weights(ctx(), dev(w), wb, C, K, 3, 3, B.MATH_3XTF32)
+    wb = torch.empty(B.small_conv_weight_elems(C, K, 3, 3, m), device="cuda")
+    B.small_pack_conv_weights(ctx(), dev(w), wb, C, K, 3, 3, m)
 
     def err():
         out = torch.empty(B.small_packed_elems(N, K, H, H), device="cuda")
-        B.small_conv2d(ctx(), to_blk(x), wb, None, out, N, C, K, H, H, 3, 3, 1, (1, 1, 1, 1), B.MATH_3XTF32)
+        B.small_conv2d(ctx(), to_blk(x), wb, None, out, N, C, K, H, H, 3, 3, 1, (1, 1, 1, 1), m)
         return rel_err(from_blk(out, N, K, H, H), ref)
 
     split = err()
-    with conv_path("tensor"):
-        assert split < err()        # 144 steps of one accumulator against 9 of 16
+    with conv_path(path):
+        assert split < err()        # a chain of 2304 products (288 steps of 8) against 16 of a sixteenth
