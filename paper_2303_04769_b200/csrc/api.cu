@@ -424,7 +424,7 @@ constexpr int kSplit = 8;
 static int choose_path(const small_ctx *ctx, const Geom &g, unsigned math, bool out_aligned32) {
     const int path = choose_whole(ctx, g, math, out_aligned32), sms = ctx ? ctx->sm_count : kSmCount;
     if (path == 0 || (ctx && ctx->conv_path != SMALL_CONV_PATH_AUTO)) return path;
-    const bool split = path >= 3 ? conv_split_preferred(g, math == SMALL_MATH_3XTF32, path == 4, sms) : conv_split_fp32_preferred(g, sms);
+    const bool split = path >= 3 ? conv_split_preferred(g, math == SMALL_MATH_3XTF32, path == 4, sms) : conv_split_fp32_us(g, sms) > 0.0;
     return split ? path + kSplit : path;
 }
 

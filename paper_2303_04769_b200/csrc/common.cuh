@@ -200,9 +200,13 @@ bool conv_split_preferred(const Geom &, bool x3, bool warp_level, int sms);     
 int launch_conv_split(small_ctx *, const float *in, const float *w_hi, const float *w_lo, const float *bias, float *out,
                       const Geom &, bool relu, bool accumulate, unsigned mode, cudaStream_t);
 // FP32 kernel for few pixels (conv_split_fp32.cu): the same for the layers that the other FP32 kernels would take
-bool conv_split_fp32_preferred(const Geom &, int sms);
+double conv_split_fp32_us(const Geom &, int sms);          // the time expected, 0 where another kernel is preferred
 int launch_conv_split_fp32(small_ctx *, const float *in, const float *w, const float *bias, float *out, const Geom &,
                            bool relu, bool accumulate, cudaStream_t);
+// a depthwise 3x3 and the 1x1 layer behind it as that kernel: the time expected (0: not taken), and the launch; gd / gp: the two layers
+double split_pair_us(const Geom &gp, int sms);
+int launch_split_pair(small_ctx *, const float *in, const float *dw, const float *dw_bias, bool dw_relu, const float *w, const float *bias,
+                      float *out, const Geom &gd, const Geom &gp, bool relu, cudaStream_t);
 // a run of layers up to the end of the list as one kernel (net_resident.cu): the first layer of the run at or behind `from`
 // (-1: none), and its launch, which reads and writes whole tensors through rd / wr (slot -> address)
 int resident_from(small_ctx *, const small_layer *layers, int n, int from, int N);

@@ -29,6 +29,9 @@ struct SplitFp32Args {
     int K, KB, CB, H, W, OH, OW, FH, FW, S, pt, pl;
     int pixels, chunks;          // output pixels of all images; (channel block, window position) pairs
     int relu, accumulate, late;
+    // DW: a depthwise 3x3 in front of a 1x1 layer; H, W, S, pt, pl above are its input's and its own, FH = FW = 1
+    const float *dw, *dw_bias;
+    int C, dw_relu;
 };
 
 __device__ __forceinline__ void fma2(uint64_t &c, uint64_t a, uint64_t b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b)); }
@@ -42,11 +45,12 @@ __device__ __forceinline__ float2 plus(uint64_t a, uint64_t b) {
 constexpr int P = 8;             // pixels of a tile: 16 take twice as long per step and leave room for fewer warps
 constexpr int kMaxWarps = 16;
 
-// CI: channels of a block that are computed (16: layers of at most 16 channels)
+// CI: channels of a block that are computed (16: layers of at most 16 channels).  DW: the pixels are a depthwise 3x3's results, which a
+// lane computes where it would load them - once more for every block of 32 filters, in place of a launch and a tensor.
 template <int CI>
 struct Room { static constexpr int kFloats = CI * (P + 4) > P * 32 ? CI * (P + 4) : P * 32; };     // of a warp
 
-template <int CI>
+template <int CI, bool DW>
 __global__ void __launch_bounds__(32 * kMaxWarps) conv_split_fp32_kernel(const SplitFp32Args a) {
     constexpr int PITCH = P + 4, NX = P * CI / 128, NC = CI / 4;    // floats from channel to channel; 16-byte pixel loads of a lane; its channels
     extern __shared__ __align__(16) float smem[];                   // a warp's pixels [channel][pixel], then its sums [pixel][filter]
@@ -66,6 +70,31 @@ __global__ void __launch_bounds__(32 * kMaxWarps) conv_split_fp32_kernel(const S
     float4 px[NX], w[NC];
     auto load_w = [&](const int c, const int i) { w[i] = *reinterpret_cast<const float4 *>(w_lane + (size_t)c * 1024 + i * 32); };
     auto load_px = [&](const int c) {
+        if constexpr (DW) {
+            const float *s = img + (size_t)c * plane + lane / P * 4, *f = a.dw + (size_t)c * 288 + lane / P * 4;
+#pragma unroll
+            for (int j = 0; j < NX; ++j) {
+                const int ch = c * 32 + (lane / P + j * (32 / P)) * 4;
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int tap = 0; tap < 9; ++tap) {
+                    const int y = iy + tap / 3, x = ix + tap % 3;
+                    const bool in = (unsigned)y < (unsigned)a.H && (unsigned)x < (unsigned)a.W;
+                    const float4 d = in ? *reinterpret_cast<const float4 *>(s + (size_t)(y * a.W + x) * 32 + j * (32 / P) * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    const float4 g = *reinterpret_cast<const float4 *>(f + tap * 32 + j * (32 / P) * 4);
+                    v.x = fmaf(d.x, g.x, v.x); v.y = fmaf(d.y, g.y, v.y); v.z = fmaf(d.z, g.z, v.z); v.w = fmaf(d.w, g.w, v.w);
+                }
+                if (a.dw_bias) {                  // C entries
+                    if (ch < a.C) v.x += a.dw_bias[ch];
+                    if (ch + 1 < a.C) v.y += a.dw_bias[ch + 1];
+                    if (ch + 2 < a.C) v.z += a.dw_bias[ch + 2];
+                    if (ch + 3 < a.C) v.w += a.dw_bias[ch + 3];
+                }
+                if (a.dw_relu) { v.x = v.x > 0.f ? v.x : 0.f; v.y = v.y > 0.f ? v.y : 0.f; v.z = v.z > 0.f ? v.z : 0.f; v.w = v.w > 0.f ? v.w : 0.f; }
+                px[j] = v;
+            }
+            return;
+        }
         const int cb = c / taps, tap = c - cb * taps, dy = tap / a.FW, y = iy + dy, x = ix + tap - dy * a.FW;
         const bool in = (unsigned)y < (unsigned)a.H && (unsigned)x < (unsigned)a.W;
         const float *s = img + (size_t)cb * plane + (size_t)(in ? y * a.W + x : 0) * 32 + lane / P * 4;
@@ -156,18 +185,22 @@ __global__ void __launch_bounds__(32 * kMaxWarps) conv_split_fp32_kernel(const S
     }
 }
 
-template <int CI>
+template <bool DW>
 void launch_form(small_ctx *ctx, const SplitFp32Args &a, dim3 grid, int warps, cudaStream_t st) {
-    launch_kernel(ctx, conv_split_fp32_kernel<CI>, grid, dim3(32 * warps), (size_t)warps * Room<CI>::kFloats * sizeof(float), st, a);
+    if (a.C <= 16) launch_kernel(ctx, conv_split_fp32_kernel<16, DW>, grid, dim3(32 * warps), (size_t)warps * Room<16>::kFloats * sizeof(float), st, a);
+    else launch_kernel(ctx, conv_split_fp32_kernel<32, DW>, grid, dim3(32 * warps), (size_t)warps * Room<32>::kFloats * sizeof(float), st, a);
 }
 
 // How a layer is cut: warps that share a tile's reduction, and the time expected of it in us (of 88 measured layers, most within a fifth).
-struct SplitFp32Plan { int warps; unsigned px_tiles; double us; };
+struct SplitFp32Plan { int warps; long long waves; unsigned px_tiles; double us; };
 
-SplitFp32Plan plan_split_fp32(const Geom &g, int sms) {
+SplitFp32Plan plan_split_fp32(const Geom &g, int sms, bool dw) {
     SplitFp32Plan best{};
     const int chunks = g.CB * g.FH * g.FW, resident = g.C <= 16 ? 20 : 16;     // warps an SM's registers hold
     const long long px = ((long long)g.N * g.OH * g.OW + P - 1) / P, tiles = px * g.KB, on_sm = (tiles + sms - 1) / sms;
+    // a round: its latency, and what a resident warp is handed from cache and shared memory (a depthwise layer's pixels and filters
+    // are another 36 loads of 16 bytes per lane)
+    const double latency = dw ? 1.2 : g.C <= 16 ? 0.42 : 0.46, warp = (g.C <= 16 ? 0.04 : 0.062) * (dw ? 6.0 : 1.0);
     int last = 0;
     for (int rounds = 1; rounds <= chunks; ++rounds) {
         const int warps = (chunks + rounds - 1) / rounds;
@@ -176,12 +209,13 @@ SplitFp32Plan plan_split_fp32(const Geom &g, int sms) {
         const int per_sm = resident / warps;       // blocks
         const long long waves = (tiles + (long long)sms * per_sm - 1) / ((long long)sms * per_sm);
         const int busy = (int)(on_sm < per_sm ? on_sm : per_sm) * warps;
-        // a round: its latency, and what the resident warps are handed from cache and shared memory
-        const double us = 0.6 + (double)waves * (1.2 + rounds * (g.C <= 16 ? 0.42 + 0.04 * busy : 0.46 + 0.062 * busy));
-        if (!best.warps || us < best.us) best = SplitFp32Plan{warps, (unsigned)px, us};
+        const double us = 0.6 + (double)waves * (1.2 + rounds * (latency + warp * busy));
+        if (!best.warps || us < best.us) best = SplitFp32Plan{warps, waves, (unsigned)px, us};
     }
     return best;
 }
+
+bool fits(const Geom &g) { return (long long)g.N * g.OH * g.OW <= 1 << 20 && (long long)g.H * g.W <= 1 << 24 && g.K <= 1 << 16; }
 
 }  // namespace
 
@@ -190,21 +224,38 @@ SplitFp32Plan plan_split_fp32(const Geom &g, int sms) {
 // pixels that fits the chip at once.  us, whole-tile against split, 1 / 4 / 16 / 37 images: 64 -> 64 3x3 on 16x16 30.8 / 30.9 / 31.1 / 31.3
 // against 3.8 / 5.6 / 16.0 / 30.2; 16 -> 16 on 32x32 10.3 / 10.5 / 10.6 against 2.5 / 5.6 / 17.8; 256 -> 256 1x1 on 14x14 32.8 / 32.9 / 30.8 /
 // 39.2 against 3.5 / 9.0 / 29.3 / 64.2; 64 -> 64 1x1 on 28x28 9.8 / 10.0 / 11.1 / 15.1 against 2.4 / 4.0 / 10.1 / 20.5.
-bool conv_split_fp32_preferred(const Geom &g, int sms) {
-    if ((long long)g.N * g.OH * g.OW > 1 << 20 || (long long)g.H * g.W > 1 << 24 || g.K > 1 << 16) return false;
+double conv_split_fp32_us(const Geom &g, int sms) {
+    if (!fits(g)) return 0.0;
     const int taps = g.FH * g.FW;
     const double whole = taps > 1 ? 4.5 + 0.043 * g.C * taps : 5.0 + 0.07 * g.C < 40.0 ? 5.0 + 0.07 * g.C : 40.0;
-    return plan_split_fp32(g, sms).us < 0.75 * whole;
+    const double us = plan_split_fp32(g, sms, false).us;
+    return us < 0.75 * whole ? us : 0.0;
 }
 
 int launch_conv_split_fp32(small_ctx *ctx, const float *in, const float *w, const float *bias, float *out, const Geom &g,
                            bool relu, bool accumulate, cudaStream_t st) {
     const SplitFp32Args a{in, w, bias, out, g.K, g.KB, g.CB, g.H, g.W, g.OH, g.OW, g.FH, g.FW, g.S, g.pt, g.pl,
-                          g.N * g.OH * g.OW, g.CB * g.FH * g.FW, relu, accumulate, ctx->dependent == 2};
-    const SplitFp32Plan p = plan_split_fp32(g, ctx->sm_count);
-    const dim3 grid(p.px_tiles, (unsigned)g.KB);
-    if (g.C <= 16) launch_form<16>(ctx, a, grid, p.warps, st);
-    else launch_form<32>(ctx, a, grid, p.warps, st);
+                          g.N * g.OH * g.OW, g.CB * g.FH * g.FW, relu, accumulate, ctx->dependent == 2, nullptr, nullptr, g.C, 0};
+    const SplitFp32Plan p = plan_split_fp32(g, ctx->sm_count, false);
+    launch_form<false>(ctx, a, dim3(p.px_tiles, (unsigned)g.KB), p.warps, st);
+    return check_launch(ctx);
+}
+
+// One launch instead of two costs the host half, and the device a depthwise layer per 32 filters.  us per pair of the keyword-spotting
+// network (64 channels on 25x5), two launches against one, 1 / 8 / 16 / 37 images: 4.2 / 4.8 / 5.8 / 6.9 against 3.5 / 4.4 / 6.1 / 8.4; a
+// depthwise layer on its own takes some 2.8, and 0.8 more are given for the host's time.
+double split_pair_us(const Geom &gp, int sms) {
+    if (!fits(gp)) return 0.0;
+    const double us = plan_split_fp32(gp, sms, true).us;
+    return us < 3.6 + plan_split_fp32(gp, sms, false).us ? us : 0.0;
+}
+
+int launch_split_pair(small_ctx *ctx, const float *in, const float *dw, const float *dw_bias, bool dw_relu, const float *w, const float *bias,
+                      float *out, const Geom &gd, const Geom &gp, bool relu, cudaStream_t st) {
+    const SplitFp32Args a{in, w, bias, out, gp.K, gp.KB, gp.CB, gd.H, gd.W, gp.OH, gp.OW, 1, 1, gd.S, gd.pt, gd.pl,
+                          gp.N * gp.OH * gp.OW, gp.CB, relu, 0, ctx->dependent == 2, dw, dw_bias, gp.C, dw_relu};
+    const SplitFp32Plan p = plan_split_fp32(gp, ctx->sm_count, true);
+    launch_form<true>(ctx, a, dim3(p.px_tiles, (unsigned)gp.KB), p.warps, st);
     return check_launch(ctx);
 }
 

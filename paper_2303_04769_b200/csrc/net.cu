@@ -163,6 +163,42 @@ static int fc_chain_len(const small_ctx *ctx, const small_layer *layers, int n_l
     return L >= 2 ? L : 0;
 }
 
+// Layers i and i + 1 as a depthwise 3x3 and a 1x1 layer in FP32 that run as one launch (conv_split_fp32.cu): the time expected, 0 where
+// they do not.
+static double split_pair(const small_ctx *ctx, const small_layer *layers, int n_layers, int i, int N, Geom &gd, Geom &gp) {
+    if (i + 1 >= n_layers) return 0.0;
+    const small_layer &A = layers[i], &Bn = layers[i + 1];
+    if (A.op != SMALL_OP_DWCONV || Bn.op != SMALL_OP_CONV || A.FH != 3 || A.FW != 3 || Bn.FH != 1 || Bn.FW != 1 || Bn.stride != 1 ||
+        (Bn.pad_t | Bn.pad_b | Bn.pad_l | Bn.pad_r) || (Bn.flags & (SMALL_ACCUMULATE | SMALL_MATH_MASK)) || Bn.C != A.C)
+        return 0.0;
+    if (A.dst < 0 || Bn.src != A.dst || Bn.dst == A.src || Bn.dst == A.dst || !slot_dead_after(layers, n_layers, i + 2, A.dst)) return 0.0;
+    if (make_geom(gd, N, A.C, A.C, A.H, A.W, 3, 3, A.stride, A.pad_t, A.pad_b, A.pad_l, A.pad_r)) return 0.0;
+    if (Bn.H != gd.OH || Bn.W != gd.OW || make_geom(gp, N, A.C, Bn.K, gd.OH, gd.OW, 1, 1, 1, 0, 0, 0, 0)) return 0.0;
+    return split_pair_us(gp, ctx->sm_count);
+}
+
+// A run with depthwise layers that could stay on chip in FP32 (net_resident.cu), launch by launch instead: whether that is the faster form
+// for its batch.  An operation costs the on-chip kernel 4.3 to 6.7 us whatever the batch - barriers, filters passing by - and the kernels
+// of few pixels 2 to 9, growing with it.  us, on chip against launches: stem and two pairs of 64 channels on 25 x 5, batch 1 / 18 / 74 31.5 /
+// 29.5 / 31.2 against 13.4 / 19.7 / 29.1; the keyword-spotting network (four pairs) 1 / 37 / 64 / 128 47.9 / 50.1 / 51.0 / 53.7 against 20.8 /
+// 35.6 / 48.3 / 82; depthwise-separable network 1 / 16 / 64 115.7 / 142 / 208 against 55.8 / 94 / 164.
+static bool launches_beat_on_chip(const small_ctx *ctx, const small_layer *layers, int n_layers, int from, int N) {
+    double us = 4.0;                              // the average pool and the classifier
+    bool depthwise = false;
+    for (int i = from; i + 2 < n_layers; ++i) {
+        Geom g, gp;
+        const small_layer &L = layers[i];
+        depthwise |= L.op == SMALL_OP_DWCONV;
+        if (const double t = split_pair(ctx, layers, n_layers, i, N, g, gp)) { us += t; ++i; continue; }
+        if ((L.op != SMALL_OP_CONV && L.op != SMALL_OP_DWCONV) || make_geom(g, N, L.C, L.K, L.H, L.W, L.FH, L.FW, L.stride, L.pad_t, L.pad_b, L.pad_l, L.pad_r)) return false;
+        const double out = (double)N * g.OH * g.OW * L.K;
+        if (L.op == SMALL_OP_DWCONV) us += 2.5 + (out + (double)N * L.C * L.H * L.W) / 1e6;
+        else if (const double t = conv_split_fp32_us(g, ctx->sm_count)) us += t;
+        else us += 5.0 + (0.07 + out / 15e6) * L.C * L.FH * L.FW;
+    }
+    return depthwise && us < 4.5 * (n_layers - from);
+}
+
 // Runs of layers are kept on chip as one kernel where every kind of fusion is on.
 static bool runs_allowed(const small_ctx *ctx) {
     const unsigned rest = SMALL_FUSE_CONVPOOL | SMALL_FUSE_FC_CHAIN | SMALL_FUSE_POOLFC;
@@ -282,10 +318,12 @@ static int run_layers(small_ctx *ctx, const small_layer *layers, int n_layers, i
     bool after_join = false;
     // a run of depthwise / 1x1 pairs (sep_chain.cu); without one, a run up to the end of the list (net_resident.cu)
     int chain = -1, chain_layers = 0, on_chip = -1;
-    if (runs_allowed(ctx)) {
+    const bool runs = runs_allowed(ctx);
+    if (runs) {
         for (int i = from; i < n_layers && !chain_layers; ++i)
             if ((chain_layers = sep_chain_layers(ctx, layers, n_layers, i, N)) > 0) chain = i;
         if (!chain_layers) on_chip = resident_from(ctx, layers, n_layers, from, N);
+        if (on_chip >= 0 && (layers[n_layers - 1].flags & SMALL_MATH_MASK) == SMALL_MATH_FP32 && launches_beat_on_chip(ctx, layers, n_layers, on_chip, N)) on_chip = -1;
     }
     for (int i = from; i < n_layers; ++i) {
         const small_layer &L = layers[i];
@@ -304,6 +342,18 @@ static int run_layers(small_ctx *ctx, const small_layer *layers, int n_layers, i
             s = launch_resident(ctx, layers, n_layers, from, N, rd, wr, static_cast<cudaStream_t>(stream));
             ctx->dependent = 0;
             return s;
+        }
+        if (runs && chain < 0 && on_chip < 0) {
+            Geom gd, gp;
+            if (split_pair(ctx, layers, n_layers, i, N, gd, gp) > 0.0) {
+                const small_layer &Nx = layers[i + 1];
+                s = launch_split_pair(ctx, rd(L.src), L.w_blk, L.bias, L.flags & SMALL_RELU, Nx.w_blk, Nx.bias, wr(Nx.dst), gd, gp, Nx.flags & SMALL_RELU,
+                                      static_cast<cudaStream_t>(stream));
+                ctx->dependent = 0;
+                if (s != SMALL_OK) return s;
+                ++i;
+                continue;
+            }
         }
         {
             int widths[13];

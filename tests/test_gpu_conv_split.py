@@ -5,7 +5,10 @@ import torch
 
 import oracle
 import synth
+from oracle import nets
 from paper_2303_04769_b200 import binding as B
+from paper_2303_04769_b200.net import Net
+from synth import configs
 from gpu_util import ctx, dev, to_blk, from_blk, rel_err, pad_lanes_are_zero, conv_path
 
 pytestmark = pytest.mark.gpu
@@ -80,3 +83,19 @@ def test_split_sums_are_closer_than_one_chain(math, path):
     split = err()
     with conv_path(path):
         assert split < err()        # a chain of 2304 products (288 steps of 8) against 16 of a sixteenth
+
+
+@pytest.mark.parametrize("C,K,H,W,S,relu,batch", [(64, 64, 25, 5, 1, True, 2), (33, 70, 9, 7, 2, False, 3), (8, 24, 1, 1, 1, True, 1), (100, 9, 6, 5, 2, True, 4)])
+def test_fp32_pairs_as_one_launch(C, K, H, W, S, relu, batch):
+    """A depthwise 3x3 and a 1x1 layer of a small batch in FP32: ragged channels and planes, strides, one pixel."""
+    layers = [dict(op="dwconv", name="d", src="in", dst="m", C=C, K=C, FH=3, FW=3, stride=S, pad=(1, 1, 1, 1), relu=relu, accumulate=False),
+              configs._conv("c", "m", "out", C, K, 1, 1, configs.P0, True)]
+    net = dict(name="pair", batch=batch, input=(C, H, W), input_dist=("uniform", -1.0, 1.0), weight_dist="he_normal", layers=layers)
+    params, x = configs.make_params(net), configs.make_input(net, batch)
+    ref = nets.run_net(net, params, x)["out"]
+    gnet = Net(ctx(), net, params, batch=batch)
+    got = gnet.run(to_blk(x))
+    assert rel_err(from_blk(got, *ref.shape), ref) <= TOL["fp32"]
+    assert pad_lanes_are_zero(got, *ref.shape)
+    apart = Net(ctx(), net, params, batch=batch, fuse_dwpw=False).run(to_blk(x))
+    assert rel_err(from_blk(apart, *ref.shape), ref) <= TOL["fp32"]
