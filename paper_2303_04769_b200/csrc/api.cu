@@ -441,6 +441,25 @@ static int conv2d_path(small_ctx *ctx, const Geom &g, unsigned math, bool out_al
     return cache[key] = choose_path(ctx, g, math, out_aligned32);
 }
 
+namespace small {
+
+// Both layers on the same one of the two kernels.
+bool joined_split(small_ctx *ctx, const Geom &sc, const Geom &g, unsigned math, bool out_aligned32) {
+    const int a = conv2d_path(ctx, sc, math, out_aligned32), b = conv2d_path(ctx, g, math, out_aligned32);
+    return a > kSplit && b > kSplit && (a - kSplit >= 3) == (b - kSplit >= 3);
+}
+
+int launch_joined(small_ctx *ctx, Shortcut sc, const float *in, const float *w, const float *bias, float *out, const Geom &g, bool relu, unsigned math, cudaStream_t st) {
+    if (conv2d_path(ctx, g, math, (reinterpret_cast<uintptr_t>(out) & 31u) == 0) - kSplit < 3)
+        return launch_conv_split_fp32(ctx, in, w, bias, out, g, relu, false, st, &sc);
+    const float *w_hi = w + conv_w_fp32_elems(g.C, g.K, g.FH, g.FW), *w_lo = w_hi + conv_w_tc_elems(g.C, g.K, g.FH, g.FW);
+    sc.w_hi = sc.w + conv_w_fp32_elems(sc.g.C, sc.g.K, 1, 1);
+    sc.w_lo = sc.w_hi + conv_w_tc_elems(sc.g.C, sc.g.K, 1, 1);
+    return launch_conv_split(ctx, in, w_hi, w_lo, bias, out, g, relu, false, math, st, &sc);
+}
+
+}  // namespace small
+
 SMALL_API int small_conv2d_uses_tensor_cores(int N, int C, int K, int H, int W, int FH, int FW, int stride,
                                              int pt, int pb, int pl, int pr) {
     Geom g;

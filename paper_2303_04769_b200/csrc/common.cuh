@@ -194,15 +194,20 @@ int launch_conv_tc(small_ctx *, const float *in, const float *w_hi, const float 
 bool conv_mma_supported(const Geom &, bool x3);
 int launch_conv_mma(small_ctx *, const float *in, const float *w_hi, const float *w_lo, const float *bias, float *out,
                     const Geom &, bool relu, bool accumulate, unsigned mode, cudaStream_t);
+// A 1x1 layer without padding and activation whose result a layer of few pixels is added to (a residual stage's shortcut); g: that layer
+struct Shortcut { const float *in, *w, *w_hi, *w_lo, *bias; Geom g; };
 // warp-level tensor-core kernel for few pixels (conv_split.cu), whose rule says where it is the fastest of the tensor-core kernels;
 // any channels, filters, window and stride; reads the same filter sections
 bool conv_split_preferred(const Geom &, bool x3, bool warp_level, int sms);     // warp_level: instead of conv_mma.cu, else conv_tc.cu
 int launch_conv_split(small_ctx *, const float *in, const float *w_hi, const float *w_lo, const float *bias, float *out,
-                      const Geom &, bool relu, bool accumulate, unsigned mode, cudaStream_t);
+                      const Geom &, bool relu, bool accumulate, unsigned mode, cudaStream_t, const Shortcut * = nullptr);
 // FP32 kernel for few pixels (conv_split_fp32.cu): the same for the layers that the other FP32 kernels would take
 double conv_split_fp32_us(const Geom &, int sms);          // the time expected, 0 where another kernel is preferred
 int launch_conv_split_fp32(small_ctx *, const float *in, const float *w, const float *bias, float *out, const Geom &,
-                           bool relu, bool accumulate, cudaStream_t);
+                           bool relu, bool accumulate, cudaStream_t, const Shortcut * = nullptr);
+// a shortcut and the layer that is added to it as one launch of those kernels: whether both run there, and the launch (api.cu)
+bool joined_split(small_ctx *, const Geom &shortcut, const Geom &, unsigned math, bool out_aligned32);
+int launch_joined(small_ctx *, Shortcut, const float *in, const float *w, const float *bias, float *out, const Geom &, bool relu, unsigned math, cudaStream_t);
 // a depthwise 3x3 and the 1x1 layer behind it as that kernel: the time expected (0: not taken), and the launch; gd / gp: the two layers
 double split_pair_us(const Geom &gp, int sms);
 int launch_split_pair(small_ctx *, const float *in, const float *dw, const float *dw_bias, bool dw_relu, const float *w, const float *bias,

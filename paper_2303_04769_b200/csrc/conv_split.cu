@@ -28,6 +28,9 @@ struct SplitArgs {
     int K, KB, CB, H, W, OH, OW, FH, FW, S, pt, pl;
     int pixels, chunks;          // output pixels of all images; (channel block, window position) pairs
     int relu, accumulate, late;
+    // JOIN: a 1x1 layer of other pixels and filters whose result this one is added to
+    const float *in2, *w2_hi, *w2_lo, *bias2;
+    int CB2, H2, W2, S2;
 };
 
 __device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], const uint32_t b0, const uint32_t b1) {
@@ -35,8 +38,9 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], 
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// NF: fragments of 8 filters of a block's tile; CW: channels of a block that exist (16: layers of at most 16 channels)
-template <int NF, int CW, bool X3>
+// NF: fragments of 8 filters of a block's tile; CW: channels of a block that exist (16: layers of at most 16 channels); JOIN: a residual
+// stage's 1x1 shortcut as further steps of the reduction it is added to - no launch of its own, nothing written and read again
+template <int NF, int CW, bool X3, bool JOIN>
 __global__ void __launch_bounds__(512) conv_split_kernel(const SplitArgs a) {
     constexpr int V = CW / 16;                    // 16-byte loads of a lane per pixel and per filter
     extern __shared__ float2 part[];              // [warp][fragment][row half][lane]
@@ -47,8 +51,9 @@ __global__ void __launch_bounds__(512) conv_split_kernel(const SplitArgs a) {
     const size_t w_lane = (size_t)(k0 + g) * 32 + t * (CW / 4);
     const size_t plane = (size_t)a.H * a.W * 32;
 
+    const int chunks = a.chunks + (JOIN ? a.CB2 : 0);
     int iy[2], ix[2];
-    const float *img[2];
+    const float *img[2], *img2[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int p = p0 + g + 8 * h, q = p < a.pixels ? p : 0;
@@ -56,10 +61,15 @@ __global__ void __launch_bounds__(512) conv_split_kernel(const SplitArgs a) {
         iy[h] = p < a.pixels ? oy * a.S - a.pt : -0x10000000;      // rows of pixels that do not exist are outside the plane
         ix[h] = (r - oy * a.OW) * a.S - a.pl;
         img[h] = a.in + (size_t)n * a.CB * plane + t * (CW / 4);
+        img2[h] = JOIN ? a.in2 + ((size_t)n * a.CB2 * a.H2 * a.W2 + (oy * a.W2 + (r - oy * a.OW)) * a.S2) * 32 + t * (CW / 4) : nullptr;
     }
     uint4 wh[NF][V], wl[X3 ? NF : 1][V], px[2][V];
     auto load_w = [&](const int c) {
         const float *h = a.w_hi + (size_t)c * w_chunk + w_lane, *l = X3 ? a.w_lo + (size_t)c * w_chunk + w_lane : h;
+        if (JOIN && c >= a.chunks) {
+            h = a.w2_hi + (size_t)(c - a.chunks) * w_chunk + w_lane;
+            l = X3 ? a.w2_lo + (size_t)(c - a.chunks) * w_chunk + w_lane : h;
+        }
 #pragma unroll
         for (int n = 0; n < NF; ++n)
 #pragma unroll
@@ -69,6 +79,14 @@ __global__ void __launch_bounds__(512) conv_split_kernel(const SplitArgs a) {
             }
     };
     auto load_px = [&](const int c) {
+        if (JOIN && c >= a.chunks) {              // (pixels that do not exist read those of the first one)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int v = 0; v < V; ++v)
+                    px[h][v] = *reinterpret_cast<const uint4 *>(img2[h] + (size_t)(c - a.chunks) * a.H2 * a.W2 * 32 + v * 4);
+            return;
+        }
         const int cb = c / taps, tap = c - cb * taps, dy = tap / a.FW, dx = tap - dy * a.FW;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -81,17 +99,17 @@ __global__ void __launch_bounds__(512) conv_split_kernel(const SplitArgs a) {
     };
 
     if (a.late) grid_dep_sync();
-    if (warp < a.chunks) load_w(warp);            // the filters are the layer's own constants
+    if (warp < chunks) load_w(warp);            // the filters are the layer's own constants
     grid_dep_sync();
     grid_dep_trigger();
-    if (warp < a.chunks) load_px(warp);
+    if (warp < chunks) load_px(warp);
 
     float acc[NF][4], small[X3 ? NF : 1][4];
 #pragma unroll
     for (int n = 0; n < NF; ++n)
 #pragma unroll
         for (int e = 0; e < 4; ++e) { acc[n][e] = 0.0f; if (X3) small[X3 ? n : 0][e] = 0.0f; }
-    for (int c = warp; c < a.chunks; c += warps) {
+    for (int c = warp; c < chunks; c += warps) {
         uint32_t ah[2 * V][4], al[X3 ? 2 * V : 1][4], bh[2 * V][NF][2], bl[X3 ? 2 * V : 1][X3 ? NF : 1][2];
         // K step s: elements 2 s and 2 s + 1 of a lane's channels
 #pragma unroll
@@ -120,7 +138,7 @@ __global__ void __launch_bounds__(512) conv_split_kernel(const SplitArgs a) {
             }
         }
         const int next = c + warps;
-        if (next < a.chunks) { load_w(next); load_px(next); }
+        if (next < chunks) { load_w(next); load_px(next); }
 #pragma unroll
         for (int s = 0; s < 2 * V; ++s)
 #pragma unroll
@@ -150,6 +168,7 @@ __global__ void __launch_bounds__(512) conv_split_kernel(const SplitArgs a) {
         float *dst = a.out + (((size_t)n * a.KB + (k >> 5)) * a.OH * a.OW + r) * 32 + (k & 31);
         float2 v = a.accumulate ? *reinterpret_cast<const float2 *>(dst) : make_float2(0.0f, 0.0f);
         const float b0 = a.bias && k < a.K ? a.bias[k] : 0.0f, b1 = a.bias && k + 1 < a.K ? a.bias[k + 1] : 0.0f;
+        if (JOIN && a.bias2) { if (k < a.K) v.x += a.bias2[k]; if (k + 1 < a.K) v.y += a.bias2[k + 1]; }
         float2 s = part[i];
 #pragma unroll 4
         for (int w = 1; w < warps; ++w) { const float2 q = part[w * NF * 64 + i]; s.x += q.x; s.y += q.y; }
@@ -166,17 +185,18 @@ __global__ void __launch_bounds__(512) conv_split_kernel(const SplitArgs a) {
 template <int NF, int CW>
 void launch_form(small_ctx *ctx, const SplitArgs &a, bool x3, dim3 grid, int warps, cudaStream_t st) {
     const size_t smem = (size_t)warps * NF * 64 * sizeof(float2);
-    if (x3) launch_kernel(ctx, conv_split_kernel<NF, CW, true>, grid, dim3(32 * warps), smem, st, a);
-    else launch_kernel(ctx, conv_split_kernel<NF, CW, false>, grid, dim3(32 * warps), smem, st, a);
+    const auto k = a.in2 ? (x3 ? conv_split_kernel<NF, CW, true, true> : conv_split_kernel<NF, CW, false, true>)
+                         : (x3 ? conv_split_kernel<NF, CW, true, false> : conv_split_kernel<NF, CW, false, false>);
+    launch_kernel(ctx, k, grid, dim3(32 * warps), smem, st, a);
 }
 
 // How a layer is cut: filters of a tile, warps that share its reduction, and the time expected of it in us.
 struct SplitPlan { int nf, warps; unsigned px_tiles, k_tiles; double us; };
 
-SplitPlan plan_split(const Geom &g, bool x3, int sms) {
+SplitPlan plan_split(const Geom &g, bool x3, int sms, int more = 0) {      // more: steps besides the layer's own
     SplitPlan best{};
     const long long pixels = (long long)g.N * g.OH * g.OW;
-    const int chunks = g.CB * g.FH * g.FW;
+    const int chunks = g.CB * g.FH * g.FW + more;
     for (int nf = 1; nf <= 2; ++nf) {
         if (nf == 2 && g.K <= 8) break;
         const long long px = (pixels + 15) / 16, kt = (g.K + 8 * nf - 1) / (8 * nf);
@@ -219,13 +239,17 @@ bool conv_split_preferred(const Geom &g, bool x3, bool warp_level, int sms) {
 }
 
 int launch_conv_split(small_ctx *ctx, const float *in, const float *w_hi, const float *w_lo, const float *bias, float *out,
-                      const Geom &g, bool relu, bool accumulate, unsigned mode, cudaStream_t st) {
+                      const Geom &g, bool relu, bool accumulate, unsigned mode, cudaStream_t st, const Shortcut *sc) {
     const bool x3 = mode == SMALL_MATH_3XTF32;
     SplitArgs a{in, w_hi, w_lo, bias, out, g.K, g.KB, g.CB, g.H, g.W, g.OH, g.OW, g.FH, g.FW, g.S, g.pt, g.pl,
-                g.N * g.OH * g.OW, g.CB * g.FH * g.FW, relu, accumulate, ctx->dependent == 2};
-    const SplitPlan p = plan_split(g, x3, ctx->sm_count);
+                g.N * g.OH * g.OW, g.CB * g.FH * g.FW, relu, accumulate, ctx->dependent == 2, nullptr, nullptr, nullptr, nullptr, 0, 0, 0, 0};
+    if (sc) {
+        a.in2 = sc->in; a.w2_hi = sc->w_hi; a.w2_lo = sc->w_lo; a.bias2 = sc->bias;
+        a.CB2 = sc->g.CB; a.H2 = sc->g.H; a.W2 = sc->g.W; a.S2 = sc->g.S;
+    }
+    const SplitPlan p = plan_split(g, x3, ctx->sm_count, a.CB2);
     const dim3 grid(p.px_tiles, p.k_tiles);
-    if (g.C <= 16) { if (p.nf == 2) launch_form<2, 16>(ctx, a, x3, grid, p.warps, st); else launch_form<1, 16>(ctx, a, x3, grid, p.warps, st); }
+    if (g.C <= 16 && (!sc || sc->g.C <= 16)) { if (p.nf == 2) launch_form<2, 16>(ctx, a, x3, grid, p.warps, st); else launch_form<1, 16>(ctx, a, x3, grid, p.warps, st); }
     else if (p.nf == 2) launch_form<2, 32>(ctx, a, x3, grid, p.warps, st);
     else launch_form<1, 32>(ctx, a, x3, grid, p.warps, st);
     return check_launch(ctx);

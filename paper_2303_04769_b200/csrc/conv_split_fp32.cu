@@ -32,6 +32,9 @@ struct SplitFp32Args {
     // DW: a depthwise 3x3 in front of a 1x1 layer; H, W, S, pt, pl above are its input's and its own, FH = FW = 1
     const float *dw, *dw_bias;
     int C, dw_relu;
+    // JOIN: a 1x1 layer of other pixels and filters whose result this one is added to
+    const float *in2, *w2, *bias2;
+    int CB2, H2, W2, S2;
 };
 
 __device__ __forceinline__ void fma2(uint64_t &c, uint64_t a, uint64_t b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b)); }
@@ -46,11 +49,12 @@ constexpr int P = 8;             // pixels of a tile: 16 take twice as long per 
 constexpr int kMaxWarps = 16;
 
 // CI: channels of a block that are computed (16: layers of at most 16 channels).  DW: the pixels are a depthwise 3x3's results, which a
-// lane computes where it would load them - once more for every block of 32 filters, in place of a launch and a tensor.
+// lane computes where it would load them - once more for every block of 32 filters, in place of a launch and a tensor.  JOIN: a residual
+// stage's 1x1 shortcut as further steps of the reduction it is added to.
 template <int CI>
 struct Room { static constexpr int kFloats = CI * (P + 4) > P * 32 ? CI * (P + 4) : P * 32; };     // of a warp
 
-template <int CI, bool DW>
+template <int CI, bool DW, bool JOIN>
 __global__ void __launch_bounds__(32 * kMaxWarps) conv_split_fp32_kernel(const SplitFp32Args a) {
     constexpr int PITCH = P + 4, NX = P * CI / 128, NC = CI / 4;    // floats from channel to channel; 16-byte pixel loads of a lane; its channels
     extern __shared__ __align__(16) float smem[];                   // a warp's pixels [channel][pixel], then its sums [pixel][filter]
@@ -67,8 +71,15 @@ __global__ void __launch_bounds__(32 * kMaxWarps) conv_split_fp32_kernel(const S
     const int ix = (r - oy * a.OW) * a.S - a.pl;
     const float *img = a.in + (size_t)n * a.CB * plane;
 
+    const int chunks = a.chunks + (JOIN ? a.CB2 : 0);
+    const float *w2_lane = JOIN ? a.w2 + (size_t)kb * a.CB2 * 1024 + quarter * NC * 32 + (lane & 7) * 4 : nullptr;
+    const float *img2 = JOIN ? a.in2 + ((size_t)n * a.CB2 * a.H2 * a.W2 + (oy * a.W2 + (r - oy * a.OW)) * a.S2) * 32 + lane / P * 4 : nullptr;
+
     float4 px[NX], w[NC];
-    auto load_w = [&](const int c, const int i) { w[i] = *reinterpret_cast<const float4 *>(w_lane + (size_t)c * 1024 + i * 32); };
+    auto load_w = [&](const int c, const int i) {
+        const float *f = JOIN && c >= a.chunks ? w2_lane + (size_t)(c - a.chunks) * 1024 : w_lane + (size_t)c * 1024;
+        w[i] = *reinterpret_cast<const float4 *>(f + i * 32);
+    };
     auto load_px = [&](const int c) {
         if constexpr (DW) {
             const float *s = img + (size_t)c * plane + lane / P * 4, *f = a.dw + (size_t)c * 288 + lane / P * 4;
@@ -95,6 +106,12 @@ __global__ void __launch_bounds__(32 * kMaxWarps) conv_split_fp32_kernel(const S
             }
             return;
         }
+        if (JOIN && c >= a.chunks) {              // (a pixel that does not exist reads the first one's)
+#pragma unroll
+            for (int j = 0; j < NX; ++j)
+                px[j] = *reinterpret_cast<const float4 *>(img2 + (size_t)(c - a.chunks) * a.H2 * a.W2 * 32 + j * (32 / P) * 4);
+            return;
+        }
         const int cb = c / taps, tap = c - cb * taps, dy = tap / a.FW, y = iy + dy, x = ix + tap - dy * a.FW;
         const bool in = (unsigned)y < (unsigned)a.H && (unsigned)x < (unsigned)a.W;
         const float *s = img + (size_t)cb * plane + (size_t)(in ? y * a.W + x : 0) * 32 + lane / P * 4;
@@ -103,19 +120,19 @@ __global__ void __launch_bounds__(32 * kMaxWarps) conv_split_fp32_kernel(const S
     };
 
     if (a.late) grid_dep_sync();
-    if (warp < a.chunks)                          // the filters are the layer's own constants
+    if (warp < chunks)                          // the filters are the layer's own constants
 #pragma unroll
         for (int i = 0; i < NC; ++i) load_w(warp, i);
     grid_dep_sync();
     grid_dep_trigger();
-    if (warp < a.chunks) load_px(warp);
+    if (warp < chunks) load_px(warp);
 
     uint64_t acc[P / 2][4];                       // pairs of pixels x filters
 #pragma unroll
     for (int j = 0; j < P / 2; ++j)
 #pragma unroll
         for (int f = 0; f < 4; ++f) acc[j][f] = 0;
-    for (int c = warp; c < a.chunks; c += warps) {
+    for (int c = warp; c < chunks; c += warps) {
         const int next = c + warps;
         float *x_store = mine + lane / P * 4 * PITCH + lane % P;
 #pragma unroll
@@ -124,7 +141,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps) conv_split_fp32_kernel(const S
             d[0] = px[j].x; d[PITCH] = px[j].y; d[2 * PITCH] = px[j].z; d[3 * PITCH] = px[j].w;
         }
         __syncwarp();
-        if (next < a.chunks) load_px(next);
+        if (next < chunks) load_px(next);
         const float *x_lane = mine + quarter * NC * PITCH;
 #pragma unroll
         for (int i = 0; i < NC; ++i) {
@@ -139,7 +156,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps) conv_split_fp32_kernel(const S
 #pragma unroll
                 for (int f = 0; f < 4; ++f) { fma2(acc[2 * j][f], x.x, ww[f]); fma2(acc[2 * j + 1][f], x.y, ww[f]); }
             }
-            if (next < a.chunks) load_w(next, i);
+            if (next < chunks) load_w(next, i);
         }
         __syncwarp();
     }
@@ -171,7 +188,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps) conv_split_fp32_kernel(const S
     __syncthreads();
 
     const int k = kb * 32 + lane;
-    const float bv = a.bias && k < a.K ? a.bias[k] : 0.0f;
+    const float bv = (a.bias && k < a.K ? a.bias[k] : 0.0f) + (JOIN && a.bias2 && k < a.K ? a.bias2[k] : 0.0f);
     for (int i = warp; i < P && p0 + i < a.pixels; i += warps) {
         const int m = (p0 + i) / (a.OH * a.OW);
         float *dst = a.out + (((size_t)m * a.KB + kb) * a.OH * a.OW + (p0 + i - m * a.OH * a.OW)) * 32 + lane;
@@ -185,18 +202,18 @@ __global__ void __launch_bounds__(32 * kMaxWarps) conv_split_fp32_kernel(const S
     }
 }
 
-template <bool DW>
-void launch_form(small_ctx *ctx, const SplitFp32Args &a, dim3 grid, int warps, cudaStream_t st) {
-    if (a.C <= 16) launch_kernel(ctx, conv_split_fp32_kernel<16, DW>, grid, dim3(32 * warps), (size_t)warps * Room<16>::kFloats * sizeof(float), st, a);
-    else launch_kernel(ctx, conv_split_fp32_kernel<32, DW>, grid, dim3(32 * warps), (size_t)warps * Room<32>::kFloats * sizeof(float), st, a);
+template <bool DW, bool JOIN>
+void launch_form(small_ctx *ctx, const SplitFp32Args &a, bool narrow, dim3 grid, int warps, cudaStream_t st) {
+    if (narrow) launch_kernel(ctx, conv_split_fp32_kernel<16, DW, JOIN>, grid, dim3(32 * warps), (size_t)warps * Room<16>::kFloats * sizeof(float), st, a);
+    else launch_kernel(ctx, conv_split_fp32_kernel<32, DW, JOIN>, grid, dim3(32 * warps), (size_t)warps * Room<32>::kFloats * sizeof(float), st, a);
 }
 
 // How a layer is cut: warps that share a tile's reduction, and the time expected of it in us (of 88 measured layers, most within a fifth).
 struct SplitFp32Plan { int warps; long long waves; unsigned px_tiles; double us; };
 
-SplitFp32Plan plan_split_fp32(const Geom &g, int sms, bool dw) {
+SplitFp32Plan plan_split_fp32(const Geom &g, int sms, bool dw, int more = 0) {      // more: steps besides the layer's own
     SplitFp32Plan best{};
-    const int chunks = g.CB * g.FH * g.FW, resident = g.C <= 16 ? 20 : 16;     // warps an SM's registers hold
+    const int chunks = g.CB * g.FH * g.FW + more, resident = g.C <= 16 ? 20 : 16;     // warps an SM's registers hold
     const long long px = ((long long)g.N * g.OH * g.OW + P - 1) / P, tiles = px * g.KB, on_sm = (tiles + sms - 1) / sms;
     // a round: its latency, and what a resident warp is handed from cache and shared memory (a depthwise layer's pixels and filters
     // are another 36 loads of 16 bytes per lane)
@@ -233,11 +250,14 @@ double conv_split_fp32_us(const Geom &g, int sms) {
 }
 
 int launch_conv_split_fp32(small_ctx *ctx, const float *in, const float *w, const float *bias, float *out, const Geom &g,
-                           bool relu, bool accumulate, cudaStream_t st) {
-    const SplitFp32Args a{in, w, bias, out, g.K, g.KB, g.CB, g.H, g.W, g.OH, g.OW, g.FH, g.FW, g.S, g.pt, g.pl,
-                          g.N * g.OH * g.OW, g.CB * g.FH * g.FW, relu, accumulate, ctx->dependent == 2, nullptr, nullptr, g.C, 0};
-    const SplitFp32Plan p = plan_split_fp32(g, ctx->sm_count, false);
-    launch_form<false>(ctx, a, dim3(p.px_tiles, (unsigned)g.KB), p.warps, st);
+                           bool relu, bool accumulate, cudaStream_t st, const Shortcut *sc) {
+    SplitFp32Args a{in, w, bias, out, g.K, g.KB, g.CB, g.H, g.W, g.OH, g.OW, g.FH, g.FW, g.S, g.pt, g.pl,
+                    g.N * g.OH * g.OW, g.CB * g.FH * g.FW, relu, accumulate, ctx->dependent == 2, nullptr, nullptr, g.C, 0, nullptr, nullptr, nullptr, 0, 0, 0, 0};
+    if (sc) { a.in2 = sc->in; a.w2 = sc->w; a.bias2 = sc->bias; a.CB2 = sc->g.CB; a.H2 = sc->g.H; a.W2 = sc->g.W; a.S2 = sc->g.S; }
+    const SplitFp32Plan p = plan_split_fp32(g, ctx->sm_count, false, a.CB2);
+    const dim3 grid(p.px_tiles, (unsigned)g.KB);
+    if (sc) launch_form<false, true>(ctx, a, g.C <= 16 && sc->g.C <= 16, grid, p.warps, st);
+    else launch_form<false, false>(ctx, a, g.C <= 16, grid, p.warps, st);
     return check_launch(ctx);
 }
 
@@ -253,9 +273,9 @@ double split_pair_us(const Geom &gp, int sms) {
 int launch_split_pair(small_ctx *ctx, const float *in, const float *dw, const float *dw_bias, bool dw_relu, const float *w, const float *bias,
                       float *out, const Geom &gd, const Geom &gp, bool relu, cudaStream_t st) {
     const SplitFp32Args a{in, w, bias, out, gp.K, gp.KB, gp.CB, gd.H, gd.W, gp.OH, gp.OW, 1, 1, gd.S, gd.pt, gd.pl,
-                          gp.N * gp.OH * gp.OW, gp.CB, relu, 0, ctx->dependent == 2, dw, dw_bias, gp.C, dw_relu};
+                          gp.N * gp.OH * gp.OW, gp.CB, relu, 0, ctx->dependent == 2, dw, dw_bias, gp.C, dw_relu, nullptr, nullptr, nullptr, 0, 0, 0, 0};
     const SplitFp32Plan p = plan_split_fp32(gp, ctx->sm_count, true);
-    launch_form<true>(ctx, a, dim3(p.px_tiles, (unsigned)gp.KB), p.warps, st);
+    launch_form<true, false>(ctx, a, gp.C <= 16, dim3(p.px_tiles, (unsigned)gp.KB), p.warps, st);
     return check_launch(ctx);
 }
 

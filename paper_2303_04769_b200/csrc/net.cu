@@ -177,11 +177,24 @@ static double split_pair(const small_ctx *ctx, const small_layer *layers, int n_
     return split_pair_us(gp, ctx->sm_count);
 }
 
-// A run with depthwise layers that could stay on chip in FP32 (net_resident.cu), launch by launch instead: whether that is the faster form
+// Layers i and i + 1 as a residual stage's shortcut - 1x1, no padding, no activation - and the convolution that is added to its result.
+static bool shortcut_pair(const small_layer *layers, int n_layers, int i, int N, Geom &sc, Geom &g) {
+    if (i + 1 >= n_layers) return false;
+    const small_layer &A = layers[i], &Bn = layers[i + 1];
+    if (A.op != SMALL_OP_CONV || Bn.op != SMALL_OP_CONV || A.FH != 1 || A.FW != 1 || (A.pad_t | A.pad_b | A.pad_l | A.pad_r) || A.dst != Bn.dst || A.K != Bn.K ||
+        (A.flags & (SMALL_RELU | SMALL_ACCUMULATE)) || !(Bn.flags & SMALL_ACCUMULATE) || (A.flags & SMALL_MATH_MASK) != (Bn.flags & SMALL_MATH_MASK))
+        return false;
+    if (make_geom(sc, N, A.C, A.K, A.H, A.W, 1, 1, A.stride, 0, 0, 0, 0)) return false;
+    if (make_geom(g, N, Bn.C, Bn.K, Bn.H, Bn.W, Bn.FH, Bn.FW, Bn.stride, Bn.pad_t, Bn.pad_b, Bn.pad_l, Bn.pad_r)) return false;
+    return sc.OH == g.OH && sc.OW == g.OW;
+}
+
+// A run that could stay on chip in FP32 (net_resident.cu), launch by launch instead: whether that is the faster form
 // for its batch.  An operation costs the on-chip kernel 4.3 to 6.7 us whatever the batch - barriers, filters passing by - and the kernels
 // of few pixels 2 to 9, growing with it.  us, on chip against launches: stem and two pairs of 64 channels on 25 x 5, batch 1 / 18 / 74 31.5 /
 // 29.5 / 31.2 against 13.4 / 19.7 / 29.1; the keyword-spotting network (four pairs) 1 / 37 / 64 / 128 47.9 / 50.1 / 51.0 / 53.7 against 20.8 /
-// 35.6 / 48.3 / 82; depthwise-separable network 1 / 16 / 64 115.7 / 142 / 208 against 55.8 / 94 / 164.
+// 35.6 / 48.3 / 82; depthwise-separable network 1 / 16 / 64 115.7 / 142 / 208 against 55.8 / 94 / 164.  Without depthwise layers, where
+// every operation ends in an exchange, it is 9 us and more (residual network 98 at batch 1 to 105 at 12).
 static bool launches_beat_on_chip(const small_ctx *ctx, const small_layer *layers, int n_layers, int from, int N) {
     double us = 4.0;                              // the average pool and the classifier
     bool depthwise = false;
@@ -196,7 +209,7 @@ static bool launches_beat_on_chip(const small_ctx *ctx, const small_layer *layer
         else if (const double t = conv_split_fp32_us(g, ctx->sm_count)) us += t;
         else us += 5.0 + (0.07 + out / 15e6) * L.C * L.FH * L.FW;
     }
-    return depthwise && us < 4.5 * (n_layers - from);
+    return us < (depthwise ? 4.5 : 9.0) * (n_layers - from);
 }
 
 // Runs of layers are kept on chip as one kernel where every kind of fusion is on.
@@ -325,8 +338,14 @@ static int run_layers(small_ctx *ctx, const small_layer *layers, int n_layers, i
         if (!chain_layers) on_chip = resident_from(ctx, layers, n_layers, from, N);
         if (on_chip >= 0 && (layers[n_layers - 1].flags & SMALL_MATH_MASK) == SMALL_MATH_FP32 && launches_beat_on_chip(ctx, layers, n_layers, on_chip, N)) on_chip = -1;
     }
+    // a shortcut and the layer that is added to it, where both are split over warps, as one launch
+    auto joins = [&](int i, Geom &sc, Geom &g) {
+        return runs && i + 1 != chain && i + 1 != on_chip && shortcut_pair(layers, n_layers, i, N, sc, g) &&
+               joined_split(ctx, sc, g, layers[i].flags & SMALL_MATH_MASK, (reinterpret_cast<uintptr_t>(wr(layers[i].dst)) & 31u) == 0);
+    };
     for (int i = from; i < n_layers; ++i) {
         const small_layer &L = layers[i];
+        Geom sc_next, g_next;
         int s = SMALL_OK;
         // every layer may start its set-up while the kernel in front of it drains (see launch_kernel)
         ctx->dependent = !ctx->overlap || after_join ? 0 : i > 0 ? 1 : 2;
@@ -349,6 +368,18 @@ static int run_layers(small_ctx *ctx, const small_layer *layers, int n_layers, i
                 const small_layer &Nx = layers[i + 1];
                 s = launch_split_pair(ctx, rd(L.src), L.w_blk, L.bias, L.flags & SMALL_RELU, Nx.w_blk, Nx.bias, wr(Nx.dst), gd, gp, Nx.flags & SMALL_RELU,
                                       static_cast<cudaStream_t>(stream));
+                ctx->dependent = 0;
+                if (s != SMALL_OK) return s;
+                ++i;
+                continue;
+            }
+        }
+        {
+            Geom sc, g;
+            if (joins(i, sc, g)) {
+                const small_layer &Nx = layers[i + 1];
+                s = launch_joined(ctx, Shortcut{rd(L.src), L.w_blk, nullptr, nullptr, L.bias, sc}, rd(Nx.src), Nx.w_blk, Nx.bias, wr(L.dst), g, Nx.flags & SMALL_RELU,
+                                  L.flags & SMALL_MATH_MASK, static_cast<cudaStream_t>(stream));
                 ctx->dependent = 0;
                 if (s != SMALL_OK) return s;
                 ++i;
@@ -394,7 +425,7 @@ static int run_layers(small_ctx *ctx, const small_layer *layers, int n_layers, i
         // stream by events, so that a short layer hides behind a long one.  Both are ordinary launches, and so is the
         // layer behind the join.
         if (ctx->branch_overlap && ctx->side_stream && i + 1 < n_layers && i + 1 != on_chip && i + 1 != chain && independent(L, layers[i + 1]) &&
-            !fused_pair(ctx, layers, n_layers, i + 1, N)) {
+            !fused_pair(ctx, layers, n_layers, i + 1, N) && !joins(i + 1, sc_next, g_next)) {
             cudaStream_t main_st = static_cast<cudaStream_t>(stream), side = static_cast<cudaStream_t>(ctx->side_stream);
             cudaError_t e = cudaEventRecord(static_cast<cudaEvent_t>(ctx->ev_fork), main_st);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(side, static_cast<cudaEvent_t>(ctx->ev_fork), 0);

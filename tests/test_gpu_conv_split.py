@@ -99,3 +99,26 @@ def test_fp32_pairs_as_one_launch(C, K, H, W, S, relu, batch):
     assert pad_lanes_are_zero(got, *ref.shape)
     apart = Net(ctx(), net, params, batch=batch, fuse_dwpw=False).run(to_blk(x))
     assert rel_err(from_blk(apart, *ref.shape), ref) <= TOL["fp32"]
+
+
+@pytest.mark.parametrize("math", ["fp32", "tf32", "3xtf32"])
+@pytest.mark.parametrize("C,K,H,W,C2,S,relu,batch", [(32, 32, 16, 16, 16, 2, True, 1), (12, 40, 7, 5, 70, 1, False, 3), (16, 9, 1, 1, 33, 3, True, 1), (64, 64, 8, 8, 32, 2, True, 2)])
+def test_shortcut_as_part_of_the_layer_it_joins(math, C, K, H, W, C2, S, relu, batch):
+    """x -> 1x1 shortcut (stride S) and 3x3 convolution, then a 3x3 convolution added to the shortcut: one launch for the last two."""
+    H2, W2 = (H - 1) * S + 1 + (S > 2), (W - 1) * S + 1
+    layers = [configs._conv("a", "in", "m", C2, C, 1, S, configs.P0, True),
+              configs._conv("s", "in", "out", C2, K, 1, S, configs.P0, False),
+              configs._conv("b", "m", "out", C, K, 3, 1, configs.P1, relu, accumulate=True)]
+    net = dict(name="joined", batch=batch, input=(C2, H2, W2), input_dist=("uniform", -1.0, 1.0), weight_dist="he_normal", layers=layers)
+    params, x = configs.make_params(net), configs.make_input(net, batch)
+    ref = nets.run_net(net, params, x)["out"]
+    for overlap in (1, 0):
+        B.small_set_layer_overlap(ctx(), overlap)
+        try:
+            got = Net(ctx(), net, params, batch=batch, math=math).run(to_blk(x))
+            apart = Net(ctx(), net, params, batch=batch, math=math, fuse_poolfc=False).run(to_blk(x))
+        finally:
+            B.small_set_layer_overlap(ctx(), 1)
+        for y in (got, apart):
+            assert rel_err(from_blk(y, *ref.shape), ref) <= TOL[math]
+            assert pad_lanes_are_zero(y, *ref.shape)
