@@ -443,10 +443,10 @@ static int conv2d_path(small_ctx *ctx, const Geom &g, unsigned math, bool out_al
 
 namespace small {
 
-// Both layers on the same one of the two kernels.
+// Where the layer runs on one of the two kernels and its shortcut in the same arithmetic, on that kernel or, by a hair, another.
 bool joined_split(small_ctx *ctx, const Geom &sc, const Geom &g, unsigned math, bool out_aligned32) {
-    const int a = conv2d_path(ctx, sc, math, out_aligned32), b = conv2d_path(ctx, g, math, out_aligned32);
-    return a > kSplit && b > kSplit && (a - kSplit >= 3) == (b - kSplit >= 3);
+    const int a = conv2d_path(ctx, sc, math, out_aligned32) & (kSplit - 1), b = conv2d_path(ctx, g, math, out_aligned32) - kSplit;
+    return a > 0 && b > 0 && (a >= 3) == (b >= 3);
 }
 
 int launch_joined(small_ctx *ctx, Shortcut sc, const float *in, const float *w, const float *bias, float *out, const Geom &g, bool relu, unsigned math, cudaStream_t st) {

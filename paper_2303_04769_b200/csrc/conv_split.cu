@@ -193,19 +193,17 @@ void launch_form(small_ctx *ctx, const SplitArgs &a, bool x3, dim3 grid, int war
 // How a layer is cut: filters of a tile, warps that share its reduction, and the time expected of it in us.
 struct SplitPlan { int nf, warps; unsigned px_tiles, k_tiles; double us; };
 
-SplitPlan plan_split(const Geom &g, bool x3, int sms, int more = 0) {      // more: steps besides the layer's own
+SplitPlan cut(long long pixels, int K, int chunks, bool narrow, bool x3, int sms) {
     SplitPlan best{};
-    const long long pixels = (long long)g.N * g.OH * g.OW;
-    const int chunks = g.CB * g.FH * g.FW + more;
     for (int nf = 1; nf <= 2; ++nf) {
-        if (nf == 2 && g.K <= 8) break;
-        const long long px = (pixels + 15) / 16, kt = (g.K + 8 * nf - 1) / (8 * nf);
+        if (nf == 2 && K <= 8) break;
+        const long long px = (pixels + 15) / 16, kt = (K + 8 * nf - 1) / (8 * nf);
         const int resident = x3 ? (nf == 1 ? 20 : 16) : (nf == 1 ? 26 : 22);      // warps an SM's registers hold
-        const double kb = (g.C <= 16 ? 1.0 : 2.0) * (1.0 + 0.5 * nf * (x3 ? 2 : 1));
+        const double kb = (narrow ? 1.0 : 2.0) * (1.0 + 0.5 * nf * (x3 ? 2 : 1));
         int last = 0;
-        for (int rounds = 1; rounds <= chunks; ++rounds) {
+        for (int rounds = (chunks + 15) / 16; rounds <= chunks; ++rounds) {
             const int warps = (chunks + rounds - 1) / rounds;
-            if (warps > 16 || warps == last) continue;
+            if (warps == last) continue;
             last = warps;
             const int per_sm = resident / warps;       // blocks
             const long long waves = (px * kt + (long long)sms * per_sm - 1) / ((long long)sms * per_sm);
@@ -218,6 +216,18 @@ SplitPlan plan_split(const Geom &g, bool x3, int sms, int more = 0) {      // mo
         }
     }
     return best;
+}
+
+// more: steps besides the layer's own.  Every launch asks: the latest answers are kept by what they depend on.
+SplitPlan plan_split(const Geom &g, bool x3, int sms, int more = 0) {
+    struct Kept { long long pixels; int K, chunks, narrow, x3, sms; SplitPlan p; };
+    static thread_local Kept kept[64];
+    const long long pixels = (long long)g.N * g.OH * g.OW;
+    const int chunks = g.CB * g.FH * g.FW + more, narrow = g.C <= 16;
+    Kept &k = kept[(size_t)(pixels * 31 + g.K * 7 + chunks * 3 + narrow + 2 * x3) % 64];
+    if (k.pixels != pixels || k.K != g.K || k.chunks != chunks || k.narrow != narrow || k.x3 != x3 || k.sms != sms)
+        k = Kept{pixels, g.K, chunks, narrow, x3, sms, cut(pixels, g.K, chunks, narrow, x3, sms)};
+    return k.p;
 }
 
 }  // namespace

@@ -209,27 +209,39 @@ void launch_form(small_ctx *ctx, const SplitFp32Args &a, bool narrow, dim3 grid,
 }
 
 // How a layer is cut: warps that share a tile's reduction, and the time expected of it in us (of 88 measured layers, most within a fifth).
-struct SplitFp32Plan { int warps; long long waves; unsigned px_tiles; double us; };
+struct SplitFp32Plan { int warps; unsigned px_tiles; double us; };
 
-SplitFp32Plan plan_split_fp32(const Geom &g, int sms, bool dw, int more = 0) {      // more: steps besides the layer's own
+SplitFp32Plan cut(long long pixels, int KB, int chunks, bool narrow, bool dw, int sms) {
     SplitFp32Plan best{};
-    const int chunks = g.CB * g.FH * g.FW + more, resident = g.C <= 16 ? 20 : 16;     // warps an SM's registers hold
-    const long long px = ((long long)g.N * g.OH * g.OW + P - 1) / P, tiles = px * g.KB, on_sm = (tiles + sms - 1) / sms;
+    const int resident = narrow ? 20 : 16;         // warps an SM's registers hold
+    const long long px = (pixels + P - 1) / P, tiles = px * KB, on_sm = (tiles + sms - 1) / sms;
     // a round: its latency, and what a resident warp is handed from cache and shared memory (a depthwise layer's pixels and filters
     // are another 36 loads of 16 bytes per lane)
-    const double latency = dw ? 1.2 : g.C <= 16 ? 0.42 : 0.46, warp = (g.C <= 16 ? 0.04 : 0.062) * (dw ? 6.0 : 1.0);
+    const double latency = dw ? 1.2 : narrow ? 0.42 : 0.46, warp = (narrow ? 0.04 : 0.062) * (dw ? 6.0 : 1.0);
     int last = 0;
-    for (int rounds = 1; rounds <= chunks; ++rounds) {
+    for (int rounds = (chunks + kMaxWarps - 1) / kMaxWarps; rounds <= chunks; ++rounds) {
         const int warps = (chunks + rounds - 1) / rounds;
-        if (warps > kMaxWarps || warps == last) continue;
+        if (warps == last) continue;
         last = warps;
         const int per_sm = resident / warps;       // blocks
         const long long waves = (tiles + (long long)sms * per_sm - 1) / ((long long)sms * per_sm);
         const int busy = (int)(on_sm < per_sm ? on_sm : per_sm) * warps;
         const double us = 0.6 + (double)waves * (1.2 + rounds * (latency + warp * busy));
-        if (!best.warps || us < best.us) best = SplitFp32Plan{warps, waves, (unsigned)px, us};
+        if (!best.warps || us < best.us) best = SplitFp32Plan{warps, (unsigned)px, us};
     }
     return best;
+}
+
+// more: steps besides the layer's own.  Every launch asks: the latest answers are kept by what they depend on.
+SplitFp32Plan plan_split_fp32(const Geom &g, int sms, bool dw, int more = 0) {
+    struct Kept { long long pixels; int KB, chunks, narrow, dw, sms; SplitFp32Plan p; };
+    static thread_local Kept kept[64];
+    const long long pixels = (long long)g.N * g.OH * g.OW;
+    const int chunks = g.CB * g.FH * g.FW + more, narrow = g.C <= 16;
+    Kept &k = kept[(size_t)(pixels * 31 + g.KB * 7 + chunks * 3 + narrow + 2 * dw) % 64];
+    if (k.pixels != pixels || k.KB != g.KB || k.chunks != chunks || k.narrow != narrow || k.dw != dw || k.sms != sms)
+        k = Kept{pixels, g.KB, chunks, narrow, dw, sms, cut(pixels, g.KB, chunks, narrow, dw, sms)};
+    return k.p;
 }
 
 bool fits(const Geom &g) { return (long long)g.N * g.OH * g.OW <= 1 << 20 && (long long)g.H * g.W <= 1 << 24 && g.K <= 1 << 16; }
