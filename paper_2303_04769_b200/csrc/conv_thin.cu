@@ -11,7 +11,8 @@
 //   * the real channels of the next input tile are copied to shared memory while a tile is computed, and then spread over dense
 //     planes [image][channel][row][column] with every value twice: a 16-byte read brings two inputs as the pairs that the FMAs
 //     take.  The copy is one TMA box of 16 bytes of each pixel's line, zeros outside the plane (as many loads of threads wait for
-//     the few lines that an SM's first-level cache has in flight: a line per pixel); from an NCHW tensor, and for very wide planes, cp.async;
+//     the few lines that an SM's first-level cache has in flight: a line per pixel); from an NCHW tensor, cp.async;
+//   * a tile is whole rows of an image, or of several images; of wide planes, some columns of rows (see plan_tiles);
 //   * a warp computes PIX adjacent output pixels of a row: per window row it reads the (PIX - 1) S + F_W inputs it needs as
 //     shared-memory broadcasts and issues PIX x F_W packed FMAs on them.
 // Bias, accumulate (the residual join), ReLU and the zero pad lanes are handled as in the other convolution kernels.
@@ -33,13 +34,13 @@ namespace {
 struct ThinArgs {
     const float *in; const float *w; const float *bias; float *out; int *status;
     int N, K, KB, H, W, OH, OW, pt, pl;
-    int nb, TH, bands, groups, kgroups;      // images and output rows per tile; tiles per image; column groups; filter groups
+    int nb, TH, bands, kgroups;              // images and output rows per tile; row bands of an image; filter groups
+    int gt, cbands;                          // column groups (of PIX outputs) of a tile; column bands of an image
     int rows, pitch, plane;                  // shared tile: rows x pitch pairs per (image, channel); plane = rows * pitch
     uint32_t raw_bytes;                      // of the next tile's copy, in front of the planes
-    uint32_t by_pitch, by_rows, by_groups;   // divisors as multipliers (see quotient)
-    long long tiles;
+    uint32_t by_pitch, by_rows, by_gt;       // divisors as multipliers (see quotient)
+    unsigned tiles;                          // (no more than output pixels, whose tensor fits the memory: below 2^31)
     bool relu, accumulate;
-    bool tma;                                // planes of at most 256 columns with their pads, blocked
     bool nchw;                               // the input is the NCHW tensor float[N][C][H][W] itself (the network's edge)
     uint32_t wait_iters;                     // limit of the bounded waits (polls)
     int late;                                // wait for the kernel in front before reading constants
@@ -99,13 +100,22 @@ __global__ void __launch_bounds__(kThinThreads, thin_blocks(C *FH *FW, PIX, (PIX
     grid_dep_trigger();
 
     const uint32_t raw = sm100::smem_u32(smem);
+    // tile t: its first image, its row band and its first column group
+    auto place = [&](unsigned t, int &n0, int &band, int &g0) {
+        g0 = 0;
+        if (a.cbands > 1) { const unsigned q = t / (unsigned)a.cbands; g0 = (int)(t - q * a.cbands) * a.gt; t = q; }
+        const unsigned q = t / (unsigned)a.bands;
+        band = (int)(t - q * a.bands); n0 = (int)q * a.nb;
+    };
     // A tile's pixels, four floats each: [image][row][column], the columns and rows outside the plane zero.
-    auto copy = [&](long long t) {
-        const int band = (int)(t % a.bands), n0 = (int)(t / a.bands) * a.nb, ih0 = band * a.TH * S - a.pt;
-        if (a.tma) {
+    auto copy = [&](unsigned t) {
+        int n0, band, g0;
+        place(t, n0, band, g0);
+        const int ih0 = band * a.TH * S - a.pt, iw0 = g0 * PIX * S - a.pl;
+        if (!a.nchw) {
             if (threadIdx.x == 0) {
                 sm100::mbar_expect_tx(full, (uint32_t)(a.nb * a.rows * a.pitch) * 16u);
-                sm100::tma_load_5d(raw, &map, full, 0, -a.pl, ih0, 0, n0);
+                sm100::tma_load_5d(raw, &map, full, 0, iw0, ih0, 0, n0);
             }
             return;
         }
@@ -113,13 +123,8 @@ __global__ void __launch_bounds__(kThinThreads, thin_blocks(C *FH *FW, PIX, (PIX
         const size_t hw = (size_t)a.H * a.W;
         for (int e = threadIdx.x; e < total; e += kThinThreads) {
             int r = quotient(e, a.by_pitch);
-            const int gw = e - r * a.pitch - a.pl, img = quotient(r, a.by_rows), gh = ih0 + r - img * a.rows;
+            const int gw = e - r * a.pitch + iw0, img = quotient(r, a.by_rows), gh = ih0 + r - img * a.rows;
             const bool in = (unsigned)gh < (unsigned)a.H && (unsigned)gw < (unsigned)a.W;
-            if (!a.nchw) {
-                const float *p = in ? a.in + (((size_t)(n0 + img) * a.H + gh) * a.W + gw) * 32 : a.in;
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(raw + (uint32_t)(e * 16)), "l"(p), "r"(in ? 16 : 0) : "memory");
-                continue;
-            }
             const float *p = in ? a.in + ((size_t)(n0 + img) * C * a.H + gh) * a.W + gw : a.in;
 #pragma unroll
             for (int c = 0; c < C; ++c)
@@ -129,10 +134,12 @@ __global__ void __launch_bounds__(kThinThreads, thin_blocks(C *FH *FW, PIX, (PIX
     uint32_t parity = 0;
     bool alive = true;
     if (blockIdx.x < a.tiles) copy(blockIdx.x);
-    for (long long t = blockIdx.x; t < a.tiles; t += gridDim.x) {
-        const int band = (int)(t % a.bands), n0 = (int)(t / a.bands) * a.nb, imgs = min(a.nb, a.N - n0), oh0 = band * a.TH;
+    for (unsigned t = blockIdx.x; t < a.tiles; t += gridDim.x) {
+        int n0, band, g0;
+        place(t, n0, band, g0);
+        const int imgs = min(a.nb, a.N - n0), oh0 = band * a.TH;
         const int th = min(a.TH, a.OH - oh0), total = imgs * a.rows * a.pitch;
-        if (!a.tma) asm volatile("cp.async.wait_all;" ::: "memory");
+        if (a.nchw) asm volatile("cp.async.wait_all;" ::: "memory");
         else alive = sm100::mbar_wait_uniform(full, parity, &abort_flag, a.status, a.wait_iters);
         parity ^= 1u;
         if (!__syncthreads_and(alive)) break;  // the tile is there, and the planes are no longer read
@@ -148,12 +155,12 @@ __global__ void __launch_bounds__(kThinThreads, thin_blocks(C *FH *FW, PIX, (PIX
         }
         __syncthreads();
         if (t + gridDim.x < a.tiles) copy(t + gridDim.x);
-        const int per_img = th * a.groups, items = imgs * per_img;      // (image, output row, column group)
+        const int per_img = th * a.gt, items = imgs * per_img;      // (image, output row, column group; some of the last column band's may lie outside)
         for (int it0 = warp * PIECES; it0 < items; it0 += PIECES * (kThinThreads / 32)) {
             const int it = min(it0 + sub, items - 1);
             int img = 0, rg = it;
             if (imgs > 1) { img = it / per_img; rg = it - img * per_img; }
-            const int r = quotient(rg, a.by_groups), cg = rg - r * a.groups;
+            const int r = quotient(rg, a.by_gt), cg = rg - r * a.gt;
             const uint32_t piece = raw + a.raw_bytes + (uint32_t)(img * C * a.plane + r * S * a.pitch + cg * PIX * S) * 8u;
             uint64_t acc[PIX];
 #pragma unroll
@@ -175,7 +182,7 @@ __global__ void __launch_bounds__(kThinThreads, thin_blocks(C *FH *FW, PIX, (PIX
                 }
             }
             if (it0 + sub >= items || !line_exists) continue;
-            const int oh = oh0 + r, ow0 = cg * PIX;
+            const int oh = oh0 + r, ow0 = (g0 + cg) * PIX;
             float *dst = a.out + ((((size_t)(n0 + img) * a.KB + kb) * a.OH + oh) * a.OW + ow0) * 32;
 #pragma unroll
             for (int p = 0; p < PIX; ++p) {
@@ -239,14 +246,54 @@ int thin_pix(const Geom &g) {
     return 8;
 }
 
-struct ThinLaunch { CUtensorMap map; ThinArgs a; ThinKernel kern; dim3 grid; size_t smem; };
-typedef std::unordered_map<std::string, ThinLaunch> ThinCache;
+// What a layer needs besides its tensors, made once per shape (a new buffer of a known shape costs a tensor map): the launch, and the
+// tensor maps of the inputs seen.
+struct ThinPlan { ThinArgs a; ThinKernel kern; dim3 grid; size_t smem; std::unordered_map<const float *, CUtensorMap> maps; };
+typedef std::unordered_map<std::string, ThinPlan> ThinCache;
 
-int thin_pitch(const Geom &g) {
-    const int pix = thin_pix(g), groups = ceil_div(g.OW, pix), seg2 = ((pix - 1) * g.S + g.FW + 1) / 2;
-    int pitch = (groups - 1) * pix * g.S + 2 * seg2;          // the last column group's reads stay inside the row
-    if (pitch < g.W + g.pl) pitch = g.W + g.pl;
-    return (pitch + 1) & ~1;
+// Columns that `groups` column groups read.
+int tile_pitch(const Geom &g, int groups) {
+    const int pix = thin_pix(g);
+    return (groups - 1) * pix * g.S + 2 * (((pix - 1) * g.S + g.FW + 1) / 2);
+}
+
+// The tile: whole rows of an image, several images where planes are small.  Estimated cycles of an SM: its tiles in rounds of as many
+// blocks as it holds; a warp alone issues every third or fourth cycle (a window row's reads, then chains of FMAs), more share the
+// scheduler (FMA pairs take two slots).
+// Of planes so wide that four rows of outputs need more than kRowTile, some columns of the rows: whole rows bring in two or three rows
+// for one computed, leave an SM one block from some 300 columns on, and from 640 on can need more than a block has.  These
+// tiles are at most kCutTile, so that the registers decide how many blocks an SM holds, and a tile costs some 100 cycles besides (21
+// layers, each with up to 60 tiles: the one taken is within 5 % of the best on average).  us, whole rows / columns cut: 3 channels,
+// 3 x 3 stride 2, 32 filters on 224 x 224, batch 8 / 64 10.0 / 9.6, 85.1 / 84.2, on 512 x 512, batch 8 113 / 56; stride 1 on 224 x 224, batch 8
+// 30.1 / 24.8; 10 x 4, 64 filters on 500 x 128, batch 16 48.5 / 48.9, on 1000 x 257 255 / 158.
+constexpr size_t kRowTile = 44 * 1024, kCutTile = 24 * 1024;
+bool plan_tiles(const small_ctx *ctx, const Geom &g, int by_regs, ThinArgs &a) {
+    const int pix = thin_pix(g), seg2 = ((pix - 1) * g.S + g.FW + 1) / 2, pieces = 32 / thin_lanes(g.K), groups = ceil_div(g.OW, pix);
+    const double per_piece = g.C * g.FH * (seg2 + 2.0 * g.FW * pix) + 8.0 * pix;
+    auto rows = [&](int th) { return (th - 1) * g.S + g.FH; };
+    auto bytes = [&](int nb, int th, int pitch) { return (size_t)nb * rows(th) * pitch * (16 + 8 * g.C); };
+    const bool cut = tile_pitch(g, groups) > 256 || bytes(1, g.OH < 4 ? g.OH : 4, tile_pitch(g, groups)) > kRowTile;
+    const size_t most = cut ? kCutTile : kRowTile;
+    double best = 0.0;
+    for (int cbands = 1; cbands <= (cut ? groups : 1); ++cbands) {
+        const int gt = ceil_div(groups, cbands), pitch = tile_pitch(g, gt);
+        if (ceil_div(groups, gt) != cbands || pitch > 256) continue;
+        for (int bands = 1; bands <= g.OH; ++bands) {
+            const int th = ceil_div(g.OH, bands);
+            if (ceil_div(g.OH, th) != bands || rows(th) > 256) continue;
+            if (th < 4 && bands > 1 && best > 0.0) break;
+            for (int nb = 1; nb <= (bands * cbands == 1 ? (g.N < 16 ? g.N : 16) : 1) && bytes(nb, th, pitch) <= most; ++nb) {
+                const long long tiles = (long long)ceil_div(g.N, nb) * bands * cbands * a.kgroups, on_sm = (tiles + ctx->sm_count - 1) / ctx->sm_count;
+                long long held = (long long)(ctx->max_smem_optin / (bytes(nb, th, pitch) + 1024));
+                if (held > by_regs) held = by_regs;
+                if (held > on_sm) held = on_sm;
+                const double work = ceil_div(nb * th * gt, 4 * pieces) * per_piece + (double)nb * rows(th) * pitch * (g.C + 2) * 0.1 + (cut ? 100.0 : 0.0), alone = work * 3.3 + 600.0;
+                const double cost = (double)((on_sm + held - 1) / held) * (held * work > alone ? held * work : alone);
+                if (best == 0.0 || cost < best) { best = cost; a.TH = th; a.nb = nb; a.bands = bands; a.gt = gt; a.cbands = cbands; a.pitch = pitch; }
+            }
+        }
+    }
+    return best > 0.0;
 }
 
 }  // namespace
@@ -254,8 +301,10 @@ int thin_pitch(const Geom &g) {
 bool conv_thin_supported(const Geom &g) {
     if (g.C > 4 || g.CB != 1) return false;
     if (!pick_thin(g, thin_pix(g), 32)) return false;
-    // at least one output row of one image must fit the shared tile
-    return (size_t)g.C * g.FH * thin_pitch(g) * sizeof(float) <= 40 * 1024;
+    // rows of up to some 850 (four channels) to 3400 columns (one); wider planes take the other kernels
+    int pitch = tile_pitch(g, ceil_div(g.OW, thin_pix(g)));
+    if (pitch < g.W + g.pl) pitch = (g.W + g.pl + 1) & ~1;
+    return (size_t)g.C * g.FH * pitch * sizeof(float) <= 40 * 1024;
 }
 
 void free_thin_cache(small_ctx *ctx) {
@@ -263,99 +312,75 @@ void free_thin_cache(small_ctx *ctx) {
     ctx->thin_cache = nullptr;
 }
 
+static int make_plan(small_ctx *ctx, const Geom &g, bool nchw_in, ThinPlan &p) {
+    ThinArgs &a = p.a;
+    a = ThinArgs{};
+    a.status = ctx->dev_status; a.nchw = nchw_in;
+    a.N = g.N; a.K = g.K; a.KB = g.KB; a.H = g.H; a.W = g.W; a.OH = g.OH; a.OW = g.OW; a.pt = g.pt; a.pl = g.pl;
+    a.kgroups = ceil_div(g.KB, 2);
+    p.kern = pick_thin(g, thin_pix(g), thin_lanes(g.K));
+    if (!p.kern) return SMALL_ERR_UNSUPPORTED;
+    int by_regs = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&by_regs, p.kern, kThinThreads, 0) != cudaSuccess || by_regs < 1) by_regs = 1;
+    if (!plan_tiles(ctx, g, by_regs, a)) return SMALL_ERR_UNSUPPORTED;
+    a.rows = (a.TH - 1) * g.S + g.FH;
+    a.plane = a.rows * a.pitch;
+    a.raw_bytes = (uint32_t)(a.nb * a.plane * 16);
+    auto multiplier = [](int d) { return d <= 1 ? 0u : (uint32_t)((1ull << 32) / (unsigned)d) + 1u; };
+    a.by_pitch = multiplier(a.pitch); a.by_rows = multiplier(a.rows);
+    a.by_gt = multiplier(a.gt);
+    a.tiles = (unsigned)((long long)ceil_div(g.N, a.nb) * a.bands * a.cbands);
+    p.smem = (size_t)a.nb * a.plane * (16 + 8 * g.C);      // at most kRowTile: within what every launch may have
+    // blocks that run at once: the grid is that many (or fewer), each walking the tile list
+    int per_sm = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, p.kern, kThinThreads, p.smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+    long long gx = (long long)per_sm * ctx->sm_count / a.kgroups;
+    if (gx < 1) gx = 1;
+    p.grid = dim3(a.tiles < gx ? a.tiles : (unsigned)gx, (unsigned)a.kgroups);
+    return SMALL_OK;
+}
+
 int launch_conv_thin(small_ctx *ctx, const float *in, const float *w, const float *bias, float *out, const Geom &g,
                      bool relu, bool accumulate, cudaStream_t st, bool nchw_in) {
     if (!conv_thin_supported(g)) return SMALL_ERR_UNSUPPORTED;
-    // a launch seen before (same shape, flags and tensors): everything is ready
     std::string key;
     {
-        const int f[] = {g.N, g.C, g.K, g.H, g.W, g.FH, g.FW, g.S, g.pt, g.pb, g.pl, g.pr, relu ? 1 : 0, accumulate ? 1 : 0, nchw_in ? 1 : 0, (int)ctx->wait_iters};
-        const void *ptrs[] = {in, w, bias, out};
+        const int f[] = {g.N, g.C, g.K, g.H, g.W, g.FH, g.FW, g.S, g.pt, g.pb, g.pl, g.pr, nchw_in ? 1 : 0};
         key.append(reinterpret_cast<const char *>(f), sizeof(f));
-        key.append(reinterpret_cast<const char *>(ptrs), sizeof(ptrs));
     }
     if (!ctx->thin_cache) ctx->thin_cache = new ThinCache();
     ThinCache &cache = *static_cast<ThinCache *>(ctx->thin_cache);
-    {
-        auto it = cache.find(key);
-        if (it != cache.end()) {
-            ThinLaunch &L = it->second;
-            L.a.late = ctx->dependent == 2;
-            launch_kernel(ctx, L.kern, L.grid, dim3(kThinThreads), L.smem, st, L.map, L.a);
-            return check_launch(ctx);
+    auto it = cache.find(key);
+    if (it == cache.end()) {
+        ThinPlan made{};
+        if (int s = make_plan(ctx, g, nchw_in, made)) return s;
+        if (cache.size() >= 512) cache.clear();
+        it = cache.emplace(std::move(key), std::move(made)).first;
+    }
+    ThinPlan &p = it->second;
+    const CUtensorMap *map;
+    static const CUtensorMap none{};
+    if (nchw_in) {
+        map = &none;
+    } else {
+        auto m = p.maps.find(in);
+        if (m == p.maps.end()) {
+            cuuint64_t dims[5] = {32, (cuuint64_t)g.W, (cuuint64_t)g.H, 1, (cuuint64_t)g.N};
+            cuuint64_t strides[4] = {128, (cuuint64_t)g.W * 128, (cuuint64_t)g.H * g.W * 128, (cuuint64_t)g.H * g.W * 128};
+            cuuint32_t box[5] = {4, (cuuint32_t)p.a.pitch, (cuuint32_t)p.a.rows, 1, (cuuint32_t)p.a.nb}, es[5] = {1, 1, 1, 1, 1};
+            CUtensorMap made;
+            CUresult r = reinterpret_cast<sm100::EncodeTiledFn>(ctx->encode_tiled)(&made, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<float *>(in), dims, strides, box, es,
+                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+            if (r != CUDA_SUCCESS) { ctx->last_cuda = (int)r; return SMALL_ERR_CUDA; }
+            if (p.maps.size() >= 64) p.maps.clear();
+            m = p.maps.emplace(in, made).first;
         }
+        map = &m->second;
     }
-    ThinLaunch made{};
-    ThinArgs &a = made.a;
-    a.late = ctx->dependent == 2;
-    a.in = in; a.w = w; a.bias = bias; a.out = out; a.status = ctx->dev_status; a.wait_iters = ctx->wait_iters;
-    a.N = g.N; a.K = g.K; a.KB = g.KB; a.H = g.H; a.W = g.W; a.OH = g.OH; a.OW = g.OW; a.pt = g.pt; a.pl = g.pl;
-    a.relu = relu; a.accumulate = accumulate; a.nchw = nchw_in;
-    a.tma = !nchw_in && thin_pitch(g) <= 256;
-    const int pix = thin_pix(g), seg2 = ((pix - 1) * g.S + g.FW + 1) / 2;
-    const int lanes = thin_lanes(g.K);
-    a.groups = ceil_div(g.OW, pix);
-    a.kgroups = ceil_div(g.KB, 2);
-    a.pitch = thin_pitch(g);
-    const ThinKernel kern = pick_thin(g, pix, lanes);
-    if (!kern) return SMALL_ERR_UNSUPPORTED;
-    // The tile: whole rows of an image, several images where planes are small.  Estimated cycles of an SM: its tiles in rounds of as many
-    // blocks as it holds; a warp alone issues every third or fourth cycle (a window row's reads, then chains of FMAs), more share the
-    // scheduler (FMA pairs take two slots).
-    const int pieces = 32 / lanes;
-    auto pixels = [&](int nb, int th) { return (size_t)nb * ((th - 1) * g.S + g.FH) * a.pitch; };
-    auto bytes = [&](int nb, int th) { return pixels(nb, th) * (16 + 8 * g.C); };
-    const size_t budget = (bytes(1, 1) > 44 * 1024 ? 240 : 44) * 1024;      // (an output row of one image fits: conv_thin_supported)
-    const double per_piece = g.C * g.FH * (seg2 + 2.0 * g.FW * pix) + 8.0 * pix;
-    int by_regs = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&by_regs, kern, kThinThreads, 0) != cudaSuccess || by_regs < 1) by_regs = 1;
-    double best = 0.0;
-    for (int bands = 1; bands <= g.OH; ++bands) {
-        const int th = ceil_div(g.OH, bands);
-        if (ceil_div(g.OH, th) != bands || (th < 4 && bands > 1 && best > 0.0)) continue;
-        for (int nb = 1; nb <= (bands == 1 ? (g.N < 16 ? g.N : 16) : 1) && bytes(nb, th) <= budget; ++nb) {
-            if (a.tma && (th - 1) * g.S + g.FH > 256) continue;
-            const long long tiles = (long long)ceil_div(g.N, nb) * bands * a.kgroups, on_sm = (tiles + ctx->sm_count - 1) / ctx->sm_count;
-            long long held = (long long)(ctx->max_smem_optin / (bytes(nb, th) + 1024));
-            if (held > by_regs) held = by_regs;
-            if (held < 1) held = 1;
-            if (held > on_sm) held = on_sm;
-            const double work = ceil_div(nb * th * a.groups, 4 * pieces) * per_piece + pixels(nb, th) * (g.C + 2) * 0.1, alone = work * 3.3 + 600.0;
-            const double cost = (double)((on_sm + held - 1) / held) * (held * work > alone ? held * work : alone);
-            if (best == 0.0 || cost < best) { best = cost; a.TH = th; a.nb = nb; a.bands = bands; }
-        }
-    }
-    if (best == 0.0) return SMALL_ERR_UNSUPPORTED;
-    a.rows = (a.TH - 1) * g.S + g.FH;
-    a.plane = a.rows * a.pitch;
-    a.raw_bytes = (uint32_t)(pixels(a.nb, a.TH) * 16);
-    auto multiplier = [](int d) { return d <= 1 ? 0u : (uint32_t)((1ull << 32) / (unsigned)d) + 1u; };
-    a.by_pitch = multiplier(a.pitch); a.by_rows = multiplier(a.rows); a.by_groups = multiplier(a.groups);
-    a.tiles = (long long)ceil_div(g.N, a.nb) * a.bands;
-    const size_t smem = bytes(a.nb, a.TH);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->max_smem_optin - 1024);
-        if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SMALL_ERR_CUDA; }
-    }
-    // blocks that run at once: the grid is that many (or fewer), each walking the tile list
-    int per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThinThreads, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
-    long long gx_ll = (long long)per_sm * ctx->sm_count / a.kgroups;
-    if (gx_ll < 1) gx_ll = 1;
-    made.grid = dim3((unsigned)(a.tiles < gx_ll ? a.tiles : gx_ll), (unsigned)a.kgroups);
-    made.kern = kern;
-    made.smem = smem;
-    if (a.tma) {
-        cuuint64_t dims[5] = {32, (cuuint64_t)g.W, (cuuint64_t)g.H, 1, (cuuint64_t)g.N};
-        cuuint64_t strides[4] = {128, (cuuint64_t)g.W * 128, (cuuint64_t)g.H * g.W * 128, (cuuint64_t)g.H * g.W * 128};
-        cuuint32_t box[5] = {4, (cuuint32_t)a.pitch, (cuuint32_t)a.rows, 1, (cuuint32_t)a.nb}, es[5] = {1, 1, 1, 1, 1};
-        CUresult r = reinterpret_cast<sm100::EncodeTiledFn>(ctx->encode_tiled)(&made.map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<float *>(in), dims, strides, box, es,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) { ctx->last_cuda = (int)r; return SMALL_ERR_CUDA; }
-    }
-    if (cache.size() >= 4096) cache.clear();
-    const ThinLaunch &L = cache[key] = made;
-    launch_kernel(ctx, L.kern, L.grid, dim3(kThinThreads), L.smem, st, L.map, L.a);
+    ThinArgs a = p.a;
+    a.in = in; a.w = w; a.bias = bias; a.out = out; a.relu = relu; a.accumulate = accumulate;
+    a.wait_iters = ctx->wait_iters; a.late = ctx->dependent == 2;
+    launch_kernel(ctx, p.kern, p.grid, dim3(kThinThreads), p.smem, st, *map, a);
     return check_launch(ctx);
 }
 

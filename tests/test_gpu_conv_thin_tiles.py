@@ -47,3 +47,28 @@ def test_nchw_and_blocked_inputs_give_the_same_bits(name, batch):
     gnet.run_host(torch.from_numpy(x).pin_memory(), host)
     torch.cuda.synchronize()
     np.testing.assert_array_equal(host.numpy(), from_blk(gnet.run(to_blk(x)), batch, *gnet.out_shape))
+
+
+WIDE = [  # planes whose rows are cut into column bands: one channel to four, every window; last bands of one column group and of a few columns
+    (1, 1, 16, 8, 3300, 3, 3, 1, P1), (1, 1, 16, 8, 1680, 3, 3, 1, P1), (1, 3, 16, 1000, 1000, 3, 3, 1, P1), (1, 3, 9, 672, 672, 3, 3, 2, P1),
+    (2, 4, 70, 19, 720, 3, 3, 2, (0, 1, 0, 1)), (1, 2, 24, 840, 840, 3, 3, 2, P1), (1, 1, 40, 600, 1000, 10, 4, 2, (4, 5, 1, 1)), (1, 4, 5, 448, 448, 3, 3, 2, P1),
+    (3, 3, 33, 5, 225, 3, 3, 1, (2, 0, 2, 0)), (1, 3, 64, 7, 265, 3, 3, 1, (0, 0, 0, 0)), (1, 4, 8, 3, 851, 3, 3, 1, (0, 0, 0, 0)),
+]
+
+
+@pytest.mark.parametrize("case", WIDE)
+def test_wide_planes_match_the_oracle(case):
+    """Rows too long for a tile of whole ones (a tile of one row was more than a block's shared memory for some of these widths)."""
+    test_tiles_match_the_oracle(case)
+
+
+@pytest.mark.parametrize("C,H,W,S", [(3, 30, 672, 2), (1, 9, 1680, 1), (4, 40, 300, 1)])
+def test_wide_planes_from_nchw_give_the_same_bits(C, H, W, S):
+    layers = [configs._conv("stem", "in", "a", C, 20, 3, S, P1, True), configs._conv("p", "a", "out", 20, 8, 1, 1, configs.P0, False)]
+    net = dict(name="wide", batch=2, input=(C, H, W), input_dist=("uniform", -1.0, 1.0), weight_dist="he_normal", layers=layers)
+    x = configs.make_input(net, 2)
+    gnet = Net(ctx(), net, configs.make_params(net), batch=2)
+    host = torch.full((2,) + tuple(gnet.out_shape), float("nan")).pin_memory()
+    gnet.run_host(torch.from_numpy(x).pin_memory(), host)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(host.numpy(), from_blk(gnet.run(to_blk(x)), 2, *gnet.out_shape))
