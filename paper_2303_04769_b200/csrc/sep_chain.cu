@@ -206,13 +206,14 @@ __device__ __forceinline__ void read_columns(const uint32_t t0, const uint32_t t
 
 // A pair's result: accumulators -> + bias, ReLU -> plane (or global memory behind the last pair: `out` is the image's tensor).
 // `sums`: the sums over the pixels instead, per filter, in four parts of 256.  The warps of a quarter of the tensor-memory lanes
-// share out the columns.
+// share out the columns.  ReLU is a maximum with 0, and without one the maximum is with NaN, which leaves numbers and NaNs as they are
+// (that with -infinity makes numbers of NaNs).  Pad filters are products of zeros, a NaN where a channel is infinite: with 0, they stay +0.
 template <bool X3>
 __device__ __forceinline__ void epilogue(const PairOp &o, const uint32_t tmem, const uint32_t plane, float *out, float *sums, const float *bias_s) {
     constexpr int G = 2, CW = 32;                         // warps of a quarter; columns read at a time
     const int lane = threadIdx.x & 31, warp = warp_index(), quarter = warp & 3, group = warp >> 2;
     const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
-    const float floor = o.relu ? 0.0f : -__int_as_float(0x7f800000);
+    const float floor = o.relu ? 0.0f : __int_as_float(0x7fffffff);
     const int px = o.px, rows = o.rows, out_stride = (int)o.out_stride, b_at = o.b_at;
     if (o.pix_m) {
         // lane = pixel, CW filters at a time
@@ -227,6 +228,9 @@ __device__ __forceinline__ void epilogue(const PairOp &o, const uint32_t tmem, c
                 v[4 * i] = fmaxf(v[4 * i] + b.x, floor); v[4 * i + 1] = fmaxf(v[4 * i + 1] + b.y, floor);
                 v[4 * i + 2] = fmaxf(v[4 * i + 2] + b.z, floor); v[4 * i + 3] = fmaxf(v[4 * i + 3] + b.w, floor);
             }
+            if (k + CW > o.K)
+#pragma unroll
+                for (int e = 0; e < CW; ++e) v[e] = k + e < o.K ? v[e] : 0.0f;
             if (sums) {
                 // over the warp's pixels: halves change places until a lane holds one filter's sum
 #pragma unroll
@@ -258,6 +262,7 @@ __device__ __forceinline__ void epilogue(const PairOp &o, const uint32_t tmem, c
         if (kb >= o.KB) continue;
         const uint32_t d = tmem + lanes + (uint32_t)mt * o.d_cols;
         const float b = bias_s[b_at + kb * 32 + lane];
+        const float least = kb * 32 + lane < o.K ? floor : 0.0f;
         const uint32_t blk = plane + (uint32_t)(kb * out_stride + lane * 4);
         float *line = out + (size_t)kb * px * 32 + lane;
         float s[4] = {0.f, 0.f, 0.f, 0.f};
@@ -267,7 +272,7 @@ __device__ __forceinline__ void epilogue(const PairOp &o, const uint32_t tmem, c
             if (X3 && o.wide) read_columns<true>(d + (uint32_t)p0, d + (uint32_t)(o.pxp + p0), v);
             else read_columns<false>(d + (uint32_t)p0, 0, v);
 #pragma unroll
-            for (int e = 0; e < CW; ++e) v[e] = fmaxf(v[e] + b, floor);
+            for (int e = 0; e < CW; ++e) v[e] = fmaxf(v[e] + b, least);
             const int left = p_to - p0;
             if (sums) {
 #pragma unroll

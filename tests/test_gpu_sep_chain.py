@@ -94,3 +94,23 @@ def test_a_result_that_is_read_again_stays():
     ref = nets.run_net(net, params, x)["out"]
     got = from_blk(Net(ctx(), net, params, batch=3, math="3xtf32").run(to_blk(x)), 3, *ref.shape[1:])
     assert rel_err(got, ref) <= TOL["3xtf32"]
+
+
+@pytest.mark.parametrize("head", [False, True])
+@pytest.mark.parametrize("math", ["tf32", "3xtf32"])
+@pytest.mark.parametrize("C,H,W,K", [(64, 25, 5, 64), (64, 25, 5, 40), (40, 6, 7, 70)])      # pixels on M, with pad filters; filters on M
+def test_values_without_a_number_pass_as_in_the_layers_one_by_one(C, H, W, K, math, head):
+    """Layers without ReLU hand a NaN and an infinity on, and pad filters stay zero beside them."""
+    net = run_of(C, H, W, [(K, 1, SAME, False, False)] * 3, 12 if head else None)
+    params, x = configs.make_params(net), configs.make_input(net, 4)
+    x[0, 3, 2, 1], x[2, C - 1, H - 1, 0] = float("nan"), float("inf")
+    shape, got = None, []
+    for kw in ({}, dict(fuse_dwpw=False)):
+        gnet = Net(ctx(), net, params, batch=4, math=math, **kw)
+        shape = (4,) + tuple(gnet.out_shape)
+        out = gnet.run(to_blk(x))
+        assert pad_lanes_are_zero(out, *shape)
+        got.append(torch.from_numpy(from_blk(out, *shape)))
+    run, layers = got
+    assert torch.equal(run.isnan(), layers.isnan()) and torch.equal(run.isinf(), layers.isinf())
+    assert not run[1].isnan().any() and run[0].isnan().any() and not run[2].isfinite().all()
