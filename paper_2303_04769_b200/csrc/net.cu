@@ -11,6 +11,7 @@ struct SlotPlan {
     std::vector<size_t> bytes;    // per slot
     std::vector<size_t> offset;   // per slot, 256-byte aligned
     size_t total = 0;
+    size_t in_bytes = 0, out_bytes = 0;      // of the network's input and output, as far as layers reach
 };
 
 static size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -47,7 +48,11 @@ static bool layer_out_shape(const small_layer &L, int N, int &oc, int &oh, int &
 static bool plan_slots(const small_layer *layers, int n_layers, int N, SlotPlan &plan) {
     if (!layers || n_layers < 1 || N < 1) return false;
     auto need = [&](int slot, size_t bytes) {
-        if (slot < 0) return slot == SMALL_SLOT_INPUT || slot == SMALL_SLOT_OUTPUT;
+        if (slot < 0) {
+            size_t &most = slot == SMALL_SLOT_INPUT ? plan.in_bytes : plan.out_bytes;
+            if (most < bytes) most = bytes;
+            return slot == SMALL_SLOT_INPUT || slot == SMALL_SLOT_OUTPUT;
+        }
         if (slot > 4096) return false;
         if ((size_t)slot >= plan.bytes.size()) plan.bytes.resize(slot + 1, 0);
         if (plan.bytes[slot] < bytes) plan.bytes[slot] = bytes;
@@ -212,6 +217,14 @@ static bool launches_beat_on_chip(const small_ctx *ctx, const small_layer *layer
     return us < (depthwise ? 4.5 : 9.0) * (n_layers - from);
 }
 
+// Do the network's input, its output and the slots lie apart?  Then tensors overlap only where they share a slot, which the forms of
+// several layers look at.  Where the caller's tensors meet - an output over the input, say, which is no longer read by then - the layers are
+// called one by one: each compares the addresses it is given.
+static bool tensors_apart(const SlotPlan &plan, const void *in, const void *out, const void *slots) {
+    return !ranges_overlap(in, plan.in_bytes, out, plan.out_bytes) && !ranges_overlap(in, plan.in_bytes, slots, plan.total) &&
+           !ranges_overlap(out, plan.out_bytes, slots, plan.total);
+}
+
 // Runs of layers are kept on chip as one kernel where every kind of fusion is on.
 static bool runs_allowed(const small_ctx *ctx) {
     const unsigned rest = SMALL_FUSE_CONVPOOL | SMALL_FUSE_FC_CHAIN | SMALL_FUSE_POOLFC;
@@ -331,7 +344,7 @@ static int run_layers(small_ctx *ctx, const small_layer *layers, int n_layers, i
     bool after_join = false;
     // a run of depthwise / 1x1 pairs (sep_chain.cu); without one, a run up to the end of the list (net_resident.cu)
     int chain = -1, chain_layers = 0, on_chip = -1;
-    const bool runs = runs_allowed(ctx);
+    const bool apart = tensors_apart(plan, in_blk, out_blk, workspace), runs = apart && runs_allowed(ctx);
     if (runs) {
         for (int i = from; i < n_layers && !chain_layers; ++i)
             if ((chain_layers = sep_chain_layers(ctx, layers, n_layers, i, N)) > 0) chain = i;
@@ -388,7 +401,7 @@ static int run_layers(small_ctx *ctx, const small_layer *layers, int n_layers, i
         }
         {
             int widths[13];
-            if (const int Lc = fc_chain_len(ctx, layers, n_layers, i, N, widths)) {
+            if (const int Lc = apart ? fc_chain_len(ctx, layers, n_layers, i, N, widths) : 0) {
                 const float *w[12], *b[12];
                 int relu[12];
                 for (int j = 0; j < Lc; ++j) { w[j] = layers[i + j].w_blk; b[j] = layers[i + j].bias; relu[j] = (layers[i + j].flags & SMALL_RELU) ? 1 : 0; }
@@ -424,7 +437,7 @@ static int run_layers(small_ctx *ctx, const small_layer *layers, int n_layers, i
         // shortcut) run side by side: the second one on the context's side stream, forked from and joined to the caller's
         // stream by events, so that a short layer hides behind a long one.  Both are ordinary launches, and so is the
         // layer behind the join.
-        if (ctx->branch_overlap && ctx->side_stream && i + 1 < n_layers && i + 1 != on_chip && i + 1 != chain && independent(L, layers[i + 1]) &&
+        if (apart && ctx->branch_overlap && ctx->side_stream && i + 1 < n_layers && i + 1 != on_chip && i + 1 != chain && independent(L, layers[i + 1]) &&
             !fused_pair(ctx, layers, n_layers, i + 1, N) && !joins(i + 1, sc_next, g_next)) {
             cudaStream_t main_st = static_cast<cudaStream_t>(stream), side = static_cast<cudaStream_t>(ctx->side_stream);
             cudaError_t e = cudaEventRecord(static_cast<cudaEvent_t>(ctx->ev_fork), main_st);

@@ -254,3 +254,44 @@ def test_depthwise_pairs_fuse_for_a_few_images_only():
         gnet = Net(ctx(), pair, pair_params, math=math)
         assert gnet.launches() == launches, (c, hw, math)
         assert rel_err(from_blk(gnet.run(to_blk(x)), 1, 64, hw, hw), nets.run_net(pair, pair_params, x)["out"]) <= TOL[math]
+
+
+@pytest.mark.parametrize("math", ["fp32", "tf32", "3xtf32"])
+@pytest.mark.parametrize("form", ["pairs", "pair", "chain"])
+def test_an_output_over_the_input_is_no_hazard(form, math):
+    """The input is read by the first layer alone, and the last one writes over it: layer by layer that is in order.  A form that reads
+    the one while it writes the other is not taken."""
+    if form == "chain":
+        layers = [configs._fc(f"f{i}", "in" if i == 0 else f"a{i}", "out" if i == 2 else f"a{i + 1}", 128, 128) for i in range(3)]
+        net = dict(name="over", batch=300, input=(128, 1, 1), input_dist=("uniform", -1.0, 1.0), weight_dist="he_normal", layers=layers)
+    else:
+        layers, n = [], 3 if form == "pairs" else 1
+        for i in range(n):
+            layers += [configs._dw(f"d{i}", "in" if i == 0 else f"p{i}", f"m{i}", 40, 1),
+                       configs._conv(f"c{i}", f"m{i}", "out" if i == n - 1 else f"p{i + 1}", 40, 40, 1, 1, configs.P0, True)]
+        net = dict(name="over", batch=600 if form == "pairs" else 5, input=(40, 9, 8), input_dist=("uniform", -1.0, 1.0), weight_dist="he_normal", layers=layers)
+    N = net["batch"]
+    params, x = configs.make_params(net), configs.make_input(net, N)
+    ref = nets.run_net(net, params, x)["out"]
+    gnet = Net(ctx(), net, params, math=math)
+    C, H, W = net["input"]
+    n_in, n_out = B.small_packed_elems(N, C, H, W), B.small_packed_elems(N, *ref.shape[1:])
+    # the same memory, and an output that begins inside the input: over images that a run of pairs reads in a second round
+    for shift in (0, n_in // N * (350 if form == "pairs" else 1)):
+        room = torch.empty(n_in + n_out, device="cuda")
+        room[:n_in] = to_blk(x)
+        out = room[shift:shift + n_out]
+        B.small_run_net(ctx(), gnet.layers, N, room[:n_in], out, gnet.workspace, gnet.ws_bytes)
+        assert rel_err(from_blk(out, *ref.shape), ref) <= TOL[math]
+
+
+def test_a_shortcut_onto_the_input_is_refused():
+    """Found by the layer that reads and writes the same memory, also where the shortcut and the layer behind it would be one launch."""
+    layers = [configs._conv("a", "in", "m", 16, 16, 3, 1, configs.P1, True), configs._conv("s", "in", "out", 16, 16, 1, 1, configs.P0, False),
+              configs._conv("b", "m", "out", 16, 16, 3, 1, configs.P1, True, accumulate=True)]
+    net = dict(name="over", batch=1, input=(16, 8, 8), input_dist=("uniform", -1.0, 1.0), weight_dist="he_normal", layers=layers)
+    for math in ("fp32", "3xtf32"):
+        gnet = Net(ctx(), net, configs.make_params(net), math=math)
+        blk = to_blk(configs.make_input(net, 1))
+        with pytest.raises(B.SmallError, match="OVERLAP|overlap"):
+            B.small_run_net(ctx(), gnet.layers, 1, blk, blk, gnet.workspace, gnet.ws_bytes)
