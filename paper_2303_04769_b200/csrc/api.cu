@@ -443,6 +443,8 @@ static int conv2d_path(small_ctx *ctx, const Geom &g, unsigned math, bool out_al
 
 namespace small {
 
+bool conv_in_fp32(small_ctx *ctx, const Geom &g, unsigned math) { return (conv2d_path(ctx, g, math, true) & (kSplit - 1)) < 3; }
+
 // Where the layer runs on one of the two kernels and its shortcut in the same arithmetic, on that kernel or, by a hair, another.
 bool joined_split(small_ctx *ctx, const Geom &sc, const Geom &g, unsigned math, bool out_aligned32) {
     const int a = conv2d_path(ctx, sc, math, out_aligned32) & (kSplit - 1), b = conv2d_path(ctx, g, math, out_aligned32) - kSplit;

@@ -205,6 +205,8 @@ int launch_conv_split(small_ctx *, const float *in, const float *w_hi, const flo
 double conv_split_fp32_us(const Geom &, int sms);          // the time expected, 0 where another kernel is preferred
 int launch_conv_split_fp32(small_ctx *, const float *in, const float *w, const float *bias, float *out, const Geom &,
                            bool relu, bool accumulate, cudaStream_t, const Shortcut * = nullptr);
+// whether a layer called on its own (with a 32-byte aligned output) computes in FP32 under this math mode (api.cu)
+bool conv_in_fp32(small_ctx *, const Geom &, unsigned math);
 // a shortcut and the layer that is added to it as one launch of those kernels: whether they run there, and the launch (api.cu)
 bool joined_split(small_ctx *, const Geom &shortcut, const Geom &, unsigned math, bool out_aligned32);
 int launch_joined(small_ctx *, Shortcut, const float *in, const float *w, const float *bias, float *out, const Geom &, bool relu, unsigned math, cudaStream_t);

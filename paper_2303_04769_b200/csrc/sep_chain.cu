@@ -609,8 +609,9 @@ bool plan_pair(const small_layer &A, const small_layer &Bn, int N, bool x3, int 
     return true;
 }
 
-// Structure of the list: does layer i start a pair of the run, reading slot `src` (any, where the run starts)?
-bool is_pair(const small_layer *layers, int n, int i, unsigned &math) {
+// Structure of the list: does layer i start a pair of the run, reading slot `src` (any, where the run starts)?  Not where the 1x1 layer
+// called on its own computes in FP32 (few products per pixel): its results stay FP32's.
+bool is_pair(small_ctx *ctx, const small_layer *layers, int n, int i, int N, unsigned &math) {
     if (i + 1 >= n) return false;
     const small_layer &A = layers[i], &Bn = layers[i + 1];
     if (A.op != SMALL_OP_DWCONV || Bn.op != SMALL_OP_CONV) return false;
@@ -619,20 +620,22 @@ bool is_pair(const small_layer *layers, int n, int i, unsigned &math) {
     if (math == ~0u) math = m;
     if (m != math || A.FH != 3 || A.FW != 3 || A.stride < 1 || A.stride > 2) return false;
     if (Bn.FH != 1 || Bn.FW != 1 || Bn.stride != 1 || (Bn.pad_t | Bn.pad_b | Bn.pad_l | Bn.pad_r) || (Bn.flags & SMALL_ACCUMULATE)) return false;
-    Geom g;
-    if (make_geom(g, 1, A.C, A.C, A.H, A.W, 3, 3, A.stride, A.pad_t, A.pad_b, A.pad_l, A.pad_r)) return false;
-    return A.dst >= 0 && Bn.src == A.dst && Bn.dst != A.dst && Bn.C == A.C && Bn.H == g.OH && Bn.W == g.OW && Bn.K >= 1 &&
-           slot_dead_after(layers, n, i + 2, A.dst);
+    Geom g, gp;
+    if (make_geom(g, N, A.C, A.C, A.H, A.W, 3, 3, A.stride, A.pad_t, A.pad_b, A.pad_l, A.pad_r)) return false;
+    return A.dst >= 0 && Bn.src == A.dst && Bn.dst != A.dst && Bn.C == A.C && Bn.H == g.OH && Bn.W == g.OW &&
+           make_geom(gp, N, A.C, Bn.K, g.OH, g.OW, 1, 1, 1, 0, 0, 0, 0) == SMALL_OK && slot_dead_after(layers, n, i + 2, A.dst) && !conv_in_fp32(ctx, gp, m);
 }
 
 // The longest run at layer i (pairs = 0: none).  Results that fit are in p.
-void plan_run(const small_layer *layers, int n, int i, int N, size_t max_smem, int sms, Plan &p) {
+void plan_run(small_ctx *ctx, const small_layer *layers, int n, int i, int N, Plan &p) {
+    const size_t max_smem = ctx->max_smem_optin;
+    const int sms = ctx->sm_count;
     p = Plan{};
     unsigned math = ~0u;
     Args &a = p.a;
     std::vector<int> ends;                               // structure: pairs that could follow one another
     int at = i;
-    while ((int)ends.size() < kMaxPairs && is_pair(layers, n, at, math)) {
+    while ((int)ends.size() < kMaxPairs && is_pair(ctx, layers, n, at, N, math)) {
         if (at > i) {                                    // reads what the pair before it wrote, as its only reader
             const small_layer &P = layers[at - 1], &A = layers[at];
             if (A.src != P.dst || P.dst < 0 || A.C != P.K || A.H != P.H || A.W != P.W || !slot_dead_after(layers, n, at + 1, P.dst)) break;
@@ -755,7 +758,7 @@ Entry &entry_of(small_ctx *ctx, const small_layer *layers, int n, int i, int N) 
     memcpy(e.key.data(), head, sizeof(head));
     memcpy(e.key.data() + sizeof(head), layers + i, lb);
     Plan p;
-    plan_run(layers, n, i, N, ctx->max_smem_optin, ctx->sm_count, p);
+    plan_run(ctx, layers, n, i, N, p);
     if (p.layers) e.p.reset(new Plan(p));
     if (s.size() >= 512) s.clear();
     return s.emplace(words, std::move(e))->second;

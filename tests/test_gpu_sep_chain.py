@@ -114,3 +114,15 @@ def test_values_without_a_number_pass_as_in_the_layers_one_by_one(C, H, W, K, ma
     run, layers = got
     assert torch.equal(run.isnan(), layers.isnan()) and torch.equal(run.isinf(), layers.isinf())
     assert not run[1].isnan().any() and run[0].isnan().any() and not run[2].isfinite().all()
+
+
+@pytest.mark.parametrize("math", ["tf32", "3xtf32"])
+@pytest.mark.parametrize("C,K", [(64, 8), (40, 12), (100, 5)])
+def test_layers_computed_in_fp32_are_no_part_of_a_run(C, K, math):
+    """A 1x1 layer of so few products per pixel that it computes in FP32 whatever the mode keeps its bits: it ends a run."""
+    batch = 600
+    net = run_of(C, 8, 8, [(C, 1, SAME, True, True), (K, 1, SAME, True, True), (C, 1, SAME, True, True)])
+    assert B.small_conv2d_path(ctx(), batch, C, K, 8, 8, 1, 1, 1, NONE, B.MATH[math]) in (1, 2)
+    params, blk = configs.make_params(net), to_blk(configs.make_input(net, batch))
+    run, apart = (Net(ctx(), net, params, batch=batch, math=math, **kw).run(blk).clone() for kw in ({}, dict(fuse_dwpw=False)))
+    assert torch.equal(run, apart)
