@@ -95,8 +95,9 @@ int small_out_size(int I, int F, int stride, int pad_before, int pad_after);
 const char *small_strerror(int status);
 /* Last cudaError_t / CUresult seen by this context (0 if none). */
 int small_last_cuda_error(small_ctx *ctx);
-/* Layer overlap (on by default; `on` = 0 switches it off).  When on, layers - called on their own or by small_run_net - are
- * launched with programmatic stream serialisation: their thread blocks may become resident and set up shared memory,
+/* Layer overlap (on by default; `on` = 0 switches it off).  When on, layers - called on their own or by small_run_net; except the
+ * general FP32 kernel, scale-shift, upsampling, the uint8 ReLU and generic depthwise kernels, full reductions called on their own and a run
+ * kept on chip that is a call's first kernel - are launched with programmatic stream serialisation: their thread blocks may become resident and set up shared memory,
  * barriers and tensor memory while the kernel in front of them in the stream is still draining, and they wait on the
  * device until that kernel has completed before they read or write a tensor.  (Filters and biases are read earlier only
  * behind a layer of the same network.)  Results are the same either way.  The paper has no counterpart. */
@@ -128,10 +129,14 @@ int small_set_conv_path(small_ctx *ctx, int path);
 /* Which kernel small_conv2d runs for this shape and math mode (with a 32-byte aligned output) under the context's
  * path setting: 0 = few-input-channel kernel (network stems), 1 = register-tiled FP32 kernel, 2 = general FP32 kernel,
  * 3 = block-level tensor-core kernel (tcgen05), 4 = warp-level tensor-core kernel (few channels and filters);
- * -1 for invalid arguments.  Under AUTO, layers of 3 and 4 with so few output pixels that their tiles would leave most of the
- * GPU idle run as warp-level MMAs with the reduction split over warps; the number reported stays the one of the shape's family. */
+ * -1 for invalid arguments.  The number is that of the shape's family: under AUTO, layers of 1 to 4 with so few output pixels that
+ * tiles with a whole reduction would leave most of the GPU idle run with the reduction split over warps (small_conv2d_split). */
 int small_conv2d_path(small_ctx *ctx, int N, int C, int K, int H, int W, int FH, int FW, int stride,
                       int pad_t, int pad_b, int pad_l, int pad_r, unsigned math);
+/* 1 where small_conv2d runs this shape with its reduction split over warps instead of the kernel small_conv2d_path names: families 1 and
+ * 2 in FP32 arithmetic, 3 and 4 as warp-level MMAs; 0 otherwise, -1 for invalid arguments. */
+int small_conv2d_split(small_ctx *ctx, int N, int C, int K, int H, int W, int FH, int FW, int stride,
+                       int pad_t, int pad_b, int pad_l, int pad_r, unsigned math);
 /* Synchronises `stream`, then reads and clears the device status word: *status is SMALL_OK or
  * SMALL_ERR_TIMEOUT (a tensor-core pipeline wait gave up; the affected outputs are undefined). */
 int small_device_status(small_ctx *ctx, int *status, void *stream);
@@ -391,16 +396,31 @@ typedef struct small_layer {
  * full reductions whose inner widths are at most 128 under a tensor-core math mode (SMALL_FUSE_FC_CHAIN, see small_fc_chain), and
  * a global average pool with the full reduction behind it, in every math mode (SMALL_FUSE_POOLFC, see small_gap_fc).  The skipped
  * intermediate tensors are then not written.  Default: all four (without DWPW_ALWAYS); 0 runs every layer on its own.
- * With every kind on, a whole run of convolutions and depthwise 3x3 layers that ends the list in a global average pool and a full
- * reduction may run as one kernel that keeps each image's activations on chip (small batches; where it was measured to pay), and so
- * may, at any batch and place of the list, a run of three or more depthwise 3x3 -> 1x1 pairs under a tensor-core math mode.
+ * With every kind on (DWPW or DWPW_ALWAYS, and the other three), the convolution path on AUTO and the caller's tensors apart from one
+ * another, whole runs may be one kernel where it was measured to pay: convolutions and depthwise 3x3 layers that end the list in a
+ * global average pool and a full reduction, each image's activations kept on chip (small batches); three or more depthwise 3x3 -> 1x1
+ * pairs under a tensor-core math mode, at any batch and place of the list.  So may, at few output pixels, a depthwise 3x3 -> 1x1 pair in
+ * FP32, and a 1x1 shortcut with the convolution that is added to its result.  small_net_forms tells which.
  * Results stay within each math mode's tolerance either way. */
 enum { SMALL_FUSE_DWPW = 1u, SMALL_FUSE_DWPW_ALWAYS = 2u, SMALL_FUSE_CONVPOOL = 4u, SMALL_FUSE_FC_CHAIN = 8u,
        SMALL_FUSE_POOLFC = 16u };   /* a global average pool and the full reduction behind it (small_gap_fc) */
 int small_set_net_fusion(small_ctx *ctx, unsigned mask);
-/* Number of kernel launches small_run_net makes for these layers at batch N under the context's fusion setting (one per
- * layer or fused pair; fewer are made where a run of layers is kept on chip as one kernel); -1 for invalid arguments. */
+/* Number of kernels these layers are at batch N under the context's fusion setting, one per layer, fused pair or chain of full
+ * reductions; -1 for invalid arguments.  Runs of layers kept on chip, FP32 pairs and joined shortcuts are counted layer by layer here:
+ * small_net_forms knows them. */
 int small_net_launches(small_ctx *ctx, const small_layer *layers, int n_layers, int N);
+/* How small_run_net takes the layers of the list at batch N under the context's settings, for tensors that lie apart from one another and
+ * an output aligned to 32 bytes: forms (HOST, n_layers entries, may be null) receives each layer's form.  Returns the number of kernel
+ * launches, -1 for invalid arguments.  Decides as small_run_net does and launches nothing.  The paper has no counterpart. */
+enum { SMALL_FORM_LAYER = 0,         /* on its own */
+       SMALL_FORM_FUSED_PAIR = 1,    /* with its neighbour as a fused layer: depthwise + 1x1, convolution + max pool, average pool + full reduction */
+       SMALL_FORM_FC_CHAIN = 2,      /* a chain of full reductions as one kernel */
+       SMALL_FORM_SIDE_BY_SIDE = 3,  /* a launch of its own, beside its neighbour on another stream */
+       SMALL_FORM_PAIR_RUN = 4,      /* a run of depthwise 3x3 -> 1x1 pairs as one kernel (tensor-core modes) */
+       SMALL_FORM_ON_CHIP = 5,       /* a run up to the end of the list as one kernel that keeps the activations on chip */
+       SMALL_FORM_PAIR_FP32 = 6,     /* a depthwise 3x3 and a 1x1 layer of few pixels as one launch (FP32) */
+       SMALL_FORM_JOINED = 7 };      /* a 1x1 shortcut and the layer of few pixels that is added to its result as one launch */
+int small_net_forms(small_ctx *ctx, const small_layer *layers, int n_layers, int N, int *forms);
 /* Bytes of workspace for `layers` at batch N: slot s is as large as the largest tensor any layer reads
  * from or writes to it, rounded up to 256 bytes; slots are laid out back to back.  0 on invalid input. */
 size_t small_net_workspace_bytes(const small_layer *layers, int n_layers, int N);

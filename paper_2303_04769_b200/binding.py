@@ -25,11 +25,11 @@ MATH = {"fp32": MATH_FP32, "tf32": MATH_TF32, "3xtf32": MATH_3XTF32}
 
 EXPORTS = [
     "small_init", "small_shutdown", "small_channel_block", "small_packed_elems", "small_out_size", "small_strerror",
-    "small_last_cuda_error", "small_set_layer_overlap", "small_set_conv_path", "small_set_branch_overlap", "small_conv2d_path", "small_set_wait_limit", "small_set_fc_chain_tile", "small_selftest_wait_timeout", "small_device_status", "small_measure_tf32_peak", "small_pack", "small_unpack", "small_conv_weight_elems",
+    "small_last_cuda_error", "small_set_layer_overlap", "small_set_conv_path", "small_set_branch_overlap", "small_conv2d_path", "small_conv2d_split", "small_set_wait_limit", "small_set_fc_chain_tile", "small_selftest_wait_timeout", "small_device_status", "small_measure_tf32_peak", "small_pack", "small_unpack", "small_conv_weight_elems",
     "small_pack_conv_weights", "small_group_count", "small_group_conv_weight_elems", "small_pack_group_conv_weights",
     "small_group_conv2d", "small_dwpw_conv2d", "small_dwpw_fused", "small_conv_maxpool2d", "small_conv_maxpool_fused", "small_dw_weight_elems", "small_pack_dw_weights", "small_fc_weight_elems",
     "small_pack_fc_weights", "small_fc_uses_tensor_cores", "small_fc_chain", "small_fc_chain_fused", "small_conv2d", "small_conv2d_uses_tensor_cores", "small_dwconv2d", "small_pool2d",
-    "small_relu", "small_scale_shift", "small_upsample_nearest", "small_add", "small_fc", "small_gap_fc", "small_gap_fc_fused", "small_net_workspace_bytes", "small_run_net", "small_set_net_fusion", "small_net_launches",
+    "small_relu", "small_scale_shift", "small_upsample_nearest", "small_add", "small_fc", "small_gap_fc", "small_gap_fc_fused", "small_net_workspace_bytes", "small_run_net", "small_set_net_fusion", "small_net_launches", "small_net_forms",
     "small_net_host_staging_bytes", "small_run_net_host", "small_static_workspace_bytes", "small_run_net_static",
     "small_q_packed_bytes", "small_q_pack", "small_q_unpack", "small_q_conv_weight_bytes", "small_q_pack_conv_weights", "small_q_conv2d",
     "small_q_dw_weight_bytes", "small_q_pack_dw_weights", "small_q_dwconv2d", "small_q_maxpool2d", "small_q_relu",
@@ -81,6 +81,7 @@ def lib():
     L.small_set_fc_chain_tile.argtypes = [P, I]
     L.small_selftest_wait_timeout.argtypes = [P, P]
     L.small_conv2d_path.argtypes = [P] + [I] * 12 + [U]
+    L.small_conv2d_split.argtypes = [P] + [I] * 12 + [U]
     L.small_pack.argtypes = [P, P, P, I, I, I, I, P]
     L.small_unpack.argtypes = [P, P, P, I, I, I, I, P]
     L.small_conv_weight_elems.argtypes = [I, I, I, I, U]
@@ -120,6 +121,7 @@ def lib():
     L.small_run_net.argtypes = [P, ctypes.POINTER(small_layer), I, I, P, P, P, Z, P]
     L.small_set_net_fusion.argtypes = [P, U]
     L.small_net_launches.argtypes = [P, ctypes.POINTER(small_layer), I, I]
+    L.small_net_forms.argtypes = [P, ctypes.POINTER(small_layer), I, I, ctypes.POINTER(I)]
     L.small_net_host_staging_bytes.argtypes = [I] * 7
     L.small_net_host_staging_bytes.restype = Z
     L.small_run_net_host.argtypes = [P, ctypes.POINTER(small_layer), I, I, P, I, I, I, P, I, I, I, P, Z, P]
@@ -241,6 +243,11 @@ def small_selftest_wait_timeout(ctx, stream=None):
 def small_conv2d_path(ctx, N, C, K, H, W, FH, FW, stride, pad, math):
     pt, pb, pl, pr = pad
     return int(lib().small_conv2d_path(ctx, N, C, K, H, W, FH, FW, stride, pt, pb, pl, pr, math))
+
+
+def small_conv2d_split(ctx, N, C, K, H, W, FH, FW, stride, pad, math):
+    pt, pb, pl, pr = pad
+    return int(lib().small_conv2d_split(ctx, N, C, K, H, W, FH, FW, stride, pt, pb, pl, pr, math))
 
 
 def small_device_status(ctx, stream=None):
@@ -394,6 +401,16 @@ def small_set_net_fusion(ctx, mask):
 
 def small_net_launches(ctx, layers, N):
     return int(lib().small_net_launches(ctx, layers, len(layers), N))
+
+
+FORMS = ("layer", "fused_pair", "fc_chain", "side_by_side", "pair_run", "on_chip", "pair_fp32", "joined")
+
+
+def small_net_forms(ctx, layers, N):
+    """Each layer's form (a name of FORMS) and the number of kernel launches."""
+    forms = (ctypes.c_int * len(layers))()
+    launches = int(lib().small_net_forms(ctx, layers, len(layers), N, forms))
+    return [FORMS[f] for f in forms], launches
 
 
 def small_net_workspace_bytes(layers, N):

@@ -476,6 +476,13 @@ SMALL_API int small_conv2d_path(small_ctx *ctx, int N, int C, int K, int H, int 
     return conv2d_path(ctx, g, math, true) & (kSplit - 1);
 }
 
+SMALL_API int small_conv2d_split(small_ctx *ctx, int N, int C, int K, int H, int W, int FH, int FW, int stride,
+                                 int pt, int pb, int pl, int pr, unsigned math) {
+    Geom g;
+    if (!ctx || !math_valid(math) || make_geom(g, N, C, K, H, W, FH, FW, stride, pt, pb, pl, pr) != SMALL_OK) return -1;
+    return conv2d_path(ctx, g, math, true) >= kSplit ? 1 : 0;
+}
+
 SMALL_API int small_conv2d(small_ctx *ctx, const float *in, const float *w, const float *bias, float *out,
                            int N, int C, int K, int H, int W, int FH, int FW, int stride,
                            int pt, int pb, int pl, int pr, unsigned flags, void *stream) {

@@ -30,7 +30,7 @@ struct small_ctx {
     void *encode_tiled;      // cuTensorMapEncodeTiled, resolved through the runtime
     int sm_count;
     size_t max_smem_optin;
-    int overlap;             // small_run_net launches every layer after the first as a dependent launch (see launch_kernel)
+    int overlap;             // layers are dependent launches, called on their own or by small_run_net (see launch_kernel)
     int dependent;           // how the next layer is launched: 0 the ordinary way, 1 and 2 as a dependent launch (see launch_kernel)
     int in_net;              // small_run_net is issuing layers: it sets `dependent`
     unsigned wait_iters;     // limit (polls) of every bounded device-side wait; small_set_wait_limit
@@ -91,8 +91,9 @@ static inline int check_launch(small_ctx *ctx) {
 // both instructions do nothing.  Chains stay ordered: a kernel cannot complete before its own grid_dep_sync()
 // returns, so completion of kernel i implies completion of every kernel before it.
 // What a layer may do in front of grid_dep_sync() depends on the kernel before it.  Behind a layer of the same network
-// (ctx->dependent = 1) it may read its filters and biases: that layer does not write them, and has seen to it that everything
-// older is finished (its own trigger comes behind its wait).  Behind any other kernel of the stream (2: a call of its own, a
+// (ctx->dependent = 1) it may read its filters and biases: no layer writes them, and everything older than the network is finished, since
+// a network's first kernel triggers behind its wait and no later one starts before that trigger.  (Later ones may trigger first:
+// fc_chain.cu does.)  Behind any other kernel of the stream (2: a call of its own, a
 // network's first layer) it reads nothing: the kernel in front may be what writes the filters.  Kernels that read constants early
 // take that as `late` and wait first.
 #ifdef __CUDACC__

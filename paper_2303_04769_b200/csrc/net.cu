@@ -231,6 +231,57 @@ static bool runs_allowed(const small_ctx *ctx) {
     return (ctx->net_fusion & rest) == rest && (ctx->net_fusion & (SMALL_FUSE_DWPW | SMALL_FUSE_DWPW_ALWAYS)) && ctx->conv_path == SMALL_CONV_PATH_AUTO;
 }
 
+// How the runner takes the layers of a list, decided from the list, the batch, the context's settings and whether the caller's tensors lie
+// apart (`apart`) and the output is 32-byte aligned (`out32`; slots are).
+struct Forms {
+    bool apart, out32, runs;
+    int chain = -1, chain_layers = 0, on_chip = -1;      // a run of depthwise / 1x1 pairs (sep_chain.cu); without one, a run up to the end of the list (net_resident.cu)
+    Forms(small_ctx *ctx, const small_layer *layers, int n_layers, int from, int N, bool apart, bool out32) : apart(apart), out32(out32), runs(apart && runs_allowed(ctx)) {
+        if (!runs) return;
+        for (int i = from; i < n_layers && !chain_layers; ++i)
+            if ((chain_layers = sep_chain_layers(ctx, layers, n_layers, i, N)) > 0) chain = i;
+        if (!chain_layers) on_chip = resident_from(ctx, layers, n_layers, from, N);
+        if (on_chip >= 0 && (layers[n_layers - 1].flags & SMALL_MATH_MASK) == SMALL_MATH_FP32 && launches_beat_on_chip(ctx, layers, n_layers, on_chip, N)) on_chip = -1;
+    }
+    bool aligned(int slot) const { return slot >= 0 || out32; }
+    // a shortcut and the layer that is added to it, where both are split over warps, as one launch
+    bool joins(small_ctx *ctx, const small_layer *layers, int n_layers, int i, int N, Geom &sc, Geom &g) const {
+        return runs && i + 1 != chain && i + 1 != on_chip && shortcut_pair(layers, n_layers, i, N, sc, g) &&
+               joined_split(ctx, sc, g, layers[i].flags & SMALL_MATH_MASK, aligned(layers[i].dst));
+    }
+};
+
+struct Step {
+    int form, layers;            // SMALL_FORM_*, layers covered
+    Geom a, b;                   // of a pair in FP32, or a shortcut and the layer it joins
+    int widths[13];              // of a chain of full reductions
+    int fused;                   // of a fused pair (see fused_pair)
+};
+
+static void step_at(small_ctx *ctx, const small_layer *layers, int n_layers, int i, int N, const Forms &f, Step &s) {
+    s.layers = 2;
+    if (i == f.chain) { s.form = SMALL_FORM_PAIR_RUN; s.layers = f.chain_layers; return; }
+    if (i == f.on_chip) { s.form = SMALL_FORM_ON_CHIP; s.layers = n_layers - i; return; }
+    s.form = SMALL_FORM_PAIR_FP32;
+    if (f.runs && f.chain < 0 && f.on_chip < 0 && split_pair(ctx, layers, n_layers, i, N, s.a, s.b) > 0.0) return;
+    s.form = SMALL_FORM_JOINED;
+    if (f.joins(ctx, layers, n_layers, i, N, s.a, s.b)) return;
+    s.form = SMALL_FORM_FC_CHAIN;
+    if (const int L = f.apart ? fc_chain_len(ctx, layers, n_layers, i, N, s.widths) : 0)
+        if (f.aligned(layers[i + L - 1].dst)) { s.layers = L; return; }
+    s.form = SMALL_FORM_FUSED_PAIR;
+    if ((s.fused = i + 1 == f.on_chip || i + 1 == f.chain ? 0 : fused_pair(ctx, layers, n_layers, i, N))) return;
+    // Two neighbouring layers that touch no common tensor except as readers (a residual stage's convolution and its
+    // shortcut) run side by side.
+    s.form = SMALL_FORM_SIDE_BY_SIDE;
+    Geom sc, g;
+    if (f.apart && ctx->branch_overlap && ctx->side_stream && i + 1 < n_layers && i + 1 != f.on_chip && i + 1 != f.chain && independent(layers[i], layers[i + 1]) &&
+        !fused_pair(ctx, layers, n_layers, i + 1, N) && !f.joins(ctx, layers, n_layers, i + 1, N, sc, g))
+        return;
+    s.form = SMALL_FORM_LAYER;
+    s.layers = 1;
+}
+
 }  // namespace small
 
 using namespace small;
@@ -249,6 +300,20 @@ SMALL_API int small_net_launches(small_ctx *ctx, const small_layer *layers, int 
         int widths[13];
         if (const int L = fc_chain_len(ctx, layers, n_layers, i, N, widths)) i += L - 1;
         else if (fused_pair(ctx, layers, n_layers, i, N)) ++i;
+    }
+    return launches;
+}
+
+SMALL_API int small_net_forms(small_ctx *ctx, const small_layer *layers, int n_layers, int N, int *forms) {
+    SlotPlan plan;
+    if (!ctx || !plan_slots(layers, n_layers, N, plan)) return -1;
+    const Forms f(ctx, layers, n_layers, 0, N, true, true);
+    int launches = 0;
+    Step step;
+    for (int i = 0; i < n_layers; i += step.layers) {
+        step_at(ctx, layers, n_layers, i, N, f, step);
+        launches += step.form == SMALL_FORM_SIDE_BY_SIDE ? 2 : 1;
+        for (int j = i; forms && j < i + step.layers; ++j) forms[j] = step.form;
     }
     return launches;
 }
@@ -342,119 +407,70 @@ static int run_layers(small_ctx *ctx, const small_layer *layers, int n_layers, i
     } in_net{ctx};
     ctx->in_net = 1;
     bool after_join = false;
-    // a run of depthwise / 1x1 pairs (sep_chain.cu); without one, a run up to the end of the list (net_resident.cu)
-    int chain = -1, chain_layers = 0, on_chip = -1;
-    const bool apart = tensors_apart(plan, in_blk, out_blk, workspace), runs = apart && runs_allowed(ctx);
-    if (runs) {
-        for (int i = from; i < n_layers && !chain_layers; ++i)
-            if ((chain_layers = sep_chain_layers(ctx, layers, n_layers, i, N)) > 0) chain = i;
-        if (!chain_layers) on_chip = resident_from(ctx, layers, n_layers, from, N);
-        if (on_chip >= 0 && (layers[n_layers - 1].flags & SMALL_MATH_MASK) == SMALL_MATH_FP32 && launches_beat_on_chip(ctx, layers, n_layers, on_chip, N)) on_chip = -1;
-    }
-    // a shortcut and the layer that is added to it, where both are split over warps, as one launch
-    auto joins = [&](int i, Geom &sc, Geom &g) {
-        return runs && i + 1 != chain && i + 1 != on_chip && shortcut_pair(layers, n_layers, i, N, sc, g) &&
-               joined_split(ctx, sc, g, layers[i].flags & SMALL_MATH_MASK, (reinterpret_cast<uintptr_t>(wr(layers[i].dst)) & 31u) == 0);
-    };
-    for (int i = from; i < n_layers; ++i) {
+    const Forms forms(ctx, layers, n_layers, from, N, tensors_apart(plan, in_blk, out_blk, workspace), (reinterpret_cast<uintptr_t>(out_blk) & 31u) == 0);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    Step step;
+    for (int i = from; i < n_layers; i += step.layers) {
         const small_layer &L = layers[i];
-        Geom sc_next, g_next;
         int s = SMALL_OK;
         // every layer may start its set-up while the kernel in front of it drains (see launch_kernel)
         ctx->dependent = !ctx->overlap || after_join ? 0 : i > 0 ? 1 : 2;
         after_join = false;
-        if (i == chain) {
-            s = launch_sep_chain(ctx, layers, n_layers, i, N, rd(L.src), wr(layers[i + chain_layers - 1].dst), static_cast<cudaStream_t>(stream));
-            ctx->dependent = 0;
-            if (s != SMALL_OK) return s;
-            i += chain_layers - 1;
-            continue;
-        }
-        if (i == on_chip) {
-            s = launch_resident(ctx, layers, n_layers, from, N, rd, wr, static_cast<cudaStream_t>(stream));
-            ctx->dependent = 0;
-            return s;
-        }
-        if (runs && chain < 0 && on_chip < 0) {
-            Geom gd, gp;
-            if (split_pair(ctx, layers, n_layers, i, N, gd, gp) > 0.0) {
-                const small_layer &Nx = layers[i + 1];
-                s = launch_split_pair(ctx, rd(L.src), L.w_blk, L.bias, L.flags & SMALL_RELU, Nx.w_blk, Nx.bias, wr(Nx.dst), gd, gp, Nx.flags & SMALL_RELU,
-                                      static_cast<cudaStream_t>(stream));
-                ctx->dependent = 0;
-                if (s != SMALL_OK) return s;
-                ++i;
-                continue;
-            }
-        }
-        {
-            Geom sc, g;
-            if (joins(i, sc, g)) {
-                const small_layer &Nx = layers[i + 1];
-                s = launch_joined(ctx, Shortcut{rd(L.src), L.w_blk, nullptr, nullptr, L.bias, sc}, rd(Nx.src), Nx.w_blk, Nx.bias, wr(L.dst), g, Nx.flags & SMALL_RELU,
-                                  L.flags & SMALL_MATH_MASK, static_cast<cudaStream_t>(stream));
-                ctx->dependent = 0;
-                if (s != SMALL_OK) return s;
-                ++i;
-                continue;
-            }
-        }
-        {
-            int widths[13];
-            if (const int Lc = apart ? fc_chain_len(ctx, layers, n_layers, i, N, widths) : 0) {
+        step_at(ctx, layers, n_layers, i, N, forms, step);
+        const small_layer &Nx = layers[i + step.layers - 1];      // the last one covered
+        switch (step.form) {
+            case SMALL_FORM_PAIR_RUN:
+                s = launch_sep_chain(ctx, layers, n_layers, i, N, rd(L.src), wr(Nx.dst), st);
+                break;
+            case SMALL_FORM_ON_CHIP:
+                s = launch_resident(ctx, layers, n_layers, from, N, rd, wr, st);
+                break;
+            case SMALL_FORM_PAIR_FP32:
+                s = launch_split_pair(ctx, rd(L.src), L.w_blk, L.bias, L.flags & SMALL_RELU, Nx.w_blk, Nx.bias, wr(Nx.dst), step.a, step.b, Nx.flags & SMALL_RELU, st);
+                break;
+            case SMALL_FORM_JOINED:
+                s = launch_joined(ctx, Shortcut{rd(L.src), L.w_blk, nullptr, nullptr, L.bias, step.a}, rd(Nx.src), Nx.w_blk, Nx.bias, wr(L.dst), step.b, Nx.flags & SMALL_RELU,
+                                  L.flags & SMALL_MATH_MASK, st);
+                break;
+            case SMALL_FORM_FC_CHAIN: {
                 const float *w[12], *b[12];
                 int relu[12];
-                for (int j = 0; j < Lc; ++j) { w[j] = layers[i + j].w_blk; b[j] = layers[i + j].bias; relu[j] = (layers[i + j].flags & SMALL_RELU) ? 1 : 0; }
-                float *dst = wr(layers[i + Lc - 1].dst);
-                if ((reinterpret_cast<uintptr_t>(dst) & 31u) == 0) {
-                    s = launch_fc_chain(ctx, rd(L.src), w, b, widths, relu, dst, Lc, N, L.flags & SMALL_MATH_MASK, static_cast<cudaStream_t>(stream));
-                    ctx->dependent = 0;
-                    if (s != SMALL_OK) return s;
-                    i += Lc - 1;
-                    continue;
+                for (int j = 0; j < step.layers; ++j) { w[j] = layers[i + j].w_blk; b[j] = layers[i + j].bias; relu[j] = (layers[i + j].flags & SMALL_RELU) ? 1 : 0; }
+                s = launch_fc_chain(ctx, rd(L.src), w, b, step.widths, relu, wr(Nx.dst), step.layers, N, L.flags & SMALL_MATH_MASK, st);
+                break;
+            }
+            case SMALL_FORM_FUSED_PAIR:
+                if (step.fused == SMALL_OP_DWPW) {
+                    const unsigned fl = ((L.flags & SMALL_RELU) ? SMALL_RELU_MID : 0u) | (Nx.flags & (SMALL_RELU | SMALL_MATH_MASK));
+                    s = small_dwpw_conv2d(ctx, rd(L.src), L.w_blk, L.bias, Nx.w_blk, Nx.bias, wr(Nx.dst), nullptr, N, L.C, Nx.K, L.H, L.W,
+                                          L.stride, L.pad_t, L.pad_b, L.pad_l, L.pad_r, fl, stream);
+                } else if (step.fused == kFusedPoolFc) {
+                    s = small_gap_fc(ctx, rd(L.src), Nx.w_blk, Nx.bias, wr(Nx.dst), nullptr, N, L.C, L.H, L.W, Nx.K,
+                                     Nx.flags & (SMALL_RELU | SMALL_MATH_MASK), stream);
+                } else {
+                    s = small_conv_maxpool2d(ctx, rd(L.src), L.w_blk, L.bias, wr(Nx.dst), nullptr, N, L.C, L.K, L.H, L.W, L.FH, L.FW, L.stride,
+                                             L.pad_t, L.pad_b, L.pad_l, L.pad_r, L.flags, stream);
                 }
+                break;
+            case SMALL_FORM_SIDE_BY_SIDE: {
+                // the second one on the context's side stream, forked from and joined to the caller's stream by events, so that a
+                // short layer hides behind a long one.  It is an ordinary launch, and so is the layer behind the join.
+                cudaStream_t side = static_cast<cudaStream_t>(ctx->side_stream);
+                cudaError_t e = cudaEventRecord(static_cast<cudaEvent_t>(ctx->ev_fork), st);
+                if (e == cudaSuccess) e = cudaStreamWaitEvent(side, static_cast<cudaEvent_t>(ctx->ev_fork), 0);
+                if (e != cudaSuccess) { ctx->last_cuda = (int)e; ctx->dependent = 0; return SMALL_ERR_CUDA; }
+                s = run_one(L, stream);
+                ctx->dependent = 0;
+                if (s == SMALL_OK) s = run_one(Nx, ctx->side_stream);
+                e = cudaEventRecord(static_cast<cudaEvent_t>(ctx->ev_join), side);
+                if (e == cudaSuccess) e = cudaStreamWaitEvent(st, static_cast<cudaEvent_t>(ctx->ev_join), 0);
+                if (s == SMALL_OK && e != cudaSuccess) { ctx->last_cuda = (int)e; s = SMALL_ERR_CUDA; }
+                after_join = true;
+                break;
             }
+            default:
+                s = run_one(L, stream);
         }
-        if (const int fused = i + 1 == on_chip || i + 1 == chain ? 0 : fused_pair(ctx, layers, n_layers, i, N)) {
-            const small_layer &Nx = layers[i + 1];
-            if (fused == SMALL_OP_DWPW) {
-                const unsigned fl = ((L.flags & SMALL_RELU) ? SMALL_RELU_MID : 0u) | (Nx.flags & (SMALL_RELU | SMALL_MATH_MASK));
-                s = small_dwpw_conv2d(ctx, rd(L.src), L.w_blk, L.bias, Nx.w_blk, Nx.bias, wr(Nx.dst), nullptr, N, L.C, Nx.K, L.H, L.W,
-                                      L.stride, L.pad_t, L.pad_b, L.pad_l, L.pad_r, fl, stream);
-            } else if (fused == kFusedPoolFc) {
-                s = small_gap_fc(ctx, rd(L.src), Nx.w_blk, Nx.bias, wr(Nx.dst), nullptr, N, L.C, L.H, L.W, Nx.K,
-                                 Nx.flags & (SMALL_RELU | SMALL_MATH_MASK), stream);
-            } else {
-                s = small_conv_maxpool2d(ctx, rd(L.src), L.w_blk, L.bias, wr(Nx.dst), nullptr, N, L.C, L.K, L.H, L.W, L.FH, L.FW, L.stride,
-                                         L.pad_t, L.pad_b, L.pad_l, L.pad_r, L.flags, stream);
-            }
-            ctx->dependent = 0;
-            if (s != SMALL_OK) return s;
-            ++i;
-            continue;
-        }
-        // Two neighbouring layers that touch no common tensor except as readers (a residual stage's convolution and its
-        // shortcut) run side by side: the second one on the context's side stream, forked from and joined to the caller's
-        // stream by events, so that a short layer hides behind a long one.  Both are ordinary launches, and so is the
-        // layer behind the join.
-        if (apart && ctx->branch_overlap && ctx->side_stream && i + 1 < n_layers && i + 1 != on_chip && i + 1 != chain && independent(L, layers[i + 1]) &&
-            !fused_pair(ctx, layers, n_layers, i + 1, N) && !joins(i + 1, sc_next, g_next)) {
-            cudaStream_t main_st = static_cast<cudaStream_t>(stream), side = static_cast<cudaStream_t>(ctx->side_stream);
-            cudaError_t e = cudaEventRecord(static_cast<cudaEvent_t>(ctx->ev_fork), main_st);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(side, static_cast<cudaEvent_t>(ctx->ev_fork), 0);
-            if (e != cudaSuccess) { ctx->last_cuda = (int)e; ctx->dependent = 0; return SMALL_ERR_CUDA; }
-            s = run_one(L, stream);
-            ctx->dependent = 0;
-            if (s == SMALL_OK) s = run_one(layers[i + 1], ctx->side_stream);
-            e = cudaEventRecord(static_cast<cudaEvent_t>(ctx->ev_join), side);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(main_st, static_cast<cudaEvent_t>(ctx->ev_join), 0);
-            if (s != SMALL_OK) return s;
-            if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SMALL_ERR_CUDA; }
-            ++i;
-            after_join = true;
-            continue;
-        }
-        s = run_one(L, stream);
         ctx->dependent = 0;
         if (s != SMALL_OK) return s;
     }

@@ -261,6 +261,9 @@ int clusters_of(small_ctx *ctx, unsigned math, int lg) {
     return c;
 }
 
+// What comes here: in the tensor-core modes, networks with at most two depthwise / 1x1 pairs in a row (longer runs of pairs are
+// sep_chain.cu's); in FP32, batches of some 30 images (128 channels on 25 x 5) to 100 (64 channels) and more, on one to four blocks per
+// image: smaller ones are faster as launches (launches_beat_on_chip in net.cu).
 // Where the run is faster on chip than layer by layer.  `one_round`: every image has its own thread blocks; with more images
 // than that the layer kernels, which see the whole batch, win.  Measured called directly, us, layer by layer / on chip, on stacks of
 // a 10 x 4 stem and n pairs of a depthwise and a 1x1 layer of C channels on 25 x 5 (the keyword-spotting network: C = 64, n = 4):

@@ -48,7 +48,7 @@ constexpr int kThreads = 256, kMma = 4, kCopy = 5;           // two of the eight
 constexpr int kMaxPairs = 14, kMaxRing = 8;
 constexpr uint32_t kSpin = 1u << 15;                         // polls without back-off on the layer-to-layer critical path
 constexpr int kMaxBlocks = 8;                                // channel blocks of a layer
-// Runs of at least three pairs.  (Shorter ones gain as well; they keep the kernels whose results they had, bit for bit.)
+// Runs of at least three pairs.  (Two were not measured apart; they run as they did before there were runs.)
 constexpr int kMinPairs = 3;
 
 struct PairOp {
@@ -90,7 +90,8 @@ __device__ __forceinline__ float lo_of(uint64_t v) { return __uint_as_float((uin
 __device__ __forceinline__ float hi_of(uint64_t v) { return __uint_as_float((uint32_t)(v >> 32)); }
 
 // The depthwise tiles that are compiled: columns x rows of outputs a thread holds, the stride; `full`: the columns are the whole
-// plane's with pads of one, so that what lies outside is known at compile time.
+// plane's with pads of one, so that what lies outside is known at compile time.  Compiled for planes of five columns; planes of other
+// widths take the tiles of three, and what full tiles of four, six or seven columns would give was not measured.
 struct DwTile { int nc, r, s; bool full; };
 constexpr DwTile kTiles[] = {{5, 2, 1, true}, {3, 2, 1, false}, {3, 2, 2, false}, {3, 1, 2, false}, {3, 4, 1, false}, {5, 4, 1, true}};
 constexpr int kTileCount = sizeof(kTiles) / sizeof(kTiles[0]), kTilesTwo = 4;      // two blocks on an SM: the first four (registers)
@@ -303,14 +304,14 @@ __global__ void __launch_bounds__(256, PER_SM) sep_chain_kernel(const __grid_con
     const float *bias_s = reinterpret_cast<const float *>(base_ptr + a.bias_off);
     float *head_s = reinterpret_cast<float *>(base_ptr + a.head_off);       // sums [4][256], partials [8][32]
     const uint32_t ctrl = base + a.ctrl_off;
-    const uint32_t bar_ring_full = ctrl, bar_ring_empty = ctrl + 8 * kMaxRing, bar_dww = ctrl + 16 * kMaxRing, bar_img = bar_dww + 16, bar_acc = bar_dww + 24;
+    const uint32_t bar_ring_full = ctrl, bar_ring_empty = ctrl + 8 * kMaxRing, bar_dww = ctrl + 16 * kMaxRing, bar_img = bar_dww + 16;
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(base_ptr + a.ctrl_off + 16 * kMaxRing + 64);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(base_ptr + a.ctrl_off + 16 * kMaxRing + 68);
     const int warp = warp_index(), lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxRing; ++s) { mbar_init(bar_ring_full + 8 * s, 1); mbar_init(bar_ring_empty + 8 * s, 1); }
-        mbar_init(bar_dww, 1); mbar_init(bar_dww + 8, 1); mbar_init(bar_img, 1); mbar_init(bar_acc, 1);
+        mbar_init(bar_dww, 1); mbar_init(bar_dww + 8, 1); mbar_init(bar_img, 1);
         *abort_flag = 0;
         mbar_fence_init();
     }
@@ -737,7 +738,7 @@ void plan_run(small_ctx *ctx, const small_layer *layers, int n, int i, int N, Pl
     p.pairs = p.layers = 0;
 }
 
-struct Launch { const float *in; float *out; unsigned wait_iters; Maps maps; };
+struct Launch { const float *in; float *out; Maps maps; };
 struct Entry { std::vector<unsigned char> key; std::unique_ptr<Plan> p; std::vector<Launch> made; };
 typedef std::unordered_multimap<size_t, Entry> State;
 

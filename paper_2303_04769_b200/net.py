@@ -113,10 +113,18 @@ class Net:
         torch.cuda.synchronize()      # the filters are packed, and nothing queued before still uses the workspace's memory (see run_host)
 
     def launches(self):
-        """Kernel launches of one run under this network's fusion setting."""
+        """Kernels of one run under this network's fusion setting: one per layer, fused pair or chain of full reductions."""
         B.small_set_net_fusion(self.ctx, self.fusion)
         try:
             return B.small_net_launches(self.ctx, self.layers, self.N)
+        finally:
+            B.small_set_net_fusion(self.ctx, B.FUSE_DEFAULT)
+
+    def forms(self):
+        """Each layer's form in one run under this network's fusion setting (a name of binding.FORMS), and the kernel launches."""
+        B.small_set_net_fusion(self.ctx, self.fusion)
+        try:
+            return B.small_net_forms(self.ctx, self.layers, self.N)
         finally:
             B.small_set_net_fusion(self.ctx, B.FUSE_DEFAULT)
 

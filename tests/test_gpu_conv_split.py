@@ -32,6 +32,8 @@ CASES = [  # N, C, K, H, W, FH, FW, stride, pad (t, b, l, r)
 def test_few_pixels(case, math):
     N, C, K, H, W, FH, FW, S, pad = case
     m = B.MATH[math]
+    # (one step on one pixel in TF32 is as fast as a whole tile)
+    assert B.small_conv2d_split(ctx(), N, C, K, H, W, FH, FW, S, pad, m) == (not (math == "tf32" and (C, H) == (8, 1)))
     x, w, b = synth.uniform((N, C, H, W), -1, 1, 1, seed=9), synth.uniform((K, C, FH, FW), -1, 1, 2, seed=9), synth.uniform((K,), -1, 1, 3, seed=9)
     ref = oracle.conv2d(x, w, b, S, pad, relu=True)
     OH, OW = ref.shape[2:]
@@ -53,18 +55,25 @@ def test_few_pixels(case, math):
     assert pad_lanes_are_zero(acc, N, K, OH, OW)
 
 
-def test_values_without_a_number_stay_where_they_are():
-    """FP32: an infinite or missing input reaches the pixels whose window holds it and no other."""
+@pytest.mark.parametrize("math", ["fp32", "tf32", "3xtf32"])
+def test_values_without_a_number_stay_where_they_are(math):
+    """An infinite or missing input reaches the pixels whose window holds it and no other, and no pad filter.  (3xTF32: the residual of an
+    infinity is no number.)"""
+    m = B.MATH[math]
+    assert B.small_conv2d_split(ctx(), 1, 40, 33, 9, 9, 3, 3, 1, (1, 1, 1, 1), m) == 1
     x, w = synth.uniform((1, 40, 9, 9), -1, 1, 1, seed=4), abs(synth.uniform((33, 40, 3, 3), -1, 1, 2, seed=4)) + 0.1
     x[0, 3, 0, 0], x[0, 39, 8, 4] = float("inf"), float("nan")
-    wb = torch.empty(B.small_conv_weight_elems(40, 33, 3, 3, B.MATH_FP32), device="cuda")
-    B.small_pack_conv_weights(ctx(), dev(w), wb, 40, 33, 3, 3, B.MATH_FP32)
+    wb = torch.empty(B.small_conv_weight_elems(40, 33, 3, 3, m), device="cuda")
+    B.small_pack_conv_weights(ctx(), dev(w), wb, 40, 33, 3, 3, m)
     out = torch.empty(B.small_packed_elems(1, 33, 9, 9), device="cuda")
-    B.small_conv2d(ctx(), to_blk(x), wb, None, out, 1, 40, 33, 9, 9, 3, 3, 1, (1, 1, 1, 1), B.MATH_FP32)
+    B.small_conv2d(ctx(), to_blk(x), wb, None, out, 1, 40, 33, 9, 9, 3, 3, 1, (1, 1, 1, 1), m)
+    assert pad_lanes_are_zero(out, 1, 33, 9, 9)
     got = torch.from_numpy(from_blk(out, 1, 33, 9, 9))
     want = torch.nn.functional.conv2d(torch.from_numpy(x).double(), torch.from_numpy(w).double(), padding=1)
-    assert torch.equal(got.isinf(), want.isinf()) and torch.equal(got.isnan(), want.isnan())
-    assert got.isinf().sum() == 33 * 4 and got.isnan().sum() == 33 * 6
+    assert torch.equal(got.isfinite(), want.isfinite()) and (~want.isfinite()).sum() == 33 * 10
+    if math != "3xtf32":
+        assert torch.equal(got.isinf(), want.isinf()) and torch.equal(got.isnan(), want.isnan())
+        assert got.isinf().sum() == 33 * 4 and got.isnan().sum() == 33 * 6
 
 
 @pytest.mark.parametrize("math,path", [("3xtf32", "tensor"), ("fp32", "cuda_cores")])
@@ -94,6 +103,7 @@ def test_fp32_pairs_as_one_launch(C, K, H, W, S, relu, batch):
     params, x = configs.make_params(net), configs.make_input(net, batch)
     ref = nets.run_net(net, params, x)["out"]
     gnet = Net(ctx(), net, params, batch=batch)
+    assert gnet.forms() == (["pair_fp32"] * 2, 1)
     got = gnet.run(to_blk(x))
     assert rel_err(from_blk(got, *ref.shape), ref) <= TOL["fp32"]
     assert pad_lanes_are_zero(got, *ref.shape)
@@ -112,6 +122,9 @@ def test_shortcut_as_part_of_the_layer_it_joins(math, C, K, H, W, C2, S, relu, b
     net = dict(name="joined", batch=batch, input=(C2, H2, W2), input_dist=("uniform", -1.0, 1.0), weight_dist="he_normal", layers=layers)
     params, x = configs.make_params(net), configs.make_input(net, batch)
     ref = nets.run_net(net, params, x)["out"]
+    # (33 -> 9: a 1x1 layer of few products computes in FP32 in every mode, its 3x3 does not)
+    forms, launches = Net(ctx(), net, params, batch=batch, math=math).forms()
+    assert (forms, launches) == ((["layer", "joined", "joined"], 2) if math == "fp32" or C2 != 33 else (["side_by_side"] * 2 + ["layer"], 3))
     for overlap in (1, 0):
         B.small_set_layer_overlap(ctx(), overlap)
         try:

@@ -166,6 +166,16 @@ def test_conv_fp32(case):
     assert pad_lanes_are_zero(acc, N, K, OH, OW)
 
 
+@pytest.mark.parametrize("case", [c for c in CONV_CASES if c[1] > 4])
+def test_conv_fp32_on_the_general_kernel(case):
+    """The automatic choice takes most of these to a kernel for few pixels."""
+    with conv_path("general"):
+        N, C, K, H, W, FH, FW, S, pad = case
+        assert B.small_conv2d_path(ctx(), N, C, K, H, W, FH, FW, S, pad, B.MATH_FP32) == 2
+        assert B.small_conv2d_split(ctx(), N, C, K, H, W, FH, FW, S, pad, B.MATH_FP32) == 0
+        test_conv_fp32(case)
+
+
 @pytest.mark.parametrize("N,J,K", [(4, 64, 10), (3, 256, 2), (5, 64, 12), (2, 70, 45), (1, 1, 1), (7, 128, 128)])
 def test_fc(N, J, K):
     x, w, b = rnd((N, J, 1, 1), 13), rnd((K, J), 14), rnd((K,), 15)

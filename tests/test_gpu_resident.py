@@ -23,7 +23,7 @@ def separable(H, W, C, K):
 
 
 def joined():
-    """A residual join and a strided shortcut without depthwise layers (FP32, one image on eight blocks)."""
+    """A residual join and a strided shortcut without depthwise layers."""
     L = [_conv("a", "in", "x", 20, 12, 3, 1, P1, True), _conv("b", "x", "y", 12, 40, 3, 2, P1, True), _conv("s", "x", "z", 12, 40, 1, 2, P0, False),
          _conv("c", "y", "z", 40, 40, 3, 1, P1, True, accumulate=True), _gap("gap", "z", "g", 40), _fc("fc", "g", "out", 40, 5)]
     return dict(name="joined", batch=1, input=(20, 13, 11), input_dist=("uniform", -1.0, 1.0), weight_dist="he_normal", layers=L)
@@ -37,7 +37,10 @@ def test_on_chip_runs_match(net, batch, math):
     x = configs.make_input(net, batch)
     ref = nets.run_net(net, params, x)["out"]
     blk = to_blk(x)
-    got = from_blk(Net(ctx(), net, params, batch=batch, math=math).run(blk), batch, *ref.shape[1:])
+    gnet = Net(ctx(), net, params, batch=batch, math=math)
+    # (FP32 at small batches and networks without depthwise layers run launch by launch)
+    assert (gnet.forms()[1] == 1) == (math != "fp32" and net["name"] == "separable")
+    got = from_blk(gnet.run(blk), batch, *ref.shape[1:])
     apart = from_blk(Net(ctx(), net, params, batch=batch, math=math, fuse_poolfc=False).run(blk), batch, *ref.shape[1:])
     assert rel_err(got, ref) <= TOL[math] and rel_err(apart, ref) <= TOL[math]
     assert B.small_device_status(ctx()) == 0
@@ -56,6 +59,7 @@ def test_result_in_the_slot_of_the_runs_input(batch):
     gnet.layers[0].dst = gnet.layers[1].src = gnet.layers[last].dst = slot
     size = B.small_net_workspace_bytes(gnet.layers, batch)
     workspace = torch.empty(size + 256, dtype=torch.uint8, device="cuda")
+    assert ("on_chip" in B.small_net_forms(ctx(), gnet.layers, batch)[0]) == (batch == 100)
     start = size - (B.small_packed_elems(batch, 64, 25, 5) * 4 + 255) // 256 * 256          # the last slot, as large as the input
     for _ in range(20):
         workspace[start:].fill_(255)
@@ -64,9 +68,11 @@ def test_result_in_the_slot_of_the_runs_input(batch):
         assert rel_err(from_blk(got, batch, *gnet.out_shape), from_blk(want, batch, *gnet.out_shape)) <= TOL["fp32"]
 
 
-def test_on_chip_run_repeats_its_bits_in_a_graph():
-    net = configs.kws_cnn(batch=40)
-    gnet = Net(ctx(), net, configs.make_params(net), math="3xtf32")
+@pytest.mark.parametrize("batch,math,form", [(40, "3xtf32", "pair_run"), (100, "fp32", "on_chip"), (148, "fp32", "on_chip")])
+def test_on_chip_run_repeats_its_bits_in_a_graph(batch, math, form):
+    net = configs.kws_cnn(batch=batch)
+    gnet = Net(ctx(), net, configs.make_params(net), math=math)
+    assert form in gnet.forms()[0]
     blk = to_blk(configs.make_input(net))
     want = gnet.run(blk).clone()
     torch.cuda.synchronize()
@@ -87,17 +93,32 @@ def stack(C, n):
     return dict(name="stack", batch=1, input=(1, 49, 10), input_dist=("normal", 0.0, 1.0), weight_dist="he_normal", layers=L)
 
 
-@pytest.mark.parametrize("C,batch,math,on_chip", [(64, 9, "fp32", True), (64, 148, "3xtf32", True), (64, 60, "tf32", True), (48, 9, "tf32", True),
-                                                  (64, 9, "3xtf32", False), (96, 148, "tf32", False), (128, 9, "3xtf32", False),
-                                                  (96, 9, "fp32", True), (96, 60, "fp32", False), (128, 148, "fp32", False), (160, 9, "fp32", False)])
-def test_which_runs_stay_on_chip(C, batch, math, on_chip):
-    """Either side of the lines between the two forms.  The on-chip kernel adds up in another order, so a result has the bits of
-    the layers launched one by one exactly where those run."""
+@pytest.mark.parametrize("net,batch,math", [
+    (stack(64, 3), 148, "fp32"), (stack(48, 4), 100, "fp32"), (stack(128, 4), 30, "fp32"), (stack(128, 2), 74, "fp32"), (stack(64, 1), 18, "3xtf32"), (stack(64, 2), 30, "3xtf32"),
+    (stack(24, 1), 1, "tf32"), (separable(11, 3, 33, 17), 2, "tf32"), (separable(11, 3, 33, 17), 2, "3xtf32"), (separable(9, 7, 20, 33), 19, "3xtf32")])
+def test_blocks_per_image_in_every_mode(net, batch, math):
+    """One, two, four and eight thread blocks to an image, as far as each mode comes to the on-chip kernel."""
+    params, x = configs.make_params(net), configs.make_input(net, batch)
+    gnet = Net(ctx(), net, params, batch=batch, math=math)
+    assert gnet.forms()[0][-4:] == ["on_chip"] * 4
+    ref = nets.run_net(net, params, x)["out"]
+    assert rel_err(from_blk(gnet.run(to_blk(x)), batch, *ref.shape[1:]), ref) <= TOL[math]
+    assert B.small_device_status(ctx()) == 0
+
+
+@pytest.mark.parametrize("C,batch,math,form", [(64, 9, "fp32", "pair_fp32"), (64, 100, "fp32", "on_chip"), (64, 148, "3xtf32", "on_chip"), (64, 60, "tf32", "on_chip"), (48, 9, "tf32", "on_chip"),
+                                                  (64, 9, "3xtf32", "layer"), (96, 148, "tf32", "layer"), (128, 9, "3xtf32", "layer"),
+                                                  (96, 9, "fp32", "pair_fp32"), (96, 60, "fp32", "layer"), (128, 148, "fp32", "layer"), (160, 9, "fp32", "layer")])
+def test_which_runs_stay_on_chip(C, batch, math, form):
+    """Either side of the lines between the forms.  The on-chip kernel and the pairs of few pixels add up in another order, so a result has
+    the bits of the layers launched one by one exactly where those run."""
     net = stack(C, 2)
     params, x = configs.make_params(net), configs.make_input(net, batch)
     blk = to_blk(x)
-    got = Net(ctx(), net, params, batch=batch, math=math).run(blk)
+    gnet = Net(ctx(), net, params, batch=batch, math=math)
+    assert set(gnet.forms()[0][1:5]) == {form}
+    got = gnet.run(blk)
     apart = Net(ctx(), net, params, batch=batch, math=math, fuse_dwpw=False).run(blk)
-    assert torch.equal(got, apart) == (not on_chip)
+    assert torch.equal(got, apart) == (form == "layer")
     ref = nets.run_net(net, params, x)["out"]
     assert rel_err(from_blk(got, batch, *ref.shape[1:]), ref) <= TOL[math]

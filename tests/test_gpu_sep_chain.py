@@ -50,13 +50,14 @@ def test_run_matches_the_oracle(name, math, batch):
     params, x = configs.make_params(net), configs.make_input(net, batch)
     ref = nets.run_net(net, params, x)["out"]
     gnet = Net(ctx(), net, params, batch=batch, math=math)
+    assert gnet.forms() == (["pair_run"] * len(net["layers"]), 1)
     got = gnet.run(to_blk(x))
     assert rel_err(from_blk(got, batch, *ref.shape[1:]), ref) <= TOL[math]
     assert pad_lanes_are_zero(got, batch, *ref.shape[1:])
     assert B.small_device_status(ctx()) == 0
 
 
-@pytest.mark.parametrize("name,batch", [("columns_5", 149), ("columns_5", 700), ("ragged", 297), ("plane_144", 300), ("two_filter_tiles", 200), ("px_16_edge", 1100)])
+@pytest.mark.parametrize("name,batch", [("columns_5", 149), ("columns_5", 700), ("ragged", 297), ("plane_144", 300), ("two_filter_tiles", 148), ("two_filter_tiles", 200), ("px_16_edge", 1100)])
 @pytest.mark.parametrize("math", ["tf32", "3xtf32"])
 def test_many_images_match_the_layers_one_by_one(name, math, batch):
     """Several images per thread block, two blocks per SM: the stream of filters crosses the images' ends.  Both forms round alike but
@@ -67,6 +68,8 @@ def test_many_images_match_the_layers_one_by_one(name, math, batch):
     params, x = configs.make_params(net), configs.make_input(net, batch)
     blk = to_blk(x)
     gnet, apart = (Net(ctx(), net, params, batch=batch, math=math, **kw) for kw in ({}, dict(fuse_dwpw=False)))
+    # (many filters on few pixels: layer by layer where images come in several rounds)
+    assert (gnet.forms()[1] == 1) == ((name, batch, math) != ("two_filter_tiles", 200, "3xtf32")) and apart.forms()[1] >= len(net["layers"]) - 1
     shape = (batch,) + tuple(gnet.out_shape)
     want = from_blk(apart.run(blk), *shape)
     got = gnet.run(blk)
@@ -107,6 +110,7 @@ def test_values_without_a_number_pass_as_in_the_layers_one_by_one(C, H, W, K, ma
     shape, got = None, []
     for kw in ({}, dict(fuse_dwpw=False)):
         gnet = Net(ctx(), net, params, batch=4, math=math, **kw)
+        assert ("pair_run" in gnet.forms()[0]) == (not kw)
         shape = (4,) + tuple(gnet.out_shape)
         out = gnet.run(to_blk(x))
         assert pad_lanes_are_zero(out, *shape)
@@ -124,5 +128,6 @@ def test_layers_computed_in_fp32_are_no_part_of_a_run(C, K, math):
     net = run_of(C, 8, 8, [(C, 1, SAME, True, True), (K, 1, SAME, True, True), (C, 1, SAME, True, True)])
     assert B.small_conv2d_path(ctx(), batch, C, K, 8, 8, 1, 1, 1, NONE, B.MATH[math]) in (1, 2)
     params, blk = configs.make_params(net), to_blk(configs.make_input(net, batch))
-    run, apart = (Net(ctx(), net, params, batch=batch, math=math, **kw).run(blk).clone() for kw in ({}, dict(fuse_dwpw=False)))
-    assert torch.equal(run, apart)
+    run, apart = (Net(ctx(), net, params, batch=batch, math=math, **kw) for kw in ({}, dict(fuse_dwpw=False)))
+    assert "pair_run" not in run.forms()[0]
+    assert torch.equal(run.run(blk).clone(), apart.run(blk))
