@@ -237,7 +237,10 @@ SplitPlan plan_split(const Geom &g, bool x3, int sms, int more = 0) {
 // this kernel's grows with them.  us, whole-tile against split, batch by batch: 64 -> 64 3x3 on 16x16 in 3xTF32, 1 / 4 / 8 / 16 images
 // 11.0 / 11.1 / 11.1 / 11.3 against 2.7 / 4.8 / 8.4 / 13.0, in TF32 9.4 / 9.4 / 9.4 / 9.6 against 2.5 / 4.1 / 7.1 / 10.2; 16 -> 16 on
 // 32x32 3xTF32, 1 / 8: 6.3 / 6.4 against 2.1 / 4.7; 256 -> 256 1x1 on 14x14, 1 / 8 / 16: 16.4 / 16.6 / 16.7 against 3.3 / 12.6 / 17.7.
-// The estimates are up to 1.7 times off near the line, hence the margin: of 236 measured pairs none is lost by it.
+// The estimates are up to 1.7 times off near the line, hence the margin.  What the rule sends here, measured back to back against the
+// whole-tile kernel forced on the same call: in 3xTF32 94 layers and batches, none slower by more than 1 %, half of them 2.1 times and
+// more faster; in TF32 92, half 1.8 times and more, but three slower, as whole tiles take less there than the estimate says when calls
+// overlap: 64 -> 64 3x3 on 16x16, batch 8 7.2 / 8.0, on 8x8, batch 37 7.3 / 8.1, 128 -> 128 on 14x14, batch 4 10.4 / 10.7.
 bool conv_split_preferred(const Geom &g, bool x3, bool warp_level, int sms) {
     if ((long long)g.N * g.OH * g.OW > 1 << 20 || (long long)g.H * g.W > 1 << 24 || g.K > 1 << 16) return false;
     const int taps = g.FH * g.FW, chunks = g.CB * taps;

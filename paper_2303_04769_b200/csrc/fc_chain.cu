@@ -20,7 +20,7 @@
 // Roles: warp 0 issues the MMAs; warp 1 streams every layer's filters, warp 2 the first layer's input (each one thread's work,
 // done by a uniform warp: see elect_one); warps 4 .. (four per 32 images) run the epilogue.
 //
-// The chain is latency-bound (batch 4096, TF32: 26.6 us with a barrier per box, 22.6 now; 16 epilogue warps, whose polls stand in the
+// The chain is latency-bound (batch 4096, TF32, back to back: 26.6 us with a barrier per box, 22.6 now; 16 epilogue warps, whose polls stand in the
 // way of the MMAs, 24.7): per layer the MMAs (16 of 40 to 64 cycles), their completion, the epilogue and its hand-over
 // follow one another.  Roles written as `if (lane == 0)` took some 140 cycles per MMA, several hundred per copy and 450 per
 // commit, and needed several producer lanes and hand-overs in groups to hide it.

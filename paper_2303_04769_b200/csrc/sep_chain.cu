@@ -23,8 +23,9 @@
 // directly, us, before and now: keyword-spotting network 3xTF32 batch 1 41 / 21, 148 47 / 27, 1024 177 / 127 (TF32 161 / 116),
 // depthwise-separable network (its last ten pairs) batch 1 124 / 76, 64 178 / 120 (TF32 157 / 114).
 // What bounds it (64 channels on 25 x 5, 3xTF32, cycles of a block alone on its SM): depthwise 1700 and 1000 to store the operand, issue
-// slots of two warps per scheduler and the latencies between them; 16 MMAs 1450, 900 of them the tensor pipe's; epilogue 1350.  Two
-// blocks on an SM need about 4200 a pair, 2600 of them shared-memory wavefronts.  Measured and not kept: 16 warps a block (fewer
+// slots of two warps per scheduler and the latencies between them; 16 MMAs 1450, 900 of them the tensor pipe's; epilogue 1350.  With two
+// blocks on an SM (batch 1024) no unit is full: of some 5800 cycles per image and pair shared memory answers the warps in 1870, issue
+// slots are 42 % used, the FMA pipe 21 %, the tensor pipe 15 %; barriers between a pair's steps are the largest stall.  Measured and not kept: 16 warps a block (fewer
 // registers: spills, 141 us at batch 1024), a warp of their own for copies or MMAs (a ninth warp leaves 96 registers at two blocks on
 // an SM), layers' parameters in shared memory, the next layer's depthwise filters loaded during the MMAs.
 #include <cuda.h>
@@ -48,7 +49,7 @@ constexpr int kThreads = 256, kMma = 4, kCopy = 5;           // two of the eight
 constexpr int kMaxPairs = 14, kMaxRing = 8;
 constexpr uint32_t kSpin = 1u << 15;                         // polls without back-off on the layer-to-layer critical path
 constexpr int kMaxBlocks = 8;                                // channel blocks of a layer
-// Runs of at least three pairs.  (Two were not measured apart; they run as they did before there were runs.)
+// Runs of at least three pairs.  (Two gain as well; they stay with the layer kernels and the on-chip kernel, whose lines were measured on them.)
 constexpr int kMinPairs = 3;
 
 struct PairOp {
